@@ -24,7 +24,7 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Regions {
     size_t state, bstate, bar, never, hist, db, rope, norm_w, bias, wlayers, wlm, emb, kcache, vcache, h, qkv_acc, sumsq, part_o,
-        part_ml, cand_val, cand_idx, logits, raw_out, staging, wraw, xstage, prof, succ, occ, dw, dh, dxn, dqkv, dq, datt, dact, dtok, total;
+        part_ml, cand_val, cand_idx, logits, raw_out, staging, wraw, xstage, prof, succ, occ, dw, dlm, dh, dxn, dpart, dq, datt, dact, total;
     size_t layer_stride, staging_bytes, raw_kmax;
 };
 
@@ -65,7 +65,7 @@ Regions carve(const sdv_config* c, bool own_weights = true) {
     r.never = take(256);
     r.hist = take(((size_t)c->max_seq + 64) * 4);
     r.db = take(((size_t)c->max_seq + 64) * 4);
-    r.rope = take((size_t)c->max_seq * (hd / 2) * sizeof(float2));
+    r.rope = take_w((size_t)c->max_seq * (hd / 2) * sizeof(float2));
     r.norm_w = take_w(((size_t)c->n_layers * 2 + 1) * d * 4);
     r.bias = take_w((size_t)c->n_layers * nqkv * 4);
     r.layer_stride = (nqkv * d + d * nq + 2 * f * d + d * f) * 2;
@@ -97,15 +97,21 @@ Regions carve(const sdv_config* c, bool own_weights = true) {
     r.raw_out = take_w((size_t)kMaxRows * (st / 128) * 4);  // N <= staging / (2 bytes * 64 columns)
     r.xstage = take((size_t)kMaxRows * raw_kmax * 4);
     r.prof = take((size_t)(3 + kPhasesPerLayer * c->n_layers) * kMaxGrid * kProfWords * 8);
-    // dense prefill path: row-major weight copies and the activations of one sub-chunk
+    // dense prefill path: row-major weight copies (a tied LM head is the embedding itself) and the activations of one
+    // sub-chunk; the partial sums of a product's K shares and the calibration's per-tile best logits share a region
     r.dw = take_w(r.layer_stride * c->n_layers);
+    r.dlm = c->tied_lm_head ? r.emb : take_w(V * d * 2);
     r.dh = take((size_t)kDenseMaxRows * d * 4);
     r.dxn = take((size_t)kDenseMaxRows * d * 2);
-    r.dqkv = take((size_t)kDenseMaxRows * nqkv * 4);
+    size_t dp = (size_t)(kMaxGrid / 2) * 256 * 256 * 4;                                    // K shares: one tile per pair of SMs at most
+    const size_t one = (size_t)kDenseMaxRows * (nqkv > d ? nqkv : d) * 4;                  // a product without K shares
+    const size_t tops = (size_t)kDenseMaxRows * ((V + 255) / 256) * kDenseTopMax * 8;
+    if (one > dp) dp = one;
+    if (tops > dp) dp = tops;
+    r.dpart = take(dp);
     r.dq = take((size_t)kDenseMaxRows * nq * 2);
     r.datt = take((size_t)kDenseMaxRows * nq * 2);
     r.dact = take((size_t)kDenseMaxRows * f * 2);
-    r.dtok = take((size_t)kDenseMaxRows * 4);
     r.succ = take((size_t)c->max_seq * SDV_CALIB_MAX * 4);  // calibration: sampled successors per context position
     r.occ = take((size_t)c->max_seq * SDV_CALIB_MAX * 4);   // and where each occurs in the context
     r.total = off;
@@ -271,7 +277,7 @@ struct sdv_ctx {
     long long launches;
     bool have_verify_time;
     bool poisoned;
-    std::vector<CUtensorMap>* maps;  // dense path: [0..2] activations (normalised rows, attention output, SwiGLU output), then 4 per layer
+    std::vector<CUtensorMap>* maps;  // dense path, see MapIndex
     bool dense_ok;       // the tensor maps could be built (else every chunk takes the small-row path)
     int calib_b;         // successors sampled per context position during prefill (0: calibration off)
     bool calibrated;     // the calibration tables cover the whole context
@@ -462,57 +468,114 @@ EncodeTiledFn encode_tiled_fn() {
     }
     return fn;
 }
-// bf16 matrix [rows][K] row-major on this GPU; box = 128 rows x 64 columns, 128-byte swizzle, zeros outside.
-bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t K) {
+// bf16 matrix [rows][K] row-major on this GPU; box = box_rows x 64 columns, 128-byte swizzle, zeros outside.
+bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {K, rows};
     const cuuint64_t strides[1] = {K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kDenseBK, (cuuint32_t)kDenseBM};
+    const cuuint32_t box[2] = {(cuuint32_t)kDenseBK, box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+// Tensor maps of a context: activations (normalised rows, attention output, SwiGLU output), the LM head, then per layer
+// q|k|v, o, gate|up and down with boxes of 64 rows (tiles of 128 features) and again with boxes of 128 (256 features).
+enum MapIndex { MAP_XN = 0, MAP_ATT, MAP_ACT, MAP_LM, MAP_LAYERS };
+inline size_t map_at(int layer, int matrix, int bn) { return MAP_LAYERS + 8 * (size_t)layer + 2 * matrix + (bn == 256 ? 1 : 0); }
 
-template <int EPI>
-cudaError_t launch_dense_gemm(sdv_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, float* out_f32, int ld_f32,
-                              const float* bias, __nv_bfloat16* out_bf16, int ld_bf16) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(dense_gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    dim3 grid((N + kDenseBN - 1) / kDenseBN, (M + kDenseBM - 1) / kDenseBM, 1);
-    if (EPI != EPI_SWIGLU) {
-        // few tiles and a long K (the down projection): split K so that about one block per SM runs; every share
-        // keeps at least six stages
-        const int tiles = (int)(grid.x * grid.y), nkb = K / kDenseBK;
-        int sp = ctx->G / tiles;
-        if (sp > nkb / 6) sp = nkb / 6;
-        if (sp < 1) sp = 1;
-        grid.z = (unsigned)sp;
-        if (EPI == EPI_STORE && sp > 1) {
-            cudaError_t e = cudaMemsetAsync(out_f32, 0, (size_t)M * ld_f32 * 4, ctx->stream);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    dense_gemm_kernel<EPI><<<grid, kDenseThreads, kDenseSmemBytes, ctx->stream>>>(a, b, M, N, K, out_f32, ld_f32, bias, out_bf16, ld_bf16,
-                                                                               ctx->P.state + ST_ERR, 2000000000ull);
+// A launch that may overlap the tail of the kernel before it (programmatic dependent launch), in clusters of `cluster`
+// blocks along x when > 0 (0: as the kernel declares).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(sdv_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster, Args... args) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 0 ? 2 : 1;
     ctx->launches++;
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
-// One sub-chunk of `rows` (32..256) context tokens at positions L..L+rows-1 through every layer:
-// fills their K/V rows.  The tokens are hist[L .. L+rows).
-int dense_prefill_rows(sdv_ctx* ctx, int rows, int L) {
+// How a product of M x N outputs is cut: features per tile and K shares.  Model of its time in microseconds: rounds of
+// one tile per pair of SMs, each its K stages (64 columns: 0.26 us with 128 features, 0.40 with 256) and a fixed price, and
+// the partial sums, written here and read by the next kernel (about 4 bytes per us and ns of L2 time each way).
+struct DensePlan {
+    int bn, splits;
+};
+DensePlan plan_dense(const sdv_ctx* ctx, int M, int N, int K, bool may_split) {
+    const int pairs = ctx->G / 2, mt = (M + 255) / 256, nkb = K / kDenseBK;
+    DensePlan best = {256, 1};
+    double best_t = -1.0;
+    for (int bn = 128; bn <= 256; bn *= 2) {
+        const int nt = (N + bn - 1) / bn;
+        for (int sp = 1; sp <= (may_split ? kDenseMaxSplits : 1) && sp <= nkb; ++sp) {
+            if (sp > 1 && mt * nt * sp > pairs) break;
+            const int rounds = (mt * nt * sp + pairs - 1) / pairs;
+            double t = rounds * (((nkb + sp - 1) / sp) * (bn == 256 ? 0.40 : 0.26) + 1.0);
+            if (may_split) t += 2.0 * sp * (double)M * N * 4.0 / 6.0e6;
+            if (best_t < 0 || t < best_t - 1e-9) {
+                best_t = t;
+                best.bn = bn;
+                best.splits = sp;
+            }
+        }
+    }
+    return best;
+}
+
+template <int EPI, int BN>
+cudaError_t launch_dense_tiles(sdv_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, int splits, float* part,
+                               __nv_bfloat16* out_bf16, int ld_bf16, DenseTopOut top) {
+    const int tiles = ((M + 255) / 256) * ((N + BN - 1) / BN) * splits, pairs = ctx->G / 2;
+    return launch_dependent(ctx, dense_gemm_kernel<EPI, BN>, dim3(2 * (tiles < pairs ? tiles : pairs)), dim3(kDenseThreads),
+                            DenseShape<BN>::kSmemBytes, 0, a, b, M, N, K, splits, part, out_bf16, ld_bf16, top, ctx->P.state + ST_ERR,
+                            2000000000ull);
+}
+// Product of the activations behind `a` with one of a layer's matrices into partial sums; *splits receives their number.
+cudaError_t dense_product(sdv_ctx* ctx, MapIndex a, int layer, int matrix, int M, int N, int K, int* splits) {
+    const std::vector<CUtensorMap>& m = *ctx->maps;
+    const DensePlan pl = plan_dense(ctx, M, N, K, true);
+    float* part = (float*)(ctx->ws + ctx->r.dpart);
+    *splits = pl.splits;
+    if (pl.bn == 256)
+        return launch_dense_tiles<EPI_PARTIAL, 256>(ctx, m[a], m[map_at(layer, matrix, 256)], M, N, K, pl.splits, part, nullptr, 0, DenseTopOut());
+    return launch_dense_tiles<EPI_PARTIAL, 128>(ctx, m[a], m[map_at(layer, matrix, 128)], M, N, K, pl.splits, part, nullptr, 0, DenseTopOut());
+}
+
+cudaError_t dense_attributes() {
+    static bool done = false;
+    if (done) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<128>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_SWIGLU, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_TOP, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, dense_attention_smem<128>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, dense_attention_smem<64>());
+    done = e == cudaSuccess;
+    return e;
+}
+
+// One sub-chunk of `rows` (1..kDenseMaxRows) context tokens at positions L..L+rows-1 through every layer:
+// fills their K/V rows.  The tokens are hist[L .. L+rows).  The last row's residual is also left where the LM head of
+// the forward kernel reads row 0; with `succ` the best logits of every row (calibration) go to succ[row][calib_b].
+int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     const sdv_config& c = ctx->cfg;
     const int d = c.d_model, f = c.d_ffn, hd = c.head_dim, nq = c.n_q_heads * hd, nkv = c.n_kv_heads * hd, nqkv = nq + 2 * nkv;
     uint8_t* ws = ctx->ws;
-    cudaStream_t s = ctx->stream;
     float* h = (float*)(ws + ctx->r.dh);
+    float* part = (float*)(ws + ctx->r.dpart);
     __nv_bfloat16* xn = (__nv_bfloat16*)(ws + ctx->r.dxn);
-    float* qkv = (float*)(ws + ctx->r.dqkv);
     __nv_bfloat16* q = (__nv_bfloat16*)(ws + ctx->r.dq);
     __nv_bfloat16* att = (__nv_bfloat16*)(ws + ctx->r.datt);
     __nv_bfloat16* act = (__nv_bfloat16*)(ws + ctx->r.dact);
@@ -520,34 +583,44 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L) {
     const std::vector<CUtensorMap>& maps = *ctx->maps;
     const float* norm_w = ctx->P.norm_w;
     const float* bias = ctx->P.bias;
-    const size_t att_smem = (size_t)(16 * hd * 2 + 4 * 64 * hd * 2 + 128);  // query tile + two K|V blocks
-    static bool att_attr = false;
-    if (!att_attr) {
-        CK(cudaFuncSetAttribute(dense_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 128 * 2 + 4 * 64 * 128 * 2 + 128));
-        CK(cudaFuncSetAttribute(dense_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 64 * 2 + 4 * 64 * 64 * 2 + 128));
-        att_attr = true;
-    }
-    dense_embed_kernel<<<rows, 128, 0, s>>>(hist + L, ctx->P.emb, h, d, c.vocab);
-    ctx->launches++;
+    const int g = ctx->P.g;
+    CK(dense_attributes());
+    // rows of four columns per thread
+    int nt = (d / 4 + 31) / 32 * 32;
+    if (nt > 1024) nt = 1024;
+    // attention: query groups per block so that up to eight warps share a key block; key shares so that the blocks fill the
+    // chip about twice over and keep at least two key blocks each
+    const int QT = 8 / g, qtiles = (rows + QT * 16 - 1) / (QT * 16);
+    unsigned cs = 1;
+    while (cs < 8 && (int)(qtiles * c.n_kv_heads * cs * 2) <= 2 * ctx->G && (int)(cs * 2) * 128 <= L + rows + 127) cs *= 2;
+    int splits = 0;
+    CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, hist + L, ctx->P.emb, c.vocab, h, part, 0, norm_w, xn, d,
+                        c.rms_eps, nullptr));
     for (int l = 0; l < c.n_layers; ++l) {
-        const CUtensorMap* mb = &maps[3 + 4 * l];
         const size_t layer_off = (size_t)l * c.n_kv_heads * c.max_seq * hd;
-        dense_rmsnorm_kernel<<<rows, 256, 0, s>>>(h, norm_w + (size_t)(2 * l) * d, xn, d, c.rms_eps);
-        CK(launch_dense_gemm<EPI_STORE>(ctx, maps[0], mb[0], rows, nqkv, d, qkv, nqkv, bias ? bias + (size_t)l * nqkv : nullptr, nullptr, 0));
-        dense_rope_append_kernel<<<dim3(rows, c.n_q_heads + c.n_kv_heads), hd / 2, 0, s>>>(
-            qkv, nqkv, ctx->P.rope, q, c.n_q_heads, c.n_kv_heads, hd, ctx->P.kcache, ctx->P.vcache, layer_off, c.max_seq, L);
-        const dim3 ag(c.n_q_heads, (rows + 15) / 16);
-        if (hd == 128)
-            dense_attention_kernel<128><<<ag, 128, att_smem, s>>>(q, ctx->P.kcache, ctx->P.vcache, layer_off, c.max_seq, c.n_q_heads,
-                                                                   ctx->P.g, rows, L, ctx->P.scale_log2e, att);
-        else
-            dense_attention_kernel<64><<<ag, 128, att_smem, s>>>(q, ctx->P.kcache, ctx->P.vcache, layer_off, c.max_seq, c.n_q_heads,
-                                                                  ctx->P.g, rows, L, ctx->P.scale_log2e, att);
-        CK(launch_dense_gemm<EPI_RESIDUAL>(ctx, maps[1], mb[1], rows, d, nq, h, d, nullptr, nullptr, 0));
-        dense_rmsnorm_kernel<<<rows, 256, 0, s>>>(h, norm_w + (size_t)(2 * l + 1) * d, xn, d, c.rms_eps);
-        CK(launch_dense_gemm<EPI_SWIGLU>(ctx, maps[0], mb[2], rows, 2 * f, d, nullptr, 0, nullptr, act, f));
-        CK(launch_dense_gemm<EPI_RESIDUAL>(ctx, maps[2], mb[3], rows, d, f, h, d, nullptr, nullptr, 0));
-        ctx->launches += 4;  // norms, rotary + append, attention
+        const bool last = l + 1 == c.n_layers;
+        CK(dense_product(ctx, MAP_XN, l, 0, rows, nqkv, d, &splits));
+        CK(launch_dependent(ctx, dense_qkv_finish_kernel, dim3(rows), dim3(256), 0, 0, part, splits, bias ? bias + (size_t)l * nqkv : nullptr,
+                            ctx->P.rope, q, c.n_q_heads, c.n_kv_heads, hd, ctx->P.kcache, ctx->P.vcache, layer_off, c.max_seq, L));
+        CK(launch_dependent(ctx, hd == 128 ? dense_attention_kernel<128> : dense_attention_kernel<64>, dim3(qtiles * cs, c.n_kv_heads),
+                            dim3(32 * g * QT), hd == 128 ? dense_attention_smem<128>() : dense_attention_smem<64>(), cs, q, ctx->P.kcache,
+                            ctx->P.vcache, layer_off, c.max_seq, c.n_q_heads, g, QT, rows, L, ctx->P.scale_log2e, att));
+        CK(dense_product(ctx, MAP_ATT, l, 1, rows, d, nq, &splits));
+        CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
+                            norm_w + (size_t)(2 * l + 1) * d, xn, d, c.rms_eps, nullptr));
+        CK((launch_dense_tiles<EPI_SWIGLU, 256>(ctx, maps[MAP_XN], maps[map_at(l, 2, 256)], rows, 2 * f, d, 1, nullptr, act, f, DenseTopOut())));
+        CK(dense_product(ctx, MAP_ACT, l, 3, rows, d, f, &splits));
+        // the next layer's first norm, behind the last layer the final norm (norm_w holds them in this order)
+        CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
+                            norm_w + (size_t)(2 * l + 2) * d, xn, d, c.rms_eps, last ? ctx->P.h : nullptr));
+    }
+    if (succ) {
+        DenseTopOut top;
+        const int ntile = (c.vocab + 255) / 256;
+        top.val = part;
+        top.idx = (int*)(part + (size_t)rows * ntile * kDenseTopMax);
+        CK((launch_dense_tiles<EPI_TOP, 256>(ctx, maps[MAP_XN], maps[MAP_LM], rows, c.vocab, d, 1, nullptr, nullptr, 0, top)));
+        CK(launch_dependent(ctx, dense_top_merge_kernel, dim3(rows), dim3(256), 0, 0, top, ntile, ctx->calib_b, succ));
     }
     CK(cudaGetLastError());
     return SDV_OK;
@@ -648,7 +721,7 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
         P.norm_w = (const float*)(ws + ctx->r.norm_w);
         P.bias = cfg->qkv_bias ? (const float*)(ws + ctx->r.bias) : nullptr;
     }
-    P.rope = (const float2*)(ws + ctx->r.rope);
+    P.rope = leader ? leader->P.rope : (const float2*)(ws + ctx->r.rope);
     P.kcache = (__nv_bfloat16*)(ws + ctx->r.kcache);
     P.vcache = (__nv_bfloat16*)(ws + ctx->r.vcache);
     P.h = (float*)(ws + ctx->r.h);
@@ -674,8 +747,8 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
         if (!apply_plan(probe, rows_max, false, &smem_bytes)) return fail(SDV_EINVAL);
     }
 
-    // rotary table in double, rounded once to fp32
-    {
+    // rotary table in double, rounded once to fp32 (a follower reads its leader's)
+    if (!leader) {
         const size_t n = (size_t)cfg->max_seq * (hd / 2);
         std::vector<float2> tab(n);
         for (int i = 0; i < hd / 2; ++i) {
@@ -704,21 +777,23 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return fail(SDV_ECUDA);
     // dense prefill path: tensor maps over its activation buffers and its weight copies
-    ctx->maps = new (std::nothrow) std::vector<CUtensorMap>(3 + 4 * (size_t)cfg->n_layers);
-    ctx->dense_ok = ctx->maps != nullptr;
+    ctx->maps = new (std::nothrow) std::vector<CUtensorMap>(MAP_LAYERS + 8 * (size_t)cfg->n_layers);
+    ctx->dense_ok = ctx->maps != nullptr && d <= 16384;  // four turns of 1024 threads x 4 columns in the row-wise kernels
+    if (ctx->dense_ok && leader) {  // the weight copies of the dense path are the leader's as well
+        ctx->dense_ok = leader->dense_ok;
+        if (ctx->dense_ok) *ctx->maps = *leader->maps;
+    }
     if (ctx->dense_ok) {
         std::vector<CUtensorMap>& m = *ctx->maps;
-        ctx->dense_ok = make_map(&m[0], ws + ctx->r.dxn, kDenseMaxRows, d) && make_map(&m[1], ws + ctx->r.datt, kDenseMaxRows, nq) &&
-                        make_map(&m[2], ws + ctx->r.dact, kDenseMaxRows, f);
-        if (leader) {  // the weight copies of the dense path are the leader's as well
-            ctx->dense_ok = ctx->dense_ok && leader->dense_ok;
-            for (size_t i = 3; i < m.size() && ctx->dense_ok; ++i) m[i] = (*leader->maps)[i];
-        }
+        ctx->dense_ok = make_map(&m[MAP_XN], ws + ctx->r.dxn, kDenseMaxRows, d, 128) && make_map(&m[MAP_ATT], ws + ctx->r.datt, kDenseMaxRows, nq, 128) &&
+                        make_map(&m[MAP_ACT], ws + ctx->r.dact, kDenseMaxRows, f, 128);
+        if (!leader) ctx->dense_ok = ctx->dense_ok && make_map(&m[MAP_LM], ws + ctx->r.dlm, cfg->vocab, d, 128);
         for (int l = 0; l < cfg->n_layers && ctx->dense_ok && !leader; ++l) {
             uint8_t* lb = ws + ctx->r.dw + (size_t)l * ctx->r.layer_stride;
             const size_t o1 = (size_t)nqkv * d * 2, o2 = o1 + (size_t)d * nq * 2, o3 = o2 + (size_t)2 * f * d * 2;
-            ctx->dense_ok = make_map(&m[3 + 4 * l], lb, nqkv, d) && make_map(&m[4 + 4 * l], lb + o1, d, nq) &&
-                            make_map(&m[5 + 4 * l], lb + o2, 2 * (uint64_t)f, d) && make_map(&m[6 + 4 * l], lb + o3, d, f);
+            for (int bn = 128; bn <= 256 && ctx->dense_ok; bn *= 2)
+                ctx->dense_ok = make_map(&m[map_at(l, 0, bn)], lb, nqkv, d, bn / 2) && make_map(&m[map_at(l, 1, bn)], lb + o1, d, nq, bn / 2) &&
+                                make_map(&m[map_at(l, 2, bn)], lb + o2, 2 * (uint64_t)f, d, bn / 2) && make_map(&m[map_at(l, 3, bn)], lb + o3, d, f, bn / 2);
         }
     }
     ctx->logits_src = P.logits;
@@ -824,6 +899,7 @@ int sdv_load_weights(sdv_ctx* ctx, const sdv_weights* w) {
     }
     CK(cudaMemcpyAsync(norm_w + (size_t)c.n_layers * 2 * d, w->final_norm, d * 4, cudaMemcpyDefault, s));
     CK(cudaMemcpyAsync(ws + ctx->r.emb, w->emb, V * d * 2, cudaMemcpyDefault, s));
+    if (!c.tied_lm_head) CK(cudaMemcpyAsync(ws + ctx->r.dlm, w->lm_head, V * d * 2, cudaMemcpyDefault, s));
     // LM head: packed from row blocks that fit the staging area
     {
         const uint16_t* src = c.tied_lm_head ? w->emb : w->lm_head;
@@ -851,6 +927,40 @@ int sdv_set_parity_mode(sdv_ctx* ctx, int on) {
     return SDV_OK;
 }
 
+}  // extern "C"
+
+namespace {
+constexpr int kDenseMinRows = 16;  // fewer rows take the small-row kernel
+// End of a prefill call: the context covers everything prefilled so far; behind the request's last token (whose
+// candidates are those of `row`) the greedy token becomes the pending one and the calibration looks its anchors up.
+int finish_prefill(sdv_ctx* ctx, bool is_last, int row) {
+    int* hist = (int*)(ctx->ws + ctx->r.hist);
+    ctx->n_ctx = ctx->hist_len;
+    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 0, hist);
+    ctx->launches++;
+    CK(cudaGetLastError());
+    if (!is_last) return SDV_OK;
+    // greedy token of the last context row: appended to the history as the pending token T
+    prefill_final_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, hist, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, row);
+    ctx->launches++;
+    CK(cudaGetLastError());
+    ctx->hist_len += 1;
+    ctx->prefill_done = true;
+    if (ctx->calib_b > 0) {
+        // "Search": where each sampled successor occurs in the request
+        const int total = ctx->n_ctx * ctx->calib_b;
+        anchor_search_kernel<<<(total + 255) / 256, 256, 0, ctx->stream>>>(hist, ctx->n_ctx, ctx->calib_b, (const int*)(ctx->ws + ctx->r.succ),
+                                                                           (int*)(ctx->ws + ctx->r.occ));
+        ctx->launches++;
+        CK(cudaGetLastError());
+        ctx->calibrated = true;
+    }
+    return SDV_OK;
+}
+}  // namespace
+
+extern "C" {
+
 int sdv_prefill_chunk(sdv_ctx* ctx, const int32_t* host_tokens, int n, int is_last) {
     if (!ctx || !host_tokens || n < 1) return SDV_EINVAL;
     if (ctx->poisoned) return SDV_ETIMEOUT;
@@ -861,7 +971,7 @@ int sdv_prefill_chunk(sdv_ctx* ctx, const int32_t* host_tokens, int n, int is_la
         if (host_tokens[i] < 0 || host_tokens[i] >= c.vocab) return SDV_EINVAL;
     int* hist = (int*)(ctx->ws + ctx->r.hist);
     CK(cudaMemcpyAsync(hist + ctx->hist_len, host_tokens, (size_t)n * 4, cudaMemcpyDefault, ctx->stream));
-    // rows per launch
+    // rows per launch of the small-row kernel
     int tile = 24;
     {
         // wide models: fewer rows per launch so that the token operand leaves room for the weight ring
@@ -872,22 +982,24 @@ int sdv_prefill_chunk(sdv_ctx* ctx, const int32_t* host_tokens, int n, int is_la
     const int n_ph = 1 + kPhasesPerLayer * c.n_layers;
     int done = 0;
     while (done < n) {
-        // sub-chunks of 32..256 rows go through the dense path (tokens on the tensor cores' M side, every weight
-        // streamed once); the last token of the request (its logits give the first generated token), short
-        // remainders and calibrated prefill (logits of every row) take the small-row kernel
-        const int dense_rows_avail = n - done - (is_last ? 1 : 0);
-        if (ctx->dense_ok && ctx->calib_b == 0 && dense_rows_avail >= 32) {
-            const int rows = dense_rows_avail < kDenseMaxRows ? dense_rows_avail : kDenseMaxRows;
-            int rc = dense_prefill_rows(ctx, rows, ctx->kv_len);
+        // sub-chunks of up to kDenseMaxRows rows, evenly cut, go through the dense path (tokens on the tensor cores' M
+        // side, every weight streamed once); a handful of rows takes the small-row kernel
+        const int left = n - done;
+        if (ctx->dense_ok && left >= kDenseMinRows) {
+            const int parts = (left + kDenseMaxRows - 1) / kDenseMaxRows, rows = (left + parts - 1) / parts;
+            int rc = dense_prefill_rows(ctx, rows, ctx->kv_len, ctx->calib_b > 0 ? (int*)(ctx->ws + ctx->r.succ) + (size_t)ctx->kv_len * ctx->calib_b : nullptr);
             if (rc) return rc;
             ctx->kv_len += rows;
             ctx->hist_len += rows;
             done += rows;
-            if (done == n) {   // the chunk ended here (never the last one: its final token takes the path below)
-                ctx->n_ctx = ctx->hist_len;
-                set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 0, hist);
-                ctx->launches++;
-                CK(cudaGetLastError());
+            if (done == n) {
+                if (is_last) {
+                    // the request's last token gives the first generated one: the LM head over its row alone
+                    rc = launch_forward(ctx, 1, ctx->kv_len, 1, n_ph, n_ph + 1, false);
+                    if (rc) return rc;
+                }
+                rc = finish_prefill(ctx, is_last != 0, 0);
+                if (rc) return rc;
             }
             continue;
         }
@@ -907,29 +1019,8 @@ int sdv_prefill_chunk(sdv_ctx* ctx, const int32_t* host_tokens, int n, int is_la
         ctx->hist_len += rows;
         done += rows;
         if (done == n) {
-            // the context now covers everything prefilled so far
-            ctx->n_ctx = ctx->hist_len;
-            set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 0, hist);
-            ctx->launches++;
-            CK(cudaGetLastError());
-            if (last_tile) {
-                // greedy token of the last context row: appended to the history as the pending token T
-                prefill_final_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, hist, ctx->P.cand_val, ctx->P.cand_idx,
-                                                              ctx->G, rows - 1);
-                ctx->launches++;
-                CK(cudaGetLastError());
-                ctx->hist_len += 1;
-                ctx->prefill_done = true;
-                if (ctx->calib_b > 0) {
-                    // "Search": where each sampled successor occurs in the request
-                    const int total = ctx->n_ctx * ctx->calib_b;
-                    anchor_search_kernel<<<(total + 255) / 256, 256, 0, ctx->stream>>>(
-                        hist, ctx->n_ctx, ctx->calib_b, (const int*)(ctx->ws + ctx->r.succ), (int*)(ctx->ws + ctx->r.occ));
-                    ctx->launches++;
-                    CK(cudaGetLastError());
-                    ctx->calibrated = true;
-                }
-            }
+            rc = finish_prefill(ctx, last_tile, rows - 1);
+            if (rc) return rc;
         }
     }
     return read_state(ctx);
