@@ -47,6 +47,17 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
     return d;
 }
 
+// The same for an operand whose rows (N) are contiguous: 8 K rows of 64 contiguous elements (128 bytes) form 1024-byte groups, K
+// groups follow each other, slabs of 64 N elements lie `slab` bytes apart.
+__device__ __forceinline__ uint64_t umma_desc_sw128_mn(uint32_t saddr, uint32_t slab) {
+    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
+    d |= (uint64_t)((slab >> 4) & 0x3fffu) << 16;
+    d |= (uint64_t)(1024u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
 struct DenseTopOut {   // EPI_TOP: [row][vocabulary tile][kDenseTopMax] best logits of the tile and their ids, best first
     float* val;
     int* idx;
@@ -390,217 +401,284 @@ __global__ void __launch_bounds__(256) dense_qkv_finish_kernel(const float* part
 }
 
 // Causal attention of a sub-chunk's queries (rows r = 0..M-1 at positions L + r) over cache rows 0 .. L + r of their
-// KV head.  A block holds the queries of all g heads that share a KV head: warp w takes the 16 queries of 16-row
-// group w / g (of QT per block) and head w % g, so that a 64-key block fetched into shared memory (two cp.async
-// buffers) serves g * QT warps.  The keys are cut into contiguous shares over the blocks of a cluster; every warp
-// keeps scores, online softmax (log2 domain) and P V in registers (mma.sync m16n8k16), and the cluster's blocks
-// merge their un-normalised outputs through distributed shared memory.  Output bf16 [M][n_q * hd].
-// Bound by the mma.sync rate (a chunk's share of work per SM is 128 instructions per warp and 64 keys) and, over short
-// contexts, by the chain load -> scores -> softmax -> merge.
+// KV head.  A block's 128 tile rows are the queries of all g heads that share a KV head: tile row t = query q0 + t / g, head
+// t % g.  The keys are cut into contiguous shares over the blocks of a cluster, a share into blocks of 128 keys (tensor-map
+// copies into a ring).  Even and odd key blocks are two independent streams, each with its own scores S, output O
+// and running maximum in tensor memory and a warpgroup of its own (one tile row per thread): while one warpgroup
+// turns its scores into probabilities (written back over S as bf16, the A operand of P V), the tensor core works for the
+// other.  O is rescaled only when the maximum grew by more than 2^8 (the probabilities then stay below 2^8, the sums
+// are fp32).  The streams of all blocks of the cluster merge through distributed shared memory.  Output bf16 [M][n_q * hd].
+// Bound by the exponentials (16 per cycle and SM) and, over short contexts, by the chain load -> S -> softmax -> P V ->
+// merge.  mma.sync tiles, which this replaces, issue m16n8k16 every 16 cycles per scheduler on this part: 35 us a launch at the
+// 1.5B shape, mean over the eight 256-token chunks of a 2048-token request.
 template <int HD>
-__global__ void __launch_bounds__(256) dense_attention_kernel(const __nv_bfloat16* q, const __nv_bfloat16* kcache,
-                                                              const __nv_bfloat16* vcache, size_t layer_off, int max_seq, int n_q,
-                                                              int g, int QT, int M, int L, float scale_log2e, __nv_bfloat16* out) {
-    constexpr int KSTEPS = HD / 16, UNITS = HD / 8, NT_O = HD / 8, KB = 64;
-    constexpr int KVBYTES = KB * HD * 2;
+struct DenseAttShape {
+    static constexpr int kAtoms = HD / 64;                       // 64-column swizzled slabs of a row
+    static constexpr int kTileBytes = 128 * HD * 2;              // queries, or the keys or values of a block
+    static constexpr int kStages = 3;
+    static constexpr int kLdo = HD + 4;                          // row stride (floats) of the exchange area
+    static constexpr int kExBytes = 128 * kLdo * 4;              // one stream's outputs
+    static constexpr int kRing = kStages * 2 * kTileBytes;
+    static constexpr int kSmemBytes = kTileBytes + kRing + 256 + 1024;
+    static_assert(2 * kExBytes <= kRing, "the exchange area reuses the ring");
+};
+constexpr int kDenseAttThreads = 320;   // warps 0..3 and 4..7: the two streams; 8: copies; 9: tensor-core issue
+
+template <int HD>
+__global__ void __launch_bounds__(kDenseAttThreads, 1)
+dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const __nv_bfloat16* q,
+                       int cache_row0, int max_seq, int n_q, int g, int QR, int M, int L, float scale_log2e, __nv_bfloat16* out,
+                       int* err, unsigned long long wait_limit_ns) {
+    using S = DenseAttShape<HD>;
+    constexpr int KSTEPS = HD / 16, UNITS = HD / 8;
     extern __shared__ uint8_t att_smem_raw[];
-    uint8_t* KVs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem_raw) + 127) & ~(uintptr_t)127);   // [2 buffers][K | V]
-    const int nthr = blockDim.x, nwarps = nthr >> 5;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-    const int CS = (int)cluster_size();
-    const int rank = (int)cluster_rank();
-    const int kvh = blockIdx.y, q0 = ((int)blockIdx.x / CS) * QT * 16;   // first query row of the block
-    const int head = kvh * g + warp % g, r0 = q0 + (warp / g) * 16;      // this warp's head and first query row
-    const size_t cache0 = layer_off + (size_t)kvh * max_seq * HD;
-    const int nkeys = L + min(M, q0 + QT * 16);         // keys any row of this block may see
-    const int nblk_all = (nkeys + KB - 1) / KB;
-    const int b0 = even_start(nblk_all, CS, rank), nblk = even_count(nblk_all, CS, rank);
-    auto load_block = [&](int blk) {
-        if (blk < nblk) {
-            uint8_t* Ks = KVs + (blk & 1) * 2 * KVBYTES;
-            uint8_t* Vs = Ks + KVBYTES;
-            for (int u = tid; u < KB * UNITS; u += nthr) {
-                const int key = u / UNITS, q16 = u % UNITS, kk = (b0 + blk) * KB + key;
-                const bool valid = kk < nkeys;
-                const size_t off = cache0 + (size_t)(valid ? kk : 0) * HD + q16 * 8;
-                const uint32_t so = (q16 >> 3) * (KB * 128) + swz_unit(key, q16 & 7);
-                cp_async_16_zfill(Ks + so, kcache + off, valid);
-                cp_async_16_zfill(Vs + so, vcache + off, valid);
-            }
-        }
-        cp_async_commit();
+    uint8_t* Qs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* ring = Qs + S::kTileBytes;                                  // [stage][K | V]
+    float2* ex_ml = reinterpret_cast<float2*>(Qs);   // once the products are done: [stream][tile row] (maximum in log2 units, sum)
+    struct Ctl {
+        uint64_t kfull[S::kStages], vfull[S::kStages], empty[S::kStages], s_full[2], p_ready[2], o_full;
+        uint32_t tmem_base;
+        int abort_flag;
     };
+    Ctl* ctl = reinterpret_cast<Ctl*>(ring + S::kRing);
+    static_assert(sizeof(Ctl) <= 256, "control block");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int CS = (int)cluster_size(), rank = (int)cluster_rank();
+    const int kvh = blockIdx.y, q0 = ((int)blockIdx.x / CS) * QR;       // first query of the block
+    const int nkeys = L + min(M, q0 + QR);                              // keys any row of this block may see
+    const int nblk_all = (nkeys + 127) / 128;
+    const int b0 = even_start(nblk_all, CS, rank), nblk = even_count(nblk_all, CS, rank);
+    if (tid == 0) {
+        for (int s = 0; s < S::kStages; ++s) {
+            mbar_init(&ctl->kfull[s], 1);
+            mbar_init(&ctl->vfull[s], 1);
+            mbar_init(&ctl->empty[s], 1);
+        }
+        for (int w = 0; w < 2; ++w) {
+            mbar_init(&ctl->s_full[w], 1);
+            mbar_init(&ctl->p_ready[w], 4);
+        }
+        mbar_init(&ctl->o_full, 1);
+        ctl->abort_flag = 0;
+        mbar_fence_init();
+    }
+    if (warp == 9) tmem_alloc(&ctl->tmem_base, 512);   // S0 | S1 | O0 | O1, 128 columns each
     grid_dep_launch();
     grid_dep_wait();
-    load_block(0);
-    load_block(1);
-    const int gq = lane >> 2, q2 = (lane & 3) * 2;
-    // query fragments stay in registers: rows gq and gq + 8 of the warp's 16, columns 16 ks + q2 (+ 8)
-    uint32_t qf[KSTEPS][4];
-    {
-        const int rl = min(r0 + gq, M - 1), rh = min(r0 + gq + 8, M - 1);
-        const uint32_t* pl = reinterpret_cast<const uint32_t*>(q + (size_t)rl * (n_q * HD) + head * HD + q2);
-        const uint32_t* ph = reinterpret_cast<const uint32_t*>(q + (size_t)rh * (n_q * HD) + head * HD + q2);
-#pragma unroll
-        for (int ks = 0; ks < KSTEPS; ++ks) {
-            qf[ks][0] = __ldcg(pl + ks * 8);
-            qf[ks][1] = __ldcg(ph + ks * 8);
-            qf[ks][2] = __ldcg(pl + ks * 8 + 4);
-            qf[ks][3] = __ldcg(ph + ks * 8 + 4);
-        }
+    // query tile, in the layout the copies below have: slabs of 64 columns, 128-byte swizzle
+    for (int u = tid; u < 128 * UNITS; u += kDenseAttThreads) {
+        const int t = u / UNITS, c16 = u % UNITS, qi = q0 + t / g;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (t < QR * g && qi < M) v = __ldcg(reinterpret_cast<const uint4*>(q + (size_t)qi * (n_q * HD) + (kvh * g + t % g) * HD + c16 * 8));
+        *reinterpret_cast<uint4*>(Qs + (c16 >> 3) * 16384 + swz_unit(t, c16 & 7)) = v;
     }
-    float o[NT_O][4];
-#pragma unroll
-    for (int n = 0; n < NT_O; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
-    float m_lo = -CUDART_INF_F, m_hi = -CUDART_INF_F, l_lo = 0.f, l_hi = 0.f;
-    const int lim_lo = L + r0 + gq, lim_hi = lim_lo + 8;   // last key each row sees
-    for (int blk = 0; blk < nblk; ++blk) {
-        cp_async_wait<1>();
-        __syncthreads();
-        const uint32_t kb = smem_u32(KVs + (blk & 1) * 2 * KVBYTES), vb = kb + KVBYTES;
-        const int key0 = (b0 + blk) * KB;
-        if (key0 <= L + r0 + 15) {   // some key of this block is visible to some row of the warp
-            float sc[KB / 8][4];
-#pragma unroll
-            for (int n = 0; n < KB / 8; ++n) sc[n][0] = sc[n][1] = sc[n][2] = sc[n][3] = 0.f;
-#pragma unroll
-            for (int ks = 0; ks < KSTEPS; ++ks) {
-#pragma unroll
-                for (int c = 0; c < KB / 16; ++c) {
-                    uint32_t f0, f1, f2, f3;
-                    const int krow = c * 16 + (lane & 7) + ((lane >> 4) << 3);
-                    ldsm_x4(kb + (ks >> 2) * (KB * 128) + swz_unit(krow, (ks & 3) * 2 + ((lane >> 3) & 1)), f0, f1, f2, f3);
-                    mma_bf16_16816(sc[2 * c], qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3], f0, f1);
-                    mma_bf16_16816(sc[2 * c + 1], qf[ks][0], qf[ks][1], qf[ks][2], qf[ks][3], f2, f3);
-                }
-            }
-            float mx_lo = -CUDART_INF_F, mx_hi = -CUDART_INF_F;
-            const bool whole = key0 + KB - 1 <= L + r0;   // every key is visible to every row
-#pragma unroll
-            for (int n = 0; n < KB / 8; ++n)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int key = key0 + n * 8 + q2 + (e & 1);
-                    const bool ok = whole || key <= (e >= 2 ? lim_hi : lim_lo);
-                    const float v = ok ? sc[n][e] * scale_log2e : -CUDART_INF_F;
-                    sc[n][e] = v;
-                    if (e >= 2) mx_hi = fmaxf(mx_hi, v); else mx_lo = fmaxf(mx_lo, v);
-                }
-            mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-            mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-            mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-            mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-            const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
-            const float use_lo = (mn_lo == -CUDART_INF_F) ? 0.f : mn_lo, use_hi = (mn_hi == -CUDART_INF_F) ? 0.f : mn_hi;
-            const float c_lo = exp2f(m_lo - use_lo), c_hi = exp2f(m_hi - use_hi);
-            m_lo = mn_lo;
-            m_hi = mn_hi;
-            float s_lo = 0.f, s_hi = 0.f;
-            uint32_t pf[KB / 8][2];   // probabilities, packed: the A operand of the next product
-#pragma unroll
-            for (int n = 0; n < KB / 8; ++n) {
-                const float p0 = exp2f(sc[n][0] - use_lo), p1 = exp2f(sc[n][1] - use_lo);
-                const float p2 = exp2f(sc[n][2] - use_hi), p3 = exp2f(sc[n][3] - use_hi);
-                s_lo += p0 + p1;
-                s_hi += p2 + p3;
-                pf[n][0] = pack_bf16(p0, p1);
-                pf[n][1] = pack_bf16(p2, p3);
-            }
-            l_lo = l_lo * c_lo + s_lo;
-            l_hi = l_hi * c_hi + s_hi;
-#pragma unroll
-            for (int n = 0; n < NT_O; ++n) { o[n][0] *= c_lo; o[n][1] *= c_lo; o[n][2] *= c_hi; o[n][3] *= c_hi; }
-#pragma unroll
-            for (int c = 0; c < KB / 16; ++c) {
-#pragma unroll
-                for (int cg = 0; cg < NT_O / 2; ++cg) {
-                    uint32_t f0, f1, f2, f3;
-                    const int key = c * 16 + (lane & 7) + (((lane >> 3) & 1) << 3);
-                    const int cu = cg * 2 + (lane >> 4);
-                    ldsm_x4_trans(vb + (cu >> 3) * (KB * 128) + swz_unit(key, cu & 7), f0, f1, f2, f3);
-                    mma_bf16_16816(o[2 * cg], pf[2 * c][0], pf[2 * c][1], pf[2 * c + 1][0], pf[2 * c + 1][1], f0, f1);
-                    mma_bf16_16816(o[2 * cg + 1], pf[2 * c][0], pf[2 * c][1], pf[2 * c + 1][0], pf[2 * c + 1][1], f2, f3);
-                }
-            }
-        }
-        __syncthreads();
-        load_block(blk + 2);
-    }
-    cp_async_wait<0>();
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
-    if (CS == 1) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int r = r0 + gq + half * 8;
-            if (r >= M) continue;
-            const float inv = 1.f / (half ? l_hi : l_lo);
-            __nv_bfloat16* po = out + (size_t)r * (n_q * HD) + head * HD + q2;
-#pragma unroll
-            for (int n = 0; n < NT_O; ++n)
-                *reinterpret_cast<uint32_t*>(po + n * 8) = pack_bf16(o[n][half * 2] * inv, o[n][half * 2 + 1] * inv);
-        }
-        return;
-    }
-    // the key shares meet: every block leaves its rows' outputs and statistics in its own shared memory (the K/V
-    // buffers are free now) and then merges its share of the rows from all blocks of the cluster
-    const int R = nwarps * 16;
-    constexpr int LDO = HD + 4;
-    float* ex_o = reinterpret_cast<float*>(KVs);            // [R][LDO]
-    float2* ex_ml = reinterpret_cast<float2*>(ex_o + 128 * LDO);   // [R] (at most 128 rows)
+    fence_proxy_async_smem();
+    tc_fence_before();
     __syncthreads();
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int lr = warp * 16 + gq + half * 8;
-#pragma unroll
-        for (int n = 0; n < NT_O; ++n)
-            *reinterpret_cast<float2*>(ex_o + lr * LDO + n * 8 + q2) = make_float2(o[n][half * 2], o[n][half * 2 + 1]);
-        if ((lane & 3) == 0) ex_ml[lr] = make_float2(half ? m_hi : m_lo, half ? l_hi : l_lo);
-    }
-    cluster_sync();
-    {
-        const uint32_t base_o = smem_u32(ex_o), base_ml = smem_u32(ex_ml);
-        constexpr int C8 = HD / 8;
-        const int rows_per = (R + CS - 1) / CS, rbeg = rank * rows_per, rend = min(R, rbeg + rows_per);
-        for (int it = tid; it < (rend - rbeg) * C8; it += nthr) {
-            const int lr = rbeg + it / C8, c = (it % C8) * 8;
-            const int w = lr >> 4, r = q0 + (w / g) * 16 + (lr & 15);
-            float2 ml[8];
-            float mmax = -CUDART_INF_F;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (k < CS) {
-                    ml[k] = ld_cluster_f2(map_shared_rank(base_ml + lr * 8, k));
-                    mmax = fmaxf(mmax, ml[k].x);
+    tc_fence_after();
+    const uint32_t tmem = ctl->tmem_base;
+
+    if (warp == 8) {
+        if (elect_one()) {
+            uint32_t s = 0, par = 0;
+            int issued = 0;
+            const int y0 = cache_row0 + kvh * max_seq + b0 * 128;
+            for (; issued < nblk; ++issued) {
+                if (!mbar_wait_bounded(&ctl->empty[s], par ^ 1u, &ctl->abort_flag, wait_limit_ns)) break;
+                uint8_t* ks = ring + s * 2 * S::kTileBytes;
+                const int y = y0 + issued * 128;
+                mbar_arrive_expect_tx(&ctl->kfull[s], S::kTileBytes);
+                for (int a = 0; a < S::kAtoms; ++a) tma_load_2d(ks + a * 16384, &map_k, a * 64, y, &ctl->kfull[s]);
+                mbar_arrive_expect_tx(&ctl->vfull[s], S::kTileBytes);
+                for (int a = 0; a < S::kAtoms; ++a) tma_load_2d(ks + S::kTileBytes + a * 16384, &map_v, a * 64, y, &ctl->vfull[s]);
+                if (++s == S::kStages) { s = 0; par ^= 1u; }
+            }
+            if (issued < nblk)   // abandoned: wait (bounded) for the copies still in flight
+                for (int back = 0; back < S::kStages && back < issued; ++back) {
+                    if (s == 0) { s = S::kStages; par ^= 1u; }
+                    --s;
+                    const uint64_t t0 = global_timer_ns();
+                    while (!(mbar_try_wait(&ctl->kfull[s], par) && mbar_try_wait(&ctl->vfull[s], par)) && global_timer_ns() - t0 < wait_limit_ns) {}
                 }
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+        }
+        __syncwarp();
+    } else if (warp == 9) {
+        const uint32_t id_s = umma_idesc_bf16(128u, 128u), id_o = umma_idesc_bf16(128u, (uint32_t)HD) | (1u << 16);   // B of P V: features contiguous
+        bool ok = true;
+        auto scores = [&](int j) {
+            const int s = j % S::kStages;
+            ok = ok && mbar_wait_bounded(&ctl->kfull[s], (uint32_t)(j / S::kStages) & 1u, &ctl->abort_flag, wait_limit_ns);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; return; }
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)(j & 1) * 128u, k = smem_u32(ring + s * 2 * S::kTileBytes), qa = smem_u32(Qs);
+            if (elect_one()) {
+#pragma unroll
+                for (int ks = 0; ks < KSTEPS; ++ks) {
+                    const uint32_t off = (uint32_t)((ks >> 2) * 16384 + (ks & 3) * 32);
+                    umma_bf16(d, umma_desc_sw128(qa + off), umma_desc_sw128(k + off), id_s, (uint32_t)ks);
+                }
+                umma_commit(&ctl->s_full[j & 1]);
+            }
+            __syncwarp();
+        };
+        if (nblk > 0) scores(0);
+        if (nblk > 1) scores(1);
+        for (int j = 0; j < nblk && ok; ++j) {
+            const int s = j % S::kStages, w = j & 1;
+            ok = mbar_wait_bounded(&ctl->vfull[s], (uint32_t)(j / S::kStages) & 1u, &ctl->abort_flag, wait_limit_ns) &&
+                 mbar_wait_bounded(&ctl->p_ready[w], (uint32_t)(j >> 1) & 1u, &ctl->abort_flag, wait_limit_ns);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t v = smem_u32(ring + s * 2 * S::kTileBytes + S::kTileBytes);
+            if (elect_one()) {
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks)   // 16 keys: 16 rows of 128 bytes of every slab; 8 packed columns of P
+                    umma_bf16_tmem_a(tmem + 256u + (uint32_t)w * 128u, tmem + (uint32_t)w * 128u + (uint32_t)ks * 8u,
+                                     umma_desc_sw128_mn(v + (uint32_t)ks * 2048u, 16384u), id_o, (uint32_t)((j >> 1) | ks));
+                umma_commit(&ctl->empty[s]);
+            }
+            __syncwarp();
+            if (j + 2 < nblk) scores(j + 2);
+        }
+        if (ok && elect_one()) umma_commit(&ctl->o_full);
+        __syncwarp();
+    } else {
+        const int w = warp >> 2, t = (warp & 3) * 32 + lane;   // stream, tile row
+        const uint32_t ts = tmem + (uint32_t)w * 128u + ((uint32_t)((warp & 3) * 32) << 16), to = ts + 256u;
+        const int lim = L + q0 + t / g;                        // last key this row sees
+        float m = -CUDART_INF_F, l = 0.f;
+        bool ok = true;
+        for (int j = w; j < nblk; j += 2) {
+            const int s = j % S::kStages, key0 = (b0 + j) * 128;
+            ok = ok && mbar_wait_bounded(&ctl->s_full[w], (uint32_t)(j >> 1) & 1u, &ctl->abort_flag, wait_limit_ns);
+            if (key0 + 128 > nkeys) {
+                // values behind the last key are whatever the cache holds there: cleared, since 0 x NaN is not 0
+                ok = ok && mbar_wait_bounded(&ctl->vfull[s], (uint32_t)(j / S::kStages) & 1u, &ctl->abort_flag, wait_limit_ns);
+                if (ok && key0 + t >= nkeys) {
+                    uint4* vr = reinterpret_cast<uint4*>(ring + s * 2 * S::kTileBytes + S::kTileBytes + t * 128);
+#pragma unroll
+                    for (int i = 0; i < UNITS; ++i) vr[(i >> 3) * 1024 + (i & 7)] = make_uint4(0, 0, 0, 0);
+                }
+                fence_proxy_async_smem();
+            }
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const int seen = lim - key0;                       // columns 0..seen are visible
+            float mx = -CUDART_INF_F;
+#pragma unroll
+            for (int c = 0; c < 128; c += 32) {
+                uint32_t v[32];
+                tmem_ld32(ts + (uint32_t)c, v);
+                tmem_ld_wait();
+                if (seen >= c + 31) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) mx = fmaxf(mx, __uint_as_float(v[i]));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (c + i <= seen) mx = fmaxf(mx, __uint_as_float(v[i]));
+                }
+            }
+            mx *= scale_log2e;
+            const bool grow = mx > m + 8.f;                    // also the first block that shows this row a key
+            if (__any_sync(0xffffffffu, grow && m != -CUDART_INF_F)) {
+                const float f = grow && m != -CUDART_INF_F ? exp2f(m - mx) : 1.f;
+                l *= f;
+#pragma unroll 1
+                for (int c = 0; c < HD; c += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(to + (uint32_t)c, v);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * f);
+                    tmem_st32(to + (uint32_t)c, v);
+                }
+            }
+            if (grow) m = mx;
+            const float ref = m == -CUDART_INF_F ? 0.f : m;
             float sum = 0.f;
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (k < CS) {
-                    const uint32_t src = map_shared_rank(base_o + (lr * LDO + c) * 4, k);
-                    const float4 x = ld_cluster_f4(src), y = ld_cluster_f4(src + 16);
-                    const float wt = exp2f(ml[k].x - mmax);
-                    sum += wt * ml[k].y;
-                    a.x += wt * x.x; a.y += wt * x.y; a.z += wt * x.z; a.w += wt * x.w;
-                    b.x += wt * y.x; b.y += wt * y.y; b.z += wt * y.z; b.w += wt * y.w;
+            for (int c = 0; c < 128; c += 32) {
+                uint32_t v[32], pk[16];
+                tmem_ld32(ts + (uint32_t)c, v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    float x = exp2f(fmaf(__uint_as_float(v[i]), scale_log2e, -ref));
+                    if (c + i > seen) x = 0.f;
+                    sum += x;
+                    v[i] = __float_as_uint(x);
                 }
-            if (r < M) {
-                const float inv = 1.f / sum;
-                *reinterpret_cast<uint4*>(out + (size_t)r * (n_q * HD) + (kvh * g + w % g) * HD + c) =
-                    make_uint4(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv), pack_bf16(b.x * inv, b.y * inv),
-                               pack_bf16(b.z * inv, b.w * inv));
+#pragma unroll
+                for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                tmem_st16(ts + (uint32_t)(c / 2), pk);         // over scores this thread has read
+            }
+            l += sum;
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->p_ready[w]);
+        }
+        // the stream's outputs and statistics; the ring is free once every product has completed
+        const bool any = nblk > w;
+        if (nblk > 0) ok = ok && mbar_wait_bounded(&ctl->o_full, 0, &ctl->abort_flag, wait_limit_ns);
+        ok = __all_sync(0xffffffffu, ok);
+        float* ex = reinterpret_cast<float*>(ring + w * S::kExBytes) + t * S::kLdo;
+        if (any && ok) {
+            tc_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < HD; c += 32) {
+                uint32_t v[32];
+                tmem_ld32(to + (uint32_t)c, v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; i += 4)
+                    *reinterpret_cast<uint4*>(ex + c + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
             }
         }
+        ex_ml[w * 128 + t] = any && ok ? make_float2(m, l) : make_float2(-CUDART_INF_F, 0.f);
+        tc_fence_before();
     }
+    __syncwarp();
+    cluster_sync();
+    if (warp == 9) tmem_dealloc(tmem, 512);
+    {
+        // every block merges its share of the tile rows from all streams of the cluster
+        const uint32_t base_o = smem_u32(ring), base_ml = smem_u32(ex_ml);
+        constexpr int C8 = HD / 8;
+        const int R = min(QR, M - q0) * g;
+        const int rbeg = even_start(R, CS, rank), rows = even_count(R, CS, rank);
+        for (int it = tid; it < rows * C8; it += kDenseAttThreads) {
+            const int t = rbeg + it / C8, c = (it % C8) * 8;
+            float mmax = -CUDART_INF_F;
+            for (int k = 0; k < CS; ++k) {
+                mmax = fmaxf(mmax, ld_cluster_f2(map_shared_rank(base_ml + t * 8, k)).x);
+                mmax = fmaxf(mmax, ld_cluster_f2(map_shared_rank(base_ml + (128 + t) * 8, k)).x);
+            }
+            float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sum = 0.f;
+            for (int k = 0; k < CS; ++k)
+#pragma unroll
+                for (int w = 0; w < 2; ++w) {
+                    const float2 ml = ld_cluster_f2(map_shared_rank(base_ml + (w * 128 + t) * 8, k));
+                    if (ml.x == -CUDART_INF_F) continue;       // no key: its output area was never written
+                    const uint32_t src = map_shared_rank(base_o + w * S::kExBytes + (t * S::kLdo + c) * 4, k);
+                    const float4 x = ld_cluster_f4(src), y = ld_cluster_f4(src + 16);
+                    const float wt = exp2f(ml.x - mmax);
+                    sum += wt * ml.y;
+                    o[0] += wt * x.x; o[1] += wt * x.y; o[2] += wt * x.z; o[3] += wt * x.w;
+                    o[4] += wt * y.x; o[5] += wt * y.y; o[6] += wt * y.z; o[7] += wt * y.w;
+                }
+            const float inv = 1.f / sum;
+            *reinterpret_cast<uint4*>(out + (size_t)(q0 + t / g) * (n_q * HD) + (kvh * g + t % g) * HD + c) =
+                make_uint4(pack_bf16(o[0] * inv, o[1] * inv), pack_bf16(o[2] * inv, o[3] * inv), pack_bf16(o[4] * inv, o[5] * inv),
+                           pack_bf16(o[6] * inv, o[7] * inv));
+        }
+    }
+    __syncwarp();
     cluster_sync();   // no block leaves while another still reads its shared memory
-}
-template <int HD>
-constexpr int dense_attention_smem() {
-    constexpr int kv = 4 * 64 * HD * 2, ex = 128 * (HD + 4) * 4 + 128 * 8;
-    return (kv > ex ? kv : ex) + 128;
+    if (tid == 0 && ctl->abort_flag) atomicExch(err, 1);
 }
 
 // Calibration, "Sample": the b best ids of every row from the tiles' best kDenseTopMax (largest first, lowest id among

@@ -479,9 +479,9 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t K, uint3
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-// Tensor maps of a context: activations (normalised rows, attention output, SwiGLU output), the LM head, then per layer
+// Tensor maps of a context: activations (normalised rows, attention output, SwiGLU output), key and value cache, the LM head, then per layer
 // q|k|v, o, gate|up and down with boxes of 64 rows (tiles of 128 features) and again with boxes of 128 (256 features).
-enum MapIndex { MAP_XN = 0, MAP_ATT, MAP_ACT, MAP_LM, MAP_LAYERS };
+enum MapIndex { MAP_XN = 0, MAP_ATT, MAP_ACT, MAP_K, MAP_V, MAP_LM, MAP_LAYERS };
 inline size_t map_at(int layer, int matrix, int bn) { return MAP_LAYERS + 8 * (size_t)layer + 2 * matrix + (bn == 256 ? 1 : 0); }
 
 // A launch that may overlap the tail of the kernel before it (programmatic dependent launch), in clusters of `cluster`
@@ -560,8 +560,8 @@ cudaError_t dense_attributes() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_SWIGLU, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_TOP, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, dense_attention_smem<128>());
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, dense_attention_smem<64>());
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseAttShape<128>::kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseAttShape<64>::kSmemBytes);
     done = e == cudaSuccess;
     return e;
 }
@@ -588,11 +588,13 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     // rows of four columns per thread
     int nt = (d / 4 + 31) / 32 * 32;
     if (nt > 1024) nt = 1024;
-    // attention: query groups per block so that up to eight warps share a key block; key shares so that the blocks fill the
-    // chip about twice over and keep at least two key blocks each
-    const int QT = 8 / g, qtiles = (rows + QT * 16 - 1) / (QT * 16);
-    unsigned cs = 1;
-    while (cs < 8 && (int)(qtiles * c.n_kv_heads * cs * 2) <= 2 * ctx->G && (int)(cs * 2) * 128 <= L + rows + 127) cs *= 2;
+    // attention: the queries whose g heads fill a 128-row tile; key shares so that the blocks fill the chip once (clusters of
+    // more than two leave some SMs of a group of 18 or 20 unused, hence 7/8) and keep at least one block of 128 keys each
+    const int QR = 128 / g, qtiles = (rows + QR - 1) / QR;
+    int cs = ctx->G * 7 / 8 / (qtiles * c.n_kv_heads);
+    if (cs > 8) cs = 8;
+    if (cs > (L + rows + 127) / 128) cs = (L + rows + 127) / 128;
+    if (cs < 1) cs = 1;
     int splits = 0;
     CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, hist + L, ctx->P.emb, c.vocab, h, part, 0, norm_w, xn, d,
                         c.rms_eps, nullptr));
@@ -603,8 +605,9 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
         CK(launch_dependent(ctx, dense_qkv_finish_kernel, dim3(rows), dim3(256), 0, 0, part, splits, bias ? bias + (size_t)l * nqkv : nullptr,
                             ctx->P.rope, q, c.n_q_heads, c.n_kv_heads, hd, ctx->P.kcache, ctx->P.vcache, layer_off, c.max_seq, L));
         CK(launch_dependent(ctx, hd == 128 ? dense_attention_kernel<128> : dense_attention_kernel<64>, dim3(qtiles * cs, c.n_kv_heads),
-                            dim3(32 * g * QT), hd == 128 ? dense_attention_smem<128>() : dense_attention_smem<64>(), cs, q, ctx->P.kcache,
-                            ctx->P.vcache, layer_off, c.max_seq, c.n_q_heads, g, QT, rows, L, ctx->P.scale_log2e, att));
+                            dim3(kDenseAttThreads), hd == 128 ? DenseAttShape<128>::kSmemBytes : DenseAttShape<64>::kSmemBytes, (unsigned)cs,
+                            maps[MAP_K], maps[MAP_V], q, l * c.n_kv_heads * c.max_seq, c.max_seq, c.n_q_heads, g, QR, rows, L,
+                            ctx->P.scale_log2e, att, ctx->P.state + ST_ERR, 2000000000ull));
         CK(dense_product(ctx, MAP_ATT, l, 1, rows, d, nq, &splits));
         CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
                             norm_w + (size_t)(2 * l + 1) * d, xn, d, c.rms_eps, nullptr));
@@ -786,7 +789,9 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
     if (ctx->dense_ok) {
         std::vector<CUtensorMap>& m = *ctx->maps;
         ctx->dense_ok = make_map(&m[MAP_XN], ws + ctx->r.dxn, kDenseMaxRows, d, 128) && make_map(&m[MAP_ATT], ws + ctx->r.datt, kDenseMaxRows, nq, 128) &&
-                        make_map(&m[MAP_ACT], ws + ctx->r.dact, kDenseMaxRows, f, 128);
+                        make_map(&m[MAP_ACT], ws + ctx->r.dact, kDenseMaxRows, f, 128) &&
+                        make_map(&m[MAP_K], P.kcache, (uint64_t)cfg->n_layers * cfg->n_kv_heads * cfg->max_seq, hd, 128) &&
+                        make_map(&m[MAP_V], P.vcache, (uint64_t)cfg->n_layers * cfg->n_kv_heads * cfg->max_seq, hd, 128);
         if (!leader) ctx->dense_ok = ctx->dense_ok && make_map(&m[MAP_LM], ws + ctx->r.dlm, cfg->vocab, d, 128);
         for (int l = 0; l < cfg->n_layers && ctx->dense_ok && !leader; ++l) {
             uint8_t* lb = ws + ctx->r.dw + (size_t)l * ctx->r.layer_stride;
