@@ -58,7 +58,7 @@ __device__ __forceinline__ uint64_t umma_desc_sw128_mn(uint32_t saddr, uint32_t 
     return d;
 }
 
-struct DenseTopOut {   // EPI_TOP: [row][vocabulary tile][kDenseTopMax] best logits of the tile and their ids, best first
+struct DenseTopOut {   // EPI_TOP: [row][share of the vocabulary][kDenseTopMax] best logits of the share and their ids, best first
     float* val;
     int* idx;
 };
@@ -72,8 +72,9 @@ struct DenseTopOut {   // EPI_TOP: [row][vocabulary tile][kDenseTopMax] best log
 // Pairs walk the tiles persistently: (features, 256-row tokens, K share), K shares fastest.
 //   EPI_PARTIAL: part[z][m][n] = the share's sum (row stride N)
 //   EPI_SWIGLU:  features come as 64 gate rows then the 64 matching up rows: out_bf16[m][64 t + c] = silu(gate) * up
-//   EPI_TOP:     the best kDenseTopMax values of every row in this tile of features (largest first, lowest id first
-//                among equals)
+//   EPI_TOP:     the best kDenseTopMax values of every row over the tiles this pair walks (largest first, lowest id first
+//                among equals): a pair stays with its 256 rows, so a thread keeps its row's best in registers and most
+//                values only take part in a maximum over 32
 // Rows >= M and columns >= N are computed on whatever the copies deliver (zeros outside the tensors) and
 // never written.  err: set to 1 when a bounded wait runs out.
 // Measured on B200 (BN 256, 1536 x 17920 weights): 256 tokens 18.6 us stand-alone (758 TFLOP/s; 25.4 us with
@@ -99,7 +100,10 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const uint32_t rank = cluster_rank();
     const int mt = (M + 255) / 256, nt = (N + BN - 1) / BN, ntiles = mt * nt * splits;
     const int nkb_all = K / kDenseBK;
-    const int npairs = (int)gridDim.x >> 1, pair = (int)blockIdx.x >> 1;
+    const int pair = (int)blockIdx.x >> 1;
+    int npairs = (int)gridDim.x >> 1;   // stride of the walk
+    if (EPI == EPI_TOP) npairs = npairs / mt * mt;
+    const int t0 = pair < npairs ? pair : ntiles;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S::kStages; ++s) {
             mbar_init(&ctl->full[s], 1);
@@ -123,7 +127,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         if (elect_one()) {
             uint32_t s = 0, par = 0, issued = 0;
             bool ok = true, first = true;
-            for (int t = pair; t < ntiles && ok; t += npairs) {
+            for (int t = t0; t < ntiles && ok; t += npairs) {
                 const int z = t % splits, r = t / splits;
                 const int m0 = (r % mt) * 256 + (int)rank * 128, n0 = (r / mt) * BN + (int)rank * (BN / 2);
                 const int kb0 = even_start(nkb_all, splits, z), nkb = even_count(nkb_all, splits, z);
@@ -170,7 +174,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             const uint32_t idesc = umma_idesc_bf16(256u, (uint32_t)BN);
             uint32_t s = 0, par = 0, q = 0;
             bool ok = true;
-            for (int t = pair; t < ntiles && ok; t += npairs, ++q) {
+            for (int t = t0; t < ntiles && ok; t += npairs, ++q) {
                 const int nkb = even_count(nkb_all, splits, t % splits);
                 const uint32_t buf = q & 1u;
                 if (!mbar_wait_bounded(&ctl->acc_empty[buf], ((q >> 1) & 1u) ^ 1u, &ctl->abort_flag, wait_limit_ns)) break;
@@ -200,9 +204,13 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         // writes whole 32-byte sectors of it
         const int q4 = warp & 3;
         uint32_t q = 0;
+        float bv[kDenseTopMax];
+        int bi[kDenseTopMax];
+#pragma unroll
+        for (int j = 0; j < kDenseTopMax; ++j) { bv[j] = -CUDART_INF_F; bi[j] = 0x7fffffff; }
         if (lane == 0) grid_dep_wait();   // the outputs may still be read by the kernels before
         __syncwarp();
-        for (int t = pair; t < ntiles; t += npairs, ++q) {
+        for (int t = t0; t < ntiles; t += npairs, ++q) {
             const int z = t % splits, r = t / splits, m0 = (r % mt) * 256 + (int)rank * 128, n0 = (r / mt) * BN;
             const uint32_t buf = q & 1u;
             const bool got = mbar_wait_bounded(&ctl->acc_full[buf], (q >> 1) & 1u, &ctl->abort_flag, wait_limit_ns);
@@ -246,41 +254,50 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     }
                 }
             } else {
-                float bv[kDenseTopMax];
-                int bi[kDenseTopMax];
-#pragma unroll
-                for (int j = 0; j < kDenseTopMax; ++j) { bv[j] = -CUDART_INF_F; bi[j] = 0x7fffffff; }
 #pragma unroll 1
                 for (int c = 0; c < BN; c += 32) {
                     uint32_t v[32];
                     tmem_ld32(ta + (uint32_t)c, v);
                     tmem_ld_wait();
+                    if (n0 + c + 32 > N) {   // N is a multiple of 16
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        float x = __uint_as_float(v[i]);
-                        // ids come in ascending order, so ">" keeps the lowest id among equals
-                        if (x > bv[kDenseTopMax - 1] && n0 + c + i < N) {
-                            int id = n0 + c + i;
+                        for (int i = 0; i < 32; ++i)
+                            if (n0 + c + i >= N) v[i] = 0xff800000u;   // -inf
+                    }
+                    float mx = __uint_as_float(v[0]);
 #pragma unroll
-                            for (int j = 0; j < kDenseTopMax; ++j)
-                                if (x > bv[j]) {
-                                    const float tv = bv[j];
-                                    const int ti = bi[j];
-                                    bv[j] = x; bi[j] = id;
-                                    x = tv; id = ti;
-                                }
+                    for (int i = 1; i < 32; ++i) mx = fmaxf(mx, __uint_as_float(v[i]));
+                    if (mx > bv[kDenseTopMax - 1]) {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            float x = __uint_as_float(v[i]);
+                            // ids come in ascending order, so ">" keeps the lowest id among equals
+                            if (x > bv[kDenseTopMax - 1]) {
+                                int id = n0 + c + i;
+#pragma unroll
+                                for (int j = 0; j < kDenseTopMax; ++j)
+                                    if (x > bv[j]) {
+                                        const float tv = bv[j];
+                                        const int ti = bi[j];
+                                        bv[j] = x; bi[j] = id;
+                                        x = tv; id = ti;
+                                    }
+                            }
                         }
                     }
-                }
-                if (row < M) {
-                    const size_t at = ((size_t)row * nt + r / mt) * kDenseTopMax;
-                    *reinterpret_cast<float4*>(top.val + at) = make_float4(bv[0], bv[1], bv[2], bv[3]);
-                    *reinterpret_cast<int4*>(top.idx + at) = make_int4(bi[0], bi[1], bi[2], bi[3]);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_leader(&ctl->acc_empty[buf]);  // this warp's part of the accumulator may be overwritten
+        }
+        if (EPI == EPI_TOP && pair < npairs) {
+            const int row = (pair % mt) * 256 + (int)rank * 128 + q4 * 32 + lane;
+            if (row < M) {
+                const size_t at = ((size_t)row * (npairs / mt) + pair / mt) * kDenseTopMax;
+                *reinterpret_cast<float4*>(top.val + at) = make_float4(bv[0], bv[1], bv[2], bv[3]);
+                *reinterpret_cast<int4*>(top.idx + at) = make_int4(bi[0], bi[1], bi[2], bi[3]);
+            }
         }
     }
     __syncwarp();
@@ -417,10 +434,10 @@ struct DenseAttShape {
     static constexpr int kTileBytes = 128 * HD * 2;              // queries, or the keys or values of a block
     static constexpr int kStages = 3;
     static constexpr int kLdo = HD + 4;                          // row stride (floats) of the exchange area
-    static constexpr int kExBytes = 128 * kLdo * 4;              // one stream's outputs
+    static constexpr int kExBytes = 128 * kLdo * 4;              // the block's outputs
     static constexpr int kRing = kStages * 2 * kTileBytes;
     static constexpr int kSmemBytes = kTileBytes + kRing + 256 + 1024;
-    static_assert(2 * kExBytes <= kRing, "the exchange area reuses the ring");
+    static_assert(kExBytes <= kRing, "the exchange area reuses the ring");
 };
 constexpr int kDenseAttThreads = 320;   // warps 0..3 and 4..7: the two streams; 8: copies; 9: tensor-core issue
 
@@ -434,7 +451,7 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
     extern __shared__ uint8_t att_smem_raw[];
     uint8_t* Qs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* ring = Qs + S::kTileBytes;                                  // [stage][K | V]
-    float2* ex_ml = reinterpret_cast<float2*>(Qs);   // once the products are done: [stream][tile row] (maximum in log2 units, sum)
+    float2* ex_ml = reinterpret_cast<float2*>(Qs);   // once the products are done: [stream 0, stream 1, both][tile row] (maximum in log2 units, sum)
     struct Ctl {
         uint64_t kfull[S::kStages], vfull[S::kStages], empty[S::kStages], s_full[2], p_ready[2], o_full;
         uint32_t tmem_base;
@@ -463,20 +480,33 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
         mbar_fence_init();
     }
     if (warp == 9) tmem_alloc(&ctl->tmem_base, 512);   // S0 | S1 | O0 | O1, 128 columns each
-    grid_dep_launch();
-    grid_dep_wait();
-    // query tile, in the layout the copies below have: slabs of 64 columns, 128-byte swizzle
-    for (int u = tid; u < 128 * UNITS; u += kDenseAttThreads) {
-        const int t = u / UNITS, c16 = u % UNITS, qi = q0 + t / g;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (t < QR * g && qi < M) v = __ldcg(reinterpret_cast<const uint4*>(q + (size_t)qi * (n_q * HD) + (kvh * g + t % g) * HD + c16 * 8));
-        *reinterpret_cast<uint4*>(Qs + (c16 >> 3) * 16384 + swz_unit(t, c16 & 7)) = v;
-    }
-    fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
+    grid_dep_launch();
+    grid_dep_wait();
+    if (warp < 8) {
+        // query tile, in the layout the copies have: slabs of 64 columns, 128-byte swizzle
+        constexpr int QI = 128 * UNITS / 256;   // 16-byte units per thread, all loads in flight
+        uint4 v[QI];
+#pragma unroll
+        for (int i = 0; i < QI; ++i) {
+            const int u = tid + i * 256, t = u / UNITS, qi = q0 + t / g;
+            v[i] = make_uint4(0, 0, 0, 0);
+            if (t < QR * g && qi < M)
+                v[i] = __ldcg(reinterpret_cast<const uint4*>(q + (size_t)qi * (n_q * HD) + (kvh * g + t % g) * HD + (u % UNITS) * 8));
+        }
+#pragma unroll
+        for (int i = 0; i < QI; ++i) {
+            const int u = tid + i * 256, c16 = u % UNITS;
+            *reinterpret_cast<uint4*>(Qs + (c16 >> 3) * 16384 + swz_unit(u / UNITS, c16 & 7)) = v[i];
+        }
+    }
+    if (warp != 8) {
+        fence_proxy_async_smem();
+        named_bar_sync(2, 288);   // the queries are in place for the tensor-core warp
+    }
 
     if (warp == 8) {
         if (elect_one()) {
@@ -621,59 +651,94 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctl->p_ready[w]);
         }
-        // the stream's outputs and statistics; the ring is free once every product has completed
-        const bool any = nblk > w;
+        // The two streams of a row meet: statistics through shared memory, outputs straight from tensor memory (each
+        // warpgroup takes half of the columns).  The ring and the queries are free once every product has completed.
         if (nblk > 0) ok = ok && mbar_wait_bounded(&ctl->o_full, 0, &ctl->abort_flag, wait_limit_ns);
         ok = __all_sync(0xffffffffu, ok);
-        float* ex = reinterpret_cast<float*>(ring + w * S::kExBytes) + t * S::kLdo;
-        if (any && ok) {
+        ex_ml[w * 128 + t] = ok ? make_float2(m, l) : make_float2(-CUDART_INF_F, 0.f);
+        named_bar_sync(1, 256);
+        const float2 o0 = ex_ml[t], o1 = ex_ml[128 + t];
+        const float mx = fmaxf(o0.x, o1.x), ref = mx == -CUDART_INF_F ? 0.f : mx;
+        const float w0 = exp2f(o0.x - ref), w1 = exp2f(o1.x - ref);
+        const float sum = w0 * o0.y + w1 * o1.y;
+        const float sc = CS == 1 ? 1.f / sum : 1.f;   // a block that saw all keys writes the result itself
+        const int qi = q0 + t / g;
+        __nv_bfloat16* po = out + (size_t)qi * (n_q * HD) + (kvh * g + t % g) * HD;
+        if (w == 0) ex_ml[256 + t] = make_float2(mx, sum);
+        float* ex = reinterpret_cast<float*>(ring) + t * S::kLdo;
+        if (nblk > 0 && ok) {
             tc_fence_after();
 #pragma unroll 1
-            for (int c = 0; c < HD; c += 32) {
-                uint32_t v[32];
-                tmem_ld32(to + (uint32_t)c, v);
+            for (int c = w * (HD / 2); c < (w + 1) * (HD / 2); c += 32) {
+                uint32_t a[32], b[32];
+                tmem_ld32(tmem + 256u + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c, a);
+                tmem_ld32(tmem + 384u + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c, b);
                 tmem_ld_wait();
 #pragma unroll
-                for (int i = 0; i < 32; i += 4)
-                    *reinterpret_cast<uint4*>(ex + c + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                for (int i = 0; i < 32; i += 4) {
+                    float4 v = make_float4(w0 * __uint_as_float(a[i]), w0 * __uint_as_float(a[i + 1]), w0 * __uint_as_float(a[i + 2]),
+                                           w0 * __uint_as_float(a[i + 3]));
+                    if (nblk > 1) {   // the second stream wrote its output
+                        v.x += w1 * __uint_as_float(b[i]); v.y += w1 * __uint_as_float(b[i + 1]);
+                        v.z += w1 * __uint_as_float(b[i + 2]); v.w += w1 * __uint_as_float(b[i + 3]);
+                    }
+                    if (CS > 1) *reinterpret_cast<float4*>(ex + c + i) = v;
+                    else if (t < QR * g && qi < M)
+                        *reinterpret_cast<uint2*>(po + c + i) = make_uint2(pack_bf16(v.x * sc, v.y * sc), pack_bf16(v.z * sc, v.w * sc));
+                }
             }
         }
-        ex_ml[w * 128 + t] = any && ok ? make_float2(m, l) : make_float2(-CUDART_INF_F, 0.f);
         tc_fence_before();
     }
     __syncwarp();
     cluster_sync();
     if (warp == 9) tmem_dealloc(tmem, 512);
-    {
-        // every block merges its share of the tile rows from all streams of the cluster
-        const uint32_t base_o = smem_u32(ring), base_ml = smem_u32(ex_ml);
-        constexpr int C8 = HD / 8;
+    if (CS > 1) {
+        // every block merges its share of the tile rows from the cluster's CS partial results: first the rows' weights, one
+        // remote load per row and block, then the outputs with all loads of an item in flight (remote shared memory gives
+        // about 13 bytes per cycle and SM, so the fewer partial results the better)
+        const uint32_t base_o = smem_u32(ring), base_ml = smem_u32(ex_ml + 256);
+        constexpr int C8 = HD / 8, NP = 8;
         const int R = min(QR, M - q0) * g;
         const int rbeg = even_start(R, CS, rank), rows = even_count(R, CS, rank);
+        float* wt = reinterpret_cast<float*>(Qs + 4096);   // [own row][8], behind the statistics
+        for (int it = tid; it < rows * NP; it += kDenseAttThreads) {   // 8 lanes share a row
+            const int t = rbeg + it / NP, k = it % NP;
+            float2 ml = make_float2(-CUDART_INF_F, 0.f);
+            if (k < CS) ml = ld_cluster_f2(map_shared_rank(base_ml + t * 8, k));
+            const unsigned mask = 0xffu << (lane & 24);
+            float mx = ml.x;
+#pragma unroll
+            for (int off = 4; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(mask, mx, off));
+            const float e = exp2f(ml.x - mx);
+            float sum = e * ml.y;
+#pragma unroll
+            for (int off = 4; off; off >>= 1) sum += __shfl_xor_sync(mask, sum, off);
+            wt[it] = e / sum;
+        }
+        __syncthreads();
         for (int it = tid; it < rows * C8; it += kDenseAttThreads) {
             const int t = rbeg + it / C8, c = (it % C8) * 8;
-            float mmax = -CUDART_INF_F;
-            for (int k = 0; k < CS; ++k) {
-                mmax = fmaxf(mmax, ld_cluster_f2(map_shared_rank(base_ml + t * 8, k)).x);
-                mmax = fmaxf(mmax, ld_cluster_f2(map_shared_rank(base_ml + (128 + t) * 8, k)).x);
-            }
-            float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sum = 0.f;
-            for (int k = 0; k < CS; ++k)
+            float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int k0 = 0; k0 < CS; k0 += 4) {   // four partial results' loads in flight (past the last: the last again)
+                float4 x[4], y[4];
 #pragma unroll
-                for (int w = 0; w < 2; ++w) {
-                    const float2 ml = ld_cluster_f2(map_shared_rank(base_ml + (w * 128 + t) * 8, k));
-                    if (ml.x == -CUDART_INF_F) continue;       // no key: its output area was never written
-                    const uint32_t src = map_shared_rank(base_o + w * S::kExBytes + (t * S::kLdo + c) * 4, k);
-                    const float4 x = ld_cluster_f4(src), y = ld_cluster_f4(src + 16);
-                    const float wt = exp2f(ml.x - mmax);
-                    sum += wt * ml.y;
-                    o[0] += wt * x.x; o[1] += wt * x.y; o[2] += wt * x.z; o[3] += wt * x.w;
-                    o[4] += wt * y.x; o[5] += wt * y.y; o[6] += wt * y.z; o[7] += wt * y.w;
+                for (int i = 0; i < 4; ++i) {
+                    const int k = min(k0 + i, CS - 1);
+                    const uint32_t src = map_shared_rank(base_o + (t * S::kLdo + c) * 4, k);
+                    x[i] = ld_cluster_f4(src);
+                    y[i] = ld_cluster_f4(src + 16);
                 }
-            const float inv = 1.f / sum;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float w = k0 + i < CS ? wt[(it / C8) * NP + k0 + i] : 0.f;
+                    const bool use = w > 0.f;   // a block without a key never wrote its area
+                    o[0] += use ? w * x[i].x : 0.f; o[1] += use ? w * x[i].y : 0.f; o[2] += use ? w * x[i].z : 0.f; o[3] += use ? w * x[i].w : 0.f;
+                    o[4] += use ? w * y[i].x : 0.f; o[5] += use ? w * y[i].y : 0.f; o[6] += use ? w * y[i].z : 0.f; o[7] += use ? w * y[i].w : 0.f;
+                }
+            }
             *reinterpret_cast<uint4*>(out + (size_t)(q0 + t / g) * (n_q * HD) + (kvh * g + t % g) * HD + c) =
-                make_uint4(pack_bf16(o[0] * inv, o[1] * inv), pack_bf16(o[2] * inv, o[3] * inv), pack_bf16(o[4] * inv, o[5] * inv),
-                           pack_bf16(o[6] * inv, o[7] * inv));
+                make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
         }
     }
     __syncwarp();
@@ -681,12 +746,12 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
     if (tid == 0 && ctl->abort_flag) atomicExch(err, 1);
 }
 
-// Calibration, "Sample": the b best ids of every row from the tiles' best kDenseTopMax (largest first, lowest id among
+// Calibration, "Sample": the b best ids of every row from the shares' best kDenseTopMax (largest first, lowest id among
 // equals).  One block per row.
-__global__ void __launch_bounds__(256) dense_top_merge_kernel(DenseTopOut top, int ntiles, int b, int* succ /* [rows][b] */) {
+__global__ void __launch_bounds__(256) dense_top_merge_kernel(DenseTopOut top, int shares, int b, int* succ /* [rows][b] */) {
     __shared__ float bv_s[8];
     __shared__ int bi_s[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = ntiles * kDenseTopMax;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = shares * kDenseTopMax;
     grid_dep_launch();
     grid_dep_wait();
     const float* val = top.val + (size_t)blockIdx.x * n;

@@ -103,11 +103,9 @@ Regions carve(const sdv_config* c, bool own_weights = true) {
     r.dlm = c->tied_lm_head ? r.emb : take_w(V * d * 2);
     r.dh = take((size_t)kDenseMaxRows * d * 4);
     r.dxn = take((size_t)kDenseMaxRows * d * 2);
-    size_t dp = (size_t)(kMaxGrid / 2) * 256 * 256 * 4;                                    // K shares: one tile per pair of SMs at most
+    size_t dp = (size_t)(kMaxGrid / 2) * 256 * 256 * 4;                                    // K shares: one tile per pair of SMs at most (the best logits are fewer)
     const size_t one = (size_t)kDenseMaxRows * (nqkv > d ? nqkv : d) * 4;                  // a product without K shares
-    const size_t tops = (size_t)kDenseMaxRows * ((V + 255) / 256) * kDenseTopMax * 8;
     if (one > dp) dp = one;
-    if (tops > dp) dp = tops;
     r.dpart = take(dp);
     r.dq = take((size_t)kDenseMaxRows * nq * 2);
     r.datt = take((size_t)kDenseMaxRows * nq * 2);
@@ -589,11 +587,11 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     int nt = (d / 4 + 31) / 32 * 32;
     if (nt > 1024) nt = 1024;
     // attention: the queries whose g heads fill a 128-row tile; key shares so that the blocks fill the chip once (clusters of
-    // more than two leave some SMs of a group of 18 or 20 unused, hence 7/8) and keep at least one block of 128 keys each
+    // more than two leave some SMs of a group of 18 or 20 unused, hence 7/8) and keep two blocks of 128 keys each, one per stream
     const int QR = 128 / g, qtiles = (rows + QR - 1) / QR;
     int cs = ctx->G * 7 / 8 / (qtiles * c.n_kv_heads);
     if (cs > 8) cs = 8;
-    if (cs > (L + rows + 127) / 128) cs = (L + rows + 127) / 128;
+    if (cs > (L + rows + 255) / 256) cs = (L + rows + 255) / 256;
     if (cs < 1) cs = 1;
     int splits = 0;
     CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, hist + L, ctx->P.emb, c.vocab, h, part, 0, norm_w, xn, d,
@@ -619,11 +617,11 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     }
     if (succ) {
         DenseTopOut top;
-        const int ntile = (c.vocab + 255) / 256;
+        const int mt = (rows + 255) / 256, tiles = mt * ((c.vocab + 255) / 256), pairs = tiles < ctx->G / 2 ? tiles : ctx->G / 2;
         top.val = part;
-        top.idx = (int*)(part + (size_t)rows * ntile * kDenseTopMax);
+        top.idx = (int*)(part + (size_t)rows * (pairs / mt) * kDenseTopMax);
         CK((launch_dense_tiles<EPI_TOP, 256>(ctx, maps[MAP_XN], maps[MAP_LM], rows, c.vocab, d, 1, nullptr, nullptr, 0, top)));
-        CK(launch_dependent(ctx, dense_top_merge_kernel, dim3(rows), dim3(256), 0, 0, top, ntile, ctx->calib_b, succ));
+        CK(launch_dependent(ctx, dense_top_merge_kernel, dim3(rows), dim3(256), 0, 0, top, pairs / mt, ctx->calib_b, succ));
     }
     CK(cudaGetLastError());
     return SDV_OK;
