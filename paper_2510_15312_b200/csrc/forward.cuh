@@ -6,7 +6,7 @@
 //                and keeps a ring of 32 KB shared-memory stages full with bulk asynchronous copies.
 //                It never waits for activations or grid barriers, only for free ring slots, so HBM
 //                traffic continues across operation boundaries.
-//   warp 10      one elected lane issues the tensor-core instructions (tcgen05.mma, M = 128 weight
+//   warp 10      one thread issues the tensor-core instructions (tcgen05.mma, M = 128 weight
 //                rows x N = 16 or 32 token rows x K = 16 per instruction): the streamed stage is the A
 //                operand, the token rows, resident in shared memory for the whole operation, the
 //                B operand; accumulators live in tensor memory (two buffers of two 128-row
@@ -15,7 +15,7 @@
 //                first accumulator of a pass, warps 4..7 the second (or, for passes of up to 128
 //                rows, alternate pairs of token columns of the one accumulator).
 //   warps 0..9   build the token operand at the start of an operation (RMSNorm scale, merge of the
-//                split-KV partial results, ...); warps 0..10 run the attention step.
+//                split-KV partial results, ...), run the attention step and meet the other blocks.
 // A layer is four operations separated by a bounded grid barrier: QKV projection; attention;
 // output projection (+ residual); gate|up with SwiGLU followed, inside the same block and without
 // a barrier, by the slice of the down projection (+ residual) that consumes this block's SwiGLU
@@ -61,6 +61,7 @@ __device__ __forceinline__ const uint8_t* op_weights(const FwdParams& P, int op,
 struct Misc {
     uint64_t full[kMaxStages], empty[kMaxStages];
     uint64_t tmem_full[2], tmem_empty[2];
+    uint64_t op_ready;    // the token operand of this block's next operation is complete (one arrival per builder warp)
     uint64_t act_ready;   // the SwiGLU operand of this block is complete (one arrival per epilogue warp)
     uint64_t done_bar;    // last tensor-core instruction of the launch has completed
     uint32_t tmem_base;
@@ -164,7 +165,7 @@ __device__ __forceinline__ uint32_t operand_off(int k8, int row, int M) {
 
 // Operand = residual rows scaled by the RMSNorm weight (the per-row factor rsqrt(mean + eps)
 // commutes with the GEMM and is applied by the consumer of the result), or, for the stand-alone
-// GEMM, the caller's fp32 rows as they are.  Warp w converts rows w, w + 11, ...; all loads of a
+// GEMM, the caller's fp32 rows as they are.  Warp w converts rows w, w + 10, ...; all loads of a
 // batch are issued before the first use.  Leaves the rows' sums of squares over this block's
 // columns in misc->sumsq; QKV blocks of row partition 0 also add them to the global sums the
 // attention step reads.
@@ -281,18 +282,38 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
 }
 
 // ------------------------------------------------------------------------------------------
-// Tensor-core issue.  The whole warp walks the loop so that ring positions and operand descriptors
-// stay warp-uniform values; one elected lane issues the instructions.  Pipeline positions: (slot, par) is the ring position (slot
-// index and parity of the current trip round the ring), `q` counts accumulator passes; all advance
-// over the whole launch, identically in every role.  The issuing thread is bound by its own
-// instruction latency, so the loop keeps ready-made descriptors and advances them by additions.
+// Tensor-core issue, by one thread of the warp for a whole operation.  The pipe takes an instruction (M = 128, N <= 32)
+// every 31 cycles, the time shared memory needs for its 4 KB of weights; what used to set the pace was the code around
+// it.  Stand-alone, a 32 KB stage of eight instructions cost 596 cycles with an election, a wait and a fence per stage, 583
+// by one thread, 520 with the instructions unrolled and 348 with the next stage's barrier looked at (without waiting)
+// before the instructions of this one are issued; the floor without any handshake is 313.
+// Pipeline positions: (slot, par) is the ring position (slot index and parity of the current trip round the ring), `q`
+// counts accumulator passes, `ops` token operands; all advance over the whole launch, identically in every role.
 struct PipePos {
-    uint32_t slot, par, q, act_uses;
+    uint32_t slot, par, q, ops;
     uint32_t w_full, w_acc;  // cycles the tensor-core thread waited for weights / for a free accumulator (profile)
 };
 
+// The instructions of one stage: nks column steps, one or (TWO) two 128-row accumulators.
+template <bool TWO>
+__device__ __forceinline__ void mma_stage(uint32_t d_tmem, uint64_t adesc, uint64_t astep, uint64_t bdesc, uint64_t bstep, uint32_t idesc,
+                                          int nks, uint32_t acc) {
+    auto step = [&]() {
+        umma_bf16(d_tmem, adesc, bdesc, idesc, acc);
+        if (TWO) umma_bf16(d_tmem + 32u, adesc + 128u, bdesc, idesc, acc);
+        acc = 1u;
+        adesc += astep;
+        bdesc += bstep;
+    };
+    int ks = 0;
+    for (; ks + 4 <= nks; ks += 4) {
+        step(); step(); step(); step();
+    }
+    for (; ks < nks; ++ks) step();
+}
+
 __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8_t* smem, const uint8_t* B, Misc* misc,
-                                       PipePos& pos, bool& dead, bool& synced) {
+                                       PipePos& pos, bool& dead, bool& ready) {
     const uint32_t nstage = (uint32_t)P.nstage;
     const uint32_t idesc = umma_idesc_bf16_m128((uint32_t)P.NB);
     const uint64_t wait_limit = P.wait_limit_ns;
@@ -301,8 +322,8 @@ __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8
     const uint64_t bdesc0 = umma_smem_desc(smem_u32(B), lbo_b, 128u);
     const uint32_t ring0 = smem_u32(smem);
     const uint32_t tmem0 = misc->tmem_base;
-    const int nst = pt.nst, SK = pt.SK, nk = pt.nk;
-    for (int p = 0; p < pt.npass; ++p, ++pos.q) {
+    const int nst = pt.nst, SK = pt.SK, nk = pt.nk, npass = pt.npass;
+    for (int p = 0; p < npass; ++p, ++pos.q) {
         const int pcount = pass_count(pt, p);
         const uint32_t buf = pos.q & 1u;
         const long long tq0 = clock64();
@@ -310,7 +331,6 @@ __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8
             dead = true;
         pos.w_acc += (uint32_t)(clock64() - tq0);
         const uint32_t d_tmem = tmem0 + buf * 64u;
-        const bool two = pcount > 8;  // rows 128.. of the pass go to the buffer's second accumulator
         const uint32_t lbo_a = (uint32_t)(2 * pcount) * 128u;
         const uint64_t astep = (uint64_t)((2u * lbo_a) >> 4);
         const uint64_t adesc0 = umma_smem_desc(ring0, lbo_a, 128u);
@@ -319,45 +339,25 @@ __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8
         for (int st = 0; st < nst; ++st, kleft -= SK) {
             const uint32_t slot = pos.slot, par = pos.par;
             if (++pos.slot == nstage) { pos.slot = 0; pos.par ^= 1u; }
-            const int nks = min(SK, kleft);
-            if (!synced) {
-                // everything above ran while the other warps were still building the token operand
-                named_bar_sync(1, kWorkerThreads);
-                synced = true;
-            }
             if (dead) continue;
-            const long long tw0 = clock64();
-            if (!mbar_wait_bounded(&misc->full[slot], par, &misc->abort_flag, wait_limit)) {
-                dead = true;
-                continue;
+            if (!ready) {
+                const long long tw0 = clock64();
+                if (!mbar_wait_bounded(&misc->full[slot], par, &misc->abort_flag, wait_limit)) {
+                    dead = true;
+                    continue;
+                }
+                pos.w_full += (uint32_t)(clock64() - tw0);
             }
-            pos.w_full += (uint32_t)(clock64() - tw0);
             tc_fence_after();
-            uint64_t adesc = adesc0 + (uint64_t)((slot * (uint32_t)kStageBytes) >> 4);
-            if (elect_one()) {
-                if (st == 0) {
-                    umma_bf16_first(d_tmem, adesc, bdesc, idesc);
-                    if (two) umma_bf16_first(d_tmem + 32u, adesc + 128u, bdesc, idesc);
-                } else {
-                    umma_bf16_acc(d_tmem, adesc, bdesc, idesc);
-                    if (two) umma_bf16_acc(d_tmem + 32u, adesc + 128u, bdesc, idesc);
-                }
-#pragma unroll 3
-                for (int ks = 1; ks < nks; ++ks) {
-                    adesc += astep;
-                    bdesc += bstep;
-                    umma_bf16_acc(d_tmem, adesc, bdesc, idesc);
-                    if (two) umma_bf16_acc(d_tmem + 32u, adesc + 128u, bdesc, idesc);
-                }
-                bdesc += bstep;
-                umma_commit(&misc->empty[slot]);  // the slot is free once these instructions have read it
-            } else {
-                bdesc += (uint64_t)nks * bstep;
-            }
-            __syncwarp();
+            ready = mbar_test(&misc->full[pos.slot], pos.par);   // the next stage, of this operation or the one after
+            const int nks = min(SK, kleft);
+            const uint64_t adesc = adesc0 + (uint64_t)((slot * (uint32_t)kStageBytes) >> 4);
+            if (pcount > 8) mma_stage<true>(d_tmem, adesc, astep, bdesc, bstep, idesc, nks, st > 0 ? 1u : 0u);   // rows 128..: second accumulator
+            else mma_stage<false>(d_tmem, adesc, astep, bdesc, bstep, idesc, nks, st > 0 ? 1u : 0u);
+            bdesc += (uint64_t)nks * bstep;
+            umma_commit(&misc->empty[slot]);  // the slot is free once these instructions have read it
         }
-        if (!dead && elect_one()) umma_commit(&misc->tmem_full[buf]);
-        __syncwarp();
+        if (!dead) umma_commit(&misc->tmem_full[buf]);
     }
 }
 
@@ -586,7 +586,7 @@ __device__ __forceinline__ void attn_split_compute(const FwdParams& P, int& S, i
 // MODE 0: the new rows are a chain; 1: a tree (positions and visibility from the state block); 2: the chain of
 // sequence `b` of a batched step (its rows, length and KV cache from P.seq[b]).
 template <int HD, int MODE>
-__device__ __noinline__ void attention_unit(const FwdParams& P, int layer, int hk, int qg, int gh, int s, int S, int kps, uint8_t* att,
+__device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, int hk, int qg, int gh, int s, int S, int kps, uint8_t* att,
                                             int wtid, unsigned long long* prof, int b) {
     constexpr bool TREE = MODE == 1, BATCH = MODE == 2;
     constexpr int HD2 = HD / 2;
@@ -903,7 +903,8 @@ __device__ __noinline__ void attention_unit(const FwdParams& P, int layer, int h
     }
 }
 
-__device__ void attention_phase(const FwdParams& P, int layer, uint8_t* att, int wtid, unsigned long long* prof) {
+template <int HD, int MODE>
+__device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, uint8_t* att, int wtid, unsigned long long* prof) {
     int S, kps;
     attn_split(P, S, kps);
     const int S1 = S + 1;
@@ -919,17 +920,8 @@ __device__ void attention_phase(const FwdParams& P, int layer, uint8_t* att, int
             qg = rem / S1;
             s = rem % S1;
         }
-        if (P.nseq > 0) {
-            // every sequence takes the key ranges of the longest one; a range past its own length holds no key
-            if (P.hd == 128) attention_unit<128, 2>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, b);
-            else attention_unit<64, 2>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, b);
-        } else if (P.tree) {
-            if (P.hd == 128) attention_unit<128, 1>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, 0);
-            else attention_unit<64, 1>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, 0);
-        } else {
-            if (P.hd == 128) attention_unit<128, 0>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, 0);
-            else attention_unit<64, 0>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, 0);
-        }
+        // batched: every sequence takes the key ranges of the longest one; a range past its own length holds no key
+        attention_unit<HD, MODE>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, b);
         named_bar_sync(1, kWorkerThreads);  // the unit's shared-memory tiles are free again
         if (prof && wtid == 0) { prof[6] = global_timer_ns(); prof[7] = (unsigned long long)(s == S); }
     }
@@ -977,6 +969,7 @@ __device__ __forceinline__ void advance_pos(PipePos& pos, const Part& pt, uint32
     pos.q += (uint32_t)pt.npass;
 }
 
+template <int NBT>
 __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int layer, uint8_t* smem, Misc* misc, PipePos& pos, int wtid,
                                         unsigned long long* prof) {
     const int warp = wtid >> 5, lane = wtid & 31;
@@ -988,67 +981,85 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int lay
     const bool have0 = p0.ntiles > 0 && p0.nk > 0;
     bool dead = *(volatile int*)&misc->abort_flag != 0;
     if (wtid == 0) misc->prof_ptr = prof;
-
-    if (warp == kMmaWarp) {
-        // the tensor-core warp builds nothing: it prepares its descriptors and meets the others at the
-        // operand barrier just before its first instruction
-        PipePos mp = pos;
-        mp.w_full = mp.w_acc = 0;
-        const long long tc0 = clock64();
-        bool synced = false;
-        for (int oi = 0; oi < nops; ++oi) {
-            const Part& pt = misc->part[ops[oi]];
-            if (pt.ntiles == 0 || pt.nk == 0) continue;
-            if (ops[oi] == OP_DOWN) {
-                if (prof && lane == 0) prof[5] = global_timer_ns();
-                if (!dead && !mbar_wait_bounded(&misc->act_ready, mp.act_uses & 1u, &misc->abort_flag, P.wait_limit_ns))
-                    dead = true;
-                dead = __any_sync(0xffffffffu, dead);
-                tc_fence_after();
-                if (prof && lane == 0) prof[6] = global_timer_ns();
-            }
-            mma_op(P, pt, smem, ops[oi] == OP_DOWN ? act : U, misc, mp, dead, synced);
-        }
-        if (!synced) named_bar_sync(1, kWorkerThreads);
-        if (prof && lane == 0) {
-            prof[3] = global_timer_ns();
-            prof[7] = mp.w_full;
-            prof[8] = mp.w_acc;
-            prof[9] = (unsigned long long)(clock64() - tc0);  // cycles of the whole issue loop
-        }
-    } else {
-        if (have0 && !dead) {
+    if (have0) {
+        if (!dead) {
             if (kind == PH_O) build_merged_operand(P, p0, U, wtid);
             else build_norm_operand(P, kind, layer, p0, U, misc, wtid);
-            fence_proxy_async_smem();
         }
-        if (kind == PH_O && warp >= 4) {
-            // clear the accumulators the next QKV projection adds into (idle warps)
-            const int n4 = kMaxRows * P.n_qkv / 4, nth = (kBuilderWarps - 4) * 32;
-            for (int i = blockIdx.x * nth + (wtid - 4 * 32); i < n4; i += P.G * nth)
-                __stcg(reinterpret_cast<float4*>(P.qkv_acc) + i, make_float4(0.f, 0.f, 0.f, 0.f));
-            if (blockIdx.x == 0 && wtid < 4 * 32 + kMaxRows)
-                __stcg(P.sumsq + ((layer + 1) & 1) * kMaxRows + (wtid - 4 * 32), 0.f);
-        }
-        named_bar_sync(1, kWorkerThreads);  // the operand is complete and visible to the tensor core
-        if (prof && wtid == 0) prof[2] = global_timer_ns();
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&misc->op_ready);   // this warp's part of the operand may be read by the tensor core
     }
+    if (kind == PH_O && warp >= 4) {
+        // clear the accumulators the next QKV projection adds into (idle warps)
+        const int n4 = kMaxRows * P.n_qkv / 4, nth = (kBuilderWarps - 4) * 32;
+        for (int i = blockIdx.x * nth + (wtid - 4 * 32); i < n4; i += P.G * nth)
+            __stcg(reinterpret_cast<float4*>(P.qkv_acc) + i, make_float4(0.f, 0.f, 0.f, 0.f));
+        if (blockIdx.x == 0 && wtid < 4 * 32 + kMaxRows)
+            __stcg(P.sumsq + ((layer + 1) & 1) * kMaxRows + (wtid - 4 * 32), 0.f);
+    }
+    if (prof && wtid == 0) prof[2] = global_timer_ns();
     if (warp < kEpilogueWarps) {
+        // the rows' sums of squares the epilogue scales with come from all builder warps
+        if (have0 && !dead && !mbar_wait_bounded(&misc->op_ready, pos.ops & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
         PipePos ep = pos;
-        if (P.NB == 32) epilogue_phase<32>(P, kind, layer, act, misc, ep, dead, warp, lane);
-        else epilogue_phase<16>(P, kind, layer, act, misc, ep, dead, warp, lane);
+        epilogue_phase<NBT>(P, kind, layer, act, misc, ep, dead, warp, lane);
         if (prof && wtid == 0) prof[4] = global_timer_ns();
     }
     // pipeline positions advance identically for every role
+    if (have0) ++pos.ops;
     for (int oi = 0; oi < nops; ++oi) {
         const Part& pt = misc->part[ops[oi]];
         if (pt.ntiles == 0 || pt.nk == 0) continue;
         advance_pos(pos, pt, (uint32_t)P.nstage);
-        if (ops[oi] == OP_GU) ++pos.act_uses;
     }
 }
 
+// The tensor-core thread: all operations of the launch in order.  It waits for operands, never for grid barriers.
+__device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc* misc) {
+    PipePos pos;
+    pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
+    uint32_t act_uses = 0;
+    bool dead = false, ready = false;
+    for (int ph = P.ph_begin; ph < P.ph_end && !dead; ++ph) {
+        int layer, ops[2];
+        const int kind = decode_phase(ph, P.n_layers, layer);
+        const int nops = phase_ops(kind, ops);
+        unsigned long long* prof = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
+        pos.w_full = pos.w_acc = 0;
+        long long tc0 = 0;
+        for (int oi = 0; oi < nops && !dead; ++oi) {
+            const Part& pt = misc->part[ops[oi]];
+            if (pt.ntiles == 0 || pt.nk == 0) continue;
+            const bool down = ops[oi] == OP_DOWN;
+            if (down && prof) prof[5] = global_timer_ns();
+            if (!mbar_wait_bounded(down ? &misc->act_ready : &misc->op_ready, (down ? act_uses++ : pos.ops++) & 1u, &misc->abort_flag,
+                                   P.wait_limit_ns)) {
+                dead = true;
+                break;
+            }
+            tc_fence_after();
+            if (prof) {
+                if (down) prof[6] = global_timer_ns();
+                else tc0 = clock64();
+            }
+            mma_op(P, pt, smem, smem + (down ? P.act_off : P.u_off), misc, pos, dead, ready);
+        }
+        if (prof && nops > 0) {
+            prof[3] = global_timer_ns();
+            prof[7] = pos.w_full;
+            prof[8] = pos.w_acc;
+            prof[9] = (unsigned long long)(clock64() - tc0);  // cycles of the whole issue loop
+        }
+    }
+    // all tensor-core work must have completed before tensor memory is returned
+    umma_commit(&misc->done_bar);
+    mbar_wait_bounded(&misc->done_bar, 0, &misc->abort_flag, P.wait_limit_ns);
+}
+
 // ------------------------------------------------------------------------------------------
+// NBT: N of the tensor-core instruction (16 or 32); HD: head dimension; MODE: chain, tree or batch (see attention_unit).
+template <int NBT, int HD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg) {
     static_assert(sizeof(FwdParams) % 4 == 0, "parameter block is copied word by word");
     extern __shared__ uint8_t smem_raw[];
@@ -1077,6 +1088,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
             mbar_init(&misc->tmem_full[b], 1);
             mbar_init(&misc->tmem_empty[b], kEpilogueWarps);
         }
+        mbar_init(&misc->op_ready, kBuilderWarps);
         mbar_init(&misc->act_ready, kEpilogueWarps);
         mbar_init(&misc->done_bar, 1);
         misc->abort_flag = 0;
@@ -1108,10 +1120,19 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         if (lane == 0) producer_loop(P, smem, misc);
         return;
     }
+    if (warp == kMmaWarp) {
+        if (elect_one()) mma_loop(P, smem, misc);
+        __syncwarp();
+        tc_fence_before();
+        named_bar_sync(3, kWorkerThreads + 32);   // the workers have read the last accumulators
+        tc_fence_after();
+        tmem_dealloc(misc->tmem_base, kTmemCols);
+        return;
+    }
 
     const int wtid = tid;  // 0 .. kWorkerThreads-1
     PipePos pos;
-    pos.slot = pos.par = pos.q = pos.act_uses = pos.w_full = pos.w_acc = 0;
+    pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
     int nbar = 0;
     bool skip = false;
     for (int ph = P.ph_begin; ph < P.ph_end; ++ph) {
@@ -1125,9 +1146,9 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
             embed_phase(P, wtid);
             zero_qkv_acc(P, 0, wtid);
         } else if (kind == PH_ATTN) {
-            attention_phase(P, layer, smem + P.u_off, wtid, pp);
+            attention_phase<HD, MODE>(P, layer, smem + P.u_off, wtid, pp);
         } else {
-            gemm_phase(P, kind, layer, smem, misc, pos, wtid, pp);
+            gemm_phase<NBT>(P, kind, layer, smem, misc, pos, wtid, pp);
         }
         if (pp) {
             named_bar_sync(1, kWorkerThreads);
@@ -1138,15 +1159,8 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
             skip = grid_barrier(P, P.bar_base + (unsigned)(nbar * P.G), misc, wtid);
         }
     }
-    // all tensor-core work must have completed before tensor memory is returned
-    if (warp == kMmaWarp && lane == 0) {
-        umma_commit(&misc->done_bar);
-        mbar_wait_bounded(&misc->done_bar, 0, &misc->abort_flag, P.wait_limit_ns);
-    }
     tc_fence_before();
-    named_bar_sync(1, kWorkerThreads);
-    tc_fence_after();
-    if (warp == kMmaWarp) tmem_dealloc(misc->tmem_base, kTmemCols);
+    named_bar_sync(3, kWorkerThreads + 32);
     if (*(volatile int*)&misc->abort_flag) {
         if (wtid == 0) atomicExch(P.state + ST_ERR, 1);
     }

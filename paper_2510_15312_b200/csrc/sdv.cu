@@ -299,14 +299,26 @@ int cuda_fail(sdv_ctx* ctx, cudaError_t e) {
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_); \
     } while (0)
 
+typedef void (*ForwardKernel)(const FwdParams);
+// The forward kernel compiled for this launch's instruction width, head dimension and kind of attention.
+ForwardKernel forward_kernel(const FwdParams& P) {
+    const int mode = P.nseq > 0 ? 2 : (P.tree ? 1 : 0);
+    static const ForwardKernel table[2][2][3] = {
+        {{sdv_forward_kernel<16, 64, 0>, sdv_forward_kernel<16, 64, 1>, sdv_forward_kernel<16, 64, 2>},
+         {sdv_forward_kernel<16, 128, 0>, sdv_forward_kernel<16, 128, 1>, sdv_forward_kernel<16, 128, 2>}},
+        {{sdv_forward_kernel<32, 64, 0>, sdv_forward_kernel<32, 64, 1>, sdv_forward_kernel<32, 64, 2>},
+         {sdv_forward_kernel<32, 128, 0>, sdv_forward_kernel<32, 128, 1>, sdv_forward_kernel<32, 128, 2>}}};
+    return table[P.NB == 32][P.hd == 128][mode];
+}
 cudaError_t launch_kernel(const FwdParams& P, int smem_bytes, cudaStream_t stream) {
-    cudaError_t e = cudaFuncSetAttribute(sdv_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    const ForwardKernel k = forward_kernel(P);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&P};
     // phases meet at grid barriers, so more than one phase needs all blocks co-resident
     if (P.ph_end - P.ph_begin > 1)
-        return cudaLaunchCooperativeKernel((const void*)sdv_forward_kernel, dim3(P.G), dim3(kThreads), args, smem_bytes, stream);
-    return cudaLaunchKernel((const void*)sdv_forward_kernel, dim3(P.G), dim3(kThreads), args, smem_bytes, stream);
+        return cudaLaunchCooperativeKernel((const void*)k, dim3(P.G), dim3(kThreads), args, smem_bytes, stream);
+    return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, smem_bytes, stream);
 }
 
 bool apply_plan(FwdParams& P, int rows, bool raw_only, int* smem_bytes) {
