@@ -104,34 +104,86 @@ __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target
 }
 
 // ------------------------------------------------------------------------------------------
-// Weight streamer (one thread).
+// Weight streamer (one thread).  The ring holds 128 KB of the 590 KB a layer of the 1.5B shape streams per block, and HBM
+// would idle through the attention half of a layer (24 us) once it is full.  So while the streamer waits for a free slot it reads
+// ahead into L2, at most kLookaheadBytes beyond the ring and no faster than one piece per kLookaheadCycles (1.5 TB/s over the
+// grid): a burst would queue in front of the other warps' loads, which cost more than it gave, the trickle does not.
+// 10050 -> 9680 us for eight steps of the 1.5B shape, 12130 -> 11970 us for four of the 7B shape; 128 KB: 9720, 256 KB: 9660.
+struct Lookahead {   // cursor over the block's weight stream: operation by operation, each one contiguous range of bytes
+    int ph, oi;
+    const uint8_t* src;
+    unsigned long long begin, end;   // the running operation's place in the stream
+};
+__device__ __forceinline__ bool lookahead_next(const FwdParams& P, Misc* misc, Lookahead& c) {
+    for (;;) {
+        int layer, ops[2];
+        if (c.ph >= P.ph_end) return false;
+        const int nops = phase_ops(decode_phase(c.ph, P.n_layers, layer), ops);
+        if (++c.oi >= nops) { c.oi = -1; ++c.ph; continue; }
+        const Part& pt = misc->part[ops[c.oi]];
+        if (pt.ntiles == 0 || pt.nk == 0) continue;
+        c.src = op_weights(P, ops[c.oi], layer) + pt.off;
+        c.begin = c.end;
+        c.end += (unsigned long long)pt.ntiles * pt.nk * kStepBytes;
+        return true;
+    }
+}
 __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem, Misc* misc) {
     const uint64_t policy = l2_policy_evict_first();
     const uint32_t nstage = (uint32_t)P.nstage;
     uint32_t slot = 0, par = 0, issued = 0;  // ring position; parity of the current trip round the ring
     bool ok = true;
+    unsigned long long streamed = 0, ahead = 0;   // bytes copied / read ahead so far
+    Lookahead la;
+    la.ph = P.ph_begin; la.oi = -1; la.begin = la.end = 0; la.src = nullptr;
+    bool more = lookahead_next(P, misc, la);
+    long long last = clock64();
+#pragma unroll 1
     for (int ph = P.ph_begin; ph < P.ph_end && ok; ++ph) {
         int layer, ops[2];
         const int kind = decode_phase(ph, P.n_layers, layer);
         const int nops = phase_ops(kind, ops);
+#pragma unroll 1
         for (int oi = 0; oi < nops && ok; ++oi) {
             const Part& pt = misc->part[ops[oi]];
             if (pt.ntiles == 0 || pt.nk == 0) continue;
             const uint8_t* src = op_weights(P, ops[oi], layer) + pt.off;
             const int nst = pt.nst, SK = pt.SK, nk = pt.nk;
+#pragma unroll 1
             for (int p = 0; p < pt.npass && ok; ++p) {
                 const uint32_t pbytes = (uint32_t)pass_count(pt, p) * kStepBytes;
                 int kleft = nk;
+#pragma unroll 1
                 for (int st = 0; st < nst; ++st, kleft -= SK) {
                     const uint32_t bytes = pbytes * (uint32_t)min(SK, kleft);
                     // the slot's previous contents must have been consumed (first trip: free at once)
-                    if (!mbar_wait_bounded(&misc->empty[slot], par ^ 1u, &misc->abort_flag, P.wait_limit_ns)) {
-                        ok = false;
-                        break;
+                    uint64_t t0 = 0;
+                    uint32_t spins = 0;
+                    while (!mbar_test(&misc->empty[slot], par ^ 1u)) {
+                        const long long now = clock64();
+                        if (now - last > kLookaheadCycles && more) {
+                            if (ahead < streamed) ahead = streamed;
+                            while (more && ahead >= la.end) more = lookahead_next(P, misc, la);
+                            if (more && ahead < streamed + kLookaheadBytes) {
+                                const unsigned long long left = la.end - ahead;
+                                const uint32_t piece = left < kLookaheadPiece ? (uint32_t)left : kLookaheadPiece;
+                                bulk_prefetch_l2(la.src + (ahead - la.begin), piece);
+                                ahead += piece;
+                                last = now;
+                            }
+                        }
+                        if ((++spins & 255u) == 0) {
+                            if (*(volatile int*)&misc->abort_flag) { ok = false; break; }
+                            const uint64_t t = global_timer_ns();
+                            if (t0 == 0) t0 = t;
+                            if (t - t0 > P.wait_limit_ns) { *(volatile int*)&misc->abort_flag = 1; ok = false; break; }
+                        }
                     }
+                    if (!ok) break;
                     mbar_arrive_expect_tx(&misc->full[slot], bytes);
                     bulk_g2s(smem + slot * kStageBytes, src, bytes, &misc->full[slot], policy);
                     src += bytes;
+                    streamed += bytes;
                     ++issued;
                     if (++slot == nstage) { slot = 0; par ^= 1u; }
                 }
@@ -180,11 +232,13 @@ __device__ __forceinline__ void build_norm_operand(const FwdParams& P, int kind,
     const float* xbase = raw ? P.raw_x : P.h;
     const float* wn = raw ? nullptr
                           : P.norm_w + (size_t)(kind == PH_QKV ? layer * 2 : (kind == PH_GUD ? layer * 2 + 1 : P.n_layers * 2)) * P.d;
+#pragma unroll 1
     for (int row = warp; row < M; row += kBuilderWarps) {
         const float4* src = reinterpret_cast<const float4*>(xbase + (size_t)row * stride) + k4_0;
         const float4* wsrc = wn ? reinterpret_cast<const float4*>(wn) + k4_0 : nullptr;
         const float4* wld = wsrc ? wsrc : src;  // without norm weights the loaded value is not used
         float ss = 0.f;
+#pragma unroll 1
         for (int base = lane; base < nk4; base += 32 * UB) {
             float4 a[UB], w[UB];
             // every unit loads (past the end: the row's last unit again, not used), so that the loads are one
@@ -229,6 +283,7 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
     const int M = P.M, hd = P.hd;
     const int k8_0 = pt.k0 * 2, nk8 = pt.nk * 2;
     const int nitems = M * nk8, sub = wtid & 3;
+#pragma unroll 1
     for (int it0 = 0; it0 < nitems; it0 += kBuilderWarps * 32 / 4) {
         const int item = it0 + (wtid >> 2);
         const bool live = item < nitems;
@@ -306,9 +361,11 @@ __device__ __forceinline__ void mma_stage(uint32_t d_tmem, uint64_t adesc, uint6
         bdesc += bstep;
     };
     int ks = 0;
+#pragma unroll 1
     for (; ks + 4 <= nks; ks += 4) {
         step(); step(); step(); step();
     }
+#pragma unroll 1
     for (; ks < nks; ++ks) step();
 }
 
@@ -323,19 +380,22 @@ __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8
     const uint32_t ring0 = smem_u32(smem);
     const uint32_t tmem0 = misc->tmem_base;
     const int nst = pt.nst, SK = pt.SK, nk = pt.nk, npass = pt.npass;
+#pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
         const int pcount = pass_count(pt, p);
         const uint32_t buf = pos.q & 1u;
-        const long long tq0 = clock64();
-        if (!dead && !mbar_wait_bounded(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u, &misc->abort_flag, wait_limit))
-            dead = true;
-        pos.w_acc += (uint32_t)(clock64() - tq0);
+        if (!dead && !mbar_test(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u)) {
+            const long long tq0 = clock64();
+            if (!mbar_wait_bounded(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u, &misc->abort_flag, wait_limit)) dead = true;
+            pos.w_acc += (uint32_t)(clock64() - tq0);
+        }
         const uint32_t d_tmem = tmem0 + buf * 64u;
         const uint32_t lbo_a = (uint32_t)(2 * pcount) * 128u;
         const uint64_t astep = (uint64_t)((2u * lbo_a) >> 4);
         const uint64_t adesc0 = umma_smem_desc(ring0, lbo_a, 128u);
         uint64_t bdesc = bdesc0;
         int kleft = nk;
+#pragma unroll 1
         for (int st = 0; st < nst; ++st, kleft -= SK) {
             const uint32_t slot = pos.slot, par = pos.par;
             if (++pos.slot == nstage) { pos.slot = 0; pos.par ^= 1u; }
@@ -363,17 +423,17 @@ __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8
 
 // ------------------------------------------------------------------------------------------
 // Epilogues (warps 0..7).  Thread t = 32 * (warp & 3) + lane owns row t of its 128-row accumulator,
-// i.e. one weight row (output feature), for the token columns its warp group takes.
+// i.e. one weight row (output feature), for the token columns its warp group takes.  Token columns are taken 16 at a time.
 // SwiGLU on one accumulator row per thread.  Rows 0..7 of a 16-row tile are gate rows, rows 8..15 the
 // matching up rows, so the two values of an output sit 8 lanes apart.  Token columns are taken in
 // pairs: the gate lane evaluates the even column of a pair, the up lane the odd one; one shuffle per
 // pair hands each lane the partner's value it needs.  All pairs are independent and written without
 // branches, so that their shuffles, exponentials and divisions overlap.  SEL >= 0: only pairs j with
-// (j & 1) == SEL (the other group of epilogue warps takes the rest).
-template <int NBT, int SEL>
-__device__ __forceinline__ void swiglu_pairs(const float (&v)[NBT], const float (&rstd)[NBT], int t, bool valid, int M,
-                                             uint8_t* dst) {
-    constexpr int STEP = SEL < 0 ? 1 : 2, J0 = SEL < 0 ? 0 : SEL, NP = (NBT / 2 - J0 + STEP - 1) / STEP;
+// (j & 1) == SEL (the other group of epilogue warps takes the rest).  rs: lane n holds the norm factor of token n;
+// n0: first token column of v, M: token columns from there on.
+template <int SEL>
+__device__ __forceinline__ void swiglu_pairs(const float (&v)[16], float rs, int n0, int t, bool valid, int M, uint8_t* dst) {
+    constexpr int STEP = SEL < 0 ? 1 : 2, J0 = SEL < 0 ? 0 : SEL, NP = (8 - J0 + STEP - 1) / STEP;
     const bool is_up = (t & 8) != 0;
     float got[NP], out[NP];
 #pragma unroll
@@ -384,7 +444,7 @@ __device__ __forceinline__ void swiglu_pairs(const float (&v)[NBT], const float 
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
         const int j = J0 + i * STEP;
-        const float mine = is_up ? v[2 * j + 1] : v[2 * j], r = is_up ? rstd[2 * j + 1] : rstd[2 * j];
+        const float mine = is_up ? v[2 * j + 1] : v[2 * j], r = __shfl_sync(0xffffffffu, rs, n0 + 2 * j + (is_up ? 1 : 0));
         const float x = (is_up ? got[i] : mine) * r, y = (is_up ? mine : got[i]) * r;
         out[i] = __fdividef(x, 1.f + __expf(-x)) * y;
     }
@@ -395,30 +455,32 @@ __device__ __forceinline__ void swiglu_pairs(const float (&v)[NBT], const float 
     }
 }
 
-// LM: the operation is the LM head (bv / bi carry the running best logit per token row); the other operations
-// are compiled without that state, which would otherwise occupy 2 x NBT registers through every phase.
-template <int NBT, bool LM>  // NBT: token columns read, 16 or 32
-__device__ __forceinline__ void epilogue_op(const FwdParams& P, int kind, int op, int layer, const Part& pt, uint8_t* act, Misc* misc,
-                                            PipePos& pos, bool& dead, int warp, int lane, float (&bv)[LM ? NBT : 1],
-                                            int (&bi)[LM ? NBT : 1]) {
+// Running best logit of each token row (LM head), per thread.
+struct Best {
+    float v[2][16];
+    int i[2][16];
+};
+
+// LM: the operation is the LM head (`best` carries the running best logits); the other operations are compiled
+// without that state.
+template <bool LM>
+__device__ __forceinline__ void epilogue_op(const FwdParams& P, int op, const Part& pt, uint8_t* act, Misc* misc, PipePos& pos, bool& dead,
+                                            int warp, int lane, Best& best) {
     const int M = P.M;
     const int quarter = warp & 3, myhalf = warp >> 2;  // this warp's 32 accumulator lanes; which of the two accumulators
     const int t = quarter * 32 + lane;
     const uint64_t wait_limit = P.wait_limit_ns;
     const uint32_t tmem_lane = misc->tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const int npass = pt.npass, tile0 = pt.tile0;
-    float rstd[NBT];
-    if (op == OP_GU || LM) {
-        const float inv_d = 1.f / (float)P.d, eps = P.eps;
-#pragma unroll
-        for (int n = 0; n < NBT; ++n) rstd[n] = (n < M) ? rsqrtf(misc->sumsq[n] * inv_d + eps) : 0.f;
-    }
+    const int npass = pt.npass, tile0 = pt.tile0, nchunk = M > 16 ? 2 : 1;
+    float rs = 0.f;   // lane n: norm factor of token n
+    if ((op == OP_GU || LM) && lane < M) rs = rsqrtf(misc->sumsq[lane] * (1.f / (float)P.d) + P.eps);
     float* out = P.h;
     int stride = P.d;
     bool add = true;  // residual add (O, down)
     if (op == OP_QKV) { out = P.qkv_acc; stride = P.n_qkv; add = P.op[OP_QKV].P_k > 1; }
     else if (op == OP_RAW) { out = P.raw_out; stride = P.raw_N; add = P.op[OP_RAW].P_k > 1; }
     const int store_logits = P.store_logits;
+#pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
         const int pcount = pass_count(pt, p), pstart = pass_start(pt, p);
         const uint32_t buf = pos.q & 1u;
@@ -431,56 +493,52 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, int kind, int op
         // two accumulators: warps 0..3 read the first, 4..7 the second; one accumulator: both groups read
         // it and share its token columns (pairs of columns alternate between the groups)
         const int nsel = (nhalf == 2) ? -1 : myhalf;
-        {
-            const int half = (nhalf == 2) ? myhalf : 0;
-            float v[NBT];
-            {
-                const uint32_t taddr = tmem_lane + buf * 64u + (uint32_t)half * 32u;
-                float lo[16];
-                tmem_ld16(taddr, lo);
+        const int half = (nhalf == 2) ? myhalf : 0;
+        const uint32_t taddr = tmem_lane + buf * 64u + (uint32_t)half * 32u;
+        const int tt = half * 128 + t;         // row within the pass
+        const bool valid = tt < 16 * pcount;
+        const int row = (tile0 + pstart) * 16 + tt;  // weight row = output feature
 #pragma unroll
-                for (int n = 0; n < 16; ++n) v[n] = lo[n];
-                if (NBT == 32) {
-                    float hi[16];
-                    tmem_ld16(taddr + 16u, hi);
-#pragma unroll
-                    for (int n = 0; n < 16; ++n) v[(NBT == 32 ? 16 : 0) + n] = hi[n];
+        for (int h = 0; h < 2; ++h) {
+            if (h == 0 || nchunk == 2) {
+                float v[16];
+                tmem_ld16(taddr + (uint32_t)(h * 16), v);
+                if (h + 1 == nchunk) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&misc->tmem_empty[buf]);  // this warp's part of the accumulators may be overwritten
                 }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&misc->tmem_empty[buf]);  // this warp's part of the accumulators may be overwritten
-            const int tt = half * 128 + t;         // row within the pass
-            const bool valid = tt < 16 * pcount;
-            const int row = (tile0 + pstart) * 16 + tt;  // weight row = output feature
-            if (!LM && op == OP_GU) {
-                // rows 0..7 of a tile are gate rows, 8..15 the matching up rows, 8 lanes apart: the gate
-                // lane evaluates the even token columns, the up lane the odd ones
-                const int col = (pstart + (tt >> 4)) * 8 + (tt & 7);  // SwiGLU column within this block's slice
-                uint8_t* dst = act + operand_off(col >> 3, 0, M) + (col & 7) * 2;
-                if (nsel < 0) swiglu_pairs<NBT, -1>(v, rstd, t, valid, M, dst);
-                else if (nsel == 0) swiglu_pairs<NBT, 0>(v, rstd, t, valid, M, dst);
-                else swiglu_pairs<NBT, 1>(v, rstd, t, valid, M, dst);
-            } else if (LM) {
+                const int n0 = h * 16, Mh = M - n0;
+                if (LM) {
 #pragma unroll
-                for (int n = 0; n < NBT; ++n) {
-                    if (valid && n < M && (nsel < 0 || ((n >> 1) & 1) == nsel)) {
-                        const float x = v[n] * rstd[n];
-                        if (store_logits) __stcg(P.logits + (size_t)n * P.V + row, x);
-                        // rows come in ascending order per thread, so ">" keeps the lowest id among equals
-                        if (x > bv[LM ? n : 0]) { bv[LM ? n : 0] = x; bi[LM ? n : 0] = row; }
+                    for (int n = 0; n < 16; ++n) {
+                        const float r = __shfl_sync(0xffffffffu, rs, n0 + n);
+                        if (valid && n < Mh && (nsel < 0 || ((n >> 1) & 1) == nsel)) {
+                            const float x = v[n] * r;
+                            if (store_logits) __stcg(P.logits + (size_t)(n0 + n) * P.V + row, x);
+                            // rows come in ascending order per thread, so ">" keeps the lowest id among equals
+                            if (x > best.v[h][n]) { best.v[h][n] = x; best.i[h][n] = row; }
+                        }
                     }
-                }
-            } else if (valid) {
-                float* d2 = out + row;
-                if (add) {
+                } else if (op == OP_GU) {
+                    // rows 0..7 of a tile are gate rows, 8..15 the matching up rows, 8 lanes apart: the gate
+                    // lane evaluates the even token columns, the up lane the odd ones
+                    const int col = (pstart + (tt >> 4)) * 8 + (tt & 7);  // SwiGLU column within this block's slice
+                    uint8_t* dst = act + operand_off(col >> 3, n0, M) + (col & 7) * 2;
+                    if (nsel < 0) swiglu_pairs<-1>(v, rs, n0, t, valid, Mh, dst);
+                    else if (nsel == 0) swiglu_pairs<0>(v, rs, n0, t, valid, Mh, dst);
+                    else swiglu_pairs<1>(v, rs, n0, t, valid, Mh, dst);
+                } else if (valid) {
+                    float* d2 = out + (size_t)n0 * stride + row;
+                    if (add) {
 #pragma unroll
-                    for (int n = 0; n < NBT; ++n, d2 += stride)
-                        if (n < M && (nsel < 0 || ((n >> 1) & 1) == nsel)) red_add_f32(d2, v[n]);
-                } else {
+                        for (int n = 0; n < 16; ++n, d2 += stride)
+                            if (n < Mh && (nsel < 0 || ((n >> 1) & 1) == nsel)) red_add_f32(d2, v[n]);
+                    } else {
 #pragma unroll
-                    for (int n = 0; n < NBT; ++n, d2 += stride)
-                        if (n < M && (nsel < 0 || ((n >> 1) & 1) == nsel)) __stcg(d2, v[n]);
+                        for (int n = 0; n < 16; ++n, d2 += stride)
+                            if (n < Mh && (nsel < 0 || ((n >> 1) & 1) == nsel)) __stcg(d2, v[n]);
+                    }
                 }
             }
         }
@@ -493,30 +551,31 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, int kind, int op
     }
 }
 
-// Best logit per token row over the block: lanes, then the four epilogue warps.
-template <int NBT>
-__device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, int warp, int lane, float (&bv)[NBT], int (&bi)[NBT],
-                                              bool dead) {
+// Best logit per token row over the block: lanes, then the eight epilogue warps.
+__device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, int warp, int lane, const Best& best, bool dead) {
 #pragma unroll
-    for (int n = 0; n < NBT; ++n) {
-        float v = bv[n];
-        int i = bi[n];
+    for (int n = 0; n < kMaxRows; ++n) {
+        if (n < P.M) {
+            float v = best.v[n >> 4][n & 15];
+            int i = best.i[n >> 4][n & 15];
 #pragma unroll
-        for (int off = 1; off <= 16; off <<= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, v, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, i, off);
-            if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
-        }
-        if (lane == 0) {
-            misc->best_v[warp][n] = v;
-            misc->best_i[warp][n] = i;
+            for (int off = 1; off <= 16; off <<= 1) {
+                const float ov = __shfl_xor_sync(0xffffffffu, v, off);
+                const int oi = __shfl_xor_sync(0xffffffffu, i, off);
+                if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
+            }
+            if (lane == 0) {
+                misc->best_v[warp][n] = v;
+                misc->best_i[warp][n] = i;
+            }
         }
     }
     named_bar_sync(2, kEpilogueWarps * 32);
     const int t = warp * 32 + lane;
-    if (t < NBT && t < P.M && !dead) {
+    if (t < P.M && !dead) {
         float v = misc->best_v[0][t];
         int i = misc->best_i[0][t];
+#pragma unroll 1
         for (int w = 1; w < kEpilogueWarps; ++w) {
             const float ov = misc->best_v[w][t];
             const int oi = misc->best_i[w][t];
@@ -527,27 +586,24 @@ __device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, in
     }
 }
 
-template <int NBT>
-__device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, int layer, uint8_t* act, Misc* misc, PipePos& pos,
-                                            bool& dead, int warp, int lane) {
+__device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, uint8_t* act, Misc* misc, PipePos& pos, bool& dead, int warp,
+                                               int lane) {
+    Best best;
     if (kind == PH_LM) {
-        float bv[NBT];
-        int bi[NBT];
 #pragma unroll
-        for (int n = 0; n < NBT; ++n) { bv[n] = -CUDART_INF_F; bi[n] = 0x7fffffff; }
+        for (int n = 0; n < kMaxRows; ++n) { best.v[n >> 4][n & 15] = -CUDART_INF_F; best.i[n >> 4][n & 15] = 0x7fffffff; }
         const Part& pt = misc->part[OP_LM];
-        if (pt.ntiles > 0 && pt.nk > 0) epilogue_op<NBT, true>(P, kind, OP_LM, layer, pt, act, misc, pos, dead, warp, lane, bv, bi);
-        argmax_finish<NBT>(P, misc, warp, lane, bv, bi, dead);
+        if (pt.ntiles > 0 && pt.nk > 0) epilogue_op<true>(P, OP_LM, pt, act, misc, pos, dead, warp, lane, best);
+        argmax_finish(P, misc, warp, lane, best, dead);
         return;
     }
-    float none_v[1];
-    int none_i[1];
     int ops[2];
     const int nops = phase_ops(kind, ops);
+#pragma unroll 1
     for (int oi = 0; oi < nops; ++oi) {
         const Part& pt = misc->part[ops[oi]];
         if (pt.ntiles == 0 || pt.nk == 0) continue;
-        epilogue_op<NBT, false>(P, kind, ops[oi], layer, pt, act, misc, pos, dead, warp, lane, none_v, none_i);
+        epilogue_op<false>(P, ops[oi], pt, act, misc, pos, dead, warp, lane, best);
     }
 }
 
@@ -654,6 +710,7 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
     {
         constexpr int QI = 2;  // items per thread and batch: all loads are issued before the first use
         const int items = RP * (HD2 / 4);
+#pragma unroll 1
         for (int base = wtid; base < items; base += QI * kWorkerThreads) {
             float4 qa[QI], qb[QI], c0[QI], c1[QI];
             float ssq[QI];
@@ -709,6 +766,7 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
         uint8_t* Ks = KVs;
         uint8_t* Vs = Ks + KVBYTES;
         // K and V rows of the new tokens: finish the projection, rotate K, append to the cache
+#pragma unroll 1
         for (int u = wtid; u < KB * UNITS; u += kWorkerThreads) {
             const int key = u / UNITS, q16 = u % UNITS, kk = key;
             uint4 kv4 = make_uint4(0, 0, 0, 0), vv4 = make_uint4(0, 0, 0, 0);
@@ -769,12 +827,14 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
     float m_lo = -CUDART_INF_F, m_hi = -CUDART_INF_F, l_lo = 0.f, l_hi = 0.f;
     const uint32_t qb = smem_u32(Qs);
 
+#pragma unroll 1
     for (int blk = 0; blk < nblk; ++blk) {
         if (!is_new) cp_async_wait<NBUF - 1>();
         named_bar_sync(1, kWorkerThreads);  // the block (and, first time, the Q tile) is in place
         if (prof && wtid == 0 && blk == 0) prof[4] = global_timer_ns();
         if (active) {
             const uint32_t kb = smem_u32(KVs + (blk % NBUF) * 2 * KVBYTES), vb = kb + KVBYTES;
+#pragma unroll 1
             for (int c = kgp; c < KB / 16; c += KG) {
                 if (blk * KB + c * 16 >= nkeys) break;
                 // ---- scores of 16 rows x 16 keys
@@ -862,6 +922,7 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
         }
         named_bar_sync(1, kWorkerThreads);
         if (active && kgp == 0) {
+#pragma unroll 1
             for (int og = 0; og < KG - 1; ++og) {
                 const float4 ml = ex_ml[(og * MT + mt) * 32 + lane];
                 const float mn_lo = fmaxf(m_lo, ml.x), mn_hi = fmaxf(m_hi, ml.y);
@@ -911,6 +972,7 @@ __device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, u
     const int gh = P.att_gh, QG = P.att_QG;
     const int per_seq = P.att_per_seq;
     const int nunits = per_seq * (P.nseq > 0 ? P.nseq : 1);
+#pragma unroll 1
     for (int unit = blockIdx.x; unit < nunits; unit += P.G) {
         int b = P.att_b0, hk = P.att_hk0, qg = P.att_qg0, s = P.att_s0;
         if (unit != (int)blockIdx.x) {  // further units of this block (more units than blocks: batched steps)
@@ -930,6 +992,7 @@ __device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, u
 __device__ void embed_phase(const FwdParams& P, int wtid) {
     // residual rows from the embedding table; rows beyond M are cleared
     const int units = kMaxRows * (P.d / 8);
+#pragma unroll 1
     for (int u = blockIdx.x * kWorkerThreads + wtid; u < units; u += P.G * kWorkerThreads) {
         const int row = u / (P.d / 8), c8 = u % (P.d / 8);
         float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
@@ -953,6 +1016,7 @@ __device__ void embed_phase(const FwdParams& P, int wtid) {
 }
 __device__ void zero_qkv_acc(const FwdParams& P, int sumsq_buf, int wtid) {
     const int n4 = kMaxRows * P.n_qkv / 4;
+#pragma unroll 1
     for (int i = blockIdx.x * kWorkerThreads + wtid; i < n4; i += P.G * kWorkerThreads)
         __stcg(reinterpret_cast<float4*>(P.qkv_acc) + i, make_float4(0.f, 0.f, 0.f, 0.f));
     if (blockIdx.x == 0 && wtid < kMaxRows) __stcg(P.sumsq + sumsq_buf * kMaxRows + wtid, 0.f);
@@ -969,7 +1033,6 @@ __device__ __forceinline__ void advance_pos(PipePos& pos, const Part& pt, uint32
     pos.q += (uint32_t)pt.npass;
 }
 
-template <int NBT>
 __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int layer, uint8_t* smem, Misc* misc, PipePos& pos, int wtid,
                                         unsigned long long* prof) {
     const int warp = wtid >> 5, lane = wtid & 31;
@@ -993,6 +1056,7 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int lay
     if (kind == PH_O && warp >= 4) {
         // clear the accumulators the next QKV projection adds into (idle warps)
         const int n4 = kMaxRows * P.n_qkv / 4, nth = (kBuilderWarps - 4) * 32;
+#pragma unroll 1
         for (int i = blockIdx.x * nth + (wtid - 4 * 32); i < n4; i += P.G * nth)
             __stcg(reinterpret_cast<float4*>(P.qkv_acc) + i, make_float4(0.f, 0.f, 0.f, 0.f));
         if (blockIdx.x == 0 && wtid < 4 * 32 + kMaxRows)
@@ -1003,11 +1067,12 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int lay
         // the rows' sums of squares the epilogue scales with come from all builder warps
         if (have0 && !dead && !mbar_wait_bounded(&misc->op_ready, pos.ops & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
         PipePos ep = pos;
-        epilogue_phase<NBT>(P, kind, layer, act, misc, ep, dead, warp, lane);
+        epilogue_phase(P, kind, act, misc, ep, dead, warp, lane);
         if (prof && wtid == 0) prof[4] = global_timer_ns();
     }
     // pipeline positions advance identically for every role
     if (have0) ++pos.ops;
+#pragma unroll 1
     for (int oi = 0; oi < nops; ++oi) {
         const Part& pt = misc->part[ops[oi]];
         if (pt.ntiles == 0 || pt.nk == 0) continue;
@@ -1021,6 +1086,7 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
     pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
     uint32_t act_uses = 0;
     bool dead = false, ready = false;
+#pragma unroll 1
     for (int ph = P.ph_begin; ph < P.ph_end && !dead; ++ph) {
         int layer, ops[2];
         const int kind = decode_phase(ph, P.n_layers, layer);
@@ -1028,7 +1094,9 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
         unsigned long long* prof = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
         pos.w_full = pos.w_acc = 0;
         long long tc0 = 0;
-        for (int oi = 0; oi < nops && !dead; ++oi) {
+#pragma unroll 1
+    #pragma unroll 1
+    for (int oi = 0; oi < nops && !dead; ++oi) {
             const Part& pt = misc->part[ops[oi]];
             if (pt.ntiles == 0 || pt.nk == 0) continue;
             const bool down = ops[oi] == OP_DOWN;
@@ -1058,13 +1126,13 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
 }
 
 // ------------------------------------------------------------------------------------------
-// NBT: N of the tensor-core instruction (16 or 32); HD: head dimension; MODE: chain, tree or batch (see attention_unit).
-template <int NBT, int HD, int MODE>
+// HD: head dimension; MODE: chain, tree or batch (see attention_unit).
+template <int HD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg) {
     static_assert(sizeof(FwdParams) % 4 == 0, "parameter block is copied word by word");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    Misc* misc = reinterpret_cast<Misc*>(smem + Pg.misc_off);
+    Misc* misc = reinterpret_cast<Misc*>(smem + kMiscOff);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (Pg.l_from_state && Pg.state[ST_BUDGET] == 0) {
         // a step enqueued behind the end of its run: nothing to do, but the barrier counter moves as the host assumed
@@ -1076,7 +1144,19 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         int* dst = reinterpret_cast<int*>(&misc->P);
         for (int i = tid; i < (int)(sizeof(FwdParams) / 4); i += kThreads) dst[i] = src[i];
     }
+    __syncthreads();
     const FwdParams& P = misc->P;
+    if (tid == 0) {
+        // Rows past the draft the device holds would be padding: they are not computed.  The shared-memory plan follows the
+        // rows (fewer rows leave room for more ring slots).
+        FwdParams& Q = misc->P;
+        if (Pg.rows_from_state) {
+            Q.M = min(Pg.M, Pg.state[ST_DRAFT_LEN] + 1);
+            Q.att_gh = Pg.att_gh_rows[Q.M - 1];
+        }
+        Q.NB = Q.M > 16 ? 32 : 16;
+        plan_smem_rows(Q, Q.M);
+    }
     if (tid >= 32 && tid < 32 + OP_COUNT) misc->part[tid - 32] = get_part(Pg.op[tid - 32], Pg.op[OP_GU], blockIdx.x, Pg.G);
 
     if (tid == 0) {
@@ -1135,6 +1215,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
     int nbar = 0;
     bool skip = false;
+#pragma unroll 1
     for (int ph = P.ph_begin; ph < P.ph_end; ++ph) {
         int layer;
         const int kind = decode_phase(ph, P.n_layers, layer);
@@ -1148,7 +1229,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         } else if (kind == PH_ATTN) {
             attention_phase<HD, MODE>(P, layer, smem + P.u_off, wtid, pp);
         } else {
-            gemm_phase<NBT>(P, kind, layer, smem, misc, pos, wtid, pp);
+            gemm_phase(P, kind, layer, smem, misc, pos, wtid, pp);
         }
         if (pp) {
             named_bar_sync(1, kWorkerThreads);

@@ -34,6 +34,10 @@ constexpr int kSmemBudget = 232448;                    // 227 KB
 constexpr int kAttnSmemBytes = 81920;                  // Q tile (up to 16 KB) + two K|V blocks of 64 keys (64 KB)
 constexpr int kActSmemMax = 32768;                     // SwiGLU output of this block (operand of its down-projection slice) at most
 constexpr int kMiscSmemBytes = 4096;
+constexpr int kMiscOff = kSmemBudget - 1024 - kMiscSmemBytes;  // bookkeeping lies behind everything else, at the same place whatever the rows
+constexpr unsigned long long kLookaheadBytes = 393216;  // how far ahead of the ring the weight streamer reads into L2,
+constexpr unsigned kLookaheadPiece = 8192;             //   in pieces of this size
+constexpr int kLookaheadCycles = 800;                  //   and no more often than this
 constexpr int kMaxDraftWords = 32;
 constexpr int kProfWords = 12;                         // timestamps per (phase, block)
 constexpr int kTmemCols = 128;                         // two buffers of two 128-row accumulators of up to 32 fp32 columns
@@ -231,12 +235,32 @@ struct FwdParams {
     int nstage;        // ring slots of kStageBytes, at offset 0
     int u_off;         // operand region (token operand of the running GEMM; attention tiles)
     int act_off;       // SwiGLU output operand
-    int misc_off;
+    int plan_ks;       // what the plan follows from besides the rows: column steps of the widest token operand,
+    int plan_act;      //   SwiGLU column steps per block at most (0: no SwiGLU operand)
+    int plan_attn;     //   bytes the attention tiles need (0: no attention)
+    int rows_from_state;  // 1: at most M rows; the draft in the state block says how many
+    uint8_t att_gh_rows[kMaxRows];  // att_gh for 1, 2, ... rows (rows_from_state)
     unsigned long long wait_limit_ns;
     int l_from_state;  // 1: L is read from the state block when the kernel starts (steps enqueued without the host in between)
     // batched verify: nseq > 0 sequences share the launch (chains only); L is then the longest length
     int nseq;
     BatchSeq seq[kMaxBatch];
 };
+
+// Shared-memory plan of a launch over `rows` token rows: ring of weight stages | operand region | SwiGLU operand |
+// bookkeeping (at kMiscOff).  The operand region holds the token operand of the widest GEMM share (or the attention
+// tiles); the ring takes what is left.  Fewer than two ring slots: the rows do not fit.
+__host__ __device__ inline void plan_smem_rows(FwdParams& P, int rows) {
+    const int step_bytes = 32 * rows;  // token operand bytes per column step: 16 columns x rows x bf16
+    int u = P.plan_ks * step_bytes;
+    if (u < P.plan_attn) u = P.plan_attn;
+    u = (u + 1023) / 1024 * 1024;
+    const int act = P.plan_act > 0 ? (P.plan_act * step_bytes + 1023) / 1024 * 1024 : 1024;
+    const int ring = kMiscOff - act - u;
+    P.nstage = ring < 0 ? 0 : ring / kStageBytes;
+    if (P.nstage > kMaxStages) P.nstage = kMaxStages;
+    P.u_off = P.nstage * kStageBytes;
+    P.act_off = P.u_off + u;
+}
 
 }  // namespace sdv

@@ -97,6 +97,11 @@ __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gmem_src, u
 }
 
 
+// global -> L2 only (address and size multiples of 16).
+__device__ __forceinline__ void bulk_prefetch_l2(const void* gmem, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gmem), "r"(bytes) : "memory");
+}
+
 // ---------------------------------------------------------------- tcgen05: tensor memory and MMA
 // Shared-memory operand descriptor, K-major, no swizzle: the operand is made of 8-row x 16-byte
 // core matrices (128 contiguous bytes each); `lbo` is the byte distance between the two core

@@ -175,44 +175,31 @@ void full_k_partition(OpDesc& o, int G, int unit) {
     o.P_row = o.T / unit < G ? o.T / unit : G;
 }
 
-// Shared-memory plan of a launch over `rows` token rows: ring of weight stages | operand region |
-// SwiGLU operand | bookkeeping.  The operand region holds the token operand of the widest GEMM
-// share (or the attention tiles); the ring takes what is left.
+// Shared-memory plan of a launch over `rows` token rows (plan_smem_rows), and whether they fit.
 struct SmemPlan {
-    int NG, NB, nstage, u_off, act_off, misc_off, total;
+    int NG, NB, nstage, u_bytes;
     bool ok;
 };
-SmemPlan plan_smem(const FwdParams& P, int rows, bool raw_only) {
-    SmemPlan s;
-    s.NG = (rows + 7) / 8;
-    s.NB = rows > 16 ? 32 : 16;
-    const int step_bytes = 32 * rows;  // token operand bytes per column step: 16 columns x rows x bf16
-    int max_ks = 0;
+SmemPlan plan_smem(FwdParams& P, int rows, bool raw_only) {
+    P.plan_ks = P.plan_act = P.plan_attn = 0;
     for (int i = 0; i < OP_COUNT; ++i) {
         const OpDesc& o = P.op[i];
         if (o.T == 0 || o.follow || (raw_only != (i == OP_RAW))) continue;
         const int ks = (o.K16 + o.P_k - 1) / o.P_k;
-        if (ks > max_ks) max_ks = ks;
+        if (ks > P.plan_ks) P.plan_ks = ks;
     }
-    int u = max_ks * step_bytes;
-    if (!raw_only && u < kAttnSmemBytes) u = kAttnSmemBytes;
-    u = (u + 1023) / 1024 * 1024;
-    s.ok = true;
-    int act = 1024;
     if (!raw_only) {
         const OpDesc& gu = P.op[OP_GU];
-        const int units = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;  // SwiGLU column steps per block at most
-        act = (units * step_bytes + 1023) / 1024 * 1024;
-        if (act > kActSmemMax) s.ok = false;
+        P.plan_act = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;  // SwiGLU column steps per block at most
+        P.plan_attn = kAttnSmemBytes;
     }
-    const int ring = kSmemBudget - 1024 - kMiscSmemBytes - act - u;
-    s.nstage = ring / kStageBytes;
-    if (s.nstage > kMaxStages) s.nstage = kMaxStages;
-    if (s.nstage < 2) s.ok = false;
-    s.u_off = s.nstage * kStageBytes;
-    s.act_off = s.u_off + u;
-    s.misc_off = s.act_off + act;
-    s.total = s.misc_off + kMiscSmemBytes + 1024;  // + slack for 1024-byte alignment
+    plan_smem_rows(P, rows);
+    SmemPlan s;
+    s.NG = (rows + 7) / 8;
+    s.NB = rows > 16 ? 32 : 16;
+    s.nstage = P.nstage;
+    s.u_bytes = P.act_off - P.u_off;
+    s.ok = P.nstage >= 2 && P.plan_act * 32 * rows <= kActSmemMax;
     return s;
 }
 
@@ -300,38 +287,29 @@ int cuda_fail(sdv_ctx* ctx, cudaError_t e) {
     } while (0)
 
 typedef void (*ForwardKernel)(const FwdParams);
-// The forward kernel compiled for this launch's instruction width, head dimension and kind of attention.
+// The forward kernel compiled for this launch's head dimension and kind of attention.
 ForwardKernel forward_kernel(const FwdParams& P) {
     const int mode = P.nseq > 0 ? 2 : (P.tree ? 1 : 0);
-    static const ForwardKernel table[2][2][3] = {
-        {{sdv_forward_kernel<16, 64, 0>, sdv_forward_kernel<16, 64, 1>, sdv_forward_kernel<16, 64, 2>},
-         {sdv_forward_kernel<16, 128, 0>, sdv_forward_kernel<16, 128, 1>, sdv_forward_kernel<16, 128, 2>}},
-        {{sdv_forward_kernel<32, 64, 0>, sdv_forward_kernel<32, 64, 1>, sdv_forward_kernel<32, 64, 2>},
-         {sdv_forward_kernel<32, 128, 0>, sdv_forward_kernel<32, 128, 1>, sdv_forward_kernel<32, 128, 2>}}};
-    return table[P.NB == 32][P.hd == 128][mode];
+    static const ForwardKernel table[2][3] = {{sdv_forward_kernel<64, 0>, sdv_forward_kernel<64, 1>, sdv_forward_kernel<64, 2>},
+                                              {sdv_forward_kernel<128, 0>, sdv_forward_kernel<128, 1>, sdv_forward_kernel<128, 2>}};
+    return table[P.hd == 128][mode];
 }
-cudaError_t launch_kernel(const FwdParams& P, int smem_bytes, cudaStream_t stream) {
+cudaError_t launch_kernel(const FwdParams& P, cudaStream_t stream) {
     const ForwardKernel k = forward_kernel(P);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&P};
     // phases meet at grid barriers, so more than one phase needs all blocks co-resident
     if (P.ph_end - P.ph_begin > 1)
-        return cudaLaunchCooperativeKernel((const void*)k, dim3(P.G), dim3(kThreads), args, smem_bytes, stream);
-    return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, smem_bytes, stream);
+        return cudaLaunchCooperativeKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
+    return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
 }
 
-bool apply_plan(FwdParams& P, int rows, bool raw_only, int* smem_bytes) {
+bool apply_plan(FwdParams& P, int rows, bool raw_only) {
     const SmemPlan sp = plan_smem(P, rows, raw_only);
-    if (!sp.ok) return false;
     P.M = rows;
     P.NB = sp.NB;
-    P.nstage = sp.nstage;
-    P.u_off = sp.u_off;
-    P.act_off = sp.act_off;
-    P.misc_off = sp.misc_off;
-    *smem_bytes = sp.total;
-    return true;
+    return sp.ok;
 }
 
 // Attention split of a launch: heads per unit (a unit's rows, heads x M, fill at most four 16-row
@@ -339,10 +317,8 @@ bool apply_plan(FwdParams& P, int rows, bool raw_only, int* smem_bytes) {
 // 16-key steps a warp walks one after another: blocks of 64 keys per range x steps per block; with
 // more units than blocks (several sequences, each with its own units) the blocks take them in rounds,
 // each round paying a unit's fixed cost (about three such steps) again.
-void plan_attention(FwdParams& P, int rows, int L, int nseq = 1) {
-    P.att_gh = 1;
-    if (P.g < 1) return;
-    int best = -1;
+int plan_attention(const FwdParams& P, int rows, int L, int nseq) {
+    int best = -1, best_gh = 1;
     for (int gh = 1; gh <= P.g; ++gh) {
         if (gh * rows > 64 && gh > 1) break;
         const int MT = (gh * rows + 15) / 16, KG = MT <= 2 ? 4 : (MT == 3 ? 3 : 2);
@@ -360,9 +336,10 @@ void plan_attention(FwdParams& P, int rows, int L, int nseq = 1) {
         cost = rounds * (3 + cost);
         if (best < 0 || cost <= best) {  // ties: more heads per unit (fewer reloads of the keys)
             best = cost;
-            P.att_gh = gh;
+            best_gh = gh;
         }
     }
+    return best_gh;
 }
 
 // `batch`: the sequences of a batched step (then `rows` is their total, `L` the longest length, and the launch
@@ -375,11 +352,13 @@ int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph
                    bool tree = false, const BatchPlan* batch = nullptr, bool l_from_state = false, cudaEvent_t* run_ev = nullptr) {
     FwdParams P = ctx->P;
     P.l_from_state = l_from_state ? 1 : 0;
-    int smem_bytes = 0;
     const bool raw_only = (ph_begin == 2 + kPhasesPerLayer * ctx->cfg.n_layers);
-    if (!apply_plan(P, rows, raw_only, &smem_bytes)) return SDV_EINVAL;
+    if (!apply_plan(P, rows, raw_only)) return SDV_EINVAL;
+    P.rows_from_state = (mode == 0 && !batch) ? 1 : 0;
     P.L = L;
-    plan_attention(P, batch ? batch->max_rows : rows, L, batch ? batch->n : 1);
+    P.att_gh = P.g < 1 ? 1 : plan_attention(P, batch ? batch->max_rows : rows, L, batch ? batch->n : 1);
+    if (P.rows_from_state)   // for every number of rows the draft may turn out to have
+        for (int r = 1; r <= rows; ++r) P.att_gh_rows[r - 1] = (uint8_t)plan_attention(P, r, L, 1);
     P.nseq = 0;
     if (batch) {
         P.nseq = batch->n;
@@ -397,7 +376,7 @@ int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph
     const int nbar = ph_end - ph_begin - 1;
     ctx->bar_base += (unsigned)(nbar * ctx->G);
     if (timed) CK(cudaEventRecord(run_ev ? run_ev[0] : ctx->ev0, ctx->stream));
-    cudaError_t e = launch_kernel(P, smem_bytes, ctx->stream);
+    cudaError_t e = launch_kernel(P, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     ctx->launches++;
     if (timed) {
@@ -756,8 +735,7 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
     {
         // the widest verify step must fit the shared-memory plan
         FwdParams probe = P;
-        int smem_bytes = 0;
-        if (!apply_plan(probe, rows_max, false, &smem_bytes)) return fail(SDV_EINVAL);
+        if (!apply_plan(probe, rows_max, false)) return fail(SDV_EINVAL);
     }
 
     // rotary table in double, rounded once to fp32 (a follower reads its leader's)
@@ -991,8 +969,7 @@ int sdv_prefill_chunk(sdv_ctx* ctx, const int32_t* host_tokens, int n, int is_la
     {
         // wide models: fewer rows per launch so that the token operand leaves room for the weight ring
         FwdParams probe = ctx->P;
-        int smem_bytes = 0;
-        while (tile > 8 && (!apply_plan(probe, tile, false, &smem_bytes) || probe.nstage < 4)) tile -= 8;
+        while (tile > 8 && (!apply_plan(probe, tile, false) || probe.nstage < 4)) tile -= 8;
     }
     const int n_ph = 1 + kPhasesPerLayer * c.n_layers;
     int done = 0;
@@ -1751,7 +1728,7 @@ int sdv_debug_plan(const sdv_config* cfg, int G, int rows, int* out) {
         for (int j = 0; j < 8; ++j) out[i * 8 + j] = v[j];
     }
     const SmemPlan sp = plan_smem(P, rows, false);
-    out[40] = sp.NG; out[41] = sp.NB; out[42] = sp.nstage; out[43] = sp.act_off - sp.u_off; out[44] = sp.total; out[45] = sp.ok ? 1 : 0;
+    out[40] = sp.NG; out[41] = sp.NB; out[42] = sp.nstage; out[43] = sp.u_bytes; out[44] = kSmemBudget; out[45] = sp.ok ? 1 : 0;
     return SDV_OK;
 }
 
@@ -1844,8 +1821,7 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
     P.ph_begin = 2;  // with n_layers = 0 phase 2 is the stand-alone GEMM
     P.ph_end = 3;
     P.wait_limit_ns = 2000000000ull;
-    int smem_bytes = 0;
-    if (!apply_plan(P, M, true, &smem_bytes)) return SDV_EINVAL;
+    if (!apply_plan(P, M, true)) return SDV_EINVAL;
 
     // the array keeps the previous call's contents: clear what must start at zero
     if (cudaMemsetAsync(sc + kNaOutOff, 0, (size_t)kMaxRows * N * 4, s) != cudaSuccess) return SDV_ECUDA;
@@ -1855,7 +1831,7 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
     if (blocks > 148 * 16) blocks = 148 * 16;
     pack_weights_kernel<<<blocks, 256, 0, s>>>(o, o, sc, dev_w, N, nullptr, 0, nullptr, K, 0, 0, o.T, 0);
     if (cudaGetLastError() != cudaSuccess) return SDV_ECUDA;
-    if (launch_kernel(P, smem_bytes, s) != cudaSuccess) return SDV_ECUDA;
+    if (launch_kernel(P, s) != cudaSuccess) return SDV_ECUDA;
     if (cudaMemcpyAsync(dev_y, sc + kNaOutOff, (size_t)M * N * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return SDV_ECUDA;
     int err = 0;
