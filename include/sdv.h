@@ -38,7 +38,7 @@ enum {
     SDV_ESTATE = -4,    /* call order: e.g. verify before prefill finished, commit without verify */
     SDV_ECUDA = -5,     /* CUDA runtime error, see sdv_last_cuda_error() */
     SDV_ETIMEOUT = -6,  /* a bounded device-side wait ran out; the context must be re-created */
-    SDV_ETOOBIG = -7    /* sdv_gemm_noalloc: the problem exceeds its fixed scratch area */
+    SDV_ETOOBIG = -7    /* sdv_gemm_noalloc: the problem exceeds its limits */
 };
 
 #define SDV_NGRAM_MAX 4096 /* longest history suffix the drafter can be asked to match */
@@ -373,7 +373,7 @@ long long sdv_launch_count(const sdv_ctx *ctx);
  * the context's stream; synchronises on the closing event). */
 int sdv_last_verify_ms(sdv_ctx *ctx, float *ms);
 
-/* The same GEMM as sdv_debug_gemm, Y[M][N] = X[M][K] * W[N][K]^T (operands rounded to bf16, fp32
+/* The same product as sdv_debug_gemm, Y[M][N] = X[M][K] * W[N][K]^T (operands rounded to bf16, fp32
  * accumulate), for callers that may not allocate.  The paper has no counterpart: this is a
  * library convenience.  It needs no context and asks the CUDA runtime for no memory at any point,
  * so it can be used where an allocation is unwelcome or impossible: inside a serving loop whose
@@ -390,19 +390,12 @@ int sdv_last_verify_ms(sdv_ctx *ctx, float *ms);
  * cuda_stream is a cudaStream_t (NULL = the default stream); the work is queued on it and the
  * call returns after it has finished (it synchronises that stream).
  *
- * Scratch (the weights in streaming order, the accumulators, an error word)
- * lives in a fixed array of about 2.5 MB inside the library's device image, present on every GPU
- * that loads the library for as long as it stays loaded.  Hence the limits: M <= 32, N <= 4096,
- * K <= 4096, N % 16 == 0, K % 64 == 0 and N * K * 2 <= 2 MiB; a larger problem returns
- * SDV_ETOOBIG and touches nothing, a malformed one SDV_EINVAL.  The array keeps whatever the last
- * call left in it; each call clears the parts that must start at zero (accumulators, error word)
- * itself.  There is one array per GPU, so two calls that overlap in time on one GPU (different
- * streams or threads) race on it: serialise them.
+ * The work is one kernel on the caller's operands, without scratch, so calls on different streams or from
+ * different threads may overlap.  Limits: M <= 32, N <= 4096, K <= 4096, N % 16 == 0, K % 64 == 0 and
+ * N * K * 2 <= 2 MiB; a larger problem returns SDV_ETOOBIG and touches nothing, a malformed one SDV_EINVAL.
  *
- * The first call on each device looks up the array's device address (a one-time set-up step that
- * also makes the runtime load the library's device code if it has not yet); make that first call
- * before starting any stream capture.  Returns SDV_OK, SDV_EINVAL, SDV_ETOOBIG, SDV_ECUDA, or
- * SDV_ETIMEOUT if a bounded device-side wait ran out. */
+ * The first call on each device may make the runtime load the library's device code: make it before starting
+ * any stream capture.  Returns SDV_OK, SDV_EINVAL, SDV_ETOOBIG or SDV_ECUDA. */
 int sdv_gemm_noalloc(const float *dev_x, const uint16_t *dev_w, float *dev_y, int M, int N, int K,
                      void *cuda_stream);
 

@@ -77,29 +77,39 @@ struct Misc {
 static_assert(sizeof(Misc) <= kMiscSmemBytes, "misc shared memory");
 
 // ------------------------------------------------------------------------------------------
-// Grid barrier: every block adds one to a counter (release) and waits (bounded, acquire) until all
-// have.  Called by all worker threads.  Returns, identically for all of them, whether some bounded
-// wait in this block has been abandoned (the remaining phases then do no work).
-__device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target, Misc* misc, int wtid) {
-    named_bar_sync(1, kWorkerThreads);
-    if (wtid == 0) {
-        red_release_add_u32(P.bar, 1u);  // no return value to wait for: polling starts at once
-        uint64_t t0 = 0;  // the global timer is slow to read: only once the wait has lasted a while
-        uint32_t spins = 0;
-        while ((int)(ld_acquire_gpu_u32(P.bar) - target) < 0) {  // wrap-safe: the difference, read as signed
-            if ((++spins & 63u) == 0) {
-                if (*(volatile int*)&misc->abort_flag) break;
-                const uint64_t now = global_timer_ns();
-                if (t0 == 0) t0 = now;
-                if (now - t0 > P.wait_limit_ns) {
-                    *(volatile int*)&misc->abort_flag = 1;
-                    break;
+// Grid barrier: every block adds one to a counter (release) and waits (bounded, acquire) until all have.  Called by all worker
+// threads.  The last worker warp (which has the least of the phases' work) meets the other blocks; the others only announce
+// themselves and work out what the next phase needs (`prepare`) meanwhile.  Returns, identically for all of them,
+// whether some bounded wait in this block has been abandoned (the remaining phases then do no work).
+constexpr int kBarrierWarp = kWorkerWarps - 1;
+template <typename F>
+__device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target, Misc* misc, int wtid, F prepare) {
+    if ((wtid >> 5) == kBarrierWarp) {
+        named_bar_sync(1, kWorkerThreads);
+        if ((wtid & 31) == 0) {
+            red_release_add_u32(P.bar, 1u);  // no return value to wait for: polling starts at once
+            uint64_t t0 = 0;  // the global timer is slow to read: only once the wait has lasted a while
+            uint32_t spins = 0;
+            while ((int)(ld_acquire_gpu_u32(P.bar) - target) < 0) {  // wrap-safe: the difference, read as signed
+                if ((++spins & 63u) == 0) {
+                    if (*(volatile int*)&misc->abort_flag) break;
+                    const uint64_t now = global_timer_ns();
+                    if (t0 == 0) t0 = now;
+                    if (now - t0 > P.wait_limit_ns) {
+                        *(volatile int*)&misc->abort_flag = 1;
+                        break;
+                    }
                 }
             }
+            *(volatile int*)&misc->skip = *(volatile int*)&misc->abort_flag;
         }
-        *(volatile int*)&misc->skip = *(volatile int*)&misc->abort_flag;
+        named_bar_sync(4, kWorkerThreads);
+        prepare();
+    } else {
+        named_bar_arrive(1, kWorkerThreads);
+        prepare();
+        named_bar_sync(4, kWorkerThreads);
     }
-    named_bar_sync(1, kWorkerThreads);
     return *(volatile int*)&misc->skip != 0;
 }
 
@@ -148,10 +158,10 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
             const Part& pt = misc->part[ops[oi]];
             if (pt.ntiles == 0 || pt.nk == 0) continue;
             const uint8_t* src = op_weights(P, ops[oi], layer) + pt.off;
-            const int nst = pt.nst, SK = pt.SK, nk = pt.nk;
+            const int nst = pt.nst, SK = pt.SK, nk = pt.nk / pt.slices;
 #pragma unroll 1
             for (int p = 0; p < pt.npass && ok; ++p) {
-                const uint32_t pbytes = (uint32_t)pass_count(pt, p) * kStepBytes;
+                const uint32_t pbytes = (uint32_t)(pass_count(pt, p) * pt.slices) * kStepBytes;
                 int kleft = nk;
 #pragma unroll 1
                 for (int st = 0; st < nst; ++st, kleft -= SK) {
@@ -219,54 +229,84 @@ __device__ __forceinline__ uint32_t operand_off(int k8, int row, int M) {
 // commutes with the GEMM and is applied by the consumer of the result), or, for the stand-alone
 // GEMM, the caller's fp32 rows as they are.  Warp w converts rows w, w + 10, ...; all loads of a
 // batch are issued before the first use.  Leaves the rows' sums of squares over this block's
-// columns in misc->sumsq; QKV blocks of row partition 0 also add them to the global sums the
-// attention step reads.
-__device__ __forceinline__ void build_norm_operand(const FwdParams& P, int kind, int layer, const Part& pt, uint8_t* U,
-                                                Misc* misc, int wtid) {
-    constexpr int UB = 12;  // 4-column units per lane and batch; a warp instruction reads 512 contiguous bytes
+// columns in misc->sumsq.
+// What the build needs to know is worked out while the blocks meet at the grid barrier before it (NormPrep): the look-ups and
+// index arithmetic took 740 of the 2800 cycles between a barrier and the finished operand.
+struct NormPrep {
+    const float4* src;    // this warp's first row, first column of the block's share
+    const float4* wsrc;   // norm weights of the share (nullptr: none)
+    int nk4, stride4;     // float4 columns of the share, of a row
+    // operand layout with K slices: slice of a float4 column = its product with slice_inv, upper half; 16-byte units per 8-column
+    // group; step from a slice to the next beyond that
+    uint32_t slice_inv;
+    int group, slice_adj;
+};
+__device__ __forceinline__ NormPrep norm_prep(const FwdParams& P, int kind, int layer, const Part& pt, int warp) {
+    NormPrep n;
+    const bool raw = (kind == PH_RAW);
+    const int stride = raw ? P.raw_K : P.d, k4_0 = pt.k0 * 4;
+    const float* xbase = raw ? P.raw_x : P.h;
+    n.nk4 = pt.nk * 4;
+    n.stride4 = stride >> 2;
+    n.src = reinterpret_cast<const float4*>(xbase) + (size_t)warp * n.stride4 + k4_0;
+    n.wsrc = raw ? nullptr
+                 : reinterpret_cast<const float4*>(P.norm_w + (size_t)(kind == PH_QKV ? layer * 2 : (kind == PH_GUD ? layer * 2 + 1 : P.n_layers * 2)) * P.d) + k4_0;
+    const int slices = pt.slices;
+    n.group = slices * P.M;
+    n.slice_inv = 0u;
+    n.slice_adj = 0;
+    if (slices > 1) {
+        const int per4 = n.nk4 / slices;   // float4 columns per slice (a multiple of 4)
+        n.slice_inv = 0xffffffffu / (uint32_t)per4 + 1u;
+        n.slice_adj = P.M - (per4 >> 1) * n.group;
+    }
+    return n;
+}
+// One row, UB units of 4 columns per lane and batch (a warp instruction reads 512 contiguous bytes).
+template <int UB>
+__device__ __forceinline__ float convert_row(const NormPrep& n, const float4* src, uint8_t* U, int row, int lane) {
+    const float4* wld = n.wsrc ? n.wsrc : src;  // without norm weights the loaded value is not used
+    float ss = 0.f;
+#pragma unroll 1
+    for (int base = lane; base < n.nk4; base += 32 * UB) {
+        float4 a[UB], w[UB];
+        // every unit loads (past the end: the row's last unit again, not used), so that the loads are one
+        // straight run of instructions instead of a branch per unit
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int k4 = min(base + u * 32, n.nk4 - 1);
+            a[u] = ld_cg_f4_inorder(src + k4);
+            w[u] = ld_nc_f4_inorder(wld + k4);
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int k4 = base + u * 32;
+            if (k4 < n.nk4) {
+                const float4 x = a[u];
+                const float4 g = n.wsrc ? w[u] : make_float4(1.f, 1.f, 1.f, 1.f);
+                ss += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+                const uint2 out = make_uint2(pack_bf16(x.x * g.x, x.y * g.y), pack_bf16(x.z * g.z, x.w * g.w));
+                const int sl = (int)__umulhi((uint32_t)k4, n.slice_inv);
+                *reinterpret_cast<uint2*>(U + ((k4 >> 1) * n.group + sl * n.slice_adj + row) * 16 + (k4 & 1) * 8) = out;
+            }
+        }
+    }
+    return ss;
+}
+__device__ __forceinline__ void build_norm_operand(const FwdParams& P, const NormPrep& n, uint8_t* U, Misc* misc, int wtid) {
     const int warp = wtid >> 5, lane = wtid & 31;
     const int M = P.M;
-    const int k4_0 = pt.k0 * 4, nk4 = pt.nk * 4;
-    const bool raw = (kind == PH_RAW);
-    const int stride = raw ? P.raw_K : P.d;
-    const float* xbase = raw ? P.raw_x : P.h;
-    const float* wn = raw ? nullptr
-                          : P.norm_w + (size_t)(kind == PH_QKV ? layer * 2 : (kind == PH_GUD ? layer * 2 + 1 : P.n_layers * 2)) * P.d;
+    const float4* src = n.src;
 #pragma unroll 1
-    for (int row = warp; row < M; row += kBuilderWarps) {
-        const float4* src = reinterpret_cast<const float4*>(xbase + (size_t)row * stride) + k4_0;
-        const float4* wsrc = wn ? reinterpret_cast<const float4*>(wn) + k4_0 : nullptr;
-        const float4* wld = wsrc ? wsrc : src;  // without norm weights the loaded value is not used
-        float ss = 0.f;
-#pragma unroll 1
-        for (int base = lane; base < nk4; base += 32 * UB) {
-            float4 a[UB], w[UB];
-            // every unit loads (past the end: the row's last unit again, not used), so that the loads are one
-            // straight run of instructions instead of a branch per unit
-#pragma unroll
-            for (int u = 0; u < UB; ++u) {
-                const int k4 = min(base + u * 32, nk4 - 1);
-                a[u] = ld_cg_f4_inorder(src + k4);
-                w[u] = ld_nc_f4_inorder(wld + k4);
-            }
-#pragma unroll
-            for (int u = 0; u < UB; ++u) {
-                const int k4 = base + u * 32;
-                if (k4 < nk4) {
-                    const float4 x = a[u];
-                    const float4 g = wsrc ? w[u] : make_float4(1.f, 1.f, 1.f, 1.f);
-                    ss += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
-                    const uint2 out = make_uint2(pack_bf16(x.x * g.x, x.y * g.y), pack_bf16(x.z * g.z, x.w * g.w));
-                    *reinterpret_cast<uint2*>(U + operand_off(k4 >> 1, row, M) + (k4 & 1) * 8) = out;
-                }
-            }
-        }
+    for (int row = warp; row < M; row += kBuilderWarps, src += (size_t)kBuilderWarps * n.stride4) {
+        // the batch follows the columns a block has: loads that only repeat the last unit would still cross L2
+        float ss;
+        if (n.nk4 <= 64) ss = convert_row<2>(n, src, U, row, lane);
+        else if (n.nk4 <= 256) ss = convert_row<8>(n, src, U, row, lane);
+        else ss = convert_row<12>(n, src, U, row, lane);
 #pragma unroll
         for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-        if (lane == 0) {
-            misc->sumsq[row] = ss;
-            if (kind == PH_QKV && pt.pr == 0) atomicAdd(P.sumsq + (layer & 1) * kMaxRows + row, ss);
-        }
+        if (lane == 0) misc->sumsq[row] = ss;
     }
 }
 
@@ -276,10 +316,9 @@ __device__ __forceinline__ void attn_split(const FwdParams& P, int& S, int& kps)
 // partial results (un-normalised sums with their running maximum and sum) are merged on the way.
 // Four lanes share one (row, 8 columns) item, each taking every fourth partial result.
 __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const Part& pt, uint8_t* U, int wtid) {
-    constexpr int TPL = (kMaxSplits + 1 + 3) / 4;  // partial results per lane at most
+    constexpr int TPL = (kMaxSplits + 3) / 4;  // partial results per lane at most
     int S, kps;
     attn_split(P, S, kps);
-    const int S1 = S + 1;
     const int M = P.M, hd = P.hd;
     const int k8_0 = pt.k0 * 2, nk8 = pt.nk * 2;
     const int nitems = M * nk8, sub = wtid & 3;
@@ -289,7 +328,7 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
         const bool live = item < nitems;
         const int j = live ? item / nk8 : 0, k8l = live ? item % nk8 : 0;
         const int col = (k8_0 + k8l) * 8, hq = col / hd, c = col % hd;
-        const size_t base = ((size_t)hq * (kMaxSplits + 1)) * kMaxRows + j;
+        const size_t base = ((size_t)hq * kMaxSplits) * kMaxRows + j;
         float m[TPL], l[TPL];
         float4 a[TPL], b[TPL];
         // every slot loads (beyond the last partial result: the last one again, given no weight below), so that
@@ -297,12 +336,12 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
 #pragma unroll
         for (int t = 0; t < TPL; ++t) {
             const int s = sub + 4 * t;
-            const size_t row = base + (size_t)min(s, S) * kMaxRows;
+            const size_t row = base + (size_t)min(s, S - 1) * kMaxRows;
             const float2 ml = ld_cg_f2_inorder(P.part_ml + row * 2);
             const float* op = P.part_o + row * hd + c;
             a[t] = ld_cg_f4_inorder(op);
             b[t] = ld_cg_f4_inorder(op + 4);
-            const bool use = live && s < S1;
+            const bool use = live && s < S;
             m[t] = use ? ml.x : -CUDART_INF_F;
             l[t] = use ? ml.y : 0.f;
         }
@@ -372,24 +411,25 @@ __device__ __forceinline__ void mma_stage(uint32_t d_tmem, uint64_t adesc, uint6
 __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8_t* smem, const uint8_t* B, Misc* misc,
                                        PipePos& pos, bool& dead, bool& ready) {
     const uint32_t nstage = (uint32_t)P.nstage;
-    const uint32_t idesc = umma_idesc_bf16_m128((uint32_t)P.NB);
+    const int brows = pt.slices * P.M;                          // rows of the token operand (stacked K slices)
+    const uint32_t idesc = umma_idesc_bf16_m128(pt.slices > 1 ? (uint32_t)((brows + 15) & ~15) : (uint32_t)P.NB);
     const uint64_t wait_limit = P.wait_limit_ns;
-    const uint32_t lbo_b = (uint32_t)P.M * 16u;
+    const uint32_t lbo_b = (uint32_t)brows * 16u;
     const uint64_t bstep = (uint64_t)((2u * lbo_b) >> 4);       // one column step, in descriptor address units
     const uint64_t bdesc0 = umma_smem_desc(smem_u32(B), lbo_b, 128u);
     const uint32_t ring0 = smem_u32(smem);
     const uint32_t tmem0 = misc->tmem_base;
-    const int nst = pt.nst, SK = pt.SK, nk = pt.nk, npass = pt.npass;
+    const int nst = pt.nst, SK = pt.SK, nk = pt.nk / pt.slices, npass = pt.npass;
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
-        const int pcount = pass_count(pt, p);
+        const int pcount = pass_count(pt, p) * pt.slices;   // row tiles of the pass, slices stacked
         const uint32_t buf = pos.q & 1u;
         if (!dead && !mbar_test(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u)) {
             const long long tq0 = clock64();
             if (!mbar_wait_bounded(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u, &misc->abort_flag, wait_limit)) dead = true;
             pos.w_acc += (uint32_t)(clock64() - tq0);
         }
-        const uint32_t d_tmem = tmem0 + buf * 64u;
+        const uint32_t d_tmem = tmem0 + buf * kTmemBuf;
         const uint32_t lbo_a = (uint32_t)(2 * pcount) * 128u;
         const uint64_t astep = (uint64_t)((2u * lbo_a) >> 4);
         const uint64_t adesc0 = umma_smem_desc(ring0, lbo_a, 128u);
@@ -477,8 +517,7 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, int op, const Pa
     float* out = P.h;
     int stride = P.d;
     bool add = true;  // residual add (O, down)
-    if (op == OP_QKV) { out = P.qkv_acc; stride = P.n_qkv; add = P.op[OP_QKV].P_k > 1; }
-    else if (op == OP_RAW) { out = P.raw_out; stride = P.raw_N; add = P.op[OP_RAW].P_k > 1; }
+    if (op == OP_RAW) { out = P.raw_out; stride = P.raw_N; add = P.op[OP_RAW].P_k > 1; }
     const int store_logits = P.store_logits;
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
@@ -494,7 +533,7 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, int op, const Pa
         // it and share its token columns (pairs of columns alternate between the groups)
         const int nsel = (nhalf == 2) ? -1 : myhalf;
         const int half = (nhalf == 2) ? myhalf : 0;
-        const uint32_t taddr = tmem_lane + buf * 64u + (uint32_t)half * 32u;
+        const uint32_t taddr = tmem_lane + buf * kTmemBuf + (uint32_t)half * 32u;
         const int tt = half * 128 + t;         // row within the pass
         const bool valid = tt < 16 * pcount;
         const int row = (tile0 + pstart) * 16 + tt;  // weight row = output feature
@@ -551,6 +590,104 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, int op, const Pa
     }
 }
 
+// q|k|v: the K slices' sums meet in shared memory (`ex`, free during this phase), then norm factor, bias and rotary embedding
+// finish the projection: queries go to P.q, keys and values straight into the cache at the rows' slots.  Every sum is
+// complete inside its block, so nothing is reduced in L2: a barrier behind plain stores is passed 1100 cycles sooner than one
+// behind reductions (2450 against 3550), and the attention step starts from finished bf16 rows.
+// An item is (8 rows, token): row r < 8 of a tile and row r + 8 are the two halves of a rotary pair.
+template <int HD, int MODE>
+__device__ __forceinline__ void epilogue_qkv(const FwdParams& P, int layer, const Part& pt, float* ex, Misc* misc, PipePos& pos, bool& dead,
+                                             int warp, int lane) {
+    constexpr int HD2 = HD / 2;
+    const int M = P.M, tid = warp * 32 + lane, group = warp >> 2, quarter = warp & 3;
+    const int slices = pt.slices, Mp = M | 1;   // odd row stride of the exchange area: no bank conflicts
+    const float inv_d = 1.f / (float)P.d;
+#pragma unroll 1
+    for (int p = 0; p < pt.npass; ++p, ++pos.q) {
+        const int pcount = pass_count(pt, p), RR = pcount * 16, t0 = pt.tile0 + pass_start(pt, p);
+        const uint32_t buf = pos.q & 1u;
+        // where an item's output goes and what it needs: fetched before the accumulator is there
+        struct Item { float2 cs; float b0, b1, rs; __nv_bfloat16* dst; };
+        auto fetch = [&](int it, Item& x) {
+            const int r = it & 7, m = (it >> 3) % M, T = t0 + (it >> 3) / M;
+            const int head = T / (HD / 16), i = (T % (HD / 16)) * 8 + r;
+            x.rs = rsqrtf(misc->sumsq[m] * inv_d + P.eps);
+            const float* b = P.bias ? P.bias + (size_t)layer * P.n_qkv + head * HD + i : nullptr;
+            x.b0 = b ? __ldg(b) : 0.f;
+            x.b1 = b ? __ldg(b + HD2) : 0.f;
+            x.cs = make_float2(1.f, 0.f);
+            if (head < P.n_q) x.dst = P.q + (size_t)m * (P.n_q * HD) + head * HD + i;
+            int L = P.L, slot = m, at = MODE == 1 ? __ldcg(P.state + ST_DEPTH + m) : m;   // tree drafts: a row's position is its depth
+            __nv_bfloat16 *kc = P.kcache, *vc = P.vcache;
+            if (MODE == 2) {
+                int b2 = 0;
+                while (b2 + 1 < P.nseq && m >= P.seq[b2 + 1].r0) ++b2;
+                L = P.seq[b2].L;
+                slot = at = m - P.seq[b2].r0;
+                kc = P.seq[b2].kcache;
+                vc = P.seq[b2].vcache;
+            }
+            if (head >= P.n_q) {
+                const int kvh = (head - P.n_q) % P.n_kv;
+                x.dst = (head - P.n_q < P.n_kv ? kc : vc) + (((size_t)layer * P.n_kv + kvh) * P.max_seq + L + slot) * HD + i;
+            }
+            if (head < P.n_q + P.n_kv) x.cs = __ldg(P.rope + (size_t)(L + at) * HD2 + i);
+        };
+        const int items = pcount * 8 * M;
+        Item first;
+        if (tid < items) fetch(tid, first);
+        if (!dead && !mbar_wait_bounded(&misc->tmem_full[buf], (pos.q >> 1) & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
+        dead = __any_sync(0xffffffffu, dead);
+        if (!dead) {
+            tc_fence_after();
+            if (misc->prof_ptr && tid == 0 && p == pt.npass - 1) misc->prof_ptr[10] = global_timer_ns();
+            // lanes of the accumulator: slice s * RR + row; of the columns a lane wants those of its own slice.  Where a warp's lanes
+            // span two slices, the two warps that share the lanes take one each; else they take a chunk of 16 tokens each
+            const uint32_t taddr = misc->tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kTmemBuf;
+            const int row = quarter * 32 + lane;
+            const int sl0 = (quarter * 32) / RR, sl1 = (quarter * 32 + 31) / RR;
+            const bool span = sl0 != sl1;
+            const int sl = span && group ? sl1 : sl0;
+            const bool mine = row < slices * RR && row >= sl * RR && row < (sl + 1) * RR;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                if (h * 16 < M && (span || group == h)) {
+                    float v[16];
+                    tmem_ld16(taddr + (uint32_t)((sl < slices ? sl : 0) * M + h * 16), v);
+#pragma unroll
+                    for (int n = 0; n < 16; ++n)
+                        if (mine && h * 16 + n < M) ex[row * Mp + h * 16 + n] = v[n];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&misc->tmem_empty[buf]);  // this warp's part of the accumulators may be overwritten
+        }
+        named_bar_sync(2, kEpilogueWarps * 32);
+        if (!dead) {
+#pragma unroll 1
+            for (int it = tid; it < items; it += kEpilogueWarps * 32) {
+                if (it != tid) fetch(it, first);
+                const int r = it & 7, m = (it >> 3) % M, tl = (it >> 3) / M;
+                const float* e = ex + (tl * 16 + r) * Mp + m;
+                float a = 0.f, b = 0.f;
+                if (slices == 8) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) { a += e[q * RR * Mp]; b += e[(q * RR + 8) * Mp]; }
+                } else {
+#pragma unroll 1
+                    for (int q = 0; q < slices; ++q, e += RR * Mp) { a += e[0]; b += e[8 * Mp]; }
+                }
+                a = a * first.rs + first.b0;
+                b = b * first.rs + first.b1;
+                first.dst[0] = __float2bfloat16(a * first.cs.x - b * first.cs.y);
+                first.dst[HD2] = __float2bfloat16(b * first.cs.x + a * first.cs.y);
+            }
+        }
+        if (p + 1 < pt.npass) named_bar_sync(2, kEpilogueWarps * 32);   // the exchange area is used again
+    }
+}
+
 // Best logit per token row over the block: lanes, then the eight epilogue warps.
 __device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, int warp, int lane, const Best& best, bool dead) {
 #pragma unroll
@@ -586,8 +723,14 @@ __device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, in
     }
 }
 
-__device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, uint8_t* act, Misc* misc, PipePos& pos, bool& dead, int warp,
-                                               int lane) {
+template <int HD, int MODE>
+__device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, int layer, uint8_t* act, Misc* misc, PipePos& pos, bool& dead,
+                                               int warp, int lane) {
+    if (kind == PH_QKV) {
+        const Part& pt = misc->part[OP_QKV];
+        if (pt.ntiles > 0 && pt.nk > 0) epilogue_qkv<HD, MODE>(P, layer, pt, reinterpret_cast<float*>(act), misc, pos, dead, warp, lane);
+        return;
+    }
     Best best;
     if (kind == PH_LM) {
 #pragma unroll
@@ -608,219 +751,145 @@ __device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, uin
 }
 
 // ------------------------------------------------------------------------------------------
-// Split-KV attention.  The committed cache [0, L) is cut into S key ranges of kps keys (a multiple
-// of 64, at most kMaxSplits ranges); the query heads of a KV head are cut into QG groups of up to
+// Split-KV attention.  The keys [0, L + M) (the new rows' keys and values are in the cache already) are cut into S ranges of
+// kps keys (a multiple of 64, at most kMaxSplits ranges); the query heads of a KV head are cut into QG groups of up to
 // gh heads, a group's rows (heads x M) filling at most four 16-row tiles (the host picks gh so
 // that the longest chain of 16-key steps a warp walks is shortest).
-// Unit (kv head, head group, s < S) attends the group's rows to range s; unit (kv head, head group,
-// S) covers the M new rows: it finishes their K/V projection (norm scale, bias, rotary), appends
-// them to the cache (group 0 only) and attends to them under the causal mask (row j sees new keys
-// 0..j).  Every unit leaves an un-normalised partial result with its running maximum and sum; the
-// output projection merges them while it builds its operand.
+// Unit (kv head, head group, s) attends the group's rows to range s under the causal mask (row j sees new keys 0..j; in a tree
+// the rows on its path) and leaves an un-normalised partial result with its running maximum and sum; the output
+// projection merges them while it builds its operand.
 //
-// Keys come in blocks of 64, copied asynchronously into two shared-memory buffers by all worker
-// warps.  Warp (row tile, key group) owns one row tile and every KG-th group of 16 keys of a block
+// Keys come in blocks of 64, copied asynchronously into two shared-memory buffers by warps 0..7.  Blocks that hold
+// committed keys only do not depend on the step: the first two are requested before the grid barrier in front of this phase,
+// so that the phase only waits for its queries.
+// Warp (row tile, key group) owns one row tile and every KG-th group of 16 keys of a block
 // (KG = 4 with up to two row tiles, 3 with three, 2 with four): scores (Q K^T on tensor cores), online softmax with quad
 // shuffles in the log2 domain and P V all stay in its registers; the key groups of a row tile meet
 // in shared memory at the end.
 // The heads per group are chosen on the host per launch; the key ranges follow from it: as many
 // as there are blocks to take a (KV head, head group, range) unit each, at most kMaxSplits.
+constexpr int kLoadThreads = kEpilogueWarps * 32;   // warps 0..7 copy keys and values
 __device__ __forceinline__ void attn_split(const FwdParams& P, int& S, int& kps) {
     S = P.att_S;      // worked out once per launch (attn_split_compute): the divisions are not repeated per phase
     kps = P.att_kps;
 }
-__device__ __forceinline__ void attn_split_compute(const FwdParams& P, int& S, int& kps) {
-    if (P.L <= 0) { S = 0; kps = 0; return; }
+// `keys`: of the longest sequence, new rows included.
+__device__ __forceinline__ void attn_split_compute(const FwdParams& P, int keys, int& S, int& kps) {
     const int QG = (P.g + P.att_gh - 1) / P.att_gh;
-    int cap = P.G / (P.n_kv * QG) - 1;
+    int cap = P.G / (P.n_kv * QG);
     if (cap > kMaxSplits) cap = kMaxSplits;
     if (cap < 1) cap = 1;
-    kps = ((P.L + cap - 1) / cap + 63) / 64 * 64;
-    S = (P.L + kps - 1) / kps;
+    kps = ((keys + cap - 1) / cap + 63) / 64 * 64;
+    S = (keys + kps - 1) / kps;
 }
 
-// MODE 0: the new rows are a chain; 1: a tree (positions and visibility from the state block); 2: the chain of
+// What a unit works on.
+struct AttnUnit {
+    int M, L, r0;             // rows of its sequence, committed length, first row in the launch's buffers
+    int head0, nheads;        // first query head, query heads
+    int s, t_begin, nkeys;    // key range: index, first key, keys
+    const __nv_bfloat16 *k, *v;   // cache of its sequence, at (layer 0, KV head, first key)
+};
+// MODE 0: the new rows are a chain; 1: a tree (visibility from the state block); 2: the chain of
 // sequence `b` of a batched step (its rows, length and KV cache from P.seq[b]).
 template <int HD, int MODE>
-__device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, int hk, int qg, int gh, int s, int S, int kps, uint8_t* att,
-                                            int wtid, unsigned long long* prof, int b) {
-    constexpr bool TREE = MODE == 1, BATCH = MODE == 2;
-    constexpr int HD2 = HD / 2;
-    constexpr int KSTEPS = HD / 16;
-    constexpr int UNITS = HD / 8;    // 16-byte units per K/V row
+__device__ __forceinline__ AttnUnit attn_unit(const FwdParams& P, int b, int hk, int qg, int s) {
+    AttnUnit u;
+    const __nv_bfloat16 *kc = P.kcache, *vc = P.vcache;
+    u.M = P.M; u.L = P.L; u.r0 = 0;
+    if (MODE == 2) { u.M = P.seq[b].M; u.L = P.seq[b].L; u.r0 = P.seq[b].r0; kc = P.seq[b].kcache; vc = P.seq[b].vcache; }
+    u.nheads = min(P.att_gh, P.g - qg * P.att_gh);   // the last group may hold fewer heads
+    u.head0 = hk * P.g + qg * P.att_gh;
+    u.s = s;
+    u.t_begin = s * P.att_kps;
+    u.nkeys = max(0, min(u.L + u.M, u.t_begin + P.att_kps) - u.t_begin);
+    const size_t off = ((size_t)hk * P.max_seq + u.t_begin) * HD;
+    u.k = kc + off;
+    u.v = vc + off;
+    return u;
+}
+template <int HD>
+struct AttnShape {
+    static constexpr int KB = 64, NBUF = 2, UNITS = HD / 8;   // keys per block, buffers, 16-byte units per K/V row
+    static constexpr int QBYTES = 64 * HD * 2, KVBYTES = KB * HD * 2;
+};
+// Keys and values of one block of the range: 16-byte asynchronous copies by warps 0..7, rows past the range zero-filled.
+template <int HD>
+__device__ __forceinline__ void attn_load_block(const FwdParams& P, const AttnUnit& u, int layer, int blk, uint8_t* att, int wtid) {
+    using A = AttnShape<HD>;
+    if (blk * A::KB < u.nkeys) {
+        uint8_t* Ks = att + A::QBYTES + (blk % A::NBUF) * 2 * A::KVBYTES;
+        uint8_t* Vs = Ks + A::KVBYTES;
+        const size_t base = (size_t)layer * P.n_kv * P.max_seq * HD;
+        const int q16 = wtid % A::UNITS;
+#pragma unroll
+        for (int i = 0; i < A::KB * A::UNITS / kLoadThreads; ++i) {
+            const int key = wtid / A::UNITS + i * (kLoadThreads / A::UNITS), kk = blk * A::KB + key;
+            const bool valid = kk < u.nkeys;
+            const size_t off = base + (size_t)(valid ? kk : 0) * HD + q16 * 8;
+            const uint32_t so = (q16 >> 3) * (A::KB * 128) + swz_unit(key, q16 & 7);
+            cp_async_16_zfill(Ks + so, u.k + off, valid);
+            cp_async_16_zfill(Vs + so, u.v + off, valid);
+        }
+    }
+    cp_async_commit();  // possibly empty: keeps the group count uniform
+}
+// Blocks that may be requested before the new rows' keys are there.
+template <int HD>
+__device__ __forceinline__ int attn_early_blocks(const AttnUnit& u) {
+    const int old = u.L - u.t_begin;   // committed keys of the range
+    const int n = old >= u.nkeys ? 2 : old / AttnShape<HD>::KB;
+    return n < 0 ? 0 : (n > 2 ? 2 : n);
+}
+
+template <int HD, int MODE>
+__device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, const AttnUnit& u, int loaded, uint8_t* att, int wtid,
+                                               unsigned long long* prof) {
+    using A = AttnShape<HD>;
+    constexpr bool TREE = MODE == 1;
+    constexpr int KSTEPS = HD / 16, UNITS = A::UNITS, KB = A::KB, NBUF = A::NBUF, KVBYTES = A::KVBYTES;
     constexpr int NT_O = HD / 8;     // 8-column tiles of the output
-    constexpr int KB = 64;           // keys per block
-    constexpr int NBUF = 2;
-    constexpr int QBYTES = 64 * HD * 2;
-    constexpr int KVBYTES = KB * HD * 2;  // one K (or V) block
-    static_assert(QBYTES + NBUF * 2 * KVBYTES <= kAttnSmemBytes, "attention tiles");
+    static_assert(A::QBYTES + NBUF * 2 * KVBYTES <= kAttnSmemBytes, "attention tiles");
     // exchange area of the key-group merge: (KG - 1) * MT <= 6 tiles of (output + statistics)
     static_assert(6 * (NT_O + 1) * 32 * 16 <= NBUF * 2 * KVBYTES, "exchange area of the key-group merge");
     const int warp = wtid >> 5, lane = wtid & 31;
-    const int M = BATCH ? P.seq[b].M : P.M, L = BATCH ? P.seq[b].L : P.L;
-    const int r0 = BATCH ? P.seq[b].r0 : 0;      // first row of this sequence in the launch's buffers
-    __nv_bfloat16* const kcache = BATCH ? P.seq[b].kcache : P.kcache;
-    __nv_bfloat16* const vcache = BATCH ? P.seq[b].vcache : P.vcache;
-    const int nheads = min(gh, P.g - qg * gh);   // the last group may hold fewer heads
-    const int R = nheads * M;                    // R <= 64
+    const int M = u.M;
+    const int R = u.nheads * M;                  // R <= 64
+    const uint32_t minv = 65536u / (uint32_t)M + 1u;   // row / M = row * minv >> 16 for rows below 64
     const int MT = (R + 15) >> 4, RP = MT * 16;
     const int KG = MT <= 2 ? 4 : (MT == 3 ? 3 : 2);  // key groups: 16-key chunks of a block handled side by side
-    const bool active = warp < MT * KG;
-    const int mt = active ? warp % MT : 0, kgp = active ? warp / MT : 0;
-    const int head0 = hk * P.g + qg * gh;     // first query head of this unit
-    const bool is_new = (s == S);
+    const int kgp = (MT == 1 ? warp : MT == 2 ? warp >> 1 : MT == 3 ? (warp * 11) >> 5 : warp >> 2), mt = warp - kgp * MT;
+    const bool active = kgp < KG;
     uint8_t* Qs = att;
-    uint8_t* KVs = att + QBYTES;
-    const float* sumsq = P.sumsq + (layer & 1) * kMaxRows;
-    const float* bias = P.bias ? P.bias + (size_t)layer * P.n_qkv : nullptr;
-    const int Nq = P.n_q * HD, Nkv = P.n_kv * HD;
+    uint8_t* KVs = att + A::QBYTES;
+    const int nkeys = u.nkeys, nblk = (nkeys + KB - 1) / KB;
 
-    int t_begin = 0, nkeys = M;
-    if (!is_new) {
-        t_begin = s * kps;
-        const int t_end = min(L, t_begin + kps);
-        nkeys = max(0, t_end - t_begin);
-    }
-    const int nblk = (nkeys + KB - 1) / KB;
-    const size_t cache_row0 = ((size_t)layer * P.n_kv + hk) * P.max_seq;
-
-    // cached keys and values of one block: 16-byte asynchronous copies, rows past the range zero-filled
-    auto load_block = [&](int blk) {
-        if (blk < nblk) {
-            uint8_t* Ks = KVs + (blk % NBUF) * 2 * KVBYTES;
-            uint8_t* Vs = Ks + KVBYTES;
-            for (int u = wtid; u < KB * UNITS; u += kWorkerThreads) {
-                const int key = u / UNITS, q16 = u % UNITS, kk = blk * KB + key;
-                const bool valid = kk < nkeys;
-                const size_t off = (cache_row0 + t_begin + (valid ? kk : 0)) * HD + q16 * 8;
-                const uint32_t so = (q16 >> 3) * (KB * 128) + swz_unit(key, q16 & 7);
-                cp_async_16_zfill(Ks + so, kcache + off, valid);
-                cp_async_16_zfill(Vs + so, vcache + off, valid);
-            }
-        }
-        cp_async_commit();  // possibly empty: keeps the group count uniform
-    };
     if (prof && wtid == 0) prof[2] = global_timer_ns();
-    if (!is_new) {
-#pragma unroll
-        for (int b = 0; b < NBUF; ++b) load_block(b);
+    // query tile (16-byte copies; rows past R zero-filled)
+    for (int un = wtid; un < RP * UNITS; un += kWorkerThreads) {
+        const int r = un / UNITS, q16 = un % UNITS;
+        const int hl = (int)((uint32_t)r * minv >> 16), j = r - hl * M;
+        const bool valid = r < R;
+        const __nv_bfloat16* src = P.q + (size_t)(u.r0 + (valid ? j : 0)) * (P.n_q * HD) + (u.head0 + (valid ? hl : 0)) * HD + q16 * 8;
+        cp_async_16_zfill(Qs + (q16 >> 3) * (RP * 128) + swz_unit(r, q16 & 7), src, valid);
     }
-
-    // ---- query tile: normalise, add bias, rotate, round to bf16; 4 rotary pairs per item
-    {
-        constexpr int QI = 2;  // items per thread and batch: all loads are issued before the first use
-        const int items = RP * (HD2 / 4);
+    cp_async_commit();
+    if (warp < kEpilogueWarps) {
 #pragma unroll 1
-        for (int base = wtid; base < items; base += QI * kWorkerThreads) {
-            float4 qa[QI], qb[QI], c0[QI], c1[QI];
-            float ssq[QI];
-            int rr[QI], ii[QI];
-#pragma unroll
-            for (int t = 0; t < QI; ++t) {
-                const int idx = base + t * kWorkerThreads;
-                rr[t] = idx / (HD2 / 4);
-                ii[t] = (idx % (HD2 / 4)) * 4;
-                ssq[t] = 0.f;
-                qa[t] = qb[t] = c0[t] = c1[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (idx < items && rr[t] < R) {
-                    const int hl = rr[t] / M, j = rr[t] % M, col = (head0 + hl) * HD + ii[t];
-                    ssq[t] = __ldcg(sumsq + r0 + j);
-                    qa[t] = ld_cg_f4_inorder(P.qkv_acc + (size_t)(r0 + j) * P.n_qkv + col);
-                    qb[t] = ld_cg_f4_inorder(P.qkv_acc + (size_t)(r0 + j) * P.n_qkv + col + HD2);
-                    const int pj = TREE ? __ldcg(P.state + ST_DEPTH + j) : j;  // tree drafts: a row's position is its depth
-                    const float4* rp = reinterpret_cast<const float4*>(P.rope + (size_t)(L + pj) * HD2 + ii[t]);
-                    c0[t] = ld_nc_f4_inorder(rp);
-                    c1[t] = ld_nc_f4_inorder(rp + 1);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < QI; ++t) {
-                const int idx = base + t * kWorkerThreads;
-                if (idx >= items) continue;
-                const int r = rr[t], i = ii[t];
-                uint2 lo = make_uint2(0, 0), hi = make_uint2(0, 0);
-                if (r < R) {
-                    const float rs = rsqrtf(ssq[t] / (float)P.d + P.eps);
-                    float a[4] = {qa[t].x * rs, qa[t].y * rs, qa[t].z * rs, qa[t].w * rs};
-                    float b[4] = {qb[t].x * rs, qb[t].y * rs, qb[t].z * rs, qb[t].w * rs};
-                    if (bias) {
-                        const int col = (head0 + r / M) * HD + i;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) { a[e] += bias[col + e]; b[e] += bias[col + HD2 + e]; }
-                    }
-                    const float cs[4] = {c0[t].x, c0[t].z, c1[t].x, c1[t].z}, sn[4] = {c0[t].y, c0[t].w, c1[t].y, c1[t].w};
-                    float x0[4], x1[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) { x0[e] = a[e] * cs[e] - b[e] * sn[e]; x1[e] = b[e] * cs[e] + a[e] * sn[e]; }
-                    lo = make_uint2(pack_bf16(x0[0], x0[1]), pack_bf16(x0[2], x0[3]));
-                    hi = make_uint2(pack_bf16(x1[0], x1[1]), pack_bf16(x1[2], x1[3]));
-                }
-                const int cA = i, cB = i + HD2;
-                *reinterpret_cast<uint2*>(Qs + (cA >> 6) * (RP * 128) + swz_off(r, cA & 63)) = lo;
-                *reinterpret_cast<uint2*>(Qs + (cB >> 6) * (RP * 128) + swz_off(r, cB & 63)) = hi;
-            }
-        }
+        for (int b = loaded; b < NBUF; ++b) attn_load_block<HD>(P, u, layer, b, att, wtid);
     }
-    // the new rows' own keys and values fit one block (M <= 32 <= KB)
-    if (is_new) {
-        uint8_t* Ks = KVs;
-        uint8_t* Vs = Ks + KVBYTES;
-        // K and V rows of the new tokens: finish the projection, rotate K, append to the cache
-#pragma unroll 1
-        for (int u = wtid; u < KB * UNITS; u += kWorkerThreads) {
-            const int key = u / UNITS, q16 = u % UNITS, kk = key;
-            uint4 kv4 = make_uint4(0, 0, 0, 0), vv4 = make_uint4(0, 0, 0, 0);
-            if (kk < nkeys) {
-                const float rs = rsqrtf(__ldcg(sumsq + r0 + kk) / (float)P.d + P.eps);
-                const float* accrow = P.qkv_acc + (size_t)(r0 + kk) * P.n_qkv;
-                const int colb = q16 * 8, ib = colb % HD2;  // 8 columns share one half of the rotary pairing
-                const float* pa = accrow + Nq + hk * HD + ib;
-                const float4 a0 = ldcg_f4(pa), a1 = ldcg_f4(pa + 4), b0 = ldcg_f4(pa + HD2), b1 = ldcg_f4(pa + HD2 + 4);
-                const float* pv = accrow + Nq + Nkv + hk * HD + colb;
-                const float4 v0 = ldcg_f4(pv), v1 = ldcg_f4(pv + 4);
-                const int pk = TREE ? __ldcg(P.state + ST_DEPTH + kk) : kk;
-                const float4* rp = reinterpret_cast<const float4*>(P.rope + (size_t)(L + pk) * HD2 + ib);
-                const float4 r0 = __ldg(rp), r1 = __ldg(rp + 1), r2 = __ldg(rp + 2), r3 = __ldg(rp + 3);
-                float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-                const float cs[8] = {r0.x, r0.z, r1.x, r1.z, r2.x, r2.z, r3.x, r3.z};
-                const float sn[8] = {r0.y, r0.w, r1.y, r1.w, r2.y, r2.w, r3.y, r3.w};
-                float kvals[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    a[e] *= rs; b[e] *= rs; v[e] *= rs;
-                    if (bias) {
-                        a[e] += bias[Nq + hk * HD + ib + e];
-                        b[e] += bias[Nq + hk * HD + ib + HD2 + e];
-                        v[e] += bias[Nq + Nkv + hk * HD + colb + e];
-                    }
-                    kvals[e] = (colb < HD2) ? (a[e] * cs[e] - b[e] * sn[e]) : (b[e] * cs[e] + a[e] * sn[e]);
-                }
-                kv4 = make_uint4(pack_bf16(kvals[0], kvals[1]), pack_bf16(kvals[2], kvals[3]),
-                                 pack_bf16(kvals[4], kvals[5]), pack_bf16(kvals[6], kvals[7]));
-                vv4 = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                                 pack_bf16(v[6], v[7]));
-                if (qg == 0) {  // every head group computes the rows, one appends them
-                    const size_t off = (cache_row0 + L + kk) * HD + q16 * 8;
-                    *reinterpret_cast<uint4*>(kcache + off) = kv4;
-                    *reinterpret_cast<uint4*>(vcache + off) = vv4;
-                }
-            }
-            const uint32_t so = (q16 >> 3) * (KB * 128) + swz_unit(key, q16 & 7);
-            *reinterpret_cast<uint4*>(Ks + so) = kv4;
-            *reinterpret_cast<uint4*>(Vs + so) = vv4;
-        }
-    }
+    cp_async_wait<0>();   // the queries, and with them the first blocks
     if (prof && wtid == 0) prof[3] = global_timer_ns();
 
     const int g = lane >> 2, q2 = (lane & 3) * 2;
     const int r_lo = mt * 16 + g, r_hi = r_lo + 8;
-    const int j_lo = r_lo % M, j_hi = r_hi % M;
-    // new keys a row may see: rows 0..j of a chain, its own path from the root in a tree
-    const bool tree_mask = TREE && is_new;
-    const unsigned see_lo = tree_mask ? (unsigned)__ldcg(P.state + ST_ANC + j_lo) : 0u;
-    const unsigned see_hi = tree_mask ? (unsigned)__ldcg(P.state + ST_ANC + j_hi) : 0u;
+    const int h_lo = (int)((uint32_t)r_lo * minv >> 16), h_hi = (int)((uint32_t)r_hi * minv >> 16);
+    const int j_lo = r_lo - h_lo * M, j_hi = r_hi - h_hi * M;
+    // last key (within the range) a row sees; in a tree the new keys it sees are a bit mask
+    const int new0 = u.L - u.t_begin;
+    const int lim_lo = TREE ? nkeys - 1 : min(new0 + j_lo, nkeys - 1), lim_hi = TREE ? nkeys - 1 : min(new0 + j_hi, nkeys - 1);
+    const unsigned see_lo = TREE ? (unsigned)__ldcg(P.state + ST_ANC + min(j_lo, kMaxRows - 1)) : 0u;
+    const unsigned see_hi = TREE ? (unsigned)__ldcg(P.state + ST_ANC + min(j_hi, kMaxRows - 1)) : 0u;
     float o[NT_O][4];
 #pragma unroll
     for (int n = 0; n < NT_O; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
@@ -829,7 +898,7 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
 
 #pragma unroll 1
     for (int blk = 0; blk < nblk; ++blk) {
-        if (!is_new) cp_async_wait<NBUF - 1>();
+        if (blk > 0) cp_async_wait<NBUF - 1>();
         named_bar_sync(1, kWorkerThreads);  // the block (and, first time, the Q tile) is in place
         if (prof && wtid == 0 && blk == 0) prof[4] = global_timer_ns();
         if (active) {
@@ -851,15 +920,15 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
                     mma_bf16_16816(sc[1], a0, a1, a2, a3, b2, b3);
                 }
                 float mx_lo = -CUDART_INF_F, mx_hi = -CUDART_INF_F;
+                const int key0 = blk * KB + c * 16 + q2;
 #pragma unroll
                 for (int n = 0; n < 2; ++n)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const int key = blk * KB + c * 16 + n * 8 + q2 + (e & 1);
+                        const int key = key0 + n * 8 + (e & 1);
                         const bool hi = e >= 2;
-                        const int row = hi ? r_hi : r_lo, j = hi ? j_hi : j_lo;
-                        bool ok = key < nkeys && row < R && (!is_new || key <= j);
-                        if (TREE && tree_mask) ok = key < nkeys && row < R && (((hi ? see_hi : see_lo) >> (key & 31)) & 1u);
+                        bool ok = key <= (hi ? lim_hi : lim_lo);
+                        if (TREE && key >= new0) ok = ok && (((hi ? see_hi : see_lo) >> ((key - new0) & 31)) & 1u);
                         const float v = ok ? sc[n][e] * P.scale_log2e : -CUDART_INF_F;
                         sc[n][e] = v;
                         if (hi) mx_hi = fmaxf(mx_hi, v); else mx_lo = fmaxf(mx_lo, v);
@@ -901,9 +970,10 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
             }
         }
         named_bar_sync(1, kWorkerThreads);  // the block has been consumed
-        if (!is_new) load_block(blk + NBUF);
+        if (blk + NBUF < nblk && warp < kEpilogueWarps) attn_load_block<HD>(P, u, layer, blk + NBUF, att, wtid);
+        else cp_async_commit();
     }
-    if (!is_new) cp_async_wait<0>();
+    cp_async_wait<0>();
     if (prof && wtid == 0) prof[5] = global_timer_ns();
 
     // ---- row sums over the quad; the key groups of a row tile meet in shared memory
@@ -952,8 +1022,7 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
         for (int half = 0; half < 2; ++half) {
             const int r = half ? r_hi : r_lo;
             if (r >= R) continue;
-            const int hq = head0 + r / M, j = r % M;
-            const size_t row = ((size_t)hq * (kMaxSplits + 1) + s) * kMaxRows + r0 + j;
+            const size_t row = ((size_t)(u.head0 + (half ? h_hi : h_lo)) * kMaxSplits + u.s) * kMaxRows + u.r0 + (half ? j_hi : j_lo);
             float* po = P.part_o + row * HD + q2;
 #pragma unroll
             for (int n = 0; n < NT_O; ++n)
@@ -964,29 +1033,41 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, in
     }
 }
 
+// `early`: key blocks of the block's first unit that were requested before the grid barrier.
 template <int HD, int MODE>
-__device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, uint8_t* att, int wtid, unsigned long long* prof) {
-    int S, kps;
-    attn_split(P, S, kps);
-    const int S1 = S + 1;
-    const int gh = P.att_gh, QG = P.att_QG;
-    const int per_seq = P.att_per_seq;
-    const int nunits = per_seq * (P.nseq > 0 ? P.nseq : 1);
+__device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, int early, uint8_t* att, int wtid, unsigned long long* prof) {
+    const int per_seq = P.att_per_seq, QG = P.att_QG, S = P.att_S;
+    const int nunits = per_seq * (MODE == 2 ? P.nseq : 1);
 #pragma unroll 1
     for (int unit = blockIdx.x; unit < nunits; unit += P.G) {
         int b = P.att_b0, hk = P.att_hk0, qg = P.att_qg0, s = P.att_s0;
         if (unit != (int)blockIdx.x) {  // further units of this block (more units than blocks: batched steps)
-            const int u = unit % per_seq, rem = u % (QG * S1);
+            const int u = unit % per_seq, rem = u % (QG * S);
             b = unit / per_seq;
-            hk = u / (QG * S1);
-            qg = rem / S1;
-            s = rem % S1;
+            hk = u / (QG * S);
+            qg = rem / S;
+            s = rem % S;
+            early = 0;
         }
         // batched: every sequence takes the key ranges of the longest one; a range past its own length holds no key
-        attention_unit<HD, MODE>(P, layer, hk, qg, gh, s, S, kps, att, wtid, prof, b);
+        attention_unit<HD, MODE>(P, layer, attn_unit<HD, MODE>(P, b, hk, qg, s), early, att, wtid, prof);
         named_bar_sync(1, kWorkerThreads);  // the unit's shared-memory tiles are free again
-        if (prof && wtid == 0) { prof[6] = global_timer_ns(); prof[7] = (unsigned long long)(s == S); }
+        if (prof && wtid == 0) { prof[6] = global_timer_ns(); prof[7] = (unsigned long long)(s + 1 == S); }
     }
+}
+// Before the grid barrier in front of the attention phase: requests the first key blocks of the block's unit that do not hold
+// new rows.  Only once the block's own products of the phase before have completed (their operand lies where the keys go), which
+// warps 0..7 know from their epilogue.
+template <int HD, int MODE>
+__device__ __forceinline__ int attention_early(const FwdParams& P, int layer, uint8_t* att, int wtid) {
+    if ((int)blockIdx.x >= P.att_per_seq * (MODE == 2 ? P.nseq : 1)) return 0;
+    const AttnUnit u = attn_unit<HD, MODE>(P, P.att_b0, P.att_hk0, P.att_qg0, P.att_s0);
+    const int n = attn_early_blocks<HD>(u);
+    if ((wtid >> 5) < kEpilogueWarps) {
+#pragma unroll 1
+        for (int b = 0; b < n; ++b) attn_load_block<HD>(P, u, layer, b, att, wtid);
+    }
+    return n;
 }
 // ------------------------------------------------------------------------------------------
 __device__ void embed_phase(const FwdParams& P, int wtid) {
@@ -1014,15 +1095,6 @@ __device__ void embed_phase(const FwdParams& P, int wtid) {
         __stcg(reinterpret_cast<float4*>(dst + 4), hi);
     }
 }
-__device__ void zero_qkv_acc(const FwdParams& P, int sumsq_buf, int wtid) {
-    const int n4 = kMaxRows * P.n_qkv / 4;
-#pragma unroll 1
-    for (int i = blockIdx.x * kWorkerThreads + wtid; i < n4; i += P.G * kWorkerThreads)
-        __stcg(reinterpret_cast<float4*>(P.qkv_acc) + i, make_float4(0.f, 0.f, 0.f, 0.f));
-    if (blockIdx.x == 0 && wtid < kMaxRows) __stcg(P.sumsq + sumsq_buf * kMaxRows + wtid, 0.f);
-}
-
-
 // ------------------------------------------------------------------------------------------
 // One GEMM phase as seen by the worker warps: build the token operand, then the tensor-core
 // thread walks the block's stages while the epilogue warps drain the accumulators.
@@ -1033,8 +1105,9 @@ __device__ __forceinline__ void advance_pos(PipePos& pos, const Part& pt, uint32
     pos.q += (uint32_t)pt.npass;
 }
 
-__device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int layer, uint8_t* smem, Misc* misc, PipePos& pos, int wtid,
-                                        unsigned long long* prof) {
+template <int HD, int MODE>
+__device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int layer, const NormPrep& prep, uint8_t* smem, Misc* misc,
+                                        PipePos& pos, int wtid, unsigned long long* prof) {
     const int warp = wtid >> 5, lane = wtid & 31;
     uint8_t* U = smem + P.u_off;
     uint8_t* act = smem + P.act_off;
@@ -1047,27 +1120,18 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int lay
     if (have0) {
         if (!dead) {
             if (kind == PH_O) build_merged_operand(P, p0, U, wtid);
-            else build_norm_operand(P, kind, layer, p0, U, misc, wtid);
+            else build_norm_operand(P, prep, U, misc, wtid);
         }
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&misc->op_ready);   // this warp's part of the operand may be read by the tensor core
-    }
-    if (kind == PH_O && warp >= 4) {
-        // clear the accumulators the next QKV projection adds into (idle warps)
-        const int n4 = kMaxRows * P.n_qkv / 4, nth = (kBuilderWarps - 4) * 32;
-#pragma unroll 1
-        for (int i = blockIdx.x * nth + (wtid - 4 * 32); i < n4; i += P.G * nth)
-            __stcg(reinterpret_cast<float4*>(P.qkv_acc) + i, make_float4(0.f, 0.f, 0.f, 0.f));
-        if (blockIdx.x == 0 && wtid < 4 * 32 + kMaxRows)
-            __stcg(P.sumsq + ((layer + 1) & 1) * kMaxRows + (wtid - 4 * 32), 0.f);
     }
     if (prof && wtid == 0) prof[2] = global_timer_ns();
     if (warp < kEpilogueWarps) {
         // the rows' sums of squares the epilogue scales with come from all builder warps
         if (have0 && !dead && !mbar_wait_bounded(&misc->op_ready, pos.ops & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
         PipePos ep = pos;
-        epilogue_phase(P, kind, act, misc, ep, dead, warp, lane);
+        epilogue_phase<HD, MODE>(P, kind, layer, act, misc, ep, dead, warp, lane);
         if (prof && wtid == 0) prof[4] = global_timer_ns();
     }
     // pipeline positions advance identically for every role
@@ -1183,17 +1247,22 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     // these writes before it
     if (tid == 0) {
         if (Pg.l_from_state) misc->P.L = Pg.state[ST_KV_LEN];
-        attn_split_compute(misc->P, misc->P.att_S, misc->P.att_kps);
         // the block's first attention unit: the same for every layer, so its index arithmetic is done here
         FwdParams& Q = misc->P;
-        const int S1 = Q.att_S + 1;
+        int keys = Q.L + Q.M;
+        if (MODE == 2) {
+            keys = 1;
+            for (int b = 0; b < Q.nseq; ++b) keys = max(keys, Q.seq[b].L + Q.seq[b].M);
+        }
+        attn_split_compute(Q, keys, Q.att_S, Q.att_kps);
+        const int S = Q.att_S;
         Q.att_QG = (Q.g + Q.att_gh - 1) / Q.att_gh;
-        Q.att_per_seq = Q.n_kv * Q.att_QG * S1;
-        const int unit = blockIdx.x, u = unit % Q.att_per_seq, rem = u % (Q.att_QG * S1);
+        Q.att_per_seq = Q.n_kv * Q.att_QG * S;
+        const int unit = blockIdx.x, u = unit % Q.att_per_seq, rem = u % (Q.att_QG * S);
         Q.att_b0 = unit / Q.att_per_seq;
-        Q.att_hk0 = u / (Q.att_QG * S1);
-        Q.att_qg0 = rem / S1;
-        Q.att_s0 = rem % S1;
+        Q.att_hk0 = u / (Q.att_QG * S);
+        Q.att_qg0 = rem / S;
+        Q.att_s0 = rem % S;
     }
 
     if (warp == kProducerWarp) {
@@ -1215,21 +1284,31 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
     int nbar = 0;
     bool skip = false;
+    int layer, kind = decode_phase(P.ph_begin, P.n_layers, layer);
+    NormPrep prep;
+    int early = 0;
+    auto prepare = [&](int ph) {
+        kind = decode_phase(ph, P.n_layers, layer);
+        if (kind == PH_ATTN) early = attention_early<HD, MODE>(P, layer, smem + P.u_off, wtid);
+        else if (kind != PH_EMBED && kind != PH_O) {
+            int ops[2];
+            phase_ops(kind, ops);
+            prep = norm_prep(P, kind, layer, misc->part[ops[0]], wtid >> 5);
+        }
+    };
+    prepare(P.ph_begin);
 #pragma unroll 1
     for (int ph = P.ph_begin; ph < P.ph_end; ++ph) {
-        int layer;
-        const int kind = decode_phase(ph, P.n_layers, layer);
         unsigned long long* pp = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
         if (pp && wtid == 0) pp[0] = global_timer_ns();
         // after an abandoned wait the remaining phases do no work but still meet at every barrier
         if (skip) {
         } else if (kind == PH_EMBED) {
             embed_phase(P, wtid);
-            zero_qkv_acc(P, 0, wtid);
         } else if (kind == PH_ATTN) {
-            attention_phase<HD, MODE>(P, layer, smem + P.u_off, wtid, pp);
+            attention_phase<HD, MODE>(P, layer, early, smem + P.u_off, wtid, pp);
         } else {
-            gemm_phase(P, kind, layer, smem, misc, pos, wtid, pp);
+            gemm_phase<HD, MODE>(P, kind, layer, prep, smem, misc, pos, wtid, pp);
         }
         if (pp) {
             named_bar_sync(1, kWorkerThreads);
@@ -1237,7 +1316,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         }
         if (ph + 1 < P.ph_end) {
             ++nbar;
-            skip = grid_barrier(P, P.bar_base + (unsigned)(nbar * P.G), misc, wtid);
+            skip = grid_barrier(P, P.bar_base + (unsigned)(nbar * P.G), misc, wtid, [&]() { prepare(ph + 1); });
         }
     }
     tc_fence_before();

@@ -11,6 +11,12 @@
 //     [step][half][8-row group][row][8 bf16]
 // with no padding.  Stages follow each other pass by pass, so every stage is one contiguous
 // bulk copy and a block's whole share of an operation is one contiguous byte range.
+//
+// A share of few row tiles would leave most of a 128-row instruction empty.  Such an operation is cut into K slices
+// that are stacked as rows: with `slices` = 8 the 16 rows of one tile and eighths of their columns fill the 128 rows, the token
+// operand is stacked the same way (eight times the token rows), and only the blocks on the diagonal of the product
+// are wanted (slice s of the rows against slice s of the tokens); they are added up in the epilogue.  A column step
+// of the stage then holds `slices` real column steps, one per slice.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -29,7 +35,7 @@ constexpr int kStageBytes = 32768;                     // ring slot
 constexpr int kMaxStages = 8;                          // ring slots at most
 constexpr int kMaxRows = 32;                           // token rows a buffer is sized for
 constexpr int kMaxBatch = 8;                           // sequences one batched verify step takes at most
-constexpr int kMaxSplits = 19;                         // KV key ranges per head (+1 partial result for the new rows)
+constexpr int kMaxSplits = 20;                         // key ranges per head at most
 constexpr int kSmemBudget = 232448;                    // 227 KB
 constexpr int kAttnSmemBytes = 81920;                  // Q tile (up to 16 KB) + two K|V blocks of 64 keys (64 KB)
 constexpr int kActSmemMax = 32768;                     // SwiGLU output of this block (operand of its down-projection slice) at most
@@ -40,7 +46,8 @@ constexpr unsigned kLookaheadPiece = 8192;             //   in pieces of this si
 constexpr int kLookaheadCycles = 800;                  //   and no more often than this
 constexpr int kMaxDraftWords = 32;
 constexpr int kProfWords = 12;                         // timestamps per (phase, block)
-constexpr int kTmemCols = 128;                         // two buffers of two 128-row accumulators of up to 32 fp32 columns
+constexpr int kTmemCols = 512;                         // two buffers; each two 128-row accumulators of up to 32 fp32 columns, or one of up to 256
+constexpr uint32_t kTmemBuf = 256;                     //   (stacked K slices)
 
 enum OpIndex { OP_QKV = 0, OP_O = 1, OP_GU = 2, OP_DOWN = 3, OP_LM = 4, OP_RAW = 5, OP_COUNT = 6 };
 
@@ -54,7 +61,7 @@ struct OpDesc {
     int SK;      // column steps per stage at most (RW * SK <= 64)
     int unit;    // row partitions are multiples of this many tiles (2 for gate|up: 16 SwiGLU columns)
     int follow;  // 1: one row partition; block i takes the columns that partition i of `gate|up` produces
-    int pad;
+    int slices;  // K slices stacked as rows (0 or 1: none); divides K16 and the column shares
     unsigned long long w_off;  // byte offset of the operation inside its weight region
 };
 
@@ -63,7 +70,7 @@ struct Part {
     unsigned long long off;  // byte offset of this partition from the operation's base
     int npass, nst;          // passes over the row tiles; stages per pass
     int pbase, prem;         // tiles per pass: pbase + (p < prem)
-    int SK, pad;
+    int SK, slices;
 };
 __host__ __device__ inline int pass_count(const Part& p, int i) { return p.pbase + (i < p.prem ? 1 : 0); }
 __host__ __device__ inline int pass_start(const Part& p, int i) { return i * p.pbase + (i < p.prem ? i : p.prem); }
@@ -86,8 +93,9 @@ __host__ __device__ inline void finish_part(Part& p, const OpDesc& o) {
     p.off = (unsigned long long)kStepBytes *
             ((unsigned long long)p.tile0 * o.K16 + (unsigned long long)p.ntiles * p.k0);
     p.SK = o.SK;
+    p.slices = o.slices > 1 ? o.slices : 1;
     p.npass = (p.ntiles + o.RW - 1) / o.RW;
-    p.nst = (p.nk + o.SK - 1) / o.SK;
+    p.nst = (p.nk / p.slices + o.SK - 1) / o.SK;
     p.pbase = p.npass ? p.ntiles / p.npass : 0;
     p.prem = p.npass ? p.ntiles % p.npass : 0;
 }
@@ -97,7 +105,6 @@ __host__ __device__ inline Part make_part(const OpDesc& o, const OpDesc& gu, int
     Part p;
     p.pr = pr;
     p.pk = pk;
-    p.pad = 0;
     if (o.follow) {
         p.tile0 = 0;
         p.ntiles = o.T;
@@ -120,8 +127,9 @@ __host__ __device__ inline Part get_part(const OpDesc& o, const OpDesc& gu, int 
     if (idx < 0) idx += G;
     if (idx >= nparts) {
         Part p;
-        p.tile0 = p.ntiles = p.k0 = p.nk = p.pr = p.pk = p.npass = p.nst = p.pbase = p.prem = p.pad = 0;
+        p.tile0 = p.ntiles = p.k0 = p.nk = p.pr = p.pk = p.npass = p.nst = p.pbase = p.prem = 0;
         p.SK = o.SK;
+        p.slices = 1;
         p.off = 0;
         return p;
     }
@@ -146,11 +154,12 @@ __host__ __device__ inline unsigned long long weight_offset(const OpDesc& o, con
     const int pass = even_find(p.ntiles, p.npass, lt);
     const int start = pass_start(p, pass), pcount = pass_count(p, pass);
     const int tip = lt - start, lk = ks - p.k0;
-    const int st = lk / p.SK, kin = lk % p.SK;
+    const int per = p.nk / p.slices, slice = lk / per, vk = lk % per;   // column steps per slice
+    const int st = vk / p.SK, kin = vk % p.SK, v = pcount * p.slices;   // v: row tiles of the stage, slices stacked
     const unsigned long long stage_base =
-        p.off + (unsigned long long)kStepBytes * ((unsigned long long)start * p.nk + (unsigned long long)pcount * st * p.SK);
+        p.off + (unsigned long long)kStepBytes * ((unsigned long long)start * p.nk + (unsigned long long)v * st * p.SK);
     const unsigned long long in_stage =
-        ((unsigned long long)(kin * 2 + half) * (2 * pcount) + (tip * 2 + ((row & 15) >> 3))) * 128 + (row & 7) * 16;
+        ((unsigned long long)(kin * 2 + half) * (2 * v) + ((slice * pcount + tip) * 2 + ((row & 15) >> 3))) * 128 + (row & 7) * 16;
     return stage_base + in_stage;
 }
 
@@ -204,10 +213,9 @@ struct FwdParams {
     __nv_bfloat16* vcache;
     // activations (global, L2 resident)
     float* h;          // [kMaxRows][d] residual stream
-    float* qkv_acc;    // [kMaxRows][n_qkv] un-normalised q|k|v sums
-    float* sumsq;      // [2][kMaxRows] sum of squares of h rows for the attention-side norm
-    float* part_o;     // [n_q][kMaxSplits+1][kMaxRows][hd] un-normalised split outputs
-    float* part_ml;    // [n_q][kMaxSplits+1][kMaxRows][2]  (running max in log2 units, sum)
+    __nv_bfloat16* q;  // [kMaxRows][n_q * hd] queries, rotated
+    float* part_o;     // [n_q][kMaxSplits][kMaxRows][hd] un-normalised split outputs
+    float* part_ml;    // [n_q][kMaxSplits][kMaxRows][2]  (running max in log2 units, sum)
     float* cand_val;   // [G][kMaxRows] per-block best logit
     int* cand_idx;     // [G][kMaxRows] and its token id
     float* logits;     // [kMaxRows][V]
@@ -247,7 +255,7 @@ struct FwdParams {
     BatchSeq seq[kMaxBatch];
 };
 
-// Shared-memory plan of a launch over `rows` token rows: ring of weight stages | operand region | SwiGLU operand |
+// Shared-memory plan of a launch over `rows` token rows: ring of weight stages | operand region | SwiGLU operand (or q|k|v exchange) |
 // bookkeeping (at kMiscOff).  The operand region holds the token operand of the widest GEMM share (or the attention
 // tiles); the ring takes what is left.  Fewer than two ring slots: the rows do not fit.
 __host__ __device__ inline void plan_smem_rows(FwdParams& P, int rows) {
@@ -255,7 +263,9 @@ __host__ __device__ inline void plan_smem_rows(FwdParams& P, int rows) {
     int u = P.plan_ks * step_bytes;
     if (u < P.plan_attn) u = P.plan_attn;
     u = (u + 1023) / 1024 * 1024;
-    const int act = P.plan_act > 0 ? (P.plan_act * step_bytes + 1023) / 1024 * 1024 : 1024;
+    int act = P.plan_act * step_bytes;
+    if (P.plan_attn > 0 && act < 128 * (rows | 1) * 4) act = 128 * (rows | 1) * 4;   // exchange area of the q|k|v epilogue
+    act = act > 0 ? (act + 1023) / 1024 * 1024 : 1024;
     const int ring = kMiscOff - act - u;
     P.nstage = ring < 0 ? 0 : ring / kStageBytes;
     if (P.nstage > kMaxStages) P.nstage = kMaxStages;

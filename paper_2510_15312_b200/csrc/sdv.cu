@@ -14,6 +14,7 @@
 #include "dense.cuh"
 #include "forward.cuh"
 #include "layout.cuh"
+#include "small_gemm.cuh"
 #include "small_kernels.cuh"
 
 using namespace sdv;
@@ -23,7 +24,7 @@ namespace {
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Regions {
-    size_t state, bstate, bar, never, hist, db, rope, norm_w, bias, wlayers, wlm, emb, kcache, vcache, h, qkv_acc, sumsq, part_o,
+    size_t state, bstate, bar, never, hist, db, rope, norm_w, bias, wlayers, wlm, emb, kcache, vcache, h, q, part_o,
         part_ml, cand_val, cand_idx, logits, raw_out, staging, wraw, xstage, prof, succ, occ, dw, dlm, dh, dxn, dpart, dq, datt, dact, total;
     size_t layer_stride, staging_bytes, raw_kmax;
 };
@@ -76,14 +77,13 @@ Regions carve(const sdv_config* c, bool own_weights = true) {
     r.kcache = take(kvb);
     r.vcache = take(kvb);
     r.h = take((size_t)kMaxRows * d * 4);
-    r.qkv_acc = take((size_t)kMaxRows * nqkv * 4);
-    r.sumsq = take(2 * kMaxRows * 4);
+    r.q = take((size_t)kMaxRows * nq * 2);
     size_t raw_kmax = f;  // the stand-alone GEMM takes operands of any K up to max(f, d, nq)
     if (d > raw_kmax) raw_kmax = d;
     if (nq > raw_kmax) raw_kmax = nq;
     r.raw_kmax = raw_kmax;
-    r.part_o = take((size_t)c->n_q_heads * (kMaxSplits + 1) * kMaxRows * hd * 4);
-    r.part_ml = take((size_t)c->n_q_heads * (kMaxSplits + 1) * kMaxRows * 2 * 4);
+    r.part_o = take((size_t)c->n_q_heads * kMaxSplits * kMaxRows * hd * 4);
+    r.part_ml = take((size_t)c->n_q_heads * kMaxSplits * kMaxRows * 2 * 4);
     r.cand_val = take((size_t)kMaxGrid * kMaxRows * 4);
     r.cand_idx = take((size_t)kMaxGrid * kMaxRows * 4);
     r.logits = take((size_t)kMaxRows * V * 4);
@@ -175,6 +175,18 @@ void full_k_partition(OpDesc& o, int G, int unit) {
     o.P_row = o.T / unit < G ? o.T / unit : G;
 }
 
+// q|k|v: all columns in one block as well (its epilogue finishes the projection).  A share is a tile or a few, so eighths (or
+// quarters, halves) of its columns are stacked to fill the instruction's 128 rows.
+void stacked_partition(OpDesc& o, int G) {
+    full_k_partition(o, G, 1);
+    const int per = (o.T + o.P_row - 1) / o.P_row;   // row tiles of the largest share
+    o.slices = 8;
+    while (o.slices > 1 && (o.slices * per > 8 || o.K16 % o.slices)) o.slices /= 2;
+    o.RW = 8 / o.slices;                             // one accumulator per pass
+    while (o.RW > 1 && o.RW / 2 >= per) o.RW /= 2;
+    o.SK = kStageBytes / kStepBytes / (o.RW * o.slices);
+}
+
 // Shared-memory plan of a launch over `rows` token rows (plan_smem_rows), and whether they fit.
 struct SmemPlan {
     int NG, NB, nstage, u_bytes;
@@ -218,7 +230,7 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
         o.T = ops[i].N / 16;
         o.K16 = ops[i].K / 16;
         switch (ops[i].idx) {
-            case OP_QKV: choose_partition(o, G, rows_max, false, false); break;
+            case OP_QKV: stacked_partition(o, G); break;
             case OP_O: choose_partition(o, G, rows_max, true, true); break;
             case OP_GU: full_k_partition(o, G, 2); break;   // pairs of tiles: 16 SwiGLU columns = one column step of down
             case OP_LM: full_k_partition(o, G, 1); break;
@@ -226,7 +238,7 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
                 o.RW = 16; o.SK = kStageBytes / kStepBytes / 16; o.unit = 1; o.follow = 1; o.P_row = 1; o.P_k = P.op[OP_GU].P_row;
                 break;
         }
-        fit_pass_width(o);
+        if (ops[i].idx != OP_QKV) fit_pass_width(o);
         if (ops[i].idx == OP_DOWN) {
             o.rot = P.op[OP_GU].rot;
         } else {
@@ -323,16 +335,12 @@ int plan_attention(const FwdParams& P, int rows, int L, int nseq) {
         if (gh * rows > 64 && gh > 1) break;
         const int MT = (gh * rows + 15) / 16, KG = MT <= 2 ? 4 : (MT == 3 ? 3 : 2);
         const int QG = (P.g + gh - 1) / gh;
-        int cap = P.G / (P.n_kv * QG) - 1;
+        int cap = P.G / (P.n_kv * QG);
         if (cap > kMaxSplits) cap = kMaxSplits;
         if (cap < 1) cap = 1;
-        int cost = 1, S = 0;
-        if (L > 0) {
-            const int kps = ((L + cap - 1) / cap + 63) / 64 * 64;
-            S = (L + kps - 1) / kps;
-            cost = (kps / 64) * ((4 + KG - 1) / KG);
-        }
-        const int rounds = (P.n_kv * QG * (S + 1) * nseq + P.G - 1) / P.G;
+        const int keys = L + rows, kps = ((keys + cap - 1) / cap + 63) / 64 * 64, S = (keys + kps - 1) / kps;
+        int cost = (kps / 64) * ((4 + KG - 1) / KG);
+        const int rounds = (P.n_kv * QG * S * nseq + P.G - 1) / P.G;
         cost = rounds * (3 + cost);
         if (best < 0 || cost <= best) {  // ties: more heads per unit (fewer reloads of the keys)
             best = cost;
@@ -402,7 +410,7 @@ int pack_op(sdv_ctx* ctx, const OpDesc& o, uint8_t* dst_base, const uint16_t* s0
     int blocks = (int)((total + 255) / 256);
     if (blocks > 148 * 16) blocks = 148 * 16;
     pack_weights_kernel<<<blocks, 256, 0, ctx->stream>>>(o, ctx->P.op[OP_GU], dst_base, s0, rows0, s1, rows1, s2, K, mode,
-                                                       t_begin, t_end, row_base);
+                                                       t_begin, t_end, row_base, ctx->cfg.head_dim);
     ctx->launches++;
     CK(cudaGetLastError());
     return SDV_OK;
@@ -631,7 +639,7 @@ const char* sdv_strerror(int code) {
         case SDV_ESTATE: return "call not valid in the current state";
         case SDV_ECUDA: return "CUDA runtime error";
         case SDV_ETIMEOUT: return "a bounded device-side wait ran out";
-        case SDV_ETOOBIG: return "problem larger than the fixed scratch area of the no-allocation entry point";
+        case SDV_ETOOBIG: return "problem larger than the no-allocation entry point takes";
         default: return "unknown error";
     }
 }
@@ -717,8 +725,7 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
     P.kcache = (__nv_bfloat16*)(ws + ctx->r.kcache);
     P.vcache = (__nv_bfloat16*)(ws + ctx->r.vcache);
     P.h = (float*)(ws + ctx->r.h);
-    P.qkv_acc = (float*)(ws + ctx->r.qkv_acc);
-    P.sumsq = (float*)(ws + ctx->r.sumsq);
+    P.q = (__nv_bfloat16*)(ws + ctx->r.q);
     P.part_o = (float*)(ws + ctx->r.part_o);
     P.part_ml = (float*)(ws + ctx->r.part_ml);
     P.cand_val = (float*)(ws + ctx->r.cand_val);
@@ -852,7 +859,7 @@ int sdv_load_weights(sdv_ctx* ctx, const sdv_weights* w) {
         CK(cudaMemcpyAsync(stg + nq * d, L.wk, nkv * d * 2, cudaMemcpyDefault, s));
         CK(cudaMemcpyAsync(stg + (nq + nkv) * d, L.wv, nkv * d * 2, cudaMemcpyDefault, s));
         rc = pack_op(ctx, ctx->P.op[OP_QKV], lbase + ctx->P.op[OP_QKV].w_off, stg, (int)nq, stg + nq * d, (int)nkv,
-                     stg + (nq + nkv) * d, (int)d, 0, 0, ctx->P.op[OP_QKV].T, 0);
+                     stg + (nq + nkv) * d, (int)d, 2, 0, ctx->P.op[OP_QKV].T, 0);
         if (rc) return rc;
         // row-major copies for the dense prefill path: q|k|v, o, gate|up (interleaved by 64), down
         uint16_t* dbase = (uint16_t*)(ws + ctx->r.dw + (size_t)l * ctx->r.layer_stride);
@@ -1672,10 +1679,13 @@ int sdv_debug_layout_check(const int* desc, const int* gu_desc, int G) {
     memset(&o, 0, sizeof(o));
     memset(&gu, 0, sizeof(gu));
     o.T = desc[0]; o.K16 = desc[1]; o.P_row = desc[2]; o.P_k = desc[3]; o.RW = desc[4]; o.SK = desc[5]; o.unit = desc[6];
-    o.follow = desc[7];
+    o.follow = desc[7] & 0xff;
+    o.slices = desc[7] >> 8;
     gu.T = gu_desc[0]; gu.K16 = gu_desc[1]; gu.P_row = gu_desc[2]; gu.P_k = gu_desc[3]; gu.RW = gu_desc[4]; gu.SK = gu_desc[5];
     gu.unit = gu_desc[6];
     if (o.T < 1 || o.K16 < 1 || o.RW < 1 || o.SK < 1 || o.RW * o.SK * kStepBytes > kStageBytes || o.unit < 1 || o.T % o.unit) return SDV_EINVAL;
+    const int slices = o.slices > 1 ? o.slices : 1;
+    if (o.K16 % slices || (slices > 1 && o.P_k != 1) || o.RW * slices * o.SK * kStepBytes > kStageBytes) return SDV_EINVAL;
     const size_t units = (size_t)o.T * 16 * o.K16 * 2;  // 16-byte units of the matrix
     std::vector<unsigned char> seen(units, 0);
     for (int cta = 0; cta < G; ++cta) {
@@ -1685,18 +1695,19 @@ int sdv_debug_layout_check(const int* desc, const int* gu_desc, int G) {
         for (int p = 0; p < pt.npass; ++p) {
             const int pcount = pass_count(pt, p), pstart = pass_start(pt, p);
             if (pcount < 1 || pcount > 16) return -100;
+            const int per = pt.nk / slices, v = pcount * slices;   // column steps per slice; row tiles of the pass, slices stacked
             for (int st = 0; st < pt.nst; ++st) {
-                const int nks = (pt.SK < pt.nk - st * pt.SK) ? pt.SK : pt.nk - st * pt.SK;
-                const unsigned long long bytes = (unsigned long long)pcount * nks * kStepBytes;
+                const int nks = (pt.SK < per - st * pt.SK) ? pt.SK : per - st * pt.SK;
+                const unsigned long long bytes = (unsigned long long)v * nks * kStepBytes;
                 if (bytes > (unsigned long long)kStageBytes) return -101;
-                const unsigned lbo = 2u * pcount * 128u, astep = 2u * lbo;
+                const unsigned lbo = 2u * v * 128u, astep = 2u * lbo;
                 for (int ks = 0; ks < nks; ++ks)
                     for (int half = 0; half < 2; ++half)
-                        for (int r = 0; r < 16 * pcount; ++r) {
+                        for (int r = 0; r < 16 * v; ++r) {
                             const unsigned long long in_slot = (unsigned long long)ks * astep + half * lbo + (r >> 3) * 128 + (r & 7) * 16;
                             if (in_slot + 16 > bytes) return -102;
-                            const int row = (pt.tile0 + pstart) * 16 + r;
-                            const int k8 = (pt.k0 + st * pt.SK + ks) * 2 + half;
+                            const int slice = r / (16 * pcount), row = (pt.tile0 + pstart) * 16 + r % (16 * pcount);
+                            const int k8 = (pt.k0 + slice * per + st * pt.SK + ks) * 2 + half;
                             const unsigned long long want = weight_offset(o, gu, row, k8);
                             if (want != src + in_slot) return -103;
                             const size_t u = want / 16;
@@ -1724,7 +1735,7 @@ int sdv_debug_plan(const sdv_config* cfg, int G, int rows, int* out) {
     setup_ops(P, cfg, G);
     for (int i = 0; i < 5; ++i) {
         const OpDesc& o = P.op[i];
-        const int v[8] = {o.T, o.K16, o.P_row, o.P_k, o.RW, o.SK, o.unit, o.follow};
+        const int v[8] = {o.T, o.K16, o.P_row, o.P_k, o.RW, o.SK, o.unit, o.follow | (o.slices << 8)};
         for (int j = 0; j < 8; ++j) out[i * 8 + j] = v[j];
     }
     const SmemPlan sp = plan_smem(P, rows, false);
@@ -1748,25 +1759,12 @@ int sdv_debug_timeout_probe(sdv_ctx* ctx) {
 }  // extern "C"
 
 // ------------------------------------------------------------------------------------------
-// Stand-alone GEMM without any allocation (see include/sdv.h, sdv_gemm_noalloc).
-//
-// For callers that have no memory left to give or cannot afford the device-wide stall an
-// allocation or a free brings (a serving loop whose memory is all KV cache, a plug-in with a fixed
-// budget): nothing below asks the runtime for memory.  Its scratch memory is a fixed array in the library's device image.  Host code must not hand the
-// array's name to a kernel (there it is only a host-side stand-in); the device address is looked
-// up once per device with cudaGetSymbolAddress and passed on.
+// Stand-alone GEMM without any allocation (see include/sdv.h, sdv_gemm_noalloc): one kernel on the caller's operands
+// (small_gemm.cuh), no scratch.
 namespace {
-constexpr size_t kNaWeightBytes = (size_t)2 << 20;              // packed weights: N * K * 2 <= 2 MiB
+constexpr size_t kNaWeightBytes = (size_t)2 << 20;              // N * K * 2 <= 2 MiB
 constexpr int kNaMaxK = 4096, kNaMaxN = 4096;
-constexpr size_t kNaOutOff = kNaWeightBytes;                    // fp32 accumulators [32][N]
-constexpr size_t kNaOutBytes = (size_t)kMaxRows * kNaMaxN * 4;
-constexpr size_t kNaStateOff = kNaOutOff + kNaOutBytes;         // state words (error flag)
-constexpr size_t kNaTotal = kNaStateOff + 1024;
-constexpr int kNaMaxDevices = 64;
-uint8_t* g_na_ptr[kNaMaxDevices];  // device address of the scratch array, per device (0 = not looked up yet)
 }  // namespace
-
-static __device__ __align__(256) uint8_t g_na_scratch[kNaTotal];  // ~2.5 MB per GPU that loads the library
 
 extern "C" {
 
@@ -1774,11 +1772,11 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
     if (!dev_x || !dev_w || !dev_y) return SDV_EINVAL;
     if (M < 1 || N < 16 || N % 16 || K < 64 || K % 64) return SDV_EINVAL;
     if (M > kMaxRows || N > kNaMaxN || K > kNaMaxK || (size_t)N * K * 2 > kNaWeightBytes) return SDV_ETOOBIG;
-    // the kernels read x and w with 16-byte vector loads
+    // the kernel reads x and w with 16-byte vector loads
     if ((((uintptr_t)dev_x | (uintptr_t)dev_w) & 15) || ((uintptr_t)dev_y & 3)) return SDV_EINVAL;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNaMaxDevices) return SDV_ECUDA;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SDV_ECUDA;
     {
         // host memory or another device's memory would fault inside the kernel: refuse it here
         const void* ptrs[3] = {dev_x, dev_w, dev_y};
@@ -1792,52 +1790,27 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
             if (at.type != cudaMemoryTypeDevice || at.device != dev) return SDV_EINVAL;
         }
     }
-    if (!g_na_ptr[dev]) {
-        // first call on this device: look the array's device address up (do this before any stream capture)
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_na_scratch) != cudaSuccess || !p) return SDV_ECUDA;
-        g_na_ptr[dev] = (uint8_t*)p;
-    }
-    uint8_t* sc = g_na_ptr[dev];
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return SDV_ECUDA;
-    if (sms > kMaxGrid) sms = kMaxGrid;
-
-    FwdParams P;
-    memset(&P, 0, sizeof(P));
-    P.G = sms;
-    OpDesc& o = P.op[OP_RAW];
-    o.T = N / 16;
-    o.K16 = K / 16;
-    choose_partition(o, sms, M, false, false);
-    fit_pass_width(o);
-    P.wraw = sc;
-    P.raw_x = dev_x;  // the caller's rows are read in place
-    P.raw_out = (float*)(sc + kNaOutOff);
-    P.raw_N = N;
-    P.raw_K = K;
-    P.state = (int*)(sc + kNaStateOff);
-    P.bar = (unsigned*)(P.state + 200);  // unused by a one-phase launch, kept inside the cleared words
-    P.mode = 1;
-    P.ph_begin = 2;  // with n_layers = 0 phase 2 is the stand-alone GEMM
-    P.ph_end = 3;
-    P.wait_limit_ns = 2000000000ull;
-    if (!apply_plan(P, M, true)) return SDV_EINVAL;
-
-    // the array keeps the previous call's contents: clear what must start at zero
-    if (cudaMemsetAsync(sc + kNaOutOff, 0, (size_t)kMaxRows * N * 4, s) != cudaSuccess) return SDV_ECUDA;
-    if (cudaMemsetAsync(sc + kNaStateOff, 0, 1024, s) != cudaSuccess) return SDV_ECUDA;
-    const long long total = (long long)o.T * 16 * (K / 8);
-    int blocks = (int)((total + 255) / 256);
-    if (blocks > 148 * 16) blocks = 148 * 16;
-    pack_weights_kernel<<<blocks, 256, 0, s>>>(o, o, sc, dev_w, N, nullptr, 0, nullptr, K, 0, 0, o.T, 0);
-    if (cudaGetLastError() != cudaSuccess) return SDV_ECUDA;
-    if (launch_kernel(P, s) != cudaSuccess) return SDV_ECUDA;
-    if (cudaMemcpyAsync(dev_y, sc + kNaOutOff, (size_t)M * N * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return SDV_ECUDA;
-    int err = 0;
-    if (cudaMemcpyAsync(&err, sc + kNaStateOff + ST_ERR * 4, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess) return SDV_ECUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return SDV_ECUDA;
-    return err ? SDV_ETIMEOUT : SDV_OK;
+    // blocks that share the K steps of 16 weight rows: doubled while a warp keeps two steps and the grid stays within about two
+    // blocks per SM
+    const int tiles = N / 16, steps = K / 32;
+    int cs = 1;
+    while (cs < 8 && steps >= 2 * (cs * 2) * kSmallGemmWarps && tiles * cs * 2 <= 296) cs *= 2;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(tiles * cs);
+    cfg.blockDim = dim3(kSmallGemmWarps * 32);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    typedef void (*Kernel)(const float*, const uint16_t*, float*, int, int, int);
+    static const Kernel kernels[4] = {small_gemm_kernel<1>, small_gemm_kernel<2>, small_gemm_kernel<3>, small_gemm_kernel<4>};
+    if (cudaLaunchKernelEx(&cfg, kernels[(M - 1) / 8], dev_x, dev_w, dev_y, M, N, K) != cudaSuccess) return SDV_ECUDA;
+    return cudaStreamSynchronize(s) == cudaSuccess ? SDV_OK : SDV_ECUDA;
 }
 
 }  // extern "C"

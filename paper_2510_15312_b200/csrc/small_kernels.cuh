@@ -13,10 +13,11 @@ namespace sdv {
 // 16-byte unit (8 columns of one row).
 // mode 0: the operation's rows are src0 | src1 | src2 stacked (the sources hold the rows from
 // row_base on); mode 1: every 16-row tile holds 8 rows of src0 (gate) followed by the 8 matching
-// rows of src1 (up).  Only tiles [t_begin, t_end) are written.
+// rows of src1 (up); mode 2: as mode 0, and every 16-row tile holds 8 rows of the first half of a head (of hd rows)
+// followed by the 8 rows of its second half that rotary embedding pairs them with.  Only tiles [t_begin, t_end) are written.
 __global__ void pack_weights_kernel(OpDesc o, OpDesc gu, uint8_t* dst_base, const uint16_t* src0, int rows0,
                                     const uint16_t* src1, int rows1, const uint16_t* src2, int K, int mode,
-                                    int t_begin, int t_end, int row_base) {
+                                    int t_begin, int t_end, int row_base, int hd) {
     const int K8 = K / 8;
     const long long total = (long long)(t_end - t_begin) * 16 * K8;
     for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < total;
@@ -28,7 +29,11 @@ __global__ void pack_weights_kernel(OpDesc o, OpDesc gu, uint8_t* dst_base, cons
         if (mode == 1) {
             src = (r < 8) ? src0 + (size_t)(8 * t + r) * K : src1 + (size_t)(8 * t + r - 8) * K;
         } else {
-            const int lr = row - row_base;
+            int lr = row - row_base;
+            if (mode == 2) {
+                const int in = lr % hd, j = in >> 4;
+                lr += -in + (r < 8 ? 8 * j + r : hd / 2 + 8 * j + r - 8);
+            }
             if (lr < rows0) src = src0 + (size_t)lr * K;
             else if (lr < rows0 + rows1) src = src1 + (size_t)(lr - rows0) * K;
             else src = src2 + (size_t)(lr - rows0 - rows1) * K;
