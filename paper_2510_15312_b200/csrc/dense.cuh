@@ -36,28 +36,6 @@ struct DenseShape {
     static constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 512;
 };
 
-// Shared-memory operand descriptor, K-major, 128-byte swizzle: rows of 64 bf16 (128 bytes), groups of
-// 8 rows 1024 bytes apart; a 16-element K step advances the start address by 32 bytes.
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)1 << 16;                         // leading byte offset: unused for swizzled K-major operands
-    d |= (uint64_t)(1024u >> 4) << 32;              // stride between 8-row groups
-    d |= (uint64_t)1 << 46;                         // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                         // 128-byte swizzle
-    return d;
-}
-
-// The same for an operand whose rows (N) are contiguous: 8 K rows of 64 contiguous elements (128 bytes) form 1024-byte groups, K
-// groups follow each other, slabs of 64 N elements lie `slab` bytes apart.
-__device__ __forceinline__ uint64_t umma_desc_sw128_mn(uint32_t saddr, uint32_t slab) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)((slab >> 4) & 0x3fffu) << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
 struct DenseTopOut {   // EPI_TOP: [row][share of the vocabulary][kDenseTopMax] best logits of the share and their ids, best first
     float* val;
     int* idx;

@@ -63,14 +63,20 @@ struct Misc {
     uint64_t tmem_full[2], tmem_empty[2];
     uint64_t op_ready;    // the token operand of this block's next operation is complete (one arrival per builder warp)
     uint64_t act_ready;   // the SwiGLU operand of this block is complete (one arrival per epilogue warp)
+    uint64_t att_bar;     // a product of the attention step has completed
     uint64_t done_bar;    // last tensor-core instruction of the launch has completed
     uint32_t tmem_base;
     unsigned long long* prof_ptr;  // this block's profile words of the running phase (or null)
     int abort_flag;
     int skip;  // block-uniform copy of abort_flag, refreshed inside every grid barrier
     float sumsq[kMaxRows];  // sums of squares of the residual rows (this block's operand columns)
-    float best_v[kEpilogueWarps][kMaxRows];
-    int best_i[kEpilogueWarps][kMaxRows];
+    union {
+        struct {
+            float best_v[kEpilogueWarps][kMaxRows];
+            int best_i[kEpilogueWarps][kMaxRows];
+        };
+        float att_red[kEpilogueWarps][32];  // maxima and sums of a warp's keys, one query row per lane
+    };
     Part part[OP_COUNT];  // this block's share of every operation
     FwdParams P;          // block-local copy of the launch parameters
 };
@@ -310,21 +316,20 @@ __device__ __forceinline__ void build_norm_operand(const FwdParams& P, const Nor
     }
 }
 
-__device__ __forceinline__ void attn_split(const FwdParams& P, int& S, int& kps);
-
 // Operand of the output projection = attention output of this block's columns: the split-KV
 // partial results (un-normalised sums with their running maximum and sum) are merged on the way.
-// Four lanes share one (row, 8 columns) item, each taking every fourth partial result.
+// LPI lanes share one (row, 8 columns) item, each taking every LPI-th partial result: 4 up to 20 partial results, else 8.
+template <int LPI>
 __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const Part& pt, uint8_t* U, int wtid) {
-    constexpr int TPL = (kMaxSplits + 3) / 4;  // partial results per lane at most
-    int S, kps;
-    attn_split(P, S, kps);
+    constexpr int TPL = 5;  // partial results per lane at most
+    static_assert(8 * TPL >= kMaxSplits, "partial results per lane");
+    const int S = P.att_S;
     const int M = P.M, hd = P.hd;
     const int k8_0 = pt.k0 * 2, nk8 = pt.nk * 2;
-    const int nitems = M * nk8, sub = wtid & 3;
+    const int nitems = M * nk8, sub = wtid % LPI;
 #pragma unroll 1
-    for (int it0 = 0; it0 < nitems; it0 += kBuilderWarps * 32 / 4) {
-        const int item = it0 + (wtid >> 2);
+    for (int it0 = 0; it0 < nitems; it0 += kBuilderWarps * 32 / LPI) {
+        const int item = it0 + wtid / LPI;
         const bool live = item < nitems;
         const int j = live ? item / nk8 : 0, k8l = live ? item % nk8 : 0;
         const int col = (k8_0 + k8l) * 8, hq = col / hd, c = col % hd;
@@ -335,7 +340,7 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
         // the loads are one straight run of instructions instead of a branch per slot
 #pragma unroll
         for (int t = 0; t < TPL; ++t) {
-            const int s = sub + 4 * t;
+            const int s = sub + LPI * t;
             const size_t row = base + (size_t)min(s, S - 1) * kMaxRows;
             const float2 ml = ld_cg_f2_inorder(P.part_ml + row * 2);
             const float* op = P.part_o + row * hd + c;
@@ -348,8 +353,8 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
         float mmax = m[0];
 #pragma unroll
         for (int t = 1; t < TPL; ++t) mmax = fmaxf(mmax, m[t]);
-        mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, 1));
-        mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, 2));
+#pragma unroll
+        for (int off = 1; off < LPI; off <<= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, off));
         const float ref = (mmax == -CUDART_INF_F) ? 0.f : mmax;
         float v[9];
 #pragma unroll
@@ -363,8 +368,8 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
         }
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
-            v[e] += __shfl_xor_sync(0xffffffffu, v[e], 1);
-            v[e] += __shfl_xor_sync(0xffffffffu, v[e], 2);
+#pragma unroll
+            for (int off = 1; off < LPI; off <<= 1) v[e] += __shfl_xor_sync(0xffffffffu, v[e], off);
         }
         if (live && sub == 0) {
             const float inv = 1.f / v[8];
@@ -752,34 +757,33 @@ __device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, int
 
 // ------------------------------------------------------------------------------------------
 // Split-KV attention.  The keys [0, L + M) (the new rows' keys and values are in the cache already) are cut into S ranges of
-// kps keys (a multiple of 64, at most kMaxSplits ranges); the query heads of a KV head are cut into QG groups of up to
-// gh heads, a group's rows (heads x M) filling at most four 16-row tiles (the host picks gh so
-// that the longest chain of 16-key steps a warp walks is shortest).
+// kps keys (a multiple of 128, at most kMaxSplits ranges); the query heads of a KV head are cut into QG groups of up to
+// gh heads, a group's rows (heads x M) filling at most 64 rows (the host picks gh).
 // Unit (kv head, head group, s) attends the group's rows to range s under the causal mask (row j sees new keys 0..j; in a tree
 // the rows on its path) and leaves an un-normalised partial result with its running maximum and sum; the output
 // projection merges them while it builds its operand.
 //
-// Keys come in blocks of 64, copied asynchronously into two shared-memory buffers by warps 0..7.  Blocks that hold
-// committed keys only do not depend on the step: the first two are requested before the grid barrier in front of this phase,
-// so that the phase only waits for its queries.
-// Warp (row tile, key group) owns one row tile and every KG-th group of 16 keys of a block
-// (KG = 4 with up to two row tiles, 3 with three, 2 with four): scores (Q K^T on tensor cores), online softmax with quad
-// shuffles in the log2 domain and P V all stay in its registers; the key groups of a row tile meet
-// in shared memory at the end.
-// The heads per group are chosen on the host per launch; the key ranges follow from it: as many
-// as there are blocks to take a (KV head, head group, range) unit each, at most kMaxSplits.
+// The few query rows are the N side of tcgen05.mma, the keys its 128 rows: S^T = K Q^T (lane = key, column = query row), and
+// O^T = V^T P (lane = output column, column = query row).  A thread of warps 0..7 owns one key and half of the query rows:
+// maxima over the 128 keys by redux and one exchange between warps, probabilities to shared memory as bf16 (the B operand of
+// the second product), sums by a halving exchange of 16 shuffles.  Warp 9 issues.  Tensor memory is free in this phase: S^T
+// takes columns 0..63, O^T columns 64..127.
+// mma.sync tiles, which this replaces, issue m16n8k16 every 16 cycles per scheduler on this part, 1 us per 64 keys.
+//
+// Keys and values of a chunk of 128 keys are copied asynchronously by warps 0..7.  Rows of committed keys do not depend on
+// the step: those of the first chunk are requested before the grid barrier in front of this phase, so that the phase only waits
+// for its queries and the new rows.  With more chunks per range, K of the next one loads during the softmax and V behind P V.
 constexpr int kLoadThreads = kEpilogueWarps * 32;   // warps 0..7 copy keys and values
-__device__ __forceinline__ void attn_split(const FwdParams& P, int& S, int& kps) {
-    S = P.att_S;      // worked out once per launch (attn_split_compute): the divisions are not repeated per phase
-    kps = P.att_kps;
-}
+constexpr int kIssueWarp = kWorkerWarps - 1;        // issues the attention's tensor-core instructions
+constexpr uint32_t kTmemO = 64;                     // first column of O^T
+
 // `keys`: of the longest sequence, new rows included.
 __device__ __forceinline__ void attn_split_compute(const FwdParams& P, int keys, int& S, int& kps) {
     const int QG = (P.g + P.att_gh - 1) / P.att_gh;
     int cap = P.G / (P.n_kv * QG);
     if (cap > kMaxSplits) cap = kMaxSplits;
     if (cap < 1) cap = 1;
-    kps = ((keys + cap - 1) / cap + 63) / 64 * 64;
+    kps = ((keys + cap - 1) / cap + kKeyChunk - 1) / kKeyChunk * kKeyChunk;
     S = (keys + kps - 1) / kps;
 }
 
@@ -808,234 +812,252 @@ __device__ __forceinline__ AttnUnit attn_unit(const FwdParams& P, int b, int hk,
     u.v = vc + off;
     return u;
 }
+// Shared memory of the attention step: query rows | values | keys, rows of 64 columns (128 bytes, 128-byte swizzle) in slabs.
 template <int HD>
 struct AttnShape {
-    static constexpr int KB = 64, NBUF = 2, UNITS = HD / 8;   // keys per block, buffers, 16-byte units per K/V row
-    static constexpr int QBYTES = 64 * HD * 2, KVBYTES = KB * HD * 2;
+    static constexpr int UNITS = HD / 8;                 // 16-byte units per row
+    static constexpr int QSLAB = 64 * 128, KSLAB = kKeyChunk * 128;
+    static constexpr int QBYTES = HD / 64 * QSLAB, KBYTES = HD / 64 * KSLAB;
+    static_assert(QBYTES + 2 * KBYTES == kAttnBytesPerDim * HD, "attention tiles");
 };
-// Keys and values of one block of the range: 16-byte asynchronous copies by warps 0..7, rows past the range zero-filled.
+// Rows [from, to) of a chunk of keys (or values) by warps 0..7, 16-byte asynchronous copies; rows past the range are zero-filled.
 template <int HD>
-__device__ __forceinline__ void attn_load_block(const FwdParams& P, const AttnUnit& u, int layer, int blk, uint8_t* att, int wtid) {
+__device__ __forceinline__ void attn_load(const FwdParams& P, const AttnUnit& u, const __nv_bfloat16* src, int layer, int chunk, int from,
+                                          int to, uint8_t* dst, int wtid) {
     using A = AttnShape<HD>;
-    if (blk * A::KB < u.nkeys) {
-        uint8_t* Ks = att + A::QBYTES + (blk % A::NBUF) * 2 * A::KVBYTES;
-        uint8_t* Vs = Ks + A::KVBYTES;
-        const size_t base = (size_t)layer * P.n_kv * P.max_seq * HD;
-        const int q16 = wtid % A::UNITS;
+    const __nv_bfloat16* base = src + ((size_t)layer * P.n_kv * P.max_seq + chunk * kKeyChunk) * HD;
+    const int q16 = wtid % A::UNITS, left = u.nkeys - chunk * kKeyChunk;
+    uint8_t* d = dst + (q16 >> 3) * A::KSLAB;
 #pragma unroll
-        for (int i = 0; i < A::KB * A::UNITS / kLoadThreads; ++i) {
-            const int key = wtid / A::UNITS + i * (kLoadThreads / A::UNITS), kk = blk * A::KB + key;
-            const bool valid = kk < u.nkeys;
-            const size_t off = base + (size_t)(valid ? kk : 0) * HD + q16 * 8;
-            const uint32_t so = (q16 >> 3) * (A::KB * 128) + swz_unit(key, q16 & 7);
-            cp_async_16_zfill(Ks + so, u.k + off, valid);
-            cp_async_16_zfill(Vs + so, u.v + off, valid);
+    for (int i = 0; i < kKeyChunk * A::UNITS / kLoadThreads; ++i) {
+        const int key = wtid / A::UNITS + i * (kLoadThreads / A::UNITS);
+        const bool valid = key < left;
+        if (key >= from && key < to) cp_async_16_zfill(d + swz_unit(key, q16 & 7), base + (size_t)(valid ? key : 0) * HD + q16 * 8, valid);
+    }
+}
+// Rows of the first chunk that may be requested before the new rows' keys are there.
+__device__ __forceinline__ int attn_early_rows(const AttnUnit& u) {
+    const int old = u.L - u.t_begin;   // committed keys from the range's first on
+    return old >= u.nkeys ? kKeyChunk : max(0, min(old, kKeyChunk));
+}
+
+// Largest of the warp's 32 values, handed to every lane.
+__device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+// Sums over the warp of 16 columns: lane n receives column n & 15.
+__device__ __forceinline__ float warp_sum16(float (&v)[16], int lane) {
+#pragma unroll
+    for (int off = 8; off; off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < off; ++i) {
+            const float keep = up ? v[i + off] : v[i], send = up ? v[i] : v[i + off];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
-    cp_async_commit();  // possibly empty: keeps the group count uniform
-}
-// Blocks that may be requested before the new rows' keys are there.
-template <int HD>
-__device__ __forceinline__ int attn_early_blocks(const AttnUnit& u) {
-    const int old = u.L - u.t_begin;   // committed keys of the range
-    const int n = old >= u.nkeys ? 2 : old / AttnShape<HD>::KB;
-    return n < 0 ? 0 : (n > 2 ? 2 : n);
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
+// One unit by all worker warps.  `loaded`: rows of its first chunk requested earlier; `uses`: completions of misc->att_bar so far.
 template <int HD, int MODE>
-__device__ __forceinline__ void attention_unit(const FwdParams& P, int layer, const AttnUnit& u, int loaded, uint8_t* att, int wtid,
-                                               unsigned long long* prof) {
+__device__ __forceinline__ void attention_unit(const FwdParams& P, Misc* misc, int layer, const AttnUnit& u, int loaded, uint8_t* att,
+                                               uint8_t* Ps, int wtid, uint32_t& uses, unsigned long long* prof) {
     using A = AttnShape<HD>;
     constexpr bool TREE = MODE == 1;
-    constexpr int KSTEPS = HD / 16, UNITS = A::UNITS, KB = A::KB, NBUF = A::NBUF, KVBYTES = A::KVBYTES;
-    constexpr int NT_O = HD / 8;     // 8-column tiles of the output
-    static_assert(A::QBYTES + NBUF * 2 * KVBYTES <= kAttnSmemBytes, "attention tiles");
-    // exchange area of the key-group merge: (KG - 1) * MT <= 6 tiles of (output + statistics)
-    static_assert(6 * (NT_O + 1) * 32 * 16 <= NBUF * 2 * KVBYTES, "exchange area of the key-group merge");
     const int warp = wtid >> 5, lane = wtid & 31;
-    const int M = u.M;
-    const int R = u.nheads * M;                  // R <= 64
-    const uint32_t minv = 65536u / (uint32_t)M + 1u;   // row / M = row * minv >> 16 for rows below 64
-    const int MT = (R + 15) >> 4, RP = MT * 16;
-    const int KG = MT <= 2 ? 4 : (MT == 3 ? 3 : 2);  // key groups: 16-key chunks of a block handled side by side
-    const int kgp = (MT == 1 ? warp : MT == 2 ? warp >> 1 : MT == 3 ? (warp * 11) >> 5 : warp >> 2), mt = warp - kgp * MT;
-    const bool active = kgp < KG;
-    uint8_t* Qs = att;
-    uint8_t* KVs = att + A::QBYTES;
-    const int nkeys = u.nkeys, nblk = (nkeys + KB - 1) / KB;
-
+    const int M = u.M, R = u.nheads * M, RP = (R + 15) & ~15;   // R <= 64
+    const uint32_t minv = 65536u / (uint32_t)M + 1u;            // row / M = row * minv >> 16 for rows below 64
+    uint8_t *Qs = att, *Vs = att + A::QBYTES, *Ks = Vs + A::KBYTES;
+    const int nkeys = u.nkeys, nch = (nkeys + kKeyChunk - 1) / kKeyChunk;
     if (prof && wtid == 0) prof[2] = global_timer_ns();
-    // query tile (16-byte copies; rows past R zero-filled)
-    for (int un = wtid; un < RP * UNITS; un += kWorkerThreads) {
-        const int r = un / UNITS, q16 = un % UNITS;
+    // query rows (past R: zeros) and what is missing of the first chunk
+    for (int un = wtid; un < RP * A::UNITS; un += kWorkerThreads) {
+        const int r = un / A::UNITS, q16 = un % A::UNITS;
         const int hl = (int)((uint32_t)r * minv >> 16), j = r - hl * M;
         const bool valid = r < R;
         const __nv_bfloat16* src = P.q + (size_t)(u.r0 + (valid ? j : 0)) * (P.n_q * HD) + (u.head0 + (valid ? hl : 0)) * HD + q16 * 8;
-        cp_async_16_zfill(Qs + (q16 >> 3) * (RP * 128) + swz_unit(r, q16 & 7), src, valid);
+        cp_async_16_zfill(Qs + (q16 >> 3) * A::QSLAB + swz_unit(r, q16 & 7), src, valid);
     }
+    if (nch > 0 && warp < kEpilogueWarps && loaded < kKeyChunk) attn_load<HD>(P, u, u.k, layer, 0, loaded, kKeyChunk, Ks, wtid);
     cp_async_commit();
-    if (warp < kEpilogueWarps) {
-#pragma unroll 1
-        for (int b = loaded; b < NBUF; ++b) attn_load_block<HD>(P, u, layer, b, att, wtid);
-    }
-    cp_async_wait<0>();   // the queries, and with them the first blocks
+    if (nch > 0 && warp < kEpilogueWarps && loaded < kKeyChunk) attn_load<HD>(P, u, u.v, layer, 0, loaded, kKeyChunk, Vs, wtid);
+    cp_async_commit();
+
+    // this warp's keys (accumulator lanes) and query rows: columns c0 .. c0 + 16 ng - 1; lane n looks after column c0 + n
+    const int quarter = warp & 3, half = warp >> 2;
+    const int c0 = half ? (RP >= 48 ? 32 : 16) : 0, ng = warp >= kEpilogueWarps ? 0 : half ? max(0, (RP - c0) >> 4) : min(2, (RP >= 48 ? 32 : 16) >> 4);
+    const int my_r = c0 + lane, my_h = (int)((uint32_t)my_r * minv >> 16), my_j = my_r - my_h * M;
+    const uint32_t tm = misc->tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0;
+    float* red = misc->att_red[warp & 7];
+    float m = -CUDART_INF_F, l = 0.f;
+    const int new0 = u.L - u.t_begin;   // range index of the first new key
+    bool dead = *(volatile int*)&misc->abort_flag != 0;
+
+    cp_async_wait<1>();
+    fence_proxy_async_smem();
+    named_bar_sync(1, kWorkerThreads);   // queries and keys are in place
     if (prof && wtid == 0) prof[3] = global_timer_ns();
-
-    const int g = lane >> 2, q2 = (lane & 3) * 2;
-    const int r_lo = mt * 16 + g, r_hi = r_lo + 8;
-    const int h_lo = (int)((uint32_t)r_lo * minv >> 16), h_hi = (int)((uint32_t)r_hi * minv >> 16);
-    const int j_lo = r_lo - h_lo * M, j_hi = r_hi - h_hi * M;
-    // last key (within the range) a row sees; in a tree the new keys it sees are a bit mask
-    const int new0 = u.L - u.t_begin;
-    const int lim_lo = TREE ? nkeys - 1 : min(new0 + j_lo, nkeys - 1), lim_hi = TREE ? nkeys - 1 : min(new0 + j_hi, nkeys - 1);
-    const unsigned see_lo = TREE ? (unsigned)__ldcg(P.state + ST_ANC + min(j_lo, kMaxRows - 1)) : 0u;
-    const unsigned see_hi = TREE ? (unsigned)__ldcg(P.state + ST_ANC + min(j_hi, kMaxRows - 1)) : 0u;
-    float o[NT_O][4];
-#pragma unroll
-    for (int n = 0; n < NT_O; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
-    float m_lo = -CUDART_INF_F, m_hi = -CUDART_INF_F, l_lo = 0.f, l_hi = 0.f;
-    const uint32_t qb = smem_u32(Qs);
-
 #pragma unroll 1
-    for (int blk = 0; blk < nblk; ++blk) {
-        if (blk > 0) cp_async_wait<NBUF - 1>();
-        named_bar_sync(1, kWorkerThreads);  // the block (and, first time, the Q tile) is in place
-        if (prof && wtid == 0 && blk == 0) prof[4] = global_timer_ns();
-        if (active) {
-            const uint32_t kb = smem_u32(KVs + (blk % NBUF) * 2 * KVBYTES), vb = kb + KVBYTES;
+    for (int c = 0; c < nch; ++c) {
+        const int left = nkeys - c * kKeyChunk;
+        if (warp == kIssueWarp) {
+            tc_fence_after();
+            if (elect_one()) {
+                const uint32_t ka = smem_u32(Ks), qa = smem_u32(Qs), id = umma_idesc_bf16(128u, (uint32_t)RP);
+#pragma unroll
+                for (int ks = 0; ks < HD / 16; ++ks)
+                    umma_bf16(misc->tmem_base, umma_desc_sw128(ka + (uint32_t)((ks >> 2) * A::KSLAB + (ks & 3) * 32)),
+                              umma_desc_sw128(qa + (uint32_t)((ks >> 2) * A::QSLAB + (ks & 3) * 32)), id, (uint32_t)ks);
+                umma_commit(&misc->att_bar);
+            }
+            __syncwarp();
+        }
+        if (warp < kEpilogueWarps) {
+            // the scores are complete: K is free, and with the products before them V, P and O of the chunk before
+            if (!dead && !mbar_wait_bounded(&misc->att_bar, uses & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
+            dead = __any_sync(0xffffffffu, dead);
+            tc_fence_after();
+            if (prof && wtid == 0 && c == 0) prof[4] = global_timer_ns();
+            if (c > 0) attn_load<HD>(P, u, u.v, layer, c, 0, kKeyChunk, Vs, wtid);
+            cp_async_commit();
+            if (c + 1 < nch) attn_load<HD>(P, u, u.k, layer, c + 1, 0, kKeyChunk, Ks, wtid);
+            cp_async_commit();
+            // columns (bit n: c0 + n) that see this thread's key
+            const int kk = quarter * 32 + lane, e = c * kKeyChunk + kk - new0;
+            unsigned see = kk < left ? 0xffffffffu : 0u;
+            if (c * kKeyChunk + quarter * 32 + 31 >= new0) {   // a new key among the warp's
+                const unsigned anc = TREE ? (unsigned)__ldcg(P.state + ST_ANC + min(my_j, kMaxRows - 1)) : 0u;
 #pragma unroll 1
-            for (int c = kgp; c < KB / 16; c += KG) {
-                if (blk * KB + c * 16 >= nkeys) break;
-                // ---- scores of 16 rows x 16 keys
-                float sc[2][4];
-#pragma unroll
-                for (int n = 0; n < 2; ++n) sc[n][0] = sc[n][1] = sc[n][2] = sc[n][3] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < KSTEPS; ++ks) {
-                    uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-                    ldsm_x4(qb + (ks >> 2) * (RP * 128) + swz_unit(mt * 16 + (lane & 15), (ks & 3) * 2 + (lane >> 4)), a0, a1, a2, a3);
-                    const int row = c * 16 + (lane & 7) + ((lane >> 4) << 3);
-                    ldsm_x4(kb + (ks >> 2) * (KB * 128) + swz_unit(row, (ks & 3) * 2 + ((lane >> 3) & 1)), b0, b1, b2, b3);
-                    mma_bf16_16816(sc[0], a0, a1, a2, a3, b0, b1);
-                    mma_bf16_16816(sc[1], a0, a1, a2, a3, b2, b3);
+                for (int i = 0; i < M; ++i) {
+                    const unsigned b = __ballot_sync(0xffffffffu, TREE ? ((anc >> i) & 1u) != 0 : i <= my_j);
+                    if (e == i) see &= b;
                 }
-                float mx_lo = -CUDART_INF_F, mx_hi = -CUDART_INF_F;
-                const int key0 = blk * KB + c * 16 + q2;
+            }
+            // maximum of every column over the 128 keys
+            const float scale = P.scale_log2e;
+            float mx = -CUDART_INF_F;
+            if (!dead) {
+#pragma unroll 1
+                for (int g = 0; g < ng; ++g) {
+                    float v[16];
+                    tmem_ld16(tm + (uint32_t)(g * 16), v);
+                    const unsigned sg = see >> (g * 16);
 #pragma unroll
-                for (int n = 0; n < 2; ++n)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int key = key0 + n * 8 + (e & 1);
-                        const bool hi = e >= 2;
-                        bool ok = key <= (hi ? lim_hi : lim_lo);
-                        if (TREE && key >= new0) ok = ok && (((hi ? see_hi : see_lo) >> ((key - new0) & 31)) & 1u);
-                        const float v = ok ? sc[n][e] * P.scale_log2e : -CUDART_INF_F;
-                        sc[n][e] = v;
-                        if (hi) mx_hi = fmaxf(mx_hi, v); else mx_lo = fmaxf(mx_lo, v);
+                    for (int n = 0; n < 16; ++n) {
+                        const float x = warp_max((sg >> n) & 1u ? v[n] * scale : -CUDART_INF_F);
+                        if (lane == g * 16 + n) mx = x;
                     }
-                mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-                mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-                mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-                mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-                // ---- online softmax: new maximum, rescale, probabilities
-                const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
-                const float use_lo = (mn_lo == -CUDART_INF_F) ? 0.f : mn_lo, use_hi = (mn_hi == -CUDART_INF_F) ? 0.f : mn_hi;
-                const float c_lo = exp2f(m_lo - use_lo), c_hi = exp2f(m_hi - use_hi);
-                m_lo = mn_lo;
-                m_hi = mn_hi;
-                float p[2][4];
-#pragma unroll
-                for (int n = 0; n < 2; ++n) {
-                    p[n][0] = exp2f(sc[n][0] - use_lo);
-                    p[n][1] = exp2f(sc[n][1] - use_lo);
-                    p[n][2] = exp2f(sc[n][2] - use_hi);
-                    p[n][3] = exp2f(sc[n][3] - use_hi);
-                }
-                l_lo = l_lo * c_lo + p[0][0] + p[0][1] + p[1][0] + p[1][1];
-                l_hi = l_hi * c_hi + p[0][2] + p[0][3] + p[1][2] + p[1][3];
-#pragma unroll
-                for (int n = 0; n < NT_O; ++n) { o[n][0] *= c_lo; o[n][1] *= c_lo; o[n][2] *= c_hi; o[n][3] *= c_hi; }
-                // ---- O += P V: the score accumulators are, pairwise packed, the A operand of the next product
-                const uint32_t a0 = pack_bf16(p[0][0], p[0][1]), a1 = pack_bf16(p[0][2], p[0][3]);
-                const uint32_t a2 = pack_bf16(p[1][0], p[1][1]), a3 = pack_bf16(p[1][2], p[1][3]);
-#pragma unroll
-                for (int cg = 0; cg < NT_O / 2; ++cg) {
-                    uint32_t b0, b1, b2, b3;
-                    const int key = c * 16 + (lane & 7) + (((lane >> 3) & 1) << 3);
-                    const int cu = cg * 2 + (lane >> 4);
-                    ldsm_x4_trans(vb + (cu >> 3) * (KB * 128) + swz_unit(key, cu & 7), b0, b1, b2, b3);
-                    mma_bf16_16816(o[2 * cg], a0, a1, a2, a3, b0, b1);
-                    mma_bf16_16816(o[2 * cg + 1], a0, a1, a2, a3, b2, b3);
                 }
             }
-        }
-        named_bar_sync(1, kWorkerThreads);  // the block has been consumed
-        if (blk + NBUF < nblk && warp < kEpilogueWarps) attn_load_block<HD>(P, u, layer, blk + NBUF, att, wtid);
-        else cp_async_commit();
-    }
-    cp_async_wait<0>();
-    if (prof && wtid == 0) prof[5] = global_timer_ns();
-
-    // ---- row sums over the quad; the key groups of a row tile meet in shared memory
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1);
-    l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
-    l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
-    {
-        float4* ex_o = reinterpret_cast<float4*>(KVs);          // [key group - 1][row tile][output tile][lane]
-        float4* ex_ml = ex_o + 6 * NT_O * 32;                   // [key group - 1][row tile][lane]
-        if (active && kgp > 0) {
-            float4* dst = ex_o + ((kgp - 1) * MT + mt) * NT_O * 32;
+            red[lane] = mx;
+            named_bar_sync(2, kLoadThreads);
+            mx = m;
 #pragma unroll
-            for (int n = 0; n < NT_O; ++n) dst[n * 32 + lane] = make_float4(o[n][0], o[n][1], o[n][2], o[n][3]);
-            ex_ml[((kgp - 1) * MT + mt) * 32 + lane] = make_float4(m_lo, m_hi, l_lo, l_hi);
-        }
-        named_bar_sync(1, kWorkerThreads);
-        if (active && kgp == 0) {
+            for (int w = 0; w < 4; ++w) mx = fmaxf(mx, misc->att_red[half * 4 + w][lane]);
+            const float ref = mx == -CUDART_INF_F ? 0.f : mx;   // no key so far
+            const float corr = exp2f(m - ref);
+            m = mx;
+            if (c > 0 && !dead && __any_sync(0xffffffffu, corr != 1.f)) {
+                // the output so far refers to the old maximum
 #pragma unroll 1
-            for (int og = 0; og < KG - 1; ++og) {
-                const float4 ml = ex_ml[(og * MT + mt) * 32 + lane];
-                const float mn_lo = fmaxf(m_lo, ml.x), mn_hi = fmaxf(m_hi, ml.y);
-                const float use_lo = (mn_lo == -CUDART_INF_F) ? 0.f : mn_lo, use_hi = (mn_hi == -CUDART_INF_F) ? 0.f : mn_hi;
-                const float e0_lo = exp2f(m_lo - use_lo), e1_lo = exp2f(ml.x - use_lo);
-                const float e0_hi = exp2f(m_hi - use_hi), e1_hi = exp2f(ml.y - use_hi);
-                m_lo = mn_lo;
-                m_hi = mn_hi;
-                l_lo = l_lo * e0_lo + ml.z * e1_lo;
-                l_hi = l_hi * e0_hi + ml.w * e1_hi;
-                const float4* src = ex_o + (og * MT + mt) * NT_O * 32;
+                for (int g = 0; g < ng; ++g) {
+                    float v[16];
+                    uint32_t o[16];
+                    tmem_ld16(tm + kTmemO + (uint32_t)(g * 16), v);
 #pragma unroll
-                for (int n = 0; n < NT_O; ++n) {
-                    const float4 t = src[n * 32 + lane];
-                    o[n][0] = o[n][0] * e0_lo + t.x * e1_lo;
-                    o[n][1] = o[n][1] * e0_lo + t.y * e1_lo;
-                    o[n][2] = o[n][2] * e0_hi + t.z * e1_hi;
-                    o[n][3] = o[n][3] * e0_hi + t.w * e1_hi;
+                    for (int n = 0; n < 16; ++n) o[n] = __float_as_uint(v[n] * __shfl_sync(0xffffffffu, corr, g * 16 + n));
+                    tmem_st16(tm + kTmemO + (uint32_t)(g * 16), o);
+                }
+                tmem_st_wait();
+            }
+            float sum = 0.f;
+            if (!dead) {
+                uint8_t* pd = Ps + (kk >> 6) * (RP * 128) + c0 * 128 + (kk & 7) * 2;   // row c0, column kk & 63 of its slab, without the swizzle
+                const uint32_t ku = (uint32_t)((kk >> 3) & 7) << 4;
+#pragma unroll 1
+                for (int g = 0; g < ng; ++g) {
+                    float v[16];
+                    tmem_ld16(tm + (uint32_t)(g * 16), v);
+                    const unsigned sg = see >> (g * 16);
+#pragma unroll
+                    for (int n = 0; n < 16; ++n) {
+                        const float x = exp2f(v[n] * scale - __shfl_sync(0xffffffffu, ref, g * 16 + n));
+                        v[n] = (sg >> n) & 1u ? x : 0.f;
+                        *reinterpret_cast<__nv_bfloat16*>(pd + (g * 16 + n) * 128 + (ku ^ (uint32_t)((n & 7) << 4))) = __float2bfloat16(v[n]);
+                    }
+                    const float t = warp_sum16(v, lane);
+                    if ((lane >> 4) == g) sum = t;
                 }
             }
+            l = l * corr + sum;
+            ++uses;
+        }
+        cp_async_wait<1>();   // V of this chunk
+        fence_proxy_async_smem();
+        tc_fence_before();
+        named_bar_sync(1, kWorkerThreads);   // values and probabilities are in place
+        if (warp == kIssueWarp) {
+            tc_fence_after();
+            if (elect_one()) {
+                // heads of 64: rows 64..127 of the instruction are the keys, the tile behind V, into lanes nobody reads
+                const uint32_t va = smem_u32(Vs), pa = smem_u32(Ps), id = umma_idesc_bf16(128u, (uint32_t)RP) | (1u << 15);   // A: features contiguous
+                const int steps = (min(left, kKeyChunk) + 15) >> 4;
+#pragma unroll 1
+                for (int ks = 0; ks < steps; ++ks)
+                    umma_bf16(misc->tmem_base + kTmemO, umma_desc_sw128_mn(va + (uint32_t)ks * 2048u, (uint32_t)A::KSLAB),
+                              umma_desc_sw128(pa + (uint32_t)((ks >> 2) * (RP * 128) + (ks & 3) * 32)), id, (uint32_t)(c | ks));
+                if (c + 1 == nch) umma_commit(&misc->att_bar);
+            }
+            __syncwarp();
+        }
+        if (c + 1 < nch) {
+            cp_async_wait<0>();   // K of the next chunk
+            fence_proxy_async_smem();
+            named_bar_sync(1, kWorkerThreads);
         }
     }
-
-    // ---- un-normalised partial result of this key range
-    if (active && kgp == 0) {
+    if (prof && wtid == 0) prof[5] = global_timer_ns();
+    // un-normalised partial result of this key range
+    if (warp < kEpilogueWarps) {
+        red[lane] = l;
+        named_bar_sync(2, kLoadThreads);
+        const int row = ((u.head0 + my_h) * kMaxSplits + u.s) * kMaxRows + u.r0 + my_j;   // partial result of this lane's column
+        if (quarter == 0 && lane < ng * 16 && my_r < R) {
+            float sum = 0.f;
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int r = half ? r_hi : r_lo;
-            if (r >= R) continue;
-            const size_t row = ((size_t)(u.head0 + (half ? h_hi : h_lo)) * kMaxSplits + u.s) * kMaxRows + u.r0 + (half ? j_hi : j_lo);
-            float* po = P.part_o + row * HD + q2;
+            for (int w = 0; w < 4; ++w) sum += misc->att_red[half * 4 + w][lane];
+            __stcg(reinterpret_cast<float2*>(P.part_ml) + row, make_float2(m, sum));
+        }
+        if (nch > 0) {
+            if (!dead && !mbar_wait_bounded(&misc->att_bar, uses & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
+            dead = __any_sync(0xffffffffu, dead);
+            tc_fence_after();
+            ++uses;
+            if (!dead && quarter * 32 < HD) {
+                float* po = P.part_o + quarter * 32 + lane;
+#pragma unroll 1
+                for (int g = 0; g < ng; ++g) {
+                    float v[16];
+                    tmem_ld16(tm + kTmemO + (uint32_t)(g * 16), v);
 #pragma unroll
-            for (int n = 0; n < NT_O; ++n)
-                __stcg(reinterpret_cast<float2*>(po + n * 8), make_float2(o[n][half * 2], o[n][half * 2 + 1]));
-            if ((lane & 3) == 0)
-                __stcg(reinterpret_cast<float2*>(P.part_ml + row * 2), make_float2(half ? m_hi : m_lo, half ? l_hi : l_lo));
+                    for (int n = 0; n < 16; ++n) {
+                        const int rw = __shfl_sync(0xffffffffu, row, g * 16 + n);
+                        if (c0 + g * 16 + n < R) __stcg(po + (size_t)rw * HD, v[n]);
+                    }
+                }
+            }
+            tc_fence_before();
         }
     }
 }
 
-// `early`: key blocks of the block's first unit that were requested before the grid barrier.
+// `early`: rows of the first chunk of the block's first unit that were requested before the grid barrier.
 template <int HD, int MODE>
-__device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, int early, uint8_t* att, int wtid, unsigned long long* prof) {
+__device__ __forceinline__ void attention_phase(const FwdParams& P, Misc* misc, int layer, int early, uint8_t* smem, int wtid, uint32_t& uses,
+                                                unsigned long long* prof) {
     const int per_seq = P.att_per_seq, QG = P.att_QG, S = P.att_S;
     const int nunits = per_seq * (MODE == 2 ? P.nseq : 1);
 #pragma unroll 1
@@ -1050,23 +1072,26 @@ __device__ __forceinline__ void attention_phase(const FwdParams& P, int layer, i
             early = 0;
         }
         // batched: every sequence takes the key ranges of the longest one; a range past its own length holds no key
-        attention_unit<HD, MODE>(P, layer, attn_unit<HD, MODE>(P, b, hk, qg, s), early, att, wtid, prof);
+        attention_unit<HD, MODE>(P, misc, layer, attn_unit<HD, MODE>(P, b, hk, qg, s), early, smem + P.u_off, smem + P.p_off, wtid, uses, prof);
         named_bar_sync(1, kWorkerThreads);  // the unit's shared-memory tiles are free again
         if (prof && wtid == 0) { prof[6] = global_timer_ns(); prof[7] = (unsigned long long)(s + 1 == S); }
     }
 }
-// Before the grid barrier in front of the attention phase: requests the first key blocks of the block's unit that do not hold
-// new rows.  Only once the block's own products of the phase before have completed (their operand lies where the keys go), which
+// Before the grid barrier in front of the attention phase: requests the committed keys of the first chunk of the block's unit.  Only
+// once the block's own products of the phase before have completed (their operand lies where the keys go), which
 // warps 0..7 know from their epilogue.
 template <int HD, int MODE>
 __device__ __forceinline__ int attention_early(const FwdParams& P, int layer, uint8_t* att, int wtid) {
+    using A = AttnShape<HD>;
     if ((int)blockIdx.x >= P.att_per_seq * (MODE == 2 ? P.nseq : 1)) return 0;
     const AttnUnit u = attn_unit<HD, MODE>(P, P.att_b0, P.att_hk0, P.att_qg0, P.att_s0);
-    const int n = attn_early_blocks<HD>(u);
+    if (u.nkeys <= 0) return 0;
+    const int n = attn_early_rows(u);
     if ((wtid >> 5) < kEpilogueWarps) {
-#pragma unroll 1
-        for (int b = 0; b < n; ++b) attn_load_block<HD>(P, u, layer, b, att, wtid);
+        attn_load<HD>(P, u, u.v, layer, 0, 0, n, att + A::QBYTES, wtid);
+        attn_load<HD>(P, u, u.k, layer, 0, 0, n, att + A::QBYTES + A::KBYTES, wtid);
     }
+    cp_async_commit();
     return n;
 }
 // ------------------------------------------------------------------------------------------
@@ -1119,7 +1144,10 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int lay
     if (wtid == 0) misc->prof_ptr = prof;
     if (have0) {
         if (!dead) {
-            if (kind == PH_O) build_merged_operand(P, p0, U, wtid);
+            if (kind == PH_O) {
+                if (P.att_S <= 20) build_merged_operand<4>(P, p0, U, wtid);
+                else build_merged_operand<8>(P, p0, U, wtid);
+            }
             else build_norm_operand(P, prep, U, misc, wtid);
         }
         fence_proxy_async_smem();
@@ -1194,8 +1222,7 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
 template <int HD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg) {
     static_assert(sizeof(FwdParams) % 4 == 0, "parameter block is copied word by word");
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    extern __shared__ __align__(1024) uint8_t smem[];   // the launch's only shared memory: starts on a 1024-byte boundary
     Misc* misc = reinterpret_cast<Misc*>(smem + kMiscOff);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (Pg.l_from_state && Pg.state[ST_BUDGET] == 0) {
@@ -1234,6 +1261,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         }
         mbar_init(&misc->op_ready, kBuilderWarps);
         mbar_init(&misc->act_ready, kEpilogueWarps);
+        mbar_init(&misc->att_bar, 1);
         mbar_init(&misc->done_bar, 1);
         misc->abort_flag = 0;
         misc->skip = 0;
@@ -1287,6 +1315,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     int layer, kind = decode_phase(P.ph_begin, P.n_layers, layer);
     NormPrep prep;
     int early = 0;
+    uint32_t att_uses = 0;
     auto prepare = [&](int ph) {
         kind = decode_phase(ph, P.n_layers, layer);
         if (kind == PH_ATTN) early = attention_early<HD, MODE>(P, layer, smem + P.u_off, wtid);
@@ -1306,7 +1335,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         } else if (kind == PH_EMBED) {
             embed_phase(P, wtid);
         } else if (kind == PH_ATTN) {
-            attention_phase<HD, MODE>(P, layer, early, smem + P.u_off, wtid, pp);
+            attention_phase<HD, MODE>(P, misc, layer, early, smem, wtid, att_uses, pp);
         } else {
             gemm_phase<HD, MODE>(P, kind, layer, prep, smem, misc, pos, wtid, pp);
         }

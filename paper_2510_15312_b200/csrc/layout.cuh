@@ -35,12 +35,13 @@ constexpr int kStageBytes = 32768;                     // ring slot
 constexpr int kMaxStages = 8;                          // ring slots at most
 constexpr int kMaxRows = 32;                           // token rows a buffer is sized for
 constexpr int kMaxBatch = 8;                           // sequences one batched verify step takes at most
-constexpr int kMaxSplits = 20;                         // key ranges per head at most
+constexpr int kMaxSplits = 40;                         // key ranges per head at most
 constexpr int kSmemBudget = 232448;                    // 227 KB
-constexpr int kAttnSmemBytes = 81920;                  // Q tile (up to 16 KB) + two K|V blocks of 64 keys (64 KB)
+constexpr int kKeyChunk = 128;                         // keys per attention chunk: the rows of a tensor-core instruction
+constexpr int kAttnBytesPerDim = 640;                  // attention tiles: 64 query rows, a chunk of keys and of values; bytes per column of a head
 constexpr int kActSmemMax = 32768;                     // SwiGLU output of this block (operand of its down-projection slice) at most
 constexpr int kMiscSmemBytes = 4096;
-constexpr int kMiscOff = kSmemBudget - 1024 - kMiscSmemBytes;  // bookkeeping lies behind everything else, at the same place whatever the rows
+constexpr int kMiscOff = kSmemBudget - kMiscSmemBytes;  // bookkeeping lies behind everything else, at the same place whatever the rows
 constexpr unsigned long long kLookaheadBytes = 393216;  // how far ahead of the ring the weight streamer reads into L2,
 constexpr unsigned kLookaheadPiece = 8192;             //   in pieces of this size
 constexpr int kLookaheadCycles = 800;                  //   and no more often than this
@@ -243,6 +244,7 @@ struct FwdParams {
     int nstage;        // ring slots of kStageBytes, at offset 0
     int u_off;         // operand region (token operand of the running GEMM; attention tiles)
     int act_off;       // SwiGLU output operand
+    int p_off;         // probabilities of an attention unit
     int plan_ks;       // what the plan follows from besides the rows: column steps of the widest token operand,
     int plan_act;      //   SwiGLU column steps per block at most (0: no SwiGLU operand)
     int plan_attn;     //   bytes the attention tiles need (0: no attention)
@@ -264,13 +266,23 @@ __host__ __device__ inline void plan_smem_rows(FwdParams& P, int rows) {
     if (u < P.plan_attn) u = P.plan_attn;
     u = (u + 1023) / 1024 * 1024;
     int act = P.plan_act * step_bytes;
-    if (P.plan_attn > 0 && act < 128 * (rows | 1) * 4) act = 128 * (rows | 1) * 4;   // exchange area of the q|k|v epilogue
+    bool p_in_u = false;
+    if (P.plan_attn > 0) {
+        if (act < 128 * (rows | 1) * 4) act = 128 * (rows | 1) * 4;   // exchange area of the q|k|v epilogue
+        // probabilities of 128 keys for a unit's query rows: behind the attention tiles where the operand region is wide enough
+        int pr = (P.att_gh * rows + 15) & ~15;
+        if (pr > 64) pr = 64;   // batched: a unit holds the rows of one sequence
+        const int p = pr * kKeyChunk * 2;
+        p_in_u = u >= P.plan_attn + p;
+        if (!p_in_u && act < p) act = p;
+    }
     act = act > 0 ? (act + 1023) / 1024 * 1024 : 1024;
     const int ring = kMiscOff - act - u;
     P.nstage = ring < 0 ? 0 : ring / kStageBytes;
     if (P.nstage > kMaxStages) P.nstage = kMaxStages;
     P.u_off = P.nstage * kStageBytes;
     P.act_off = P.u_off + u;
+    P.p_off = p_in_u ? P.u_off + P.plan_attn : P.act_off;
 }
 
 }  // namespace sdv

@@ -141,7 +141,7 @@ void choose_partition(OpDesc& o, int G, int rows, bool merge, bool always_add) {
                 const double stream = (double)tiles * ks * kStepBytes / 44000.0;
                 const double walk = 0.06 * stages + 0.25 * passes;
                 const double operand_bytes =
-                    merge ? (double)rows * ks * 2 * (kMaxSplits + 1) * 40.0 : (double)rows * ks * 16 * 4.0;
+                    merge ? (double)rows * ks * 2 * 21 * 40.0 : (double)rows * ks * 16 * 4.0;
                 double t = (stream > walk ? stream : walk) + 0.8 + operand_bytes / 60000.0;
                 if (pk > 1 || always_add) t += 0.7 + 0.016 * pk * (rows / 9.0);
                 if (best_t < 0 || t < best_t - 1e-9) {
@@ -203,7 +203,7 @@ SmemPlan plan_smem(FwdParams& P, int rows, bool raw_only) {
     if (!raw_only) {
         const OpDesc& gu = P.op[OP_GU];
         P.plan_act = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;  // SwiGLU column steps per block at most
-        P.plan_attn = kAttnSmemBytes;
+        P.plan_attn = kAttnBytesPerDim * P.hd;
     }
     plan_smem_rows(P, rows);
     SmemPlan s;
@@ -318,30 +318,27 @@ cudaError_t launch_kernel(const FwdParams& P, cudaStream_t stream) {
 }
 
 bool apply_plan(FwdParams& P, int rows, bool raw_only) {
+    if (!raw_only && P.att_gh < 1) P.att_gh = rows >= 64 ? 1 : 64 / rows;   // not chosen yet: room for any choice
     const SmemPlan sp = plan_smem(P, rows, raw_only);
     P.M = rows;
     P.NB = sp.NB;
     return sp.ok;
 }
 
-// Attention split of a launch: heads per unit (a unit's rows, heads x M, fill at most four 16-row
-// tiles), number of key ranges and keys per range (a multiple of 64).  Cost of a choice = the
-// 16-key steps a warp walks one after another: blocks of 64 keys per range x steps per block; with
-// more units than blocks (several sequences, each with its own units) the blocks take them in rounds,
-// each round paying a unit's fixed cost (about three such steps) again.
+// Attention split of a launch: heads per unit (a unit's rows, heads x M, fill at most 64); the key ranges follow (as in
+// attn_split_compute).  Cost of a choice in units of about 0.15 us: per round of one unit per block a fixed price, and per
+// chunk of 128 keys the latency of its products and exchanges and the softmax of its query rows, 16 at a time.
 int plan_attention(const FwdParams& P, int rows, int L, int nseq) {
     int best = -1, best_gh = 1;
     for (int gh = 1; gh <= P.g; ++gh) {
         if (gh * rows > 64 && gh > 1) break;
-        const int MT = (gh * rows + 15) / 16, KG = MT <= 2 ? 4 : (MT == 3 ? 3 : 2);
-        const int QG = (P.g + gh - 1) / gh;
+        const int QG = (P.g + gh - 1) / gh, RP = (gh * rows + 15) / 16;
         int cap = P.G / (P.n_kv * QG);
         if (cap > kMaxSplits) cap = kMaxSplits;
         if (cap < 1) cap = 1;
-        const int keys = L + rows, kps = ((keys + cap - 1) / cap + 63) / 64 * 64, S = (keys + kps - 1) / kps;
-        int cost = (kps / 64) * ((4 + KG - 1) / KG);
+        const int keys = L + rows, chunks = ((keys + cap - 1) / cap + kKeyChunk - 1) / kKeyChunk, S = (keys + chunks * kKeyChunk - 1) / (chunks * kKeyChunk);
         const int rounds = (P.n_kv * QG * S * nseq + P.G - 1) / P.G;
-        cost = rounds * (3 + cost);
+        const int cost = rounds * (6 + chunks * (4 + RP));
         if (best < 0 || cost <= best) {  // ties: more heads per unit (fewer reloads of the keys)
             best = cost;
             best_gh = gh;
@@ -361,12 +358,12 @@ int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph
     FwdParams P = ctx->P;
     P.l_from_state = l_from_state ? 1 : 0;
     const bool raw_only = (ph_begin == 2 + kPhasesPerLayer * ctx->cfg.n_layers);
-    if (!apply_plan(P, rows, raw_only)) return SDV_EINVAL;
     P.rows_from_state = (mode == 0 && !batch) ? 1 : 0;
     P.L = L;
     P.att_gh = P.g < 1 ? 1 : plan_attention(P, batch ? batch->max_rows : rows, L, batch ? batch->n : 1);
     if (P.rows_from_state)   // for every number of rows the draft may turn out to have
         for (int r = 1; r <= rows; ++r) P.att_gh_rows[r - 1] = (uint8_t)plan_attention(P, r, L, 1);
+    if (!apply_plan(P, rows, raw_only)) return SDV_EINVAL;
     P.nseq = 0;
     if (batch) {
         P.nseq = batch->n;
