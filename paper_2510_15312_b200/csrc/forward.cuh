@@ -58,6 +58,12 @@ __device__ __forceinline__ const uint8_t* op_weights(const FwdParams& P, int op,
     return P.wlayers + (unsigned long long)layer * P.layer_stride + P.op[op].w_off;
 }
 
+struct NormShape {
+    int segs, seg_inv;   // segments per row; quotients by it are products with seg_inv, shifted by 16
+    int per4, row_step;  // float4 columns per segment; warps that share a segment
+    int group, adj;      // 16-byte units per column group of the operand; step to the next K slice beyond the columns'
+    uint32_t inv;        // see norm_shape
+};
 struct Misc {
     uint64_t full[kMaxStages], empty[kMaxStages];
     uint64_t tmem_full[2], tmem_empty[2];
@@ -69,7 +75,7 @@ struct Misc {
     unsigned long long* prof_ptr;  // this block's profile words of the running phase (or null)
     int abort_flag;
     int skip;  // block-uniform copy of abort_flag, refreshed inside every grid barrier
-    float sumsq[kMaxRows];  // sums of squares of the residual rows (this block's operand columns)
+    float sumsq[2][kMaxRows];  // sums of squares of the residual rows (this block's operand columns), of this phase and the one before
     union {
         struct {
             float best_v[kEpilogueWarps][kMaxRows];
@@ -78,6 +84,7 @@ struct Misc {
         float att_red[kEpilogueWarps][32];  // maxima and sums of a warp's keys, one query row per lane
     };
     Part part[OP_COUNT];  // this block's share of every operation
+    NormShape shape[OP_COUNT];
     FwdParams P;          // block-local copy of the launch parameters
 };
 static_assert(sizeof(Misc) <= kMiscSmemBytes, "misc shared memory");
@@ -91,6 +98,7 @@ constexpr int kBarrierWarp = kWorkerWarps - 1;
 template <typename F>
 __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target, Misc* misc, int wtid, F prepare) {
     if ((wtid >> 5) == kBarrierWarp) {
+        prepare();
         named_bar_sync(1, kWorkerThreads);
         if ((wtid & 31) == 0) {
             red_release_add_u32(P.bar, 1u);  // no return value to wait for: polling starts at once
@@ -110,7 +118,6 @@ __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target
             *(volatile int*)&misc->skip = *(volatile int*)&misc->abort_flag;
         }
         named_bar_sync(4, kWorkerThreads);
-        prepare();
     } else {
         named_bar_arrive(1, kWorkerThreads);
         prepare();
@@ -222,109 +229,138 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
 // ------------------------------------------------------------------------------------------
 // Token operand of a GEMM, resident in shared memory for the whole operation, in a layout the
 // tensor core reads (K-major, no swizzle): for every 8 columns the M token rows, 16 bytes each:
-//     [8-column group][row 0..M-1][8 bf16].
+//     [8-column group][row 0..M-1, padded to an odd number where it fits][8 bf16].
 // An 8-row core matrix is 128 contiguous bytes, row groups are 128 bytes apart and the two halves
 // of a column step M * 16 bytes.  The instruction reads 16 or 32 rows: the ones past M belong to the
 // next column groups (or lie behind the operand, still inside shared memory) and only feed
 // accumulator columns nobody reads.
-__device__ __forceinline__ uint32_t operand_off(int k8, int row, int M) {
+__device__ __forceinline__ uint32_t operand_off(int k8, int row, int M) {  // M: operand_rows()
     return (uint32_t)((k8 * M + row) * 16);
 }
 
 // Operand = residual rows scaled by the RMSNorm weight (the per-row factor rsqrt(mean + eps)
 // commutes with the GEMM and is applied by the consumer of the result), or, for the stand-alone
-// GEMM, the caller's fp32 rows as they are.  Warp w converts rows w, w + 10, ...; all loads of a
-// batch are issued before the first use.  Leaves the rows' sums of squares over this block's
-// columns in misc->sumsq.
-// What the build needs to know is worked out while the blocks meet at the grid barrier before it (NormPrep): the look-ups and
-// index arithmetic took 740 of the 2800 cycles between a barrier and the finished operand.
+// GEMM, the caller's fp32 rows as they are.  The columns are cut into segments of up to kSegUnits units (32 lanes x 4 columns); a
+// warp stays with one segment and takes every row_step-th row, loading the next row while it converts the one before.  So the
+// norm weights and the places its columns go to are fixed: both are fetched or worked out while the blocks meet at
+// the grid barrier before the phase (NormPrep), and a row costs 15 instructions per unit.  (With weights and addresses
+// worked out per row and unit the build took 8 us at 32 rows of 1536 columns, 6 of them without loading a single row.)
+// Leaves the rows' sums of squares over this block's columns in misc->sumsq.
+constexpr int kSegUnits = 8;
 struct NormPrep {
-    const float4* src;    // this warp's first row, first column of the block's share
-    const float4* wsrc;   // norm weights of the share (nullptr: none)
-    int nk4, stride4;     // float4 columns of the share, of a row
-    // operand layout with K slices: slice of a float4 column = its product with slice_inv, upper half; 16-byte units per 8-column
-    // group; step from a slice to the next beyond that
-    uint32_t slice_inv;
-    int group, slice_adj;
+    const float4* src;       // first row of this warp, this lane's first column
+    int step4;               // float4 columns from one of its rows to the next
+    int row0, row_step;      // its rows
+    int rem;                 // float4 columns from the lane's first one to the segment's end
+    float4 w[kSegUnits];     // norm weights
+    uint32_t off[kSegUnits]; // where a unit goes for row 0, bytes from the operand's start
 };
-__device__ __forceinline__ NormPrep norm_prep(const FwdParams& P, int kind, int layer, const Part& pt, int warp) {
-    NormPrep n;
-    const bool raw = (kind == PH_RAW);
-    const int stride = raw ? P.raw_K : P.d, k4_0 = pt.k0 * 4;
-    const float* xbase = raw ? P.raw_x : P.h;
-    n.nk4 = pt.nk * 4;
-    n.stride4 = stride >> 2;
-    n.src = reinterpret_cast<const float4*>(xbase) + (size_t)warp * n.stride4 + k4_0;
-    n.wsrc = raw ? nullptr
-                 : reinterpret_cast<const float4*>(P.norm_w + (size_t)(kind == PH_QKV ? layer * 2 : (kind == PH_GUD ? layer * 2 + 1 : P.n_layers * 2)) * P.d) + k4_0;
-    const int slices = pt.slices;
-    n.group = slices * P.M;
-    n.slice_inv = 0u;
-    n.slice_adj = 0;
-    if (slices > 1) {
-        const int per4 = n.nk4 / slices;   // float4 columns per slice (a multiple of 4)
-        n.slice_inv = 0xffffffffu / (uint32_t)per4 + 1u;
-        n.slice_adj = P.M - (per4 >> 1) * n.group;
-    }
-    return n;
+// How the block's share of an operation is cut: the same in every layer, so its divisions are done once per launch.
+__device__ __forceinline__ NormShape norm_shape(const FwdParams& P, const Part& pt) {
+    NormShape f;
+    const int units = (pt.nk * 4 + 31) >> 5;
+    f.segs = max(1, (units + kSegUnits - 1) / kSegUnits);
+    f.seg_inv = 65536 / f.segs + 1;
+    f.per4 = (units + f.segs - 1) / f.segs * 32;
+    f.row_step = max(1, kBuilderWarps / f.segs);
+    f.group = operand_rows(P, P.M, pt.slices);
+    const int slice4 = pt.nk * 4 / pt.slices;                               // float4 columns per slice (a multiple of 4)
+    f.inv = pt.slices > 1 && slice4 > 0 ? 0xffffffffu / (uint32_t)slice4 + 1u : 0u;   // slice of a column = upper half of its product with inv
+    f.adj = P.M - (slice4 >> 1) * f.group;                                  // step from a slice to the next beyond the columns'
+    return f;
 }
-// One row, UB units of 4 columns per lane and batch (a warp instruction reads 512 contiguous bytes).
-template <int UB>
-__device__ __forceinline__ float convert_row(const NormPrep& n, const float4* src, uint8_t* U, int row, int lane) {
-    const float4* wld = n.wsrc ? n.wsrc : src;  // without norm weights the loaded value is not used
-    float ss = 0.f;
-#pragma unroll 1
-    for (int base = lane; base < n.nk4; base += 32 * UB) {
-        float4 a[UB], w[UB];
-        // every unit loads (past the end: the row's last unit again, not used), so that the loads are one
-        // straight run of instructions instead of a branch per unit
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            const int k4 = min(base + u * 32, n.nk4 - 1);
-            a[u] = ld_cg_f4_inorder(src + k4);
-            w[u] = ld_nc_f4_inorder(wld + k4);
-        }
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            const int k4 = base + u * 32;
-            if (k4 < n.nk4) {
-                const float4 x = a[u];
-                const float4 g = n.wsrc ? w[u] : make_float4(1.f, 1.f, 1.f, 1.f);
-                ss += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
-                const uint2 out = make_uint2(pack_bf16(x.x * g.x, x.y * g.y), pack_bf16(x.z * g.z, x.w * g.w));
-                const int sl = (int)__umulhi((uint32_t)k4, n.slice_inv);
-                *reinterpret_cast<uint2*>(U + ((k4 >> 1) * n.group + sl * n.slice_adj + row) * 16 + (k4 & 1) * 8) = out;
-            }
-        }
-    }
-    return ss;
-}
-__device__ __forceinline__ void build_norm_operand(const FwdParams& P, const NormPrep& n, uint8_t* U, Misc* misc, int wtid) {
+// `more` > 0: the warp's further segments, where a row has more of them than there are warps.
+template <int KIND>
+__device__ __forceinline__ void norm_prep(NormPrep& n, const FwdParams& P, const Misc* misc, int layer, int wtid, int more) {
+    constexpr bool raw = KIND == PH_RAW;
+    constexpr int op = KIND == PH_QKV ? OP_QKV : KIND == PH_GUD ? OP_GU : KIND == PH_LM ? OP_LM : OP_RAW;
+    const NormShape& f = misc->shape[op];
+    const Part& pt = misc->part[op];
     const int warp = wtid >> 5, lane = wtid & 31;
-    const int M = P.M;
-    const float4* src = n.src;
-#pragma unroll 1
-    for (int row = warp; row < M; row += kBuilderWarps, src += (size_t)kBuilderWarps * n.stride4) {
-        // the batch follows the columns a block has: loads that only repeat the last unit would still cross L2
-        float ss;
-        if (n.nk4 <= 64) ss = convert_row<2>(n, src, U, row, lane);
-        else if (n.nk4 <= 256) ss = convert_row<8>(n, src, U, row, lane);
-        else ss = convert_row<12>(n, src, U, row, lane);
+    const int stride4 = (raw ? P.raw_K : P.d) >> 2, k4_0 = pt.k0 * 4, nk4 = pt.nk * 4;
+    const int turn = (warp * f.seg_inv) >> 16, seg = warp - turn * f.segs + more;
+    n.row_step = f.row_step;
+    n.row0 = turn < f.row_step ? turn : kMaxRows;
+    const int c0 = seg * f.per4 + lane;
+    n.rem = min(f.per4, nk4 - seg * f.per4) - lane;
+    n.src = reinterpret_cast<const float4*>(raw ? P.raw_x : P.h) + n.row0 * stride4 + k4_0 + c0;
+    n.step4 = n.row_step * stride4;
+    const float4* w = reinterpret_cast<const float4*>(P.norm_w + (size_t)(KIND == PH_QKV ? layer * 2 : KIND == PH_GUD ? layer * 2 + 1 : P.n_layers * 2) * P.d) + k4_0 + c0;
 #pragma unroll
-        for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-        if (lane == 0) misc->sumsq[row] = ss;
+    for (int u = 0; u < kSegUnits; ++u) {
+        n.w[u] = raw ? make_float4(1.f, 1.f, 1.f, 1.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!raw) ld_nc_f4_gt(n.w[u], w + u * 32, n.rem, u * 32);
+    }
+#pragma unroll
+    for (int u = 0; u < kSegUnits; ++u) {
+        const int k4 = c0 + u * 32;
+        n.off[u] = (uint32_t)(((k4 >> 1) * f.group + (int)__umulhi((uint32_t)k4, f.inv) * f.adj) * 16 + (k4 & 1) * 8);
+    }
+}
+__device__ __forceinline__ void norm_load(const NormPrep& n, float4 (&a)[kSegUnits], const float4* src, bool live) {
+    const int rem = live ? n.rem : 0;
+#pragma unroll
+    for (int u = 0; u < kSegUnits; ++u) ld_cg_f4_gt(a[u], src + u * 32, rem, u * 32);
+}
+__device__ __forceinline__ void norm_convert(const NormPrep& n, const float4 (&a)[kSegUnits], uint32_t dst, float* sumsq, bool one, int lane) {
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int u = 0; u < kSegUnits; ++u) {
+        const float4 v = a[u], g = n.w[u];
+        s0 += v.x * v.x + v.y * v.y;
+        s1 += v.z * v.z + v.w * v.w;
+        st_shared_v2_gt(dst + n.off[u], pack_bf16(v.x * g.x, v.y * g.y), pack_bf16(v.z * g.z, v.w * g.w), n.rem, u * 32);
+    }
+    s0 += s1;
+#pragma unroll
+    for (int off = 16; off; off >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+    if (lane == 0) {
+        if (one) *sumsq = s0;
+        else atomicAdd(sumsq, s0);
+    }
+}
+// `buf`: which of the two sets of sums this phase uses; the other one is cleared for the next.
+template <int KIND>
+__device__ __forceinline__ void build_norm_operand(const FwdParams& P, NormPrep& n, int layer, uint8_t* U, Misc* misc, int buf, int wtid) {
+    constexpr int op = KIND == PH_QKV ? OP_QKV : KIND == PH_GUD ? OP_GU : KIND == PH_LM ? OP_LM : OP_RAW;
+    const int lane = wtid & 31, M = P.M, segs = misc->shape[op].segs;
+    float* sumsq = misc->sumsq[buf];
+    if (wtid < kMaxRows) misc->sumsq[buf ^ 1][wtid] = 0.f;
+    const uint32_t dst = smem_u32(U);
+#pragma unroll 1
+    for (int more = 0;;) {
+        float4 a[kSegUnits], b[kSegUnits];
+#pragma unroll
+        for (int u = 0; u < kSegUnits; ++u) a[u] = b[u] = make_float4(0.f, 0.f, 0.f, 0.f);   // units past the segment stay zero
+        const float4* src = n.src;
+        int row = n.row0;
+        norm_load(n, a, src, row < M);
+#pragma unroll 1
+        while (row < M) {
+            src += n.step4;
+            norm_load(n, b, src, row + n.row_step < M);
+            norm_convert(n, a, dst + (uint32_t)row * 16u, sumsq + row, segs == 1, lane);
+            row += n.row_step;
+            if (row >= M) break;
+            src += n.step4;
+            norm_load(n, a, src, row + n.row_step < M);
+            norm_convert(n, b, dst + (uint32_t)row * 16u, sumsq + row, segs == 1, lane);
+            row += n.row_step;
+        }
+        more += kBuilderWarps;
+        if (segs <= kBuilderWarps || (wtid >> 5) + more >= segs) break;
+        norm_prep<KIND>(n, P, misc, layer, wtid, more);
     }
 }
 
 // Operand of the output projection = attention output of this block's columns: the split-KV
 // partial results (un-normalised sums with their running maximum and sum) are merged on the way.
-// LPI lanes share one (row, 8 columns) item, each taking every LPI-th partial result: 4 up to 20 partial results, else 8.
-template <int LPI>
+// Four lanes share one (row, 8 columns) item, each taking every fourth partial result, TPL of them at most.
+template <int TPL>
 __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const Part& pt, uint8_t* U, int wtid) {
-    constexpr int TPL = 5;  // partial results per lane at most
-    static_assert(8 * TPL >= kMaxSplits, "partial results per lane");
+    constexpr int LPI = 4;  // lanes per item
     const int S = P.att_S;
-    const int M = P.M, hd = P.hd;
+    const int M = P.M, Mp = operand_rows(P, P.M, 1), hd = P.hd;
     const int k8_0 = pt.k0 * 2, nk8 = pt.nk * 2;
     const int nitems = M * nk8, sub = wtid % LPI;
 #pragma unroll 1
@@ -375,7 +411,7 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
             const float inv = 1.f / v[8];
             const uint4 out = make_uint4(pack_bf16(v[0] * inv, v[1] * inv), pack_bf16(v[2] * inv, v[3] * inv),
                                          pack_bf16(v[4] * inv, v[5] * inv), pack_bf16(v[6] * inv, v[7] * inv));
-            *reinterpret_cast<uint4*>(U + operand_off(k8l, j, M)) = out;
+            *reinterpret_cast<uint4*>(U + operand_off(k8l, j, Mp)) = out;
         }
     }
 }
@@ -389,7 +425,7 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
 // Pipeline positions: (slot, par) is the ring position (slot index and parity of the current trip round the ring), `q`
 // counts accumulator passes, `ops` token operands; all advance over the whole launch, identically in every role.
 struct PipePos {
-    uint32_t slot, par, q, ops;
+    uint32_t slot, par, q, ops, sums;
     uint32_t w_full, w_acc;  // cycles the tensor-core thread waited for weights / for a free accumulator (profile)
 };
 
@@ -419,7 +455,7 @@ __device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8
     const int brows = pt.slices * P.M;                          // rows of the token operand (stacked K slices)
     const uint32_t idesc = umma_idesc_bf16_m128(pt.slices > 1 ? (uint32_t)((brows + 15) & ~15) : (uint32_t)P.NB);
     const uint64_t wait_limit = P.wait_limit_ns;
-    const uint32_t lbo_b = (uint32_t)brows * 16u;
+    const uint32_t lbo_b = (uint32_t)operand_rows(P, P.M, pt.slices) * 16u;
     const uint64_t bstep = (uint64_t)((2u * lbo_b) >> 4);       // one column step, in descriptor address units
     const uint64_t bdesc0 = umma_smem_desc(smem_u32(B), lbo_b, 128u);
     const uint32_t ring0 = smem_u32(smem);
@@ -506,19 +542,19 @@ struct Best {
     int i[2][16];
 };
 
-// LM: the operation is the LM head (`best` carries the running best logits); the other operations are compiled
-// without that state.
-template <bool LM>
-__device__ __forceinline__ void epilogue_op(const FwdParams& P, int op, const Part& pt, uint8_t* act, Misc* misc, PipePos& pos, bool& dead,
+// op: the operation; with the LM head `best` carries the running best logits.
+template <int op>
+__device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, uint8_t* act, Misc* misc, PipePos& pos, bool& dead,
                                             int warp, int lane, Best& best) {
-    const int M = P.M;
+    constexpr bool LM = op == OP_LM;
+    const int M = P.M, Mp = operand_rows(P, P.M, 1);
     const int quarter = warp & 3, myhalf = warp >> 2;  // this warp's 32 accumulator lanes; which of the two accumulators
     const int t = quarter * 32 + lane;
     const uint64_t wait_limit = P.wait_limit_ns;
     const uint32_t tmem_lane = misc->tmem_base + ((uint32_t)(quarter * 32) << 16);
     const int npass = pt.npass, tile0 = pt.tile0, nchunk = M > 16 ? 2 : 1;
     float rs = 0.f;   // lane n: norm factor of token n
-    if ((op == OP_GU || LM) && lane < M) rs = rsqrtf(misc->sumsq[lane] * (1.f / (float)P.d) + P.eps);
+    if ((op == OP_GU || LM) && lane < M) rs = rsqrtf(misc->sumsq[pos.sums][lane] * (1.f / (float)P.d) + P.eps);
     float* out = P.h;
     int stride = P.d;
     bool add = true;  // residual add (O, down)
@@ -568,7 +604,7 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, int op, const Pa
                     // rows 0..7 of a tile are gate rows, 8..15 the matching up rows, 8 lanes apart: the gate
                     // lane evaluates the even token columns, the up lane the odd ones
                     const int col = (pstart + (tt >> 4)) * 8 + (tt & 7);  // SwiGLU column within this block's slice
-                    uint8_t* dst = act + operand_off(col >> 3, n0, M) + (col & 7) * 2;
+                    uint8_t* dst = act + operand_off(col >> 3, n0, Mp) + (col & 7) * 2;
                     if (nsel < 0) swiglu_pairs<-1>(v, rs, n0, t, valid, Mh, dst);
                     else if (nsel == 0) swiglu_pairs<0>(v, rs, n0, t, valid, Mh, dst);
                     else swiglu_pairs<1>(v, rs, n0, t, valid, Mh, dst);
@@ -616,7 +652,7 @@ __device__ __forceinline__ void epilogue_qkv(const FwdParams& P, int layer, cons
         auto fetch = [&](int it, Item& x) {
             const int r = it & 7, m = (it >> 3) % M, T = t0 + (it >> 3) / M;
             const int head = T / (HD / 16), i = (T % (HD / 16)) * 8 + r;
-            x.rs = rsqrtf(misc->sumsq[m] * inv_d + P.eps);
+            x.rs = rsqrtf(misc->sumsq[pos.sums][m] * inv_d + P.eps);
             const float* b = P.bias ? P.bias + (size_t)layer * P.n_qkv + head * HD + i : nullptr;
             x.b0 = b ? __ldg(b) : 0.f;
             x.b1 = b ? __ldg(b + HD2) : 0.f;
@@ -728,30 +764,27 @@ __device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, in
     }
 }
 
-template <int HD, int MODE>
-__device__ __forceinline__ void epilogue_phase(const FwdParams& P, int kind, int layer, uint8_t* act, Misc* misc, PipePos& pos, bool& dead,
+template <int HD, int MODE, int KIND>
+__device__ __forceinline__ void epilogue_phase(const FwdParams& P, int layer, uint8_t* act, uint8_t* ex, Misc* misc, PipePos& pos, bool& dead,
                                                int warp, int lane) {
-    if (kind == PH_QKV) {
-        const Part& pt = misc->part[OP_QKV];
-        if (pt.ntiles > 0 && pt.nk > 0) epilogue_qkv<HD, MODE>(P, layer, pt, reinterpret_cast<float*>(act), misc, pos, dead, warp, lane);
-        return;
-    }
     Best best;
-    if (kind == PH_LM) {
+    if (KIND == PH_QKV) {
+        const Part& pt = misc->part[OP_QKV];
+        if (pt.ntiles > 0 && pt.nk > 0) epilogue_qkv<HD, MODE>(P, layer, pt, reinterpret_cast<float*>(ex), misc, pos, dead, warp, lane);
+    } else if (KIND == PH_LM) {
 #pragma unroll
         for (int n = 0; n < kMaxRows; ++n) { best.v[n >> 4][n & 15] = -CUDART_INF_F; best.i[n >> 4][n & 15] = 0x7fffffff; }
         const Part& pt = misc->part[OP_LM];
-        if (pt.ntiles > 0 && pt.nk > 0) epilogue_op<true>(P, OP_LM, pt, act, misc, pos, dead, warp, lane, best);
+        if (pt.ntiles > 0 && pt.nk > 0) epilogue_op<OP_LM>(P, pt, act, misc, pos, dead, warp, lane, best);
         argmax_finish(P, misc, warp, lane, best, dead);
-        return;
-    }
-    int ops[2];
-    const int nops = phase_ops(kind, ops);
-#pragma unroll 1
-    for (int oi = 0; oi < nops; ++oi) {
-        const Part& pt = misc->part[ops[oi]];
-        if (pt.ntiles == 0 || pt.nk == 0) continue;
-        epilogue_op<false>(P, ops[oi], pt, act, misc, pos, dead, warp, lane, best);
+    } else if (KIND == PH_GUD) {
+        const Part &gu = misc->part[OP_GU], &dn = misc->part[OP_DOWN];
+        if (gu.ntiles > 0 && gu.nk > 0) epilogue_op<OP_GU>(P, gu, act, misc, pos, dead, warp, lane, best);
+        if (dn.ntiles > 0 && dn.nk > 0) epilogue_op<OP_DOWN>(P, dn, act, misc, pos, dead, warp, lane, best);
+    } else {
+        constexpr int op = KIND == PH_O ? OP_O : OP_RAW;
+        const Part& pt = misc->part[op];
+        if (pt.ntiles > 0 && pt.nk > 0) epilogue_op<op>(P, pt, act, misc, pos, dead, warp, lane, best);
     }
 }
 
@@ -1123,32 +1156,24 @@ __device__ void embed_phase(const FwdParams& P, int wtid) {
 // ------------------------------------------------------------------------------------------
 // One GEMM phase as seen by the worker warps: build the token operand, then the tensor-core
 // thread walks the block's stages while the epilogue warps drain the accumulators.
-__device__ __forceinline__ void advance_pos(PipePos& pos, const Part& pt, uint32_t nstage) {
-    const uint32_t at = pos.slot + (uint32_t)(pt.npass * pt.nst);
-    pos.slot = at % nstage;
-    pos.par ^= (at / nstage) & 1u;
-    pos.q += (uint32_t)pt.npass;
-}
-
-template <int HD, int MODE>
-__device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int layer, const NormPrep& prep, uint8_t* smem, Misc* misc,
-                                        PipePos& pos, int wtid, unsigned long long* prof) {
+template <int HD, int MODE, int KIND>
+__device__ __forceinline__ void gemm_phase(const FwdParams& P, int layer, NormPrep& prep, uint8_t* smem, Misc* misc, PipePos& pos, int wtid,
+                                           unsigned long long* prof) {
+    constexpr int op = KIND == PH_QKV ? OP_QKV : KIND == PH_O ? OP_O : KIND == PH_GUD ? OP_GU : KIND == PH_LM ? OP_LM : OP_RAW;
     const int warp = wtid >> 5, lane = wtid & 31;
     uint8_t* U = smem + P.u_off;
-    uint8_t* act = smem + P.act_off;
-    int ops[2];
-    const int nops = phase_ops(kind, ops);
-    const Part& p0 = misc->part[ops[0]];
+    const Part& p0 = misc->part[op];
     const bool have0 = p0.ntiles > 0 && p0.nk > 0;
     bool dead = *(volatile int*)&misc->abort_flag != 0;
     if (wtid == 0) misc->prof_ptr = prof;
     if (have0) {
         if (!dead) {
-            if (kind == PH_O) {
-                if (P.att_S <= 20) build_merged_operand<4>(P, p0, U, wtid);
-                else build_merged_operand<8>(P, p0, U, wtid);
+            if (KIND == PH_O) {
+                if (P.att_S <= 20) build_merged_operand<5>(P, p0, U, wtid);
+                else build_merged_operand<kMaxSplits / 4>(P, p0, U, wtid);
+            } else {
+                build_norm_operand<KIND>(P, prep, layer, U, misc, pos.sums, wtid);
             }
-            else build_norm_operand(P, prep, U, misc, wtid);
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -1159,23 +1184,25 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int kind, int lay
         // the rows' sums of squares the epilogue scales with come from all builder warps
         if (have0 && !dead && !mbar_wait_bounded(&misc->op_ready, pos.ops & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
         PipePos ep = pos;
-        epilogue_phase<HD, MODE>(P, kind, layer, act, misc, ep, dead, warp, lane);
+        epilogue_phase<HD, MODE, KIND>(P, layer, smem + P.act_off, smem + P.p_off, misc, ep, dead, warp, lane);
         if (prof && wtid == 0) prof[4] = global_timer_ns();
     }
-    // pipeline positions advance identically for every role
-    if (have0) ++pos.ops;
-#pragma unroll 1
-    for (int oi = 0; oi < nops; ++oi) {
-        const Part& pt = misc->part[ops[oi]];
-        if (pt.ntiles == 0 || pt.nk == 0) continue;
-        advance_pos(pos, pt, (uint32_t)P.nstage);
+    // pipeline positions advance identically for every role (a worker only follows accumulator passes and operands)
+    if (have0) {
+        ++pos.ops;
+        if (KIND != PH_O) pos.sums ^= 1u;
+        pos.q += (uint32_t)p0.npass;
+    }
+    if (KIND == PH_GUD) {
+        const Part& dn = misc->part[OP_DOWN];
+        if (dn.ntiles > 0 && dn.nk > 0) pos.q += (uint32_t)dn.npass;
     }
 }
 
 // The tensor-core thread: all operations of the launch in order.  It waits for operands, never for grid barriers.
 __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc* misc) {
     PipePos pos;
-    pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
+    pos.slot = pos.par = pos.q = pos.ops = pos.sums = pos.w_full = pos.w_acc = 0;
     uint32_t act_uses = 0;
     bool dead = false, ready = false;
 #pragma unroll 1
@@ -1265,14 +1292,13 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         mbar_init(&misc->done_bar, 1);
         misc->abort_flag = 0;
         misc->skip = 0;
+        for (int r = 0; r < kMaxRows; ++r) misc->sumsq[0][r] = 0.f;
         mbar_fence_init();
     }
     if (warp == kMmaWarp) tmem_alloc(&misc->tmem_base, kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // the first reader of L and of the key ranges (the attention phase) comes after a grid barrier, which orders
-    // these writes before it
     if (tid == 0) {
         if (Pg.l_from_state) misc->P.L = Pg.state[ST_KV_LEN];
         // the block's first attention unit: the same for every layer, so its index arithmetic is done here
@@ -1293,6 +1319,9 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         Q.att_s0 = rem % S;
     }
 
+    if (tid >= 32 && tid < 32 + OP_COUNT) misc->shape[tid - 32] = norm_shape(P, misc->part[tid - 32]);
+    __syncthreads();
+
     if (warp == kProducerWarp) {
         if (lane == 0) producer_loop(P, smem, misc);
         return;
@@ -1309,44 +1338,69 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
 
     const int wtid = tid;  // 0 .. kWorkerThreads-1
     PipePos pos;
-    pos.slot = pos.par = pos.q = pos.ops = pos.w_full = pos.w_acc = 0;
-    int nbar = 0;
-    bool skip = false;
-    int layer, kind = decode_phase(P.ph_begin, P.n_layers, layer);
-    NormPrep prep;
-    int early = 0;
+    pos.slot = pos.par = pos.q = pos.ops = pos.sums = pos.w_full = pos.w_acc = 0;
     uint32_t att_uses = 0;
-    auto prepare = [&](int ph) {
-        kind = decode_phase(ph, P.n_layers, layer);
-        if (kind == PH_ATTN) early = attention_early<HD, MODE>(P, layer, smem + P.u_off, wtid);
-        else if (kind != PH_EMBED && kind != PH_O) {
-            int ops[2];
-            phase_ops(kind, ops);
-            prep = norm_prep(P, kind, layer, misc->part[ops[0]], wtid >> 5);
-        }
-    };
-    prepare(P.ph_begin);
-#pragma unroll 1
-    for (int ph = P.ph_begin; ph < P.ph_end; ++ph) {
-        unsigned long long* pp = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
+    int ph = P.ph_begin;
+    unsigned target = P.bar_base;
+    bool skip = false;   // after an abandoned wait the remaining phases do no work but still meet at every barrier
+    unsigned long long* pp = nullptr;
+    auto enter = [&]() {
+        pp = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
         if (pp && wtid == 0) pp[0] = global_timer_ns();
-        // after an abandoned wait the remaining phases do no work but still meet at every barrier
-        if (skip) {
-        } else if (kind == PH_EMBED) {
-            embed_phase(P, wtid);
-        } else if (kind == PH_ATTN) {
-            attention_phase<HD, MODE>(P, misc, layer, early, smem, wtid, att_uses, pp);
-        } else {
-            gemm_phase<HD, MODE>(P, kind, layer, prep, smem, misc, pos, wtid, pp);
-        }
+    };
+    auto leave = [&]() {
+        ++ph;
         if (pp) {
             named_bar_sync(1, kWorkerThreads);
             if (wtid == 0) pp[1] = global_timer_ns();
         }
-        if (ph + 1 < P.ph_end) {
-            ++nbar;
-            skip = grid_barrier(P, P.bar_base + (unsigned)(nbar * P.G), misc, wtid, [&]() { prepare(ph + 1); });
+    };
+    // the grid barrier behind a phase; `prepare` works out what the next one needs
+    auto meet = [&](auto prepare) {
+        target += (unsigned)P.G;
+        skip = grid_barrier(P, target, misc, wtid, prepare);
+    };
+    const int n_layers = P.n_layers, lm = 1 + kPhasesPerLayer * n_layers;
+    NormPrep prep;
+    if (ph == 0) {
+        enter();
+        embed_phase(P, wtid);
+        leave();
+        meet([&]() { norm_prep<PH_QKV>(prep, P, misc, 0, wtid, 0); });
+#pragma unroll 1
+        for (int layer = 0; layer < n_layers; ++layer) {
+            int early = 0;
+            enter();
+            if (!skip) gemm_phase<HD, MODE, PH_QKV>(P, layer, prep, smem, misc, pos, wtid, pp);
+            leave();
+            meet([&]() { early = attention_early<HD, MODE>(P, layer, smem + P.u_off, wtid); });
+            enter();
+            if (!skip) attention_phase<HD, MODE>(P, misc, layer, early, smem, wtid, att_uses, pp);
+            leave();
+            meet([]() {});
+            enter();
+            if (!skip) gemm_phase<HD, MODE, PH_O>(P, layer, prep, smem, misc, pos, wtid, pp);
+            leave();
+            meet([&]() { norm_prep<PH_GUD>(prep, P, misc, layer, wtid, 0); });
+            enter();
+            if (!skip) gemm_phase<HD, MODE, PH_GUD>(P, layer, prep, smem, misc, pos, wtid, pp);
+            leave();
+            if (layer + 1 < n_layers) meet([&]() { norm_prep<PH_QKV>(prep, P, misc, layer + 1, wtid, 0); });
         }
+        if (ph < P.ph_end) meet([&]() { norm_prep<PH_LM>(prep, P, misc, 0, wtid, 0); });
+    } else if (ph == lm) {
+        norm_prep<PH_LM>(prep, P, misc, 0, wtid, 0);
+    }
+    if (ph == lm && ph < P.ph_end) {
+        enter();
+        if (!skip) gemm_phase<HD, MODE, PH_LM>(P, 0, prep, smem, misc, pos, wtid, pp);
+        leave();
+    }
+    if (MODE == 0 && ph == lm + 1 && ph < P.ph_end) {   // the stand-alone GEMM (a launch of its own)
+        norm_prep<PH_RAW>(prep, P, misc, 0, wtid, 0);
+        enter();
+        gemm_phase<HD, MODE, PH_RAW>(P, 0, prep, smem, misc, pos, wtid, pp);
+        leave();
     }
     tc_fence_before();
     named_bar_sync(3, kWorkerThreads + 32);

@@ -391,6 +391,32 @@ __device__ __forceinline__ float4 ld_nc_f4_inorder(const void* p) {
     asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
+// The same where n > limit; otherwise v keeps its value.
+__device__ __forceinline__ void ld_cg_f4_gt(float4& v, const void* p, int n, int limit) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.gt.s32 p, %5, %6;\n\t"
+        "@p ld.global.cg.v4.f32 {%0,%1,%2,%3}, [%4];\n\t}"
+        : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+        : "l"(p), "r"(n), "r"(limit));
+}
+__device__ __forceinline__ void ld_nc_f4_gt(float4& v, const void* p, int n, int limit) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.gt.s32 p, %5, %6;\n\t"
+        "@p ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];\n\t}"
+        : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+        : "l"(p), "r"(n), "r"(limit));
+}
+// Two words to shared memory where n > limit.
+__device__ __forceinline__ void st_shared_v2_gt(uint32_t addr, uint32_t a, uint32_t b, int n, int limit) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.gt.s32 p, %3, %4;\n\t"
+        "@p st.shared.v2.b32 [%0], {%1,%2};\n\t}"
+        ::"r"(addr), "r"(a), "r"(b), "r"(n), "r"(limit)
+        : "memory");
+}
 __device__ __forceinline__ float2 ld_cg_f2_inorder(const void* p) {
     float2 v;
     asm volatile("ld.global.cg.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));

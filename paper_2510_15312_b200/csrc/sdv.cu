@@ -1729,6 +1729,7 @@ int sdv_debug_plan(const sdv_config* cfg, int G, int rows, int* out) {
     FwdParams P;
     memset(&P, 0, sizeof(P));
     P.d = cfg->d_model;
+    P.hd = cfg->head_dim;
     setup_ops(P, cfg, G);
     for (int i = 0; i < 5; ++i) {
         const OpDesc& o = P.op[i];
