@@ -64,6 +64,10 @@ struct NormShape {
     int group, adj;      // 16-byte units per column group of the operand; step to the next K slice beyond the columns'
     uint32_t inv;        // see norm_shape
 };
+struct MmaShape {
+    uint32_t idesc, blo, bstep;            // instruction descriptor; token operand's descriptor and its column step
+    int groups, last_groups, last_steps;   // column steps of a stage: groups of four, and the last stage's
+};
 struct Misc {
     uint64_t full[kMaxStages], empty[kMaxStages];
     uint64_t tmem_full[2], tmem_empty[2];
@@ -76,15 +80,10 @@ struct Misc {
     int abort_flag;
     int skip;  // block-uniform copy of abort_flag, refreshed inside every grid barrier
     float sumsq[2][kMaxRows];  // sums of squares of the residual rows (this block's operand columns), of this phase and the one before
-    union {
-        struct {
-            float best_v[kEpilogueWarps][kMaxRows];
-            int best_i[kEpilogueWarps][kMaxRows];
-        };
-        float att_red[kEpilogueWarps][32];  // maxima and sums of a warp's keys, one query row per lane
-    };
+    float att_red[kEpilogueWarps][32];  // maxima and sums of a warp's keys, one query row per lane (attention step)
     Part part[OP_COUNT];  // this block's share of every operation
     NormShape shape[OP_COUNT];
+    MmaShape mma[OP_COUNT];
     FwdParams P;          // block-local copy of the launch parameters
 };
 static_assert(sizeof(Misc) <= kMiscSmemBytes, "misc shared memory");
@@ -171,7 +170,7 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
             const Part& pt = misc->part[ops[oi]];
             if (pt.ntiles == 0 || pt.nk == 0) continue;
             const uint8_t* src = op_weights(P, ops[oi], layer) + pt.off;
-            const int nst = pt.nst, SK = pt.SK, nk = pt.nk / pt.slices;
+            const int nst = pt.nst, SK = pt.SK, nk = pt.per;
 #pragma unroll 1
             for (int p = 0; p < pt.npass && ok; ++p) {
                 const uint32_t pbytes = (uint32_t)(pass_count(pt, p) * pt.slices) * kStepBytes;
@@ -417,89 +416,93 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
 }
 
 // ------------------------------------------------------------------------------------------
-// Tensor-core issue, by one thread of the warp for a whole operation.  The pipe takes an instruction (M = 128, N <= 32)
-// every 31 cycles, the time shared memory needs for its 4 KB of weights; what used to set the pace was the code around
-// it.  Stand-alone, a 32 KB stage of eight instructions cost 596 cycles with an election, a wait and a fence per stage, 583
-// by one thread, 520 with the instructions unrolled and 348 with the next stage's barrier looked at (without waiting)
-// before the instructions of this one are issued; the floor without any handshake is 313.
+// Tensor-core issue, by one thread for the whole launch.  The pipe takes an instruction (M = 128, N <= 32) every 31 cycles, the
+// time shared memory needs for its 4 KB of weights, 250 cycles per 32 KB stage; the code around the instructions sets the pace: a
+// lone thread pays the full latency of every dependent instruction and branch.  So what an operation needs is worked out
+// once per launch (MmaShape), descriptors advance by 32-bit additions, the next stage's barrier is looked at (without waiting)
+// before the instructions of this one are issued, and stages run in straight groups of four column steps.
 // Pipeline positions: (slot, par) is the ring position (slot index and parity of the current trip round the ring), `q`
 // counts accumulator passes, `ops` token operands; all advance over the whole launch, identically in every role.
 struct PipePos {
     uint32_t slot, par, q, ops, sums;
     uint32_t w_full, w_acc;  // cycles the tensor-core thread waited for weights / for a free accumulator (profile)
 };
-
-// The instructions of one stage: nks column steps, one or (TWO) two 128-row accumulators.
-template <bool TWO>
-__device__ __forceinline__ void mma_stage(uint32_t d_tmem, uint64_t adesc, uint64_t astep, uint64_t bdesc, uint64_t bstep, uint32_t idesc,
-                                          int nks, uint32_t acc) {
-    auto step = [&]() {
-        umma_bf16(d_tmem, adesc, bdesc, idesc, acc);
-        if (TWO) umma_bf16(d_tmem + 32u, adesc + 128u, bdesc, idesc, acc);
-        acc = 1u;
-        adesc += astep;
-        bdesc += bstep;
-    };
-    int ks = 0;
-#pragma unroll 1
-    for (; ks + 4 <= nks; ks += 4) {
-        step(); step(); step(); step();
-    }
-#pragma unroll 1
-    for (; ks < nks; ++ks) step();
+__device__ __forceinline__ MmaShape mma_shape(const FwdParams& P, const Part& pt, uint32_t operand) {
+    MmaShape f;
+    const int brows = pt.slices * P.M;                          // rows of the token operand (stacked K slices)
+    const uint32_t lbo_b = (uint32_t)operand_rows(P, P.M, pt.slices) * 16u;
+    f.idesc = umma_idesc_bf16_m128(pt.slices > 1 ? (uint32_t)((brows + 15) & ~15) : (uint32_t)P.NB);
+    f.blo = umma_smem_lo(operand, lbo_b);
+    f.bstep = (2u * lbo_b) >> 4;                                // one column step, in descriptor address units
+    f.groups = pt.SK >> 2;                                      // a full stage: groups of four column steps (SK is a multiple of 4)
+    const int last = pt.per - (pt.nst - 1) * pt.SK;             // column steps of the last stage
+    f.last_groups = last >> 2;
+    f.last_steps = last & 3;
+    return f;
 }
 
-__device__ __forceinline__ void mma_op(const FwdParams& P, const Part& pt, uint8_t* smem, const uint8_t* B, Misc* misc,
-                                       PipePos& pos, bool& dead, bool& ready) {
-    const uint32_t nstage = (uint32_t)P.nstage;
-    const int brows = pt.slices * P.M;                          // rows of the token operand (stacked K slices)
-    const uint32_t idesc = umma_idesc_bf16_m128(pt.slices > 1 ? (uint32_t)((brows + 15) & ~15) : (uint32_t)P.NB);
+// The stages of one pass; one or (TWO) two 128-row accumulators.  alo: weight descriptor of ring slot 0.
+template <bool TWO>
+__device__ __forceinline__ bool mma_pass(Misc* misc, PipePos& pos, bool& ready, uint32_t nstage, int nst, const MmaShape& f, uint32_t d, uint32_t alo,
+                                         uint32_t astep, uint64_t wait_limit) {
+    uint32_t b = f.blo, acc = 0u, slot = pos.slot, par = pos.par;
+    int groups = f.groups;
+#pragma unroll 1
+    for (; nst > 0; --nst) {
+        if (!ready) {
+            const long long t0 = clock64();
+            if (!mbar_wait_bounded(&misc->full[slot], par, &misc->abort_flag, wait_limit)) return false;
+            pos.w_full += (uint32_t)(clock64() - t0);
+        }
+        tc_fence_after();
+        uint64_t* const done = &misc->empty[slot];
+        uint32_t a = alo + slot * (uint32_t)(kStageBytes >> 4);
+        if (++slot == nstage) { slot = 0; par ^= 1u; }
+        ready = mbar_test(&misc->full[slot], par);   // the next stage, of this operation or the one after
+        int steps = 0;
+        if (nst == 1) { groups = f.last_groups; steps = f.last_steps; }
+        auto step = [&]() {
+            umma_bf16_lo(d, a, b, f.idesc, acc);
+            if (TWO) umma_bf16_lo(d + 32u, a + 128u, b, f.idesc, acc);   // rows 128.. of the pass
+            acc = 1u;
+            a += astep;
+            b += f.bstep;
+        };
+#pragma unroll 1
+        for (int g = groups; g > 0; --g) {
+            step(); step(); step(); step();
+        }
+#pragma unroll 1
+        for (; steps > 0; --steps) step();
+        umma_commit(done);  // the slot is free once these instructions have read it
+    }
+    pos.slot = slot;
+    pos.par = par;
+    return true;
+}
+// One operation; false: a wait was abandoned.
+__device__ __forceinline__ bool mma_op(const FwdParams& P, int op, uint32_t ring0, Misc* misc, PipePos& pos, bool& ready) {
+    const Part& pt = misc->part[op];
+    const MmaShape f = misc->mma[op];
+    const uint32_t nstage = (uint32_t)P.nstage, tmem0 = misc->tmem_base;
     const uint64_t wait_limit = P.wait_limit_ns;
-    const uint32_t lbo_b = (uint32_t)operand_rows(P, P.M, pt.slices) * 16u;
-    const uint64_t bstep = (uint64_t)((2u * lbo_b) >> 4);       // one column step, in descriptor address units
-    const uint64_t bdesc0 = umma_smem_desc(smem_u32(B), lbo_b, 128u);
-    const uint32_t ring0 = smem_u32(smem);
-    const uint32_t tmem0 = misc->tmem_base;
-    const int nst = pt.nst, SK = pt.SK, nk = pt.nk / pt.slices, npass = pt.npass;
+    const int nst = pt.nst, slices = pt.slices, npass = pt.npass, pbase = pt.pbase, prem = pt.prem;
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
-        const int pcount = pass_count(pt, p) * pt.slices;   // row tiles of the pass, slices stacked
-        const uint32_t buf = pos.q & 1u;
-        if (!dead && !mbar_test(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u)) {
-            const long long tq0 = clock64();
-            if (!mbar_wait_bounded(&misc->tmem_empty[buf], ((pos.q >> 1) & 1u) ^ 1u, &misc->abort_flag, wait_limit)) dead = true;
-            pos.w_acc += (uint32_t)(clock64() - tq0);
+        const uint32_t count = (uint32_t)((pbase + (p < prem ? 1 : 0)) * slices);   // row tiles of the pass, slices stacked
+        const uint32_t buf = pos.q & 1u, par = ((pos.q >> 1) & 1u) ^ 1u, d = tmem0 + buf * kTmemBuf;
+        if (!mbar_test(&misc->tmem_empty[buf], par)) {
+            const long long t0 = clock64();
+            if (!mbar_wait_bounded(&misc->tmem_empty[buf], par, &misc->abort_flag, wait_limit)) return false;
+            pos.w_acc += (uint32_t)(clock64() - t0);
         }
-        const uint32_t d_tmem = tmem0 + buf * kTmemBuf;
-        const uint32_t lbo_a = (uint32_t)(2 * pcount) * 128u;
-        const uint64_t astep = (uint64_t)((2u * lbo_a) >> 4);
-        const uint64_t adesc0 = umma_smem_desc(ring0, lbo_a, 128u);
-        uint64_t bdesc = bdesc0;
-        int kleft = nk;
-#pragma unroll 1
-        for (int st = 0; st < nst; ++st, kleft -= SK) {
-            const uint32_t slot = pos.slot, par = pos.par;
-            if (++pos.slot == nstage) { pos.slot = 0; pos.par ^= 1u; }
-            if (dead) continue;
-            if (!ready) {
-                const long long tw0 = clock64();
-                if (!mbar_wait_bounded(&misc->full[slot], par, &misc->abort_flag, wait_limit)) {
-                    dead = true;
-                    continue;
-                }
-                pos.w_full += (uint32_t)(clock64() - tw0);
-            }
-            tc_fence_after();
-            ready = mbar_test(&misc->full[pos.slot], pos.par);   // the next stage, of this operation or the one after
-            const int nks = min(SK, kleft);
-            const uint64_t adesc = adesc0 + (uint64_t)((slot * (uint32_t)kStageBytes) >> 4);
-            if (pcount > 8) mma_stage<true>(d_tmem, adesc, astep, bdesc, bstep, idesc, nks, st > 0 ? 1u : 0u);   // rows 128..: second accumulator
-            else mma_stage<false>(d_tmem, adesc, astep, bdesc, bstep, idesc, nks, st > 0 ? 1u : 0u);
-            bdesc += (uint64_t)nks * bstep;
-            umma_commit(&misc->empty[slot]);  // the slot is free once these instructions have read it
-        }
-        if (!dead) umma_commit(&misc->tmem_full[buf]);
+        const uint32_t alo = umma_smem_lo(ring0, count * 256u), astep = count * 32u;
+        if (!(count > 8u ? mma_pass<true>(misc, pos, ready, nstage, nst, f, d, alo, astep, wait_limit)
+                         : mma_pass<false>(misc, pos, ready, nstage, nst, f, d, alo, astep, wait_limit)))
+            return false;
+        umma_commit(&misc->tmem_full[buf]);
     }
+    return true;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -729,8 +732,10 @@ __device__ __forceinline__ void epilogue_qkv(const FwdParams& P, int layer, cons
     }
 }
 
-// Best logit per token row over the block: lanes, then the eight epilogue warps.
-__device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, int warp, int lane, const Best& best, bool dead) {
+// Best logit per token row over the block: lanes, then the eight epilogue warps (through `ex`, 2 KB of shared memory).
+__device__ __forceinline__ void argmax_finish(const FwdParams& P, uint8_t* ex, int warp, int lane, const Best& best, bool dead) {
+    float* best_v = reinterpret_cast<float*>(ex);   // [warp][row]
+    int* best_i = reinterpret_cast<int*>(best_v + kEpilogueWarps * kMaxRows);
 #pragma unroll
     for (int n = 0; n < kMaxRows; ++n) {
         if (n < P.M) {
@@ -743,20 +748,20 @@ __device__ __forceinline__ void argmax_finish(const FwdParams& P, Misc* misc, in
                 if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
             }
             if (lane == 0) {
-                misc->best_v[warp][n] = v;
-                misc->best_i[warp][n] = i;
+                best_v[warp * kMaxRows + n] = v;
+                best_i[warp * kMaxRows + n] = i;
             }
         }
     }
     named_bar_sync(2, kEpilogueWarps * 32);
     const int t = warp * 32 + lane;
     if (t < P.M && !dead) {
-        float v = misc->best_v[0][t];
-        int i = misc->best_i[0][t];
+        float v = best_v[t];
+        int i = best_i[t];
 #pragma unroll 1
         for (int w = 1; w < kEpilogueWarps; ++w) {
-            const float ov = misc->best_v[w][t];
-            const int oi = misc->best_i[w][t];
+            const float ov = best_v[w * kMaxRows + t];
+            const int oi = best_i[w * kMaxRows + t];
             if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
         }
         P.cand_val[(size_t)blockIdx.x * kMaxRows + t] = v;
@@ -776,7 +781,7 @@ __device__ __forceinline__ void epilogue_phase(const FwdParams& P, int layer, ui
         for (int n = 0; n < kMaxRows; ++n) { best.v[n >> 4][n & 15] = -CUDART_INF_F; best.i[n >> 4][n & 15] = 0x7fffffff; }
         const Part& pt = misc->part[OP_LM];
         if (pt.ntiles > 0 && pt.nk > 0) epilogue_op<OP_LM>(P, pt, act, misc, pos, dead, warp, lane, best);
-        argmax_finish(P, misc, warp, lane, best, dead);
+        argmax_finish(P, ex, warp, lane, best, dead);
     } else if (KIND == PH_GUD) {
         const Part &gu = misc->part[OP_GU], &dn = misc->part[OP_DOWN];
         if (gu.ntiles > 0 && gu.nk > 0) epilogue_op<OP_GU>(P, gu, act, misc, pos, dead, warp, lane, best);
@@ -874,6 +879,12 @@ __device__ __forceinline__ int attn_early_rows(const AttnUnit& u) {
     return old >= u.nkeys ? kKeyChunk : max(0, min(old, kKeyChunk));
 }
 
+// Power of two; results below the normal range become 0.
+__device__ __forceinline__ float ex2_ftz(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 // Largest of the warp's 32 values, handed to every lane.
 __device__ __forceinline__ float warp_max(float v) {
     float r;
@@ -1017,7 +1028,7 @@ __device__ __forceinline__ void attention_unit(const FwdParams& P, Misc* misc, i
                     const unsigned sg = see >> (g * 16);
 #pragma unroll
                     for (int n = 0; n < 16; ++n) {
-                        const float x = exp2f(v[n] * scale - __shfl_sync(0xffffffffu, ref, g * 16 + n));
+                        const float x = ex2_ftz(v[n] * scale - __shfl_sync(0xffffffffu, ref, g * 16 + n));
                         v[n] = (sg >> n) & 1u ? x : 0.f;
                         *reinterpret_cast<__nv_bfloat16*>(pd + (g * 16 + n) * 128 + (ku ^ (uint32_t)((n & 7) << 4))) = __float2bfloat16(v[n]);
                     }
@@ -1204,44 +1215,50 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
     PipePos pos;
     pos.slot = pos.par = pos.q = pos.ops = pos.sums = pos.w_full = pos.w_acc = 0;
     uint32_t act_uses = 0;
-    bool dead = false, ready = false;
-#pragma unroll 1
-    for (int ph = P.ph_begin; ph < P.ph_end && !dead; ++ph) {
-        int layer, ops[2];
-        const int kind = decode_phase(ph, P.n_layers, layer);
-        const int nops = phase_ops(kind, ops);
+    bool ready = false;
+    const uint32_t ring0 = smem_u32(smem);
+    const uint64_t wait_limit = P.wait_limit_ns;
+    int ph = P.ph_begin;
+    auto run = [&](int op) {   // one operation once its token operand is complete
+        const Part& pt = misc->part[op];
+        if (pt.ntiles == 0 || pt.nk == 0) return true;
+        const bool down = op == OP_DOWN;
         unsigned long long* prof = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
-        pos.w_full = pos.w_acc = 0;
-        long long tc0 = 0;
-#pragma unroll 1
-    #pragma unroll 1
-    for (int oi = 0; oi < nops && !dead; ++oi) {
-            const Part& pt = misc->part[ops[oi]];
-            if (pt.ntiles == 0 || pt.nk == 0) continue;
-            const bool down = ops[oi] == OP_DOWN;
-            if (down && prof) prof[5] = global_timer_ns();
-            if (!mbar_wait_bounded(down ? &misc->act_ready : &misc->op_ready, (down ? act_uses++ : pos.ops++) & 1u, &misc->abort_flag,
-                                   P.wait_limit_ns)) {
-                dead = true;
-                break;
-            }
-            tc_fence_after();
-            if (prof) {
-                if (down) prof[6] = global_timer_ns();
-                else tc0 = clock64();
-            }
-            mma_op(P, pt, smem, smem + (down ? P.act_off : P.u_off), misc, pos, dead, ready);
-        }
-        if (prof && nops > 0) {
+        if (down && prof) prof[5] = global_timer_ns();
+        if (!mbar_wait_bounded(down ? &misc->act_ready : &misc->op_ready, (down ? act_uses++ : pos.ops++) & 1u, &misc->abort_flag, wait_limit))
+            return false;
+        tc_fence_after();
+        if (down && prof) prof[6] = global_timer_ns();
+        if (!down) pos.w_full = pos.w_acc = 0;
+        const long long t0 = clock64();
+        const bool ok = mma_op(P, op, ring0, misc, pos, ready);
+        if (prof) {
+            prof[9] = (unsigned long long)(clock64() - t0);  // cycles of the operation's issue loop (the last one's)
             prof[3] = global_timer_ns();
             prof[7] = pos.w_full;
             prof[8] = pos.w_acc;
-            prof[9] = (unsigned long long)(clock64() - tc0);  // cycles of the whole issue loop
         }
+        return ok;
+    };
+    bool ok = true;
+    const int lm = 1 + kPhasesPerLayer * P.n_layers;
+    if (ph == 0) {
+#pragma unroll 1
+        for (int layer = 0; layer < P.n_layers && ok; ++layer) {
+#pragma unroll 1
+            for (int i = 0; i < 4 && ok; ++i) {   // q|k|v, o, gate|up, down: phases 0, 2, 3 and 3 of the layer
+                ph = 1 + kPhasesPerLayer * layer + (i == 0 ? 0 : (i < 3 ? i + 1 : 3));
+                ok = run(OP_QKV + i);
+            }
+        }
+        ph = lm;
+    }
+    if (ok && P.ph_end > lm) {
+        ok = run(ph == lm ? OP_LM : OP_RAW);
     }
     // all tensor-core work must have completed before tensor memory is returned
     umma_commit(&misc->done_bar);
-    mbar_wait_bounded(&misc->done_bar, 0, &misc->abort_flag, P.wait_limit_ns);
+    mbar_wait_bounded(&misc->done_bar, 0, &misc->abort_flag, wait_limit);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1319,7 +1336,11 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         Q.att_s0 = rem % S;
     }
 
-    if (tid >= 32 && tid < 32 + OP_COUNT) misc->shape[tid - 32] = norm_shape(P, misc->part[tid - 32]);
+    if (tid >= 32 && tid < 32 + OP_COUNT) {
+        const int op = tid - 32;
+        misc->shape[op] = norm_shape(P, misc->part[op]);
+        misc->mma[op] = mma_shape(P, misc->part[op], smem_u32(smem + (op == OP_DOWN ? P.act_off : P.u_off)));
+    }
     __syncthreads();
 
     if (warp == kProducerWarp) {

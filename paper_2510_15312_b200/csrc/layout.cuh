@@ -72,6 +72,7 @@ struct Part {
     int npass, nst;          // passes over the row tiles; stages per pass
     int pbase, prem;         // tiles per pass: pbase + (p < prem)
     int SK, slices;
+    int per, pad;        // column steps per slice
 };
 __host__ __device__ inline int pass_count(const Part& p, int i) { return p.pbase + (i < p.prem ? 1 : 0); }
 __host__ __device__ inline int pass_start(const Part& p, int i) { return i * p.pbase + (i < p.prem ? i : p.prem); }
@@ -96,7 +97,9 @@ __host__ __device__ inline void finish_part(Part& p, const OpDesc& o) {
     p.SK = o.SK;
     p.slices = o.slices > 1 ? o.slices : 1;
     p.npass = (p.ntiles + o.RW - 1) / o.RW;
-    p.nst = (p.nk / p.slices + o.SK - 1) / o.SK;
+    p.per = p.nk / p.slices;
+    p.pad = 0;
+    p.nst = (p.per + o.SK - 1) / o.SK;
     p.pbase = p.npass ? p.ntiles / p.npass : 0;
     p.prem = p.npass ? p.ntiles % p.npass : 0;
 }
@@ -131,6 +134,7 @@ __host__ __device__ inline Part get_part(const OpDesc& o, const OpDesc& gu, int 
         p.tile0 = p.ntiles = p.k0 = p.nk = p.pr = p.pk = p.npass = p.nst = p.pbase = p.prem = 0;
         p.SK = o.SK;
         p.slices = 1;
+        p.per = p.pad = 0;
         p.off = 0;
         return p;
     }

@@ -142,19 +142,18 @@ __host__ __device__ __forceinline__ uint32_t umma_idesc_bf16_m128(uint32_t n) { 
 // D[tmem] = A[smem] * B[smem]^T (first instruction of an accumulation) and D[tmem] += ..., issued by
 // one thread.  Successive column steps only advance the descriptors' address fields (the low 14
 // bits, in 16-byte units), so the issuing thread spends one addition per operand and instruction.
-__device__ __forceinline__ void umma_bf16_first(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
+// The same for operands without swizzle, given the low words of their descriptors (umma_smem_lo): successive column steps only
+// add to the address field, so the issuing thread spends one 32-bit addition per operand and instruction.
+constexpr uint32_t kUmmaPlainHi = (128u >> 4) | (1u << 14);   // 8-row groups 128 bytes apart; descriptor version of this architecture
+__device__ __forceinline__ uint32_t umma_smem_lo(uint32_t saddr, uint32_t lbo) { return ((saddr >> 4) & 0x3fffu) | (((lbo >> 4) & 0x3fffu) << 16); }
+__device__ __forceinline__ void umma_bf16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc));
-}
-__device__ __forceinline__ void umma_bf16_acc(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.eq.b32 p, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc));
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %5};\n\t"
+        "mov.b64 b, {%2, %5};\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(acc), "r"(kUmmaPlainHi));
 }
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
     asm volatile(

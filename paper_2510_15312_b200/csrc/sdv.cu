@@ -8,6 +8,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <new>
 #include <vector>
 
@@ -1761,7 +1762,7 @@ int sdv_debug_timeout_probe(sdv_ctx* ctx) {
 // (small_gemm.cuh), no scratch.
 namespace {
 constexpr size_t kNaWeightBytes = (size_t)2 << 20;              // N * K * 2 <= 2 MiB
-constexpr int kNaMaxK = 4096, kNaMaxN = 4096;
+constexpr int kNaMaxK = 4096, kNaMaxN = 4096, kNaMaxDevices = 64;
 }  // namespace
 
 extern "C" {
@@ -1807,6 +1808,15 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
     cfg.numAttrs = 1;
     typedef void (*Kernel)(const float*, const uint16_t*, float*, int, int, int);
     static const Kernel kernels[4] = {small_gemm_kernel<1>, small_gemm_kernel<2>, small_gemm_kernel<3>, small_gemm_kernel<4>};
+    static std::atomic<bool> loaded[kNaMaxDevices];
+    if (dev >= kNaMaxDevices || !loaded[dev].load(std::memory_order_relaxed)) {
+        // the runtime loads a kernel's code when it is first named: all four now, so that no later call makes it take memory
+        for (int i = 0; i < 4; ++i) {
+            cudaFuncAttributes fa;
+            if (cudaFuncGetAttributes(&fa, (const void*)kernels[i]) != cudaSuccess) return SDV_ECUDA;
+        }
+        if (dev < kNaMaxDevices) loaded[dev].store(true, std::memory_order_relaxed);
+    }
     if (cudaLaunchKernelEx(&cfg, kernels[(M - 1) / 8], dev_x, dev_w, dev_y, M, N, K) != cudaSuccess) return SDV_ECUDA;
     return cudaStreamSynchronize(s) == cudaSuccess ? SDV_OK : SDV_ECUDA;
 }
