@@ -70,7 +70,7 @@ struct MmaShape {
 };
 struct Misc {
     uint64_t full[kMaxStages], empty[kMaxStages];
-    uint64_t tmem_full[2], tmem_empty[2];
+    uint64_t tmem_full[kAccBufs], tmem_empty[kAccBufs];
     uint64_t op_ready;    // the token operand of this block's next operation is complete (one arrival per builder warp)
     uint64_t act_ready;   // the SwiGLU operand of this block is complete (one arrival per epilogue warp)
     uint64_t att_bar;     // a product of the attention step has completed
@@ -480,8 +480,10 @@ __device__ __forceinline__ bool mma_pass(Misc* misc, PipePos& pos, bool& ready, 
     pos.par = par;
     return true;
 }
-// One operation; false: a wait was abandoned.
-__device__ __forceinline__ bool mma_op(const FwdParams& P, int op, uint32_t ring0, Misc* misc, PipePos& pos, bool& ready) {
+// One operation; false: a wait was abandoned.  The token operand (`operand`, its parity) is waited for last, with everything else
+// at hand.
+__device__ __forceinline__ bool mma_op(const FwdParams& P, int op, uint32_t ring0, Misc* misc, PipePos& pos, bool& ready, uint64_t* operand,
+                                       uint32_t operand_par) {
     const Part& pt = misc->part[op];
     const MmaShape f = misc->mma[op];
     const uint32_t nstage = (uint32_t)P.nstage, tmem0 = misc->tmem_base;
@@ -490,13 +492,22 @@ __device__ __forceinline__ bool mma_op(const FwdParams& P, int op, uint32_t ring
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
         const uint32_t count = (uint32_t)((pbase + (p < prem ? 1 : 0)) * slices);   // row tiles of the pass, slices stacked
-        const uint32_t buf = pos.q & 1u, par = ((pos.q >> 1) & 1u) ^ 1u, d = tmem0 + buf * kTmemBuf;
+        const uint32_t buf = pos.q % kAccBufs, par = ((pos.q / kAccBufs) & 1u) ^ 1u, d = tmem0 + (slices > 1 ? kTmemStack : buf * kTmemBuf);
         if (!mbar_test(&misc->tmem_empty[buf], par)) {
             const long long t0 = clock64();
             if (!mbar_wait_bounded(&misc->tmem_empty[buf], par, &misc->abort_flag, wait_limit)) return false;
             pos.w_acc += (uint32_t)(clock64() - t0);
         }
         const uint32_t alo = umma_smem_lo(ring0, count * 256u), astep = count * 32u;
+        if (p == 0) {
+            if (!ready) {
+                const long long t0 = clock64();
+                if (!mbar_wait_bounded(&misc->full[pos.slot], pos.par, &misc->abort_flag, wait_limit)) return false;
+                pos.w_full += (uint32_t)(clock64() - t0);
+                ready = true;
+            }
+            if (!mbar_wait_bounded(operand, operand_par, &misc->abort_flag, wait_limit)) return false;
+        }
         if (!(count > 8u ? mma_pass<true>(misc, pos, ready, nstage, nst, f, d, alo, astep, wait_limit)
                          : mma_pass<false>(misc, pos, ready, nstage, nst, f, d, alo, astep, wait_limit)))
             return false;
@@ -566,8 +577,8 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, 
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
         const int pcount = pass_count(pt, p), pstart = pass_start(pt, p);
-        const uint32_t buf = pos.q & 1u;
-        if (!dead && !mbar_wait_bounded(&misc->tmem_full[buf], (pos.q >> 1) & 1u, &misc->abort_flag, wait_limit)) dead = true;
+        const uint32_t buf = pos.q % kAccBufs;
+        if (!dead && !mbar_wait_bounded(&misc->tmem_full[buf], (pos.q / kAccBufs) & 1u, &misc->abort_flag, wait_limit)) dead = true;
         dead = __any_sync(0xffffffffu, dead);
         if (dead) continue;
         tc_fence_after();
@@ -649,7 +660,7 @@ __device__ __forceinline__ void epilogue_qkv(const FwdParams& P, int layer, cons
 #pragma unroll 1
     for (int p = 0; p < pt.npass; ++p, ++pos.q) {
         const int pcount = pass_count(pt, p), RR = pcount * 16, t0 = pt.tile0 + pass_start(pt, p);
-        const uint32_t buf = pos.q & 1u;
+        const uint32_t buf = pos.q % kAccBufs;
         // where an item's output goes and what it needs: fetched before the accumulator is there
         struct Item { float2 cs; float b0, b1, rs; __nv_bfloat16* dst; };
         auto fetch = [&](int it, Item& x) {
@@ -680,14 +691,14 @@ __device__ __forceinline__ void epilogue_qkv(const FwdParams& P, int layer, cons
         const int items = pcount * 8 * M;
         Item first;
         if (tid < items) fetch(tid, first);
-        if (!dead && !mbar_wait_bounded(&misc->tmem_full[buf], (pos.q >> 1) & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
+        if (!dead && !mbar_wait_bounded(&misc->tmem_full[buf], (pos.q / kAccBufs) & 1u, &misc->abort_flag, P.wait_limit_ns)) dead = true;
         dead = __any_sync(0xffffffffu, dead);
         if (!dead) {
             tc_fence_after();
             if (misc->prof_ptr && tid == 0 && p == pt.npass - 1) misc->prof_ptr[10] = global_timer_ns();
             // lanes of the accumulator: slice s * RR + row; of the columns a lane wants those of its own slice.  Where a warp's lanes
             // span two slices, the two warps that share the lanes take one each; else they take a chunk of 16 tokens each
-            const uint32_t taddr = misc->tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kTmemBuf;
+            const uint32_t taddr = misc->tmem_base + ((uint32_t)(quarter * 32) << 16) + (slices > 1 ? kTmemStack : buf * kTmemBuf);
             const int row = quarter * 32 + lane;
             const int sl0 = (quarter * 32) / RR, sl1 = (quarter * 32 + 31) / RR;
             const bool span = sl0 != sl1;
@@ -1224,17 +1235,12 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
         if (pt.ntiles == 0 || pt.nk == 0) return true;
         const bool down = op == OP_DOWN;
         unsigned long long* prof = P.prof ? P.prof + ((size_t)(ph - P.ph_begin) * P.G + blockIdx.x) * kProfWords : nullptr;
-        if (down && prof) prof[5] = global_timer_ns();
-        if (!mbar_wait_bounded(down ? &misc->act_ready : &misc->op_ready, (down ? act_uses++ : pos.ops++) & 1u, &misc->abort_flag, wait_limit))
-            return false;
-        tc_fence_after();
-        if (down && prof) prof[6] = global_timer_ns();
         if (!down) pos.w_full = pos.w_acc = 0;
         const long long t0 = clock64();
-        const bool ok = mma_op(P, op, ring0, misc, pos, ready);
+        const bool ok = mma_op(P, op, ring0, misc, pos, ready, down ? &misc->act_ready : &misc->op_ready, (down ? act_uses++ : pos.ops++) & 1u);
         if (prof) {
-            prof[9] = (unsigned long long)(clock64() - t0);  // cycles of the operation's issue loop (the last one's)
-            prof[3] = global_timer_ns();
+            prof[9] = (unsigned long long)(clock64() - t0);  // cycles from turning to the operation (the phase's last one) to its last instruction
+            prof[op == OP_GU ? 5 : 3] = global_timer_ns();
             prof[7] = pos.w_full;
             prof[8] = pos.w_acc;
         }
@@ -1299,7 +1305,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
             mbar_init(&misc->full[s], 1);
             mbar_init(&misc->empty[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < (int)kAccBufs; ++b) {
             mbar_init(&misc->tmem_full[b], 1);
             mbar_init(&misc->tmem_empty[b], kEpilogueWarps);
         }

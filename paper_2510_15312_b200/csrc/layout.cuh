@@ -47,8 +47,10 @@ constexpr unsigned kLookaheadPiece = 8192;             //   in pieces of this si
 constexpr int kLookaheadCycles = 800;                  //   and no more often than this
 constexpr int kMaxDraftWords = 32;
 constexpr int kProfWords = 12;                         // timestamps per (phase, block)
-constexpr int kTmemCols = 512;                         // two buffers; each two 128-row accumulators of up to 32 fp32 columns, or one of up to 256
-constexpr uint32_t kTmemBuf = 256;                     //   (stacked K slices)
+constexpr int kTmemCols = 512;
+constexpr uint32_t kAccBufs = 4;                       // accumulator buffers: each two 128-row accumulators of up to 32 fp32 columns,
+constexpr uint32_t kTmemBuf = 64;                      //   columns 0..255; so many that the issuing thread does not wait for a pass to be read out
+constexpr uint32_t kTmemStack = 256;                   // stacked K slices (one pass, up to 256 columns): columns 256..511
 
 enum OpIndex { OP_QKV = 0, OP_O = 1, OP_GU = 2, OP_DOWN = 3, OP_LM = 4, OP_RAW = 5, OP_COUNT = 6 };
 
