@@ -135,6 +135,7 @@ struct Lookahead {   // cursor over the block's weight stream: operation by oper
     int ph, oi;
     const uint8_t* src;
     unsigned long long begin, end;   // the running operation's place in the stream
+    uint32_t bytes, first;           // its bytes, and where in its weights the block begins
 };
 __device__ __forceinline__ bool lookahead_next(const FwdParams& P, Misc* misc, Lookahead& c) {
     for (;;) {
@@ -146,7 +147,9 @@ __device__ __forceinline__ bool lookahead_next(const FwdParams& P, Misc* misc, L
         if (pt.ntiles == 0 || pt.nk == 0) continue;
         c.src = op_weights(P, ops[c.oi], layer) + pt.off;
         c.begin = c.end;
-        c.end += (unsigned long long)pt.ntiles * pt.nk * kStepBytes;
+        c.bytes = (uint32_t)(pt.ntiles * pt.nk * kStepBytes);
+        c.first = (uint32_t)(pass_start(pt, pt.rot) * pt.nk * kStepBytes);
+        c.end += c.bytes;
         return true;
     }
 }
@@ -157,7 +160,7 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
     bool ok = true;
     unsigned long long streamed = 0, ahead = 0;   // bytes copied / read ahead so far
     Lookahead la;
-    la.ph = P.ph_begin; la.oi = -1; la.begin = la.end = 0; la.src = nullptr;
+    la.ph = P.ph_begin; la.oi = -1; la.begin = la.end = 0; la.src = nullptr; la.bytes = la.first = 0;
     bool more = lookahead_next(P, misc, la);
     long long last = clock64();
 #pragma unroll 1
@@ -169,11 +172,13 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
         for (int oi = 0; oi < nops && ok; ++oi) {
             const Part& pt = misc->part[ops[oi]];
             if (pt.ntiles == 0 || pt.nk == 0) continue;
-            const uint8_t* src = op_weights(P, ops[oi], layer) + pt.off;
+            const uint8_t* const op_src = op_weights(P, ops[oi], layer) + pt.off;
             const int nst = pt.nst, SK = pt.SK, nk = pt.per;
 #pragma unroll 1
             for (int p = 0; p < pt.npass && ok; ++p) {
-                const uint32_t pbytes = (uint32_t)(pass_count(pt, p) * pt.slices) * kStepBytes;
+                const int pi = pass_index(pt, p);
+                const uint8_t* src = op_src + (size_t)pass_start(pt, pi) * (uint32_t)(pt.nk * kStepBytes);
+                const uint32_t pbytes = (uint32_t)(pass_count(pt, pi) * pt.slices) * kStepBytes;
                 int kleft = nk;
 #pragma unroll 1
                 for (int st = 0; st < nst; ++st, kleft -= SK) {
@@ -187,9 +192,11 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
                             if (ahead < streamed) ahead = streamed;
                             while (more && ahead >= la.end) more = lookahead_next(P, misc, la);
                             if (more && ahead < streamed + kLookaheadBytes) {
-                                const unsigned long long left = la.end - ahead;
-                                const uint32_t piece = left < kLookaheadPiece ? (uint32_t)left : kLookaheadPiece;
-                                bulk_prefetch_l2(la.src + (ahead - la.begin), piece);
+                                uint32_t at = (uint32_t)(ahead - la.begin) + la.first, left = (uint32_t)(la.end - ahead);
+                                if (at >= la.bytes) at -= la.bytes;
+                                if (left > la.bytes - at) left = la.bytes - at;
+                                const uint32_t piece = left < kLookaheadPiece ? left : kLookaheadPiece;
+                                bulk_prefetch_l2(la.src + at, piece);
                                 ahead += piece;
                                 last = now;
                             }
@@ -488,10 +495,11 @@ __device__ __forceinline__ bool mma_op(const FwdParams& P, int op, uint32_t ring
     const MmaShape f = misc->mma[op];
     const uint32_t nstage = (uint32_t)P.nstage, tmem0 = misc->tmem_base;
     const uint64_t wait_limit = P.wait_limit_ns;
-    const int nst = pt.nst, slices = pt.slices, npass = pt.npass, pbase = pt.pbase, prem = pt.prem;
+    const int nst = pt.nst, slices = pt.slices, npass = pt.npass, pbase = pt.pbase, prem = pt.prem, rot = pt.rot;
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
-        const uint32_t count = (uint32_t)((pbase + (p < prem ? 1 : 0)) * slices);   // row tiles of the pass, slices stacked
+        const int pi = p + rot < npass ? p + rot : p + rot - npass;
+        const uint32_t count = (uint32_t)((pbase + (pi < prem ? 1 : 0)) * slices);   // row tiles of the pass, slices stacked
         const uint32_t buf = pos.q % kAccBufs, par = ((pos.q / kAccBufs) & 1u) ^ 1u, d = tmem0 + (slices > 1 ? kTmemStack : buf * kTmemBuf);
         if (!mbar_test(&misc->tmem_empty[buf], par)) {
             const long long t0 = clock64();
@@ -576,7 +584,8 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, 
     const int store_logits = P.store_logits;
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
-        const int pcount = pass_count(pt, p), pstart = pass_start(pt, p);
+        const int pi = op == OP_GU || LM ? p : pass_index(pt, p);   // those two have no partial sums
+        const int pcount = pass_count(pt, pi), pstart = pass_start(pt, pi);
         const uint32_t buf = pos.q % kAccBufs;
         if (!dead && !mbar_wait_bounded(&misc->tmem_full[buf], (pos.q / kAccBufs) & 1u, &misc->abort_flag, wait_limit)) dead = true;
         dead = __any_sync(0xffffffffu, dead);

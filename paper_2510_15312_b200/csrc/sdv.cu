@@ -1689,9 +1689,9 @@ int sdv_debug_layout_check(const int* desc, const int* gu_desc, int G) {
     for (int cta = 0; cta < G; ++cta) {
         const Part pt = get_part(o, gu, cta, G);
         if (pt.ntiles == 0 || pt.nk == 0) continue;
-        unsigned long long src = pt.off;  // the streamer's running offset
-        for (int p = 0; p < pt.npass; ++p) {
-            const int pcount = pass_count(pt, p), pstart = pass_start(pt, p);
+        for (int i = 0; i < pt.npass; ++i) {
+            const int p = pass_index(pt, i), pcount = pass_count(pt, p), pstart = pass_start(pt, p);
+            unsigned long long src = pt.off + (unsigned long long)pstart * pt.nk * kStepBytes;  // the streamer's running offset
             if (pcount < 1 || pcount > 16) return -100;
             const int per = pt.nk / slices, v = pcount * slices;   // column steps per slice; row tiles of the pass, slices stacked
             for (int st = 0; st < pt.nst; ++st) {
