@@ -1,6 +1,7 @@
 """ctypes binding of libsdv.so.  Method names follow the C entry points (include/sdv.h)."""
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
 from typing import List, Optional, Sequence, Tuple
@@ -129,6 +130,22 @@ def config_from(cfg, k_max: Optional[int] = None, max_seq: Optional[int] = None,
                      cfg.ngram_n, cfg.ngram_min, int(search_history), cfg.rope_theta, cfg.rms_eps)
 
 
+_Tokens = C.c_int32 * (K_MAX + 1)   # room for what one call hands back
+_NO_TOKENS = (C.c_int32 * 1)()
+
+
+def _tokens(seq):
+    """(object to keep alive, its address, length) of a sequence of token ids as int32."""
+    if isinstance(seq, (list, tuple)):
+        try:
+            a = array.array("i", seq)
+            return (a, a.buffer_info()[0], len(a)) if a else (_NO_TOKENS, C.addressof(_NO_TOKENS), 0)
+        except TypeError:
+            pass
+    a = np.ascontiguousarray(seq, dtype=np.int32)
+    return (a, a.ctypes.data, len(a)) if len(a) else (_NO_TOKENS, C.addressof(_NO_TOKENS), 0)
+
+
 def _ptr(a):
     if a is None:
         return None
@@ -205,23 +222,19 @@ class Sdv:
         if not fetch:
             self._check(lib().sdv_draft(self._h, k, None, None), "sdv_draft")
             return None
-        out = np.zeros(K_MAX, dtype=np.int32)
-        dl = C.c_int(0)
-        self._check(lib().sdv_draft(self._h, k, out.ctypes.data, C.byref(dl)), "sdv_draft")
-        return out[:dl.value].tolist()
+        out, dl = _Tokens(), C.c_int(0)
+        self._check(lib().sdv_draft(self._h, k, out, C.byref(dl)), "sdv_draft")
+        return out[:dl.value]
 
     def verify(self, draft: Optional[Sequence[int]] = None, fetch: bool = True) -> Optional[Tuple[List[int], int]]:
         """draft=None verifies the device draft left by draft(); returns (y, accept_len) when fetch."""
-        d = None if draft is None else np.ascontiguousarray(draft, dtype=np.int32)
-        dp = None if d is None else (d.ctypes.data if len(d) else np.zeros(1, np.int32).ctypes.data)
-        dl = 0 if d is None else len(d)
+        d, dp, dl = (None, None, 0) if draft is None else _tokens(draft)
         if not fetch:
             self._check(lib().sdv_verify(self._h, dp, dl, None, None), "sdv_verify")
             return None
-        y = np.zeros(K_MAX + 1, dtype=np.int32)
-        a = C.c_int(0)
-        self._check(lib().sdv_verify(self._h, dp, dl, y.ctypes.data, C.byref(a)), "sdv_verify")
-        return y, a.value
+        y, a = _Tokens(), C.c_int(0)
+        self._check(lib().sdv_verify(self._h, dp, dl, y, C.byref(a)), "sdv_verify")
+        return np.frombuffer(y, dtype=np.int32), a.value
 
     @staticmethod
     def verify_batch(seqs: Sequence["Sdv"], fetch: bool = True) -> Optional[List[int]]:
@@ -235,14 +248,11 @@ class Sdv:
     def step(self, draft: Optional[Sequence[int]], k_next: int) -> Tuple[List[int], List[int], int]:
         """Verify `draft` (None: the device draft), accept, commit and draft k_next tokens for the next step:
         one call, one synchronisation.  Returns (emitted tokens, next draft, KV length)."""
-        d = None if draft is None else np.ascontiguousarray(draft, dtype=np.int32)
-        dp = None if d is None else (d.ctypes.data if len(d) else np.zeros(1, np.int32).ctypes.data)
-        em = np.zeros(K_MAX + 1, dtype=np.int32)
-        nd = np.zeros(K_MAX + 1, dtype=np.int32)
+        d, dp, dl = (None, None, 0) if draft is None else _tokens(draft)
+        em, nd = _Tokens(), _Tokens()
         n, ndl, kv = C.c_int(0), C.c_int(0), C.c_int(0)
-        self._check(lib().sdv_step(self._h, dp, 0 if d is None else len(d), k_next, em.ctypes.data, C.byref(n),
-                                   nd.ctypes.data, C.byref(ndl), C.byref(kv)), "sdv_step")
-        return em[:n.value].tolist(), nd[:ndl.value].tolist(), kv.value
+        self._check(lib().sdv_step(self._h, dp, dl, k_next, em, C.byref(n), nd, C.byref(ndl), C.byref(kv)), "sdv_step")
+        return em[:n.value], nd[:ndl.value], kv.value
 
     def decode_steps(self, k: int, n_steps: int, max_tokens: int = 0, ext_max_total: int = 0,
                      ext_max_life: int = 0) -> Tuple[List[int], int]:
@@ -348,10 +358,10 @@ class Sdv:
         return out
 
     def commit(self, max_emit: int = 0) -> Tuple[List[int], int]:
-        out = np.zeros(K_MAX + 1, dtype=np.int32)
+        out = _Tokens()
         n, kv = C.c_int(0), C.c_int(0)
-        self._check(lib().sdv_commit(self._h, max_emit, out.ctypes.data, C.byref(n), C.byref(kv)), "sdv_commit")
-        return out[:n.value].tolist(), kv.value
+        self._check(lib().sdv_commit(self._h, max_emit, out, C.byref(n), C.byref(kv)), "sdv_commit")
+        return out[:n.value], kv.value
 
     def rollback(self, new_kv_len: int):
         self._check(lib().sdv_rollback(self._h, new_kv_len), "sdv_rollback")

@@ -752,24 +752,29 @@ __device__ __forceinline__ void epilogue_qkv(const FwdParams& P, int layer, cons
     }
 }
 
+// Largest of the warp's 32 values, handed to every lane.
+__device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
 // Best logit per token row over the block: lanes, then the eight epilogue warps (through `ex`, 2 KB of shared memory).
 __device__ __forceinline__ void argmax_finish(const FwdParams& P, uint8_t* ex, int warp, int lane, const Best& best, bool dead) {
     float* best_v = reinterpret_cast<float*>(ex);   // [warp][row]
     int* best_i = reinterpret_cast<int*>(best_v + kEpilogueWarps * kMaxRows);
+    // two reductions per row (the value, then the lowest id that has it): written out as shuffles this was 70 KB of code that ran
+    // once, 7 us behind the last pass, mostly fetching itself
 #pragma unroll
-    for (int n = 0; n < kMaxRows; ++n) {
-        if (n < P.M) {
-            float v = best.v[n >> 4][n & 15];
-            int i = best.i[n >> 4][n & 15];
+    for (int h = 0; h < 2; ++h) {
+        if (h * 16 < P.M) {
 #pragma unroll
-            for (int off = 1; off <= 16; off <<= 1) {
-                const float ov = __shfl_xor_sync(0xffffffffu, v, off);
-                const int oi = __shfl_xor_sync(0xffffffffu, i, off);
-                if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
-            }
-            if (lane == 0) {
-                best_v[warp * kMaxRows + n] = v;
-                best_i[warp * kMaxRows + n] = i;
+            for (int n = 0; n < 16; ++n) {
+                const float v = warp_max(best.v[h][n]);
+                const int i = __reduce_min_sync(0xffffffffu, best.v[h][n] == v ? best.i[h][n] : 0x7fffffff);
+                if (lane == n) {
+                    best_v[warp * kMaxRows + h * 16 + n] = v;
+                    best_i[warp * kMaxRows + h * 16 + n] = i;
+                }
             }
         }
     }
@@ -903,12 +908,6 @@ __device__ __forceinline__ int attn_early_rows(const AttnUnit& u) {
 __device__ __forceinline__ float ex2_ftz(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-// Largest of the warp's 32 values, handed to every lane.
-__device__ __forceinline__ float warp_max(float v) {
-    float r;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 // Sums over the warp of 16 columns: lane n receives column n & 15.
@@ -1159,7 +1158,17 @@ __device__ __forceinline__ int attention_early(const FwdParams& P, int layer, ui
     return n;
 }
 // ------------------------------------------------------------------------------------------
-__device__ void embed_phase(const FwdParams& P, int wtid) {
+__device__ void embed_phase(const FwdParams& P, const DraftArg& draft, int wtid) {
+    if (blockIdx.x == 0 && draft.n >= 0) {
+        // the caller's draft becomes the one of the state block, for the kernels behind this one
+        if (wtid < draft.n) P.state[ST_DRAFT + wtid] = draft.tok[wtid];
+        if (wtid == 0) {
+            P.state[ST_DRAFT_LEN] = draft.n;
+            P.state[ST_BASE_LEN] = draft.n;
+            P.state[ST_SEG_USED] = 0;
+            P.state[ST_TREE_ON] = 0;
+        }
+    }
     // residual rows from the embedding table; rows beyond M are cleared
     const int units = kMaxRows * (P.d / 8);
 #pragma unroll 1
@@ -1170,6 +1179,7 @@ __device__ void embed_phase(const FwdParams& P, int wtid) {
             int tok;
             if (P.mode == 1) tok = P.hist[P.L + row];
             else if (row == 0) tok = P.state[ST_PENDING];
+            else if (draft.n >= 0) tok = draft.tok[row - 1];
             else tok = (row <= P.state[ST_DRAFT_LEN]) ? P.state[ST_DRAFT + row - 1] : 0;
             tok = min(max(tok, 0), P.V - 1);
             const uint4 raw = __ldg(reinterpret_cast<const uint4*>(P.emb + (size_t)tok * P.d + c8 * 8));
@@ -1279,7 +1289,7 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
 // ------------------------------------------------------------------------------------------
 // HD: head dimension; MODE: chain, tree or batch (see attention_unit).
 template <int HD, int MODE>
-__global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg) {
+__global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg, const __grid_constant__ DraftArg draft) {
     static_assert(sizeof(FwdParams) % 4 == 0, "parameter block is copied word by word");
     extern __shared__ __align__(1024) uint8_t smem[];   // the launch's only shared memory: starts on a 1024-byte boundary
     Misc* misc = reinterpret_cast<Misc*>(smem + kMiscOff);
@@ -1400,7 +1410,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     NormPrep prep;
     if (ph == 0) {
         enter();
-        embed_phase(P, wtid);
+        embed_phase(P, draft, wtid);
         leave();
         meet([&]() { norm_prep<PH_QKV>(prep, P, misc, 0, wtid, 0); });
 #pragma unroll 1

@@ -34,6 +34,7 @@ constexpr int kStepBytes = 512;                        // one row tile x one col
 constexpr int kStageBytes = 32768;                     // ring slot
 constexpr int kMaxStages = 8;                          // ring slots at most
 constexpr int kMaxRows = 32;                           // token rows a buffer is sized for
+constexpr int kMaxGrid = 256;                          // thread blocks at most: per-block candidate arrays are sized for them
 constexpr int kMaxBatch = 8;                           // sequences one batched verify step takes at most
 constexpr int kMaxSplits = 40;                         // key ranges per head at most
 constexpr int kSmemBudget = 232448;                    // 227 KB
@@ -196,6 +197,12 @@ enum StateWord {
     ST_ANC = 256,     // [32] bit r set: row r lies on row j's path from the root (j itself included)
     ST_PATH = 288,    // [32] accepted path (rows), root excluded
     ST_WORDS = 320
+};
+
+// Caller-supplied tokens (or other small whole numbers) by value, so that no host buffer has to outlive the call; n < 0: none.
+struct DraftArg {
+    int n;
+    int tok[kMaxDraftWords];
 };
 
 // One sequence of a batched verify step: its rows [r0, r0 + M) of the launch, its committed length

@@ -30,8 +30,6 @@ struct Regions {
     size_t layer_stride, staging_bytes, raw_kmax;
 };
 
-constexpr int kMaxGrid = 256;  // per-block candidate arrays are sized for this many blocks
-
 bool config_ok(const sdv_config* c) {
     if (!c) return false;
     if (c->n_layers < 1 || c->d_model < 64 || c->d_model % 64 || c->d_ffn < 64 || c->d_ffn % 64) return false;
@@ -299,7 +297,7 @@ int cuda_fail(sdv_ctx* ctx, cudaError_t e) {
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_); \
     } while (0)
 
-typedef void (*ForwardKernel)(const FwdParams);
+typedef void (*ForwardKernel)(const FwdParams, const DraftArg);
 // The forward kernel compiled for this launch's head dimension and kind of attention.
 ForwardKernel forward_kernel(const FwdParams& P) {
     const int mode = P.nseq > 0 ? 2 : (P.tree ? 1 : 0);
@@ -307,11 +305,21 @@ ForwardKernel forward_kernel(const FwdParams& P) {
                                               {sdv_forward_kernel<128, 0>, sdv_forward_kernel<128, 1>, sdv_forward_kernel<128, 2>}};
     return table[P.hd == 128][mode];
 }
-cudaError_t launch_kernel(const FwdParams& P, cudaStream_t stream) {
+cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_t stream) {
     const ForwardKernel k = forward_kernel(P);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    static std::atomic<unsigned long long> sized[2][3];   // bit: the kernel may use all shared memory on that device
+    std::atomic<unsigned long long>& done = sized[P.hd == 128][P.nseq > 0 ? 2 : (P.tree ? 1 : 0)];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    void* args[] = {(void*)&P};
+    if (dev >= 64 || !(done.load(std::memory_order_relaxed) >> dev & 1ull)) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) done.fetch_or(1ull << dev, std::memory_order_relaxed);
+    }
+    DraftArg none;
+    none.n = -1;
+    void* args[] = {(void*)&P, (void*)(draft ? draft : &none)};
     // phases meet at grid barriers, so more than one phase needs all blocks co-resident
     if (P.ph_end - P.ph_begin > 1)
         return cudaLaunchCooperativeKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
@@ -355,11 +363,12 @@ struct BatchPlan {
     BatchSeq seq[kMaxBatch];
 };
 int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph_end, bool timed, bool force_logits = false,
-                   bool tree = false, const BatchPlan* batch = nullptr, bool l_from_state = false, cudaEvent_t* run_ev = nullptr) {
+                   bool tree = false, const BatchPlan* batch = nullptr, bool l_from_state = false, cudaEvent_t* run_ev = nullptr,
+                   const DraftArg* draft = nullptr) {
     FwdParams P = ctx->P;
     P.l_from_state = l_from_state ? 1 : 0;
     const bool raw_only = (ph_begin == 2 + kPhasesPerLayer * ctx->cfg.n_layers);
-    P.rows_from_state = (mode == 0 && !batch) ? 1 : 0;
+    P.rows_from_state = (mode == 0 && !batch && !draft) ? 1 : 0;
     P.L = L;
     P.att_gh = P.g < 1 ? 1 : plan_attention(P, batch ? batch->max_rows : rows, L, batch ? batch->n : 1);
     if (P.rows_from_state)   // for every number of rows the draft may turn out to have
@@ -382,7 +391,7 @@ int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph
     const int nbar = ph_end - ph_begin - 1;
     ctx->bar_base += (unsigned)(nbar * ctx->G);
     if (timed) CK(cudaEventRecord(run_ev ? run_ev[0] : ctx->ev0, ctx->stream));
-    cudaError_t e = launch_kernel(P, ctx->stream);
+    cudaError_t e = launch_kernel(P, draft, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     ctx->launches++;
     if (timed) {
@@ -392,8 +401,9 @@ int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph
     return SDV_OK;
 }
 
-int read_state(sdv_ctx* ctx) {
-    CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + ctx->r.state, ST_WORDS * 4, cudaMemcpyDeviceToHost, ctx->stream));
+// `published`: the last kernel has written the state block to the page-locked copy itself.
+int read_state(sdv_ctx* ctx, bool published = false) {
+    if (!published) CK(cudaMemcpyAsync(ctx->pinned, ctx->ws + ctx->r.state, ST_WORDS * 4, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (ctx->pinned[ST_ERR] == 1) {
         ctx->poisoned = true;
@@ -430,10 +440,10 @@ int commit_common(sdv_ctx* ctx, int max_emit, int force_accept, int force_token,
         ctx->launches++;
         ctx->tree_verified = false;
     }
-    commit_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, hist, max_emit, force_accept, force_token, 0);
+    commit_kernel<<<1, 64, 0, ctx->stream>>>(ctx->P.state, hist, max_emit, force_accept, force_token, 0, ctx->pinned);
     ctx->launches++;
     CK(cudaGetLastError());
-    int rc = read_state(ctx);
+    int rc = read_state(ctx, true);
     if (rc) return rc;
     const int n = ctx->pinned[ST_N_EMITTED];
     ctx->kv_len = ctx->pinned[ST_KV_LEN];
@@ -1029,7 +1039,8 @@ int sdv_draft(sdv_ctx* ctx, int k, int32_t* host_draft, int* draft_len) {
     if (!ctx->prefill_done) return SDV_ESTATE;
     int* hist = (int*)(ctx->ws + ctx->r.hist);
     ngram_draft_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->P.state, hist, (const int*)(ctx->ws + ctx->r.db), ctx->cfg.ngram_n,
-                                                    ctx->cfg.ngram_min, k, ctx->cfg.search_history, 0);
+                                                    ctx->cfg.ngram_min, k, ctx->cfg.search_history, 0,
+                                                    host_draft || draft_len ? ctx->pinned : nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->draft_pending = true;
@@ -1037,7 +1048,7 @@ int sdv_draft(sdv_ctx* ctx, int k, int32_t* host_draft, int* draft_len) {
     ctx->draft_k = k;
     ctx->verified = false;
     if (host_draft || draft_len) {
-        int rc = read_state(ctx);
+        int rc = read_state(ctx, true);
         if (rc) return rc;
         const int dl = ctx->pinned[ST_DRAFT_LEN];
         if (draft_len) *draft_len = dl;
@@ -1062,24 +1073,21 @@ int sdv_verify(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int32_t* 
         rows = ctx->draft_pending ? ctx->draft_k + 1 : 1;
     }
     if (ctx->kv_len + rows > c.max_seq) return SDV_ECAPACITY;
-    if (host_draft) {
-        DraftArg a;
-        fill_draft_arg(a, host_draft, draft_len);
-        set_draft_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, a);
-        ctx->launches++;
-        CK(cudaGetLastError());
-    }
-    const bool tree = !host_draft && ctx->tree_pending;
-    int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, tree);
+    DraftArg a;
+    if (host_draft) fill_draft_arg(a, host_draft, draft_len);
+    const bool tree = !host_draft && ctx->tree_pending, fetch = host_y || accept_len;
+    int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, tree, nullptr, false, nullptr,
+                            host_draft ? &a : nullptr);
     if (rc) return rc;
-    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0);
+    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0,
+                                                    fetch ? ctx->pinned : nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->verified = true;
     ctx->tree_verified = tree;
     ctx->last_rows = rows;
-    if (host_y || accept_len) {
-        rc = read_state(ctx);
+    if (fetch) {
+        rc = read_state(ctx, true);
         if (rc) return rc;
         const int dl = ctx->pinned[ST_DRAFT_LEN];
         if (accept_len) *accept_len = ctx->pinned[ST_ACCEPT_LEN];
@@ -1130,7 +1138,7 @@ int sdv_verify_batch(sdv_ctx* const* ctxs, int n, int* accept_len) {
     for (int b = 0; b < n; ++b) {
         sdv_ctx* c = ctxs[b];
         accept_kernel<<<1, 32 * bp.seq[b].M, 0, ctx->stream>>>(c->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, bp.seq[b].r0,
-                                                              bstate, 0);
+                                                              bstate, 0, accept_len ? c->pinned : nullptr);
         ctx->launches++;
         c->verified = true;
         c->tree_verified = false;
@@ -1141,7 +1149,7 @@ int sdv_verify_batch(sdv_ctx* const* ctxs, int n, int* accept_len) {
     if (accept_len) {
         for (int b = 0; b < n; ++b) {
             sdv_ctx* c = ctxs[b];
-            rc = read_state(c);
+            rc = read_state(c, true);
             if (rc) return rc;
             accept_len[b] = c->pinned[ST_ACCEPT_LEN];
         }
@@ -1232,16 +1240,13 @@ int sdv_step(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int k_next,
     if (ctx->kv_len + rows > c.max_seq || ctx->hist_len + rows > c.max_seq + 64) return SDV_ECAPACITY;
     int* state = ctx->P.state;
     int* hist = (int*)(ctx->ws + ctx->r.hist);
-    if (host_draft) {
-        DraftArg a;
-        fill_draft_arg(a, host_draft, draft_len);
-        set_draft_kernel<<<1, 32, 0, ctx->stream>>>(state, a);
-        ctx->launches++;
-    }
-    int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true);
+    DraftArg a;
+    if (host_draft) fill_draft_arg(a, host_draft, draft_len);
+    int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, false, nullptr, false, nullptr,
+                            host_draft ? &a : nullptr);
     if (rc) return rc;
     step_tail_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, (const int*)(ctx->ws + ctx->r.db), ctx->P.cand_val, ctx->P.cand_idx,
-                                                  ctx->G, c.ngram_n, c.ngram_min, k_next, c.search_history, 0, 0, k_next > 0 ? 1 : 0, 0);
+                                                  ctx->G, c.ngram_n, c.ngram_min, k_next, c.search_history, 0, 0, k_next > 0 ? 1 : 0, 0, ctx->pinned);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->last_rows = rows;
@@ -1250,7 +1255,7 @@ int sdv_step(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int k_next,
     ctx->tree_verified = false;
     ctx->draft_pending = k_next > 0;
     ctx->draft_k = k_next;
-    rc = read_state(ctx);  // one copy of the state block: emitted tokens, lengths and the next draft
+    rc = read_state(ctx, true);  // the tail kernel wrote the state block to the host: emitted tokens, lengths and the next draft
     if (rc) return rc;
     const int n = ctx->pinned[ST_N_EMITTED];
     ctx->kv_len = ctx->pinned[ST_KV_LEN];
@@ -1290,7 +1295,7 @@ int sdv_decode_steps(sdv_ctx* ctx, int k, int n_steps, int max_tokens, int ext_m
     const int hist_before = ctx->hist_len;
     fill_i32_kernel<<<1, 32, 0, ctx->stream>>>(state + ST_BUDGET, max_tokens > 0 ? max_tokens : -1, 1);
     const int* db = (const int*)(ctx->ws + ctx->r.db);
-    ngram_draft_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, db, c.ngram_n, c.ngram_min, k, c.search_history, 1);
+    ngram_draft_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, db, c.ngram_n, c.ngram_min, k, c.search_history, 1, nullptr);
     if (ext_max_total > 0) extend_draft_kernel<<<1, 32, 0, ctx->stream>>>(state, ext_max_total, 1);
     ctx->launches += ext_max_total > 0 ? 3 : 2;
     const int all_phases = 2 + kPhasesPerLayer * c.n_layers;
@@ -1302,7 +1307,7 @@ int sdv_decode_steps(sdv_ctx* ctx, int k, int n_steps, int max_tokens, int ext_m
         // accept, commit and the next step's draft in one launch
         step_tail_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, db, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, c.ngram_n,
                                                       c.ngram_min, k, c.search_history, ext_max_total, ext_max_life,
-                                                      i + 1 < n_steps ? 1 : 0, 1);
+                                                      i + 1 < n_steps ? 1 : 0, 1, nullptr);
         ctx->launches++;
     }
     CK(cudaGetLastError());
@@ -1359,14 +1364,15 @@ int sdv_draft_tree(sdv_ctx* ctx, int k, int max_nodes, int32_t* host_tokens, int
     int* hist = (int*)(ctx->ws + ctx->r.hist);
     if (k > 0) {
         ngram_draft_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->P.state, hist, (const int*)(ctx->ws + ctx->r.db), ctx->cfg.ngram_n,
-                                                        ctx->cfg.ngram_min, k, ctx->cfg.search_history, 0);
+                                                        ctx->cfg.ngram_min, k, ctx->cfg.search_history, 0, nullptr);
     } else {
         DraftArg none;
         fill_draft_arg(none, nullptr, 0);
         set_draft_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, none);
     }
     tree_draft_kernel<<<1, 1024, 0, ctx->stream>>>(ctx->P.state, hist, (const int*)(ctx->ws + ctx->r.succ),
-                                                   (const int*)(ctx->ws + ctx->r.occ), ctx->calibrated ? ctx->calib_b : 0, max_nodes);
+                                                   (const int*)(ctx->ws + ctx->r.occ), ctx->calibrated ? ctx->calib_b : 0, max_nodes,
+                                                   host_tokens || host_parent || n_nodes ? ctx->pinned : nullptr);
     ctx->launches += 2;
     CK(cudaGetLastError());
     ctx->draft_pending = true;
@@ -1374,7 +1380,7 @@ int sdv_draft_tree(sdv_ctx* ctx, int k, int max_nodes, int32_t* host_tokens, int
     ctx->draft_k = max_nodes;   // rows of the next verify: the bound, or the exact count when the caller reads it
     ctx->verified = false;
     if (host_tokens || host_parent || n_nodes) {
-        int rc = read_state(ctx);
+        int rc = read_state(ctx, true);
         if (rc) return rc;
         const int n = ctx->pinned[ST_DRAFT_LEN];
         ctx->draft_k = n;
@@ -1416,14 +1422,16 @@ int sdv_verify_tree(sdv_ctx* ctx, const int32_t* host_tokens, const int32_t* hos
     }
     int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, true);
     if (rc) return rc;
-    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0);
+    const bool fetch = host_y || host_path || path_len;
+    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0,
+                                                    fetch ? ctx->pinned : nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->verified = true;
     ctx->tree_verified = true;
     ctx->last_rows = rows;
-    if (host_y || host_path || path_len) {
-        rc = read_state(ctx);
+    if (fetch) {
+        rc = read_state(ctx, true);
         if (rc) return rc;
         const int n = ctx->pinned[ST_DRAFT_LEN], a = ctx->pinned[ST_PATH_LEN];
         if (path_len) *path_len = a;
@@ -1557,7 +1565,7 @@ int sdv_debug_accept(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, con
         ctx->launches++;
     }
     set_y_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, y);
-    accept_kernel<<<1, 32 * (draft_len + 1), 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 1, 0, nullptr, 0);
+    accept_kernel<<<1, 32 * (draft_len + 1), 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 1, 0, nullptr, 0, nullptr);
     ctx->launches += 2;
     CK(cudaGetLastError());
     ctx->verified = true;

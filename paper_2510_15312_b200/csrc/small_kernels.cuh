@@ -52,6 +52,23 @@ __global__ void fill_i32_kernel(int* p, int v, long long n) {
         p[i] = v;
 }
 
+// Runs `f` (all threads of the block) on a shared-memory copy of the state block, then writes the copy back and, with `host`
+// (page-locked memory), to the host as well.  The stages of a step are chains of single-word reads and writes: against
+// global memory a step's tail took 6.3 us, and the copy to the host 6 more.
+template <typename F>
+__device__ __forceinline__ void with_state(int* state, int* host, F f) {
+    __shared__ int copy[ST_WORDS];
+    for (int i = threadIdx.x; i < ST_WORDS; i += blockDim.x) copy[i] = state[i];
+    __syncthreads();
+    f(copy);
+    __syncthreads();
+    for (int i = threadIdx.x; i < ST_WORDS; i += blockDim.x) {
+        const int v = copy[i];
+        state[i] = v;
+        if (host) host[i] = v;
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // Retrieval drafter.  One block; thread p tests search position p: the length m(p) of the common
 // suffix of search[0..p] and the history (capped at n), then a block-wide maximum of (m(p), p)
@@ -128,19 +145,14 @@ __device__ __forceinline__ void ngram_draft_body(int* state, const int* hist, co
     }
 }
 __global__ void ngram_draft_kernel(int* state, const int* hist, const int* db, int n, int n_min, int k,
-                                   int search_history, int in_run) {
+                                   int search_history, int in_run, int* host) {
     if (in_run && state[ST_BUDGET] == 0) return;
-    ngram_draft_body(state, hist, db, n, n_min, k, search_history);
+    with_state(state, host, [&](int* st) { ngram_draft_body(st, hist, db, n, n_min, k, search_history); });
 }
 
 __global__ void set_word_kernel(int* state, int word, int value) {
     if (threadIdx.x == 0) state[word] = value;
 }
-
-struct DraftArg {
-    int n;
-    int tok[kMaxDraftWords];
-};
 
 // Caller-supplied drafts (by value: no host buffer has to outlive the call).
 __global__ void set_draft_kernel(int* state, DraftArg a) {
@@ -174,17 +186,19 @@ __device__ __forceinline__ void tree_finish(int* state, int n_nodes) {
 
 // Caller-supplied tree: tokens of the draft nodes and, for node i (1-based), the row it continues.
 __global__ void set_tree_kernel(int* state, DraftArg tok, DraftArg par) {
-    if ((int)threadIdx.x < tok.n) {
-        state[ST_DRAFT + threadIdx.x] = tok.tok[threadIdx.x];
-        state[ST_PARENT + 1 + threadIdx.x] = par.tok[threadIdx.x];
-    }
-    __syncwarp();
-    if (threadIdx.x == 0) {
-        state[ST_DRAFT_LEN] = tok.n;
-        state[ST_BASE_LEN] = tok.n;
-        state[ST_SEG_USED] = 0;
-        tree_finish(state, tok.n);
-    }
+    with_state(state, nullptr, [&](int* st) {
+        if ((int)threadIdx.x < tok.n) {
+            st[ST_DRAFT + threadIdx.x] = tok.tok[threadIdx.x];
+            st[ST_PARENT + 1 + threadIdx.x] = par.tok[threadIdx.x];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            st[ST_DRAFT_LEN] = tok.n;
+            st[ST_BASE_LEN] = tok.n;
+            st[ST_SEG_USED] = 0;
+            tree_finish(st, tok.n);
+        }
+    });
 }
 
 // In-context calibration, "Sample": the b best token ids of every logits row (largest logit first,
@@ -245,7 +259,7 @@ __global__ void anchor_search_kernel(const int* hist, int n_ctx, int b, const in
 // (two levels, depth first).  A token a node already has as a child is not added twice; at most
 // max_nodes draft nodes.  One block: all threads look for the latest position of T in the context,
 // one thread builds.
-__global__ void tree_draft_kernel(int* state, const int* hist, const int* succ, const int* occ, int b, int max_nodes) {
+__device__ __forceinline__ void tree_draft_body(int* state, const int* hist, const int* succ, const int* occ, int b, int max_nodes) {
     __shared__ int best_s[32];
     const int n_ctx = state[ST_N_CTX], T = state[ST_PENDING];
     int best = -1;
@@ -281,6 +295,9 @@ __global__ void tree_draft_kernel(int* state, const int* hist, const int* succ, 
     state[ST_BASE_LEN] = n;
     state[ST_SEG_USED] = 0;
     tree_finish(state, n);
+}
+__global__ void tree_draft_kernel(int* state, const int* hist, const int* succ, const int* occ, int b, int max_nodes, int* host) {
+    with_state(state, host, [&](int* st) { tree_draft_body(st, hist, succ, occ, b, max_nodes); });
 }
 
 // The accepted path given by the caller (teacher forcing in tests): emitted = its tokens + next_token.
@@ -414,11 +431,18 @@ __device__ __forceinline__ void accept_body(int* state, const float* cand_val, c
         } else {
             float bv = -CUDART_INF_F;
             bi = 0x7fffffff;
-            for (int c = lane; c < G; c += 32) {
-                const float v = cand_val[(size_t)c * kMaxRows + row0 + warp];
-                const int i = cand_idx[(size_t)c * kMaxRows + row0 + warp];
-                if (v > bv || (v == bv && i < bi)) { bv = v; bi = i; }
+            constexpr int PER = kMaxGrid / 32;   // candidates per lane, all loads in flight
+            float v[PER];
+            int id[PER];
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const size_t at = (size_t)min(lane + k * 32, G - 1) * kMaxRows + row0 + warp;   // past the last: the last again
+                v[k] = cand_val[at];
+                id[k] = cand_idx[at];
             }
+#pragma unroll
+            for (int k = 0; k < PER; ++k)
+                if (v[k] > bv || (v[k] == bv && id[k] < bi)) { bv = v[k]; bi = id[k]; }
             for (int off = 16; off; off >>= 1) {
                 const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
                 const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
@@ -458,9 +482,9 @@ __device__ __forceinline__ void accept_body(int* state, const float* cand_val, c
     }
 }
 __global__ void accept_kernel(int* state, const float* cand_val, const int* cand_idx, int G, int from_host_y, int row0,
-                              const int* launch_state, int in_run) {
+                              const int* launch_state, int in_run, int* host) {
     if (in_run && state[ST_BUDGET] == 0) return;
-    accept_body(state, cand_val, cand_idx, G, from_host_y, row0, launch_state);
+    with_state(state, host, [&](int* st) { accept_body(st, cand_val, cand_idx, G, from_host_y, row0, launch_state); });
 }
 
 // Batched verify: the token rows of up to kMaxBatch sequences (each its pending token, then its draft, token 0
@@ -520,8 +544,8 @@ __device__ __forceinline__ void commit_body(int* state, int* hist, int max_emit,
     state[ST_VERIFIED] = 0;
     state[ST_TREE_ON] = 0;
 }
-__global__ void commit_kernel(int* state, int* hist, int max_emit, int force_accept, int force_token, int in_run) {
-    commit_body(state, hist, max_emit, force_accept, force_token, in_run);
+__global__ void commit_kernel(int* state, int* hist, int max_emit, int force_accept, int force_token, int in_run, int* host) {
+    with_state(state, host, [&](int* st) { commit_body(st, hist, max_emit, force_accept, force_token, in_run); });
 }
 
 // Everything between two forward kernels (of a run of enqueued steps, or of sdv_step), in one launch of 1024 threads: the accept
@@ -530,22 +554,24 @@ __global__ void commit_kernel(int* state, int* hist, int max_emit, int force_acc
 // meet at block barriers: what one writes to the state block and the history, the next reads.
 __global__ void __launch_bounds__(1024) step_tail_kernel(int* state, int* hist, const int* db, const float* cand_val,
                                                          const int* cand_idx, int G, int n, int n_min, int k, int search_history,
-                                                         int ext_max_total, int ext_max_life, int draft_next, int in_run) {
+                                                         int ext_max_total, int ext_max_life, int draft_next, int in_run, int* host) {
     if (in_run && state[ST_BUDGET] == 0) return;   // enqueued behind the end of the run
-    accept_body(state, cand_val, cand_idx, G, 0, 0, nullptr);
-    __syncthreads();
-    if (ext_max_total > 0) {
-        if (threadIdx.x < 32) extension_update_body(state, ext_max_life);
+    with_state(state, host, [&](int* st) {
+        accept_body(st, cand_val, cand_idx, G, 0, 0, nullptr);
         __syncthreads();
-    }
-    commit_body(state, hist, 0, -1, 0, in_run);
-    __syncthreads();
-    if (!draft_next || (in_run && state[ST_BUDGET] == 0)) return;
-    ngram_draft_body(state, hist, db, n, n_min, k, search_history);
-    if (ext_max_total > 0) {
+        if (ext_max_total > 0) {
+            if (threadIdx.x < 32) extension_update_body(st, ext_max_life);
+            __syncthreads();
+        }
+        commit_body(st, hist, 0, -1, 0, in_run);
         __syncthreads();
-        if (threadIdx.x < 32) extend_draft_body(state, ext_max_total);
-    }
+        if (!draft_next || (in_run && st[ST_BUDGET] == 0)) return;
+        ngram_draft_body(st, hist, db, n, n_min, k, search_history);
+        if (ext_max_total > 0) {
+            __syncthreads();
+            if (threadIdx.x < 32) extend_draft_body(st, ext_max_total);
+        }
+    });
 }
 
 // After the last prefill tile: the greedy token of its last row becomes the pending token.
