@@ -904,12 +904,6 @@ __device__ __forceinline__ int attn_early_rows(const AttnUnit& u) {
     return old >= u.nkeys ? kKeyChunk : max(0, min(old, kKeyChunk));
 }
 
-// Power of two; results below the normal range become 0.
-__device__ __forceinline__ float ex2_ftz(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 // Sums over the warp of 16 columns: lane n receives column n & 15.
 __device__ __forceinline__ float warp_sum16(float (&v)[16], int lane) {
 #pragma unroll

@@ -543,7 +543,7 @@ template <int EPI, int BN>
 cudaError_t launch_dense_tiles(sdv_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, int splits, float* part,
                                __nv_bfloat16* out_bf16, int ld_bf16, DenseTopOut top) {
     const int tiles = ((M + 255) / 256) * ((N + BN - 1) / BN) * splits, pairs = ctx->G / 2;
-    return launch_dependent(ctx, dense_gemm_kernel<EPI, BN>, dim3(2 * (tiles < pairs ? tiles : pairs)), dim3(kDenseThreads),
+    return launch_dependent(ctx, dense_gemm_kernel<EPI, BN>, dim3(2 * (tiles < pairs ? tiles : pairs)), dim3(kDenseThreads<EPI>),
                             DenseShape<BN>::kSmemBytes, 0, a, b, M, N, K, splits, part, out_bf16, ld_bf16, top, ctx->P.state + ST_ERR,
                             2000000000ull);
 }
@@ -625,10 +625,11 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     if (succ) {
         DenseTopOut top;
         const int mt = (rows + 255) / 256, tiles = mt * ((c.vocab + 255) / 256), pairs = tiles < ctx->G / 2 ? tiles : ctx->G / 2;
+        const int shares = kDenseHalves<EPI_TOP> * (pairs / mt);
         top.val = part;
-        top.idx = (int*)(part + (size_t)rows * (pairs / mt) * kDenseTopMax);
+        top.idx = (int*)(part + (size_t)rows * shares * kDenseTopMax);
         CK((launch_dense_tiles<EPI_TOP, 256>(ctx, maps[MAP_XN], maps[MAP_LM], rows, c.vocab, d, 1, nullptr, nullptr, 0, top)));
-        CK(launch_dependent(ctx, dense_top_merge_kernel, dim3(rows), dim3(256), 0, 0, top, pairs / mt, ctx->calib_b, succ));
+        CK(launch_dependent(ctx, dense_top_merge_kernel, dim3(rows), dim3(256), 0, 0, top, shares, ctx->calib_b, succ));
     }
     CK(cudaGetLastError());
     return SDV_OK;
