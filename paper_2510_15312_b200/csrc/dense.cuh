@@ -409,20 +409,23 @@ __global__ void __launch_bounds__(256) dense_qkv_finish_kernel(const float* part
 // and running maximum in tensor memory and a warpgroup of its own (one tile row per thread): while one warpgroup
 // turns its scores into probabilities (written back over S as bf16, the A operand of P V), the tensor core works for the
 // other.  O is rescaled only when the maximum grew by more than 2^8 (the probabilities then stay below 2^8, the sums
-// are fp32).  The streams of all blocks of the cluster merge through distributed shared memory.  Output bf16 [M][n_q * hd].
-// Bound by the exponentials (16 per cycle and SM) and, over short contexts, by the chain load -> S -> softmax -> P V ->
-// merge.  mma.sync tiles, which this replaces, issue m16n8k16 every 16 cycles per scheduler on this part: 35 us a launch at the
-// 1.5B shape, mean over the eight 256-token chunks of a 2048-token request.
+// are fp32).  The blocks of a cluster merge their rows by bulk copies between their shared memories: each finishes an
+// even share of the tile rows and is sent the others' outputs of them, with maximum and sum behind every row.  (Reading
+// them by remote loads took 4 to 6 us of a launch, 13 bytes per cycle and SM.)  Output bf16 [M][n_q * hd].
+// Bound by the exponentials (16 per cycle and SM: 1.1 us per 128 keys of both streams) and, over short contexts, by the
+// chain load -> S -> softmax -> P V -> merge.  Mean over the eight 256-token chunks of a 2048-token request at the 1.5B
+// shape: 11.5 us a launch (14.3 with remote loads, 35 with mma.sync tiles); 7B 14.2 us (18.5).
 template <int HD>
 struct DenseAttShape {
     static constexpr int kAtoms = HD / 64;                       // 64-column swizzled slabs of a row
     static constexpr int kTileBytes = 128 * HD * 2;              // queries, or the keys or values of a block
     static constexpr int kStages = 3;
-    static constexpr int kLdo = HD + 4;                          // row stride (floats) of the exchange area
+    static constexpr int kLdo = HD + 4;                          // floats of an exchanged row: output, maximum in log2 units, sum, padding
     static constexpr int kExBytes = 128 * kLdo * 4;              // the block's outputs
     static constexpr int kRing = kStages * 2 * kTileBytes;
+    static constexpr int kInBytes = (128 + 8) * kLdo * 4;        // the other blocks' outputs for this block's rows (up to eight shares, rounded up)
     static constexpr int kSmemBytes = kTileBytes + kRing + 256 + 1024;
-    static_assert(kExBytes <= kRing, "the exchange area reuses the ring");
+    static_assert(kExBytes + kInBytes <= kRing, "the exchange areas reuse the ring");
 };
 constexpr int kDenseAttThreads = 320;   // warps 0..3 and 4..7: the two streams; 8: copies; 9: tensor-core issue
 
@@ -436,9 +439,9 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
     extern __shared__ uint8_t att_smem_raw[];
     uint8_t* Qs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* ring = Qs + S::kTileBytes;                                  // [stage][K | V]
-    float2* ex_ml = reinterpret_cast<float2*>(Qs);   // once the products are done: [stream 0, stream 1, both][tile row] (maximum in log2 units, sum)
+    float2* ex_ml = reinterpret_cast<float2*>(Qs);   // once the products are done: [stream][tile row] (maximum in log2 units, sum)
     struct Ctl {
-        uint64_t kfull[S::kStages], vfull[S::kStages], empty[S::kStages], s_full[2], p_ready[2], o_full;
+        uint64_t kfull[S::kStages], vfull[S::kStages], empty[S::kStages], s_full[2], p_ready[2], o_full, in_full;
         uint32_t tmem_base;
         int abort_flag;
     };
@@ -450,6 +453,7 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
     const int nkeys = L + min(M, q0 + QR);                              // keys any row of this block may see
     const int nblk_all = (nkeys + 127) / 128;
     const int b0 = even_start(nblk_all, CS, rank), nblk = even_count(nblk_all, CS, rank);
+    const int R = min(QR, M - q0) * g, rbeg = even_start(R, CS, rank), rows = even_count(R, CS, rank);   // tile rows; those this block finishes
     if (tid == 0) {
         for (int s = 0; s < S::kStages; ++s) {
             mbar_init(&ctl->kfull[s], 1);
@@ -461,8 +465,10 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
             mbar_init(&ctl->p_ready[w], 4);
         }
         mbar_init(&ctl->o_full, 1);
+        mbar_init(&ctl->in_full, 1);
         ctl->abort_flag = 0;
         mbar_fence_init();
+        mbar_arrive_expect_tx(&ctl->in_full, (uint32_t)((CS - 1) * rows * S::kLdo * 4));
     }
     if (warp == 9) tmem_alloc(&ctl->tmem_base, 512);   // S0 | S1 | O0 | O1, 128 columns each
     tc_fence_before();
@@ -470,18 +476,19 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
     grid_dep_launch();
+    constexpr int QI = 128 * UNITS / 256;   // 16-byte units of the query tile per thread
+    int qoff[QI];                           // where they are, -1: a row without a query (worked out while the kernel before runs)
+#pragma unroll
+    for (int i = 0; i < QI; ++i) {
+        const int u = tid + i * 256, t = u / UNITS, qi = q0 + t / g;
+        qoff[i] = t < QR * g && qi < M ? qi * (n_q * HD) + (kvh * g + t % g) * HD + (u % UNITS) * 8 : -1;
+    }
     grid_dep_wait();
     if (warp < 8) {
-        // query tile, in the layout the copies have: slabs of 64 columns, 128-byte swizzle
-        constexpr int QI = 128 * UNITS / 256;   // 16-byte units per thread, all loads in flight
+        // query tile, in the layout the copies have: slabs of 64 columns, 128-byte swizzle; all loads in flight
         uint4 v[QI];
 #pragma unroll
-        for (int i = 0; i < QI; ++i) {
-            const int u = tid + i * 256, t = u / UNITS, qi = q0 + t / g;
-            v[i] = make_uint4(0, 0, 0, 0);
-            if (t < QR * g && qi < M)
-                v[i] = __ldcg(reinterpret_cast<const uint4*>(q + (size_t)qi * (n_q * HD) + (kvh * g + t % g) * HD + (u % UNITS) * 8));
-        }
+        for (int i = 0; i < QI; ++i) v[i] = qoff[i] < 0 ? make_uint4(0, 0, 0, 0) : __ldcg(reinterpret_cast<const uint4*>(q + qoff[i]));
 #pragma unroll
         for (int i = 0; i < QI; ++i) {
             const int u = tid + i * 256, c16 = u % UNITS;
@@ -639,6 +646,7 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
         ok = __all_sync(0xffffffffu, ok);
         ex_ml[w * 128 + t] = ok ? make_float2(m, l) : make_float2(-CUDART_INF_F, 0.f);
         named_bar_sync(1, 256);
+        if (CS > 1) cluster_arrive();   // nothing reads this block's ring any more
         const float2 o0 = ex_ml[t], o1 = ex_ml[128 + t];
         const float mx = fmaxf(o0.x, o1.x), ref = mx == -CUDART_INF_F ? 0.f : mx;
         const float w0 = exp2f(o0.x - ref), w1 = exp2f(o1.x - ref);
@@ -646,8 +654,8 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
         const float sc = CS == 1 ? 1.f / sum : 1.f;   // a block that saw all keys writes the result itself
         const int qi = q0 + t / g;
         __nv_bfloat16* po = out + (size_t)qi * (n_q * HD) + (kvh * g + t % g) * HD;
-        if (w == 0) ex_ml[256 + t] = make_float2(mx, sum);
         float* ex = reinterpret_cast<float*>(ring) + t * S::kLdo;
+        if (w == 0 && CS > 1) *reinterpret_cast<float2*>(ex + HD) = make_float2(mx, sum);
         if (nblk > 0 && ok) {
             tc_fence_after();
 #pragma unroll 1
@@ -671,60 +679,57 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
             }
         }
         tc_fence_before();
+        fence_proxy_async_smem();
     }
     __syncwarp();
-    cluster_sync();
-    if (warp == 9) tmem_dealloc(tmem, 512);
     if (CS > 1) {
-        // every block merges its share of the tile rows from the cluster's CS partial results: first the rows' weights, one
-        // remote load per row and block, then the outputs with all loads of an item in flight (remote shared memory gives
-        // about 13 bytes per cycle and SM, so the fewer partial results the better)
-        const uint32_t base_o = smem_u32(ring), base_ml = smem_u32(ex_ml + 256);
-        constexpr int C8 = HD / 8, NP = 8;
-        const int R = min(QR, M - q0) * g;
-        const int rbeg = even_start(R, CS, rank), rows = even_count(R, CS, rank);
-        float* wt = reinterpret_cast<float*>(Qs + 4096);   // [own row][8], behind the statistics
-        for (int it = tid; it < rows * NP; it += kDenseAttThreads) {   // 8 lanes share a row
-            const int t = rbeg + it / NP, k = it % NP;
-            float2 ml = make_float2(-CUDART_INF_F, 0.f);
-            if (k < CS) ml = ld_cluster_f2(map_shared_rank(base_ml + t * 8, k));
-            const unsigned mask = 0xffu << (lane & 24);
-            float mx = ml.x;
-#pragma unroll
-            for (int off = 4; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(mask, mx, off));
-            const float e = exp2f(ml.x - mx);
-            float sum = e * ml.y;
-#pragma unroll
-            for (int off = 4; off; off >>= 1) sum += __shfl_xor_sync(mask, sum, off);
-            wt[it] = e / sum;
-        }
-        __syncthreads();
+        if (warp >= 8) cluster_arrive();
+        cluster_wait();
+    }
+    __syncthreads();
+    if (warp == 9) tmem_dealloc(tmem, 512);
+    if (CS == 1) {
+        if (tid == 0 && ctl->abort_flag) atomicExch(err, 1);
+        return;
+    }
+    // every block finishes its share of the tile rows: the others send it their outputs and statistics of them
+    const uint32_t ex = smem_u32(ring), in = ex + S::kExBytes;
+    constexpr uint32_t kRowBytes = S::kLdo * 4;
+    if (tid < CS && tid != rank) {
+        const int n = even_count(R, CS, tid);
+        if (n) bulk_s2cluster(map_shared_rank(in + (uint32_t)(rank * n) * kRowBytes, tid), ex + (uint32_t)even_start(R, CS, tid) * kRowBytes,
+                              (uint32_t)n * kRowBytes, map_shared_rank(smem_u32(&ctl->in_full), tid));
+    }
+    __syncwarp();
+    const bool got = mbar_wait_bounded(&ctl->in_full, 0, &ctl->abort_flag, wait_limit_ns);
+    __syncwarp();
+    cluster_arrive();   // what was sent to this block has left its senders
+    if (got) {
+        constexpr int C8 = HD / 8;
         for (int it = tid; it < rows * C8; it += kDenseAttThreads) {
-            const int t = rbeg + it / C8, c = (it % C8) * 8;
+            const int i = it / C8, t = rbeg + i, c = (it % C8) * 8;
+            auto part = [&](int k) {
+                return reinterpret_cast<const float*>(k == rank ? ring + t * kRowBytes : ring + S::kExBytes + (k * rows + i) * kRowBytes);
+            };
+            float mx = -CUDART_INF_F, sum = 0.f;
+            for (int k = 0; k < CS; ++k) mx = fmaxf(mx, part(k)[HD]);
             float o[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            for (int k0 = 0; k0 < CS; k0 += 4) {   // four partial results' loads in flight (past the last: the last again)
-                float4 x[4], y[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int k = min(k0 + i, CS - 1);
-                    const uint32_t src = map_shared_rank(base_o + (t * S::kLdo + c) * 4, k);
-                    x[i] = ld_cluster_f4(src);
-                    y[i] = ld_cluster_f4(src + 16);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float w = k0 + i < CS ? wt[(it / C8) * NP + k0 + i] : 0.f;
-                    const bool use = w > 0.f;   // a block without a key never wrote its area
-                    o[0] += use ? w * x[i].x : 0.f; o[1] += use ? w * x[i].y : 0.f; o[2] += use ? w * x[i].z : 0.f; o[3] += use ? w * x[i].w : 0.f;
-                    o[4] += use ? w * y[i].x : 0.f; o[5] += use ? w * y[i].y : 0.f; o[6] += use ? w * y[i].z : 0.f; o[7] += use ? w * y[i].w : 0.f;
-                }
+            for (int k = 0; k < CS; ++k) {
+                const float* p = part(k);
+                if (p[HD] == -CUDART_INF_F) continue;   // a block without a key never wrote its outputs
+                const float w = exp2f(p[HD] - mx);
+                const float4 x = *reinterpret_cast<const float4*>(p + c), y = *reinterpret_cast<const float4*>(p + c + 4);
+                sum += w * p[HD + 1];
+                o[0] += w * x.x; o[1] += w * x.y; o[2] += w * x.z; o[3] += w * x.w;
+                o[4] += w * y.x; o[5] += w * y.y; o[6] += w * y.z; o[7] += w * y.w;
             }
+            const float sc = 1.f / sum;
             *reinterpret_cast<uint4*>(out + (size_t)(q0 + t / g) * (n_q * HD) + (kvh * g + t % g) * HD + c) =
-                make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
+                make_uint4(pack_bf16(o[0] * sc, o[1] * sc), pack_bf16(o[2] * sc, o[3] * sc), pack_bf16(o[4] * sc, o[5] * sc), pack_bf16(o[6] * sc, o[7] * sc));
         }
     }
     __syncwarp();
-    cluster_sync();   // no block leaves while another still reads its shared memory
+    cluster_wait();   // and what this block sent has left
     if (tid == 0 && ctl->abort_flag) atomicExch(err, 1);
 }
 
