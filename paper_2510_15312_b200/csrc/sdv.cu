@@ -590,9 +590,14 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     const float* bias = ctx->P.bias;
     const int g = ctx->P.g;
     CK(dense_attributes());
-    // rows of four columns per thread
-    int nt = (d / 4 + 31) / 32 * 32;
+    // rows: four columns per thread and turn
+    const int turns = d <= 2048 ? 1 : d <= 4096 ? 2 : 4;
+    int nt = ((turns <= 2 ? d / 4 / turns : d / 4) + 31) / 32 * 32;
     if (nt > 1024) nt = 1024;
+    const auto norm_kernel = turns == 1 ? dense_residual_norm_kernel<1> : turns == 2 ? dense_residual_norm_kernel<2> : dense_residual_norm_kernel<4>;
+    // four rotary pairs per thread, q|k|v of a row in one turn where a block can hold them
+    int ft = (nqkv / 8 + 31) / 32 * 32;
+    if (ft > 1024) ft = 1024;
     // attention: the queries whose g heads fill a 128-row tile; key shares so that the blocks fill the chip once (clusters of
     // more than two leave some SMs of a group of 18 or 20 unused, hence 7/8) and keep two blocks of 128 keys each, one per stream
     const int QR = 128 / g, qtiles = (rows + QR - 1) / QR;
@@ -601,25 +606,25 @@ int dense_prefill_rows(sdv_ctx* ctx, int rows, int L, int* succ) {
     if (cs > (L + rows + 255) / 256) cs = (L + rows + 255) / 256;
     if (cs < 1) cs = 1;
     int splits = 0;
-    CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, hist + L, ctx->P.emb, c.vocab, h, part, 0, norm_w, xn, d,
+    CK(launch_dependent(ctx, norm_kernel, dim3(rows), dim3(nt), 0, 0, hist + L, ctx->P.emb, c.vocab, h, part, 0, norm_w, xn, d,
                         c.rms_eps, nullptr));
     for (int l = 0; l < c.n_layers; ++l) {
         const size_t layer_off = (size_t)l * c.n_kv_heads * c.max_seq * hd;
         const bool last = l + 1 == c.n_layers;
         CK(dense_product(ctx, MAP_XN, l, 0, rows, nqkv, d, &splits));
-        CK(launch_dependent(ctx, dense_qkv_finish_kernel, dim3(rows), dim3(256), 0, 0, part, splits, bias ? bias + (size_t)l * nqkv : nullptr,
+        CK(launch_dependent(ctx, dense_qkv_finish_kernel, dim3(rows), dim3(ft), 0, 0, part, splits, bias ? bias + (size_t)l * nqkv : nullptr,
                             ctx->P.rope, q, c.n_q_heads, c.n_kv_heads, hd, ctx->P.kcache, ctx->P.vcache, layer_off, c.max_seq, L));
         CK(launch_dependent(ctx, hd == 128 ? dense_attention_kernel<128> : dense_attention_kernel<64>, dim3(qtiles * cs, c.n_kv_heads),
                             dim3(kDenseAttThreads), hd == 128 ? DenseAttShape<128>::kSmemBytes : DenseAttShape<64>::kSmemBytes, (unsigned)cs,
                             maps[MAP_K], maps[MAP_V], q, l * c.n_kv_heads * c.max_seq, c.max_seq, c.n_q_heads, g, QR, rows, L,
                             ctx->P.scale_log2e, att, ctx->P.state + ST_ERR, 2000000000ull));
         CK(dense_product(ctx, MAP_ATT, l, 1, rows, d, nq, &splits));
-        CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
+        CK(launch_dependent(ctx, norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
                             norm_w + (size_t)(2 * l + 1) * d, xn, d, c.rms_eps, nullptr));
         CK((launch_dense_tiles<EPI_SWIGLU, 256>(ctx, maps[MAP_XN], maps[map_at(l, 2, 256)], rows, 2 * f, d, 1, nullptr, act, f, DenseTopOut())));
         CK(dense_product(ctx, MAP_ACT, l, 3, rows, d, f, &splits));
         // the next layer's first norm, behind the last layer the final norm (norm_w holds them in this order)
-        CK(launch_dependent(ctx, dense_residual_norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
+        CK(launch_dependent(ctx, norm_kernel, dim3(rows), dim3(nt), 0, 0, nullptr, ctx->P.emb, c.vocab, h, part, splits,
                             norm_w + (size_t)(2 * l + 2) * d, xn, d, c.rms_eps, last ? ctx->P.h : nullptr));
     }
     if (succ) {
