@@ -244,9 +244,8 @@ def phase_timeline(s, cfg, k):
     out = [f"verify step of {k + 1} rows, KV length {s.kv_len()}, {cfg.name}: {prof_us:.1f} us with the per-phase stamps on",
            "", "| phase | launches of it | dur us (mean) | gap us (mean) | marks inside the phase, us after its start: first block / last block |",
            "|---|---|---|---|---|"]
-    legend = {"attention": ["loads issued", "Q tile and new rows ready", "first key block in place", "key loop done", "unit done"],
-              "default": ["token operand built", "tensor-core warp done issuing", "epilogue done", "reached the down projection",
-                          "SwiGLU operand complete"]}
+    legend = {"attention": ["unit begins", "queries and first keys in place", "first scores seen", "key loop done", "unit done"],
+              "default": ["token operand built", "tensor-core warp done issuing", "epilogue done", "gate and up issued"]}
     total = 0.0
     for nm, r in rows.items():
         lg = legend.get(nm, legend["default"])

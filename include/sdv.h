@@ -342,11 +342,11 @@ int sdv_debug_timeout_probe(sdv_ctx *ctx);
  * recorded, uint64 [n_phases][blocks][12] per thread block (phase 0 = embedding, then 4 per layer:
  * qkv, attention, o, gate|up + down; last = LM head).  Words 0, 1: phase work begin and end
  * (nanoseconds of the global timer).  GEMM phases: 2 token operand built, 3 last tensor-core
- * instruction issued, 4 epilogue done, 5 / 6 wait for the SwiGLU operand begins / ends (gate|up +
- * down only), 10 last accumulator seen complete by the epilogue (nanoseconds); 7, 8, 9 cycles the
- * tensor-core warp waited for weights, waited for a free accumulator, and spent in its loop.
- * Attention phase: 2 unit begins, 3 query tile built, 4 first key block in place, 5 key loop done,
- * 6 unit done, 7 whether the unit was a new-rows unit.  Then switches recording on or off for
+ * instruction issued, 4 epilogue done, 5 last instruction of gate|up issued (gate|up + down only), 10
+ * last accumulator seen complete by the epilogue (nanoseconds); 7, 8, 9 cycles the tensor-core
+ * thread waited for weights, waited for a free accumulator, and spent in its loop.
+ * Attention phase: 2 unit begins, 3 queries and first keys in place, 4 first scores seen, 5 key loop done,
+ * 6 unit done, 7 whether the unit is its head's last key range.  Then switches recording on or off for
  * later launches (it adds a block-wide barrier per phase, so timed runs keep it off).  Returns the
  * number of thread blocks, or an error. */
 int sdv_debug_profile(sdv_ctx *ctx, int on, unsigned long long *host_out, int n_phases);
@@ -355,8 +355,8 @@ int sdv_debug_profile(sdv_ctx *ctx, int on, unsigned long long *host_out, int n_
  * share of an operation the way the kernel does and checks that every 16-byte unit of the matrix
  * is met exactly once at the offset the packing step writes it to.  desc and gu_desc are
  * {row tiles, column steps, row partitions, column partitions, tiles per pass, steps per stage,
- * row granularity, follow flag}; gu_desc (the gate|up operation) is only read when the follow flag
- * of desc is set.  Returns SDV_OK, SDV_EINVAL for a malformed description, or a code <= -100. */
+ * row granularity, follow flag | slices of K stacked as rows << 8}; gu_desc (the gate|up operation) is only read when the follow flag
+ * (1) of desc is set.  Returns SDV_OK, SDV_EINVAL for a malformed description, or a code <= -100. */
 int sdv_debug_layout_check(const int *desc, const int *gu_desc, int n_blocks);
 
 /* Host-only: the work partition and the shared-memory plan a context of this configuration uses

@@ -9,13 +9,15 @@
 //   warp 10      one thread issues the tensor-core instructions (tcgen05.mma, M = 128 weight
 //                rows x N = 16 or 32 token rows x K = 16 per instruction): the streamed stage is the A
 //                operand, the token rows, resident in shared memory for the whole operation, the
-//                B operand; accumulators live in tensor memory (two buffers of two 128-row
-//                accumulators, so the next pass starts while the previous one is read out).
+//                B operand; accumulators live in tensor memory (four buffers, so the next passes run while one
+//                is read out).  A share of few weight rows (q|k|v) stacks slices of its K as rows.
 //   warps 0..7   read the accumulators back (tcgen05.ld) and run the fused epilogues: warps 0..3 the
 //                first accumulator of a pass, warps 4..7 the second (or, for passes of up to 128
-//                rows, alternate pairs of token columns of the one accumulator).
-//   warps 0..9   build the token operand at the start of an operation (RMSNorm scale, merge of the
-//                split-KV partial results, ...), run the attention step and meet the other blocks.
+//                rows, alternate pairs of token columns of the one accumulator).  The q|k|v epilogue finishes its
+//                rows: slices, norm, bias, rotary embedding, cache append.
+//   warps 0..9   build the token operand at the start of an operation (normalised rows, merge of the
+//                split-KV partial results, ...) and meet the other blocks; warps 0..7 are the softmax of the attention
+//                step, whose products (scores and outputs, keys on the M side) warp 9 issues.
 // A layer is four operations separated by a bounded grid barrier: QKV projection; attention;
 // output projection (+ residual); gate|up with SwiGLU followed, inside the same block and without
 // a barrier, by the slice of the down projection (+ residual) that consumes this block's SwiGLU

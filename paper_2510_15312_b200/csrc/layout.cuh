@@ -277,7 +277,7 @@ struct FwdParams {
 
 // Rows a column group of a token operand takes (`rows` token rows, K slices stacked).  An odd number spreads the groups over the
 // banks: with a multiple of 8 every 16-byte unit of a token row lies in the same four banks, and the build's stores (one row,
-// consecutive columns) take 16 turns instead of 2 (9.5 us of a layer's 55 at 32 rows of 1536 columns).
+// consecutive columns) take 16 turns instead of 2 (32 rows of 1536 columns: 8.6 -> 8.0 us a build).
 __host__ __device__ inline int operand_rows(const FwdParams& P, int rows, int slices) {
     const int n = rows * (slices > 1 ? slices : 1);
     return P.pad ? n | 1 : n;
