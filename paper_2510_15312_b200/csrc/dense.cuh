@@ -274,7 +274,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_leader(&ctl->acc_empty[buf]);  // this warp's part of the accumulator may be overwritten
+            if (lane == 0 && t + 2 * npairs < ntiles) mbar_arrive_leader(&ctl->acc_empty[buf]);  // this warp's part of the accumulator may be overwritten
         }
         if (EPI == EPI_TOP && pair < npairs) {
             const int row = (pair % mt) * 256 + (int)rank * 128 + q4 * 32 + lane;
@@ -287,7 +287,10 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     }
     __syncwarp();
     tc_fence_before();
-    cluster_sync();   // neither SM leaves while the other still reads its shared memory or signals its barriers
+    // Neither SM leaves while the other still reads its shared memory or signals its barriers.  Relaxed: all such accesses have been
+    // waited for (every arrival above has a later product behind it), and a release would wait for the outputs' stores.
+    cluster_arrive_relaxed();
+    cluster_wait();
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem, 512);
     if (threadIdx.x == 0 && ctl->abort_flag) atomicExch(err, 1);
