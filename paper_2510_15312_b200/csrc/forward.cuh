@@ -130,9 +130,13 @@ __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target
 // ------------------------------------------------------------------------------------------
 // Weight streamer (one thread).  The ring holds 128 KB of the 590 KB a layer of the 1.5B shape streams per block, and HBM
 // would idle through the attention half of a layer (24 us) once it is full.  So while the streamer waits for a free slot it reads
-// ahead into L2, at most kLookaheadBytes beyond the ring and no faster than one piece per kLookaheadCycles (1.5 TB/s over the
-// grid): a burst would queue in front of the other warps' loads, which cost more than it gave, the trickle does not.
+// ahead into L2, at most kLookaheadBytes beyond the ring and no faster than one piece per kLookaheadCycles or kLookaheadSlow
+// (4 or 2 TB/s over the grid if nothing else ran): a burst would queue in front of the other warps' loads, which cost more than it gave, the trickle does not.
 // 10050 -> 9680 us for eight steps of the 1.5B shape, 12130 -> 11970 us for four of the 7B shape; 128 KB: 9720, 256 KB: 9660.
+// The rate: where a layer is short the weights have to come during its waits.  Where the stream itself fills HBM (a block's share of a
+// layer above 2 MB), or the rows' operand builds are what a layer waits for (above 24 rows), the slower trickle disturbs less.
+// 600 against 1100 cycles: 1.5B shape 7570 / 7700 us for eight steps, 3B (17 rows) 7800 / 7860 for four; 7B 10880 / 10720, 27 rows of the
+// 1.5B shape 1452 / 1431 us a step.
 struct Lookahead {   // cursor over the block's weight stream: operation by operation, each one contiguous range of bytes
     int ph, oi;
     const uint8_t* src;
@@ -164,7 +168,8 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
     Lookahead la;
     la.ph = P.ph_begin; la.oi = -1; la.begin = la.end = 0; la.src = nullptr; la.bytes = la.first = 0;
     bool more = lookahead_next(P, misc, la);
-    long long last = clock64();
+    const uint32_t pause = P.M > 24 || P.layer_stride > (2ull << 20) * (unsigned)P.G ? kLookaheadSlow : kLookaheadCycles;
+    uint32_t last = (uint32_t)clock64();
 #pragma unroll 1
     for (int ph = P.ph_begin; ph < P.ph_end && ok; ++ph) {
         int layer, ops[2];
@@ -189,8 +194,8 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
                     uint64_t t0 = 0;
                     uint32_t spins = 0;
                     while (!mbar_test(&misc->empty[slot], par ^ 1u)) {
-                        const long long now = clock64();
-                        if (now - last > kLookaheadCycles && more) {
+                        const uint32_t now = (uint32_t)clock64();
+                        if (now - last > pause && more) {
                             if (ahead < streamed) ahead = streamed;
                             while (more && ahead >= la.end) more = lookahead_next(P, misc, la);
                             if (more && ahead < streamed + kLookaheadBytes) {
