@@ -128,8 +128,9 @@ int sdv_set_database(sdv_ctx *ctx, const int32_t *host_tokens, int n);
  * positions L..L+n, writing their KV rows speculatively, takes the greedy token y_{j+1} of
  * every row (lowest id wins ties) and the accept length a = number of leading x_i == y_i.
  * host_draft != NULL: verify these draft_len tokens (0 <= draft_len <= k_max).
- * host_draft == NULL: verify the draft left by the last sdv_draft (draft_len is ignored; k+1
- *   rows are computed, rows past the drafter's own draft length are padding and never accepted).
+ * host_draft == NULL: verify the draft left by the last sdv_draft (draft_len is ignored).  The kernel
+ *   takes the draft's length from the device and computes that many rows + 1; the host only knows the
+ *   bound of k + 1 rows, which the capacity check uses.
  * host_y (draft_len+1 ints; k_max+1 is always enough) and accept_len may be NULL; if either is
  * given the stream is synchronised.  Nothing is committed: L, T and the history are unchanged.
  * Errors: SDV_ESTATE before prefill has finished, SDV_ECAPACITY, SDV_EINVAL, SDV_ETIMEOUT. */
@@ -152,8 +153,8 @@ int sdv_step(sdv_ctx *ctx, const int32_t *host_draft, int draft_len, int k_next,
  * sdv_extend_draft(ext_max_total) when ext_max_total > 0] -> sdv_verify -> [sdv_extension_update(ext_max_life)]
  * -> sdv_commit on the context's stream; every kernel takes the KV length, history and drafts from the
  * device state the step before left, so nothing is read back until the run ends.  Each verify computes
- * k + 1 rows (ext_max_total + 1 with the extension; k <= ext_max_total <= k_max); between two forward kernels one
- * launch does the accept scan, the commit and the next draft.  max_tokens > 0 ends the
+ * its draft's length + 1 rows, at most `rows` = k + 1 (ext_max_total + 1 with the extension; k <= ext_max_total
+ * <= k_max); between two forward kernels one launch does the accept scan, the commit and the next draft.  max_tokens > 0 ends the
  * run after that many emitted tokens: the step that reaches it is cut like sdv_commit's max_emit and the
  * steps enqueued behind it do nothing (they cost a few microseconds each); max_tokens <= 0: no limit.
  * The emitted tokens equal those of the same calls made one by one.  host_tokens (room for
@@ -181,9 +182,11 @@ int sdv_run_kernel_ms(sdv_ctx *ctx, float *host_ms, int n);
  * itself a follower, alignment), SDV_ESTATE (leader without weights), SDV_ENOMEM, SDV_ECUDA.
  *
  * sdv_verify_batch: one verify step over ctxs[0..n) (1 <= n <= 8, distinct, a leader and followers of it
- * or followers of one leader).  Each sequence contributes the rows sdv_verify(ctx, NULL, ...) would
- * compute for it: its pending token and, after sdv_draft / sdv_extend_draft, its chain draft (k + 1 rows);
- * the rows of all sequences together may not exceed 32.  The decoder runs once over all rows, every row
+ * or followers of one leader).  Each sequence contributes its pending token and, after sdv_draft /
+ * sdv_extend_draft, as many rows as the host knows its chain draft may have tokens (k; max_total, or the exact
+ * length where the caller read the extended draft back): unlike sdv_verify(ctx, NULL, ...), rows past the
+ * draft are computed, as padding that is never accepted.  The rows of all sequences together may not
+ * exceed 32.  The decoder runs once over all rows, every row
  * attending to its own sequence's KV cache and earlier rows only, each sequence's KV rows are written
  * speculatively into its own cache, and the accept scan runs per sequence; afterwards every context
  * is in the state sdv_verify leaves it in (sdv_commit, sdv_extension_update, sdv_get_logits per context).
@@ -207,9 +210,9 @@ int sdv_verify_batch(sdv_ctx *const *ctxs, int n, int *accept_len);
  * sdv_extend_draft: call after sdv_draft.  Appends the retained segment to the device draft when
  * the result has at most max_total tokens (1 <= max_total <= k_max; the paper's threshold is 32
  * rows); a segment that does not fit is dropped, not cut.  host_draft (max_total ints) and
- * draft_len may be NULL; if either is given the stream is synchronised and the next sdv_verify
- * computes exactly draft_len + 1 rows, otherwise it computes max_total + 1 rows (rows past the
- * draft are padding and never accepted).
+ * draft_len may be NULL; if either is given the stream is synchronised.  The next sdv_verify computes
+ * the extended draft's length + 1 rows either way; without the read-back the host takes max_total + 1 as
+ * their bound (capacity; the rows of a batched step).
  *
  * sdv_extension_update: call after sdv_verify, before sdv_commit.  Among the drafts beyond the
  * reject point e = a + 1 it finds the longest run with x_i == y_i (Eq. 3; the earliest among
@@ -239,8 +242,9 @@ int sdv_extension_update(sdv_ctx *ctx, int max_life, int32_t *host_segment, int 
  * child of the root, followed at once by the successors of the position where that anchor was
  * matched (two levels, depth first).  A token a node already has as a child is not added twice.
  * Node i (1-based) continues row host_parent[i-1] < i, row 0 being T; host_tokens / host_parent
- * (k_max ints each) and n_nodes may be NULL; if any is given the stream is synchronised and the
- * next sdv_verify_tree computes exactly n_nodes + 1 rows, else max_nodes + 1.
+ * (k_max ints each) and n_nodes may be NULL; if any is given the stream is synchronised.  The next
+ * sdv_verify_tree computes n_nodes + 1 rows either way; without the read-back the host takes
+ * max_nodes + 1 as their bound for the capacity check.
  *
  * sdv_verify_tree: one forward pass over [T, nodes]: node i sits at position L + depth(i), its K/V
  * rows go to cache slot L + i, and it attends to the cache and to its own path from the root.
@@ -276,10 +280,12 @@ int sdv_rollback(sdv_ctx *ctx, int new_kv_len);
 int sdv_kv_len(const sdv_ctx *ctx);
 
 /* Parity mode: when on, every verify (and the last prefill chunk) also stores the fp32 logits of
- * all rows so that sdv_get_logits can return them.  Off by default (it adds rows x vocab x 4
- * bytes of writes per step). */
+ * its rows so that sdv_get_logits can return them, and a verify of the device's draft computes every row up
+ * to the host's bound, the ones past the draft with token 0 as padding (never accepted): k + 1 rows
+ * after sdv_draft.  Off by default (it adds those rows, and rows x vocab x 4 bytes of writes per step).
+ * sdv_get_logits: fp32 [rows][vocab] of the last verify; rows it did not compute are unspecified. */
 int sdv_set_parity_mode(sdv_ctx *ctx, int on);
-int sdv_get_logits(sdv_ctx *ctx, float *host_logits, int rows); /* [rows][vocab] of the last verify */
+int sdv_get_logits(sdv_ctx *ctx, float *host_logits, int rows);
 
 /* Frees the host-side structure; never touches the workspace. */
 int sdv_destroy(sdv_ctx *ctx);
@@ -319,10 +325,11 @@ int sdv_debug_force_commit_tree(sdv_ctx *ctx, const int32_t *host_path, int path
 int sdv_debug_top_successors(sdv_ctx *ctx, const float *host_logits, int rows, int top_b, int32_t *host_out);
 
 /* Copies rows [pos0, pos0+n) of one layer's key (which = 0) or value (which = 1) cache to the
- * host as fp32 [n_kv_heads][n][head_dim]. */
+ * host as fp32 [n_kv_heads][n][head_dim].  Rows behind the committed length are those of the last verify's rows,
+ * and beyond them whatever earlier steps left. */
 int sdv_debug_read_kv(sdv_ctx *ctx, int layer, int which, int pos0, int n, float *host_out);
 
-/* Copies the residual stream of the last forward pass, fp32 [rows][d_model]. */
+/* Copies the residual stream of the last forward pass, fp32 [rows][d_model]; rows it did not compute are zero. */
 int sdv_debug_read_hidden(sdv_ctx *ctx, int rows, float *host_out);
 
 /* Y[M][N] = X[M][K] * W[N][K]^T with the verify path's weight-streaming GEMM (bf16 operands, fp32

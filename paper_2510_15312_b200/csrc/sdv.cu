@@ -368,7 +368,9 @@ int launch_forward(sdv_ctx* ctx, int rows, int L, int mode, int ph_begin, int ph
     FwdParams P = ctx->P;
     P.l_from_state = l_from_state ? 1 : 0;
     const bool raw_only = (ph_begin == 2 + kPhasesPerLayer * ctx->cfg.n_layers);
-    P.rows_from_state = (mode == 0 && !batch && !draft) ? 1 : 0;
+    // A draft on the device may be shorter than `rows` allows: its own rows alone are computed.  In parity mode every row is, the
+    // padding (token 0) too, so that what is stored for the rows past the draft never dates from another step.
+    P.rows_from_state = (mode == 0 && !batch && !draft && !ctx->parity) ? 1 : 0;
     P.L = L;
     P.att_gh = P.g < 1 ? 1 : plan_attention(P, batch ? batch->max_rows : rows, L, batch ? batch->n : 1);
     if (P.rows_from_state)   // for every number of rows the draft may turn out to have

@@ -1,0 +1,57 @@
+"""Which rows of a verify step exist: a draft held on the device may be shorter than the bound the host knows.  What the
+read-back calls return for the rows past it."""
+import numpy as np
+import pytest
+
+from sdv_inputs import get_config, make_context, make_weights
+from paper_2510_15312_b200.binding import Sdv, config_from
+
+pytestmark = pytest.mark.gpu
+
+BOUND = 8              # drafts the host assumes
+AGAIN = 1e-2           # the same rows twice: partial sums meet in another order (fp32), a bf16 rounding behind them may flip
+
+
+@pytest.fixture(scope="module")
+def seq():
+    cfg = get_config("tiny")
+    ctx = make_context(cfg)
+    s = Sdv(config_from(cfg, k_max=24))
+    s.load_weights(make_weights(cfg))
+    for i in range(0, cfg.n_ctx, cfg.chunk):
+        s.prefill_chunk(ctx[i:i + cfg.chunk], is_last=i + cfg.chunk >= cfg.n_ctx)
+    yield s, cfg, s.kv_len()
+    s.close()
+
+
+def short_draft(s, tokens):
+    """A draft of these tokens on the device; the host only knows that it has at most BOUND."""
+    s.debug_set_draft(tokens)
+    s.extend_draft(BOUND, fetch=False)
+
+
+def rows_of(s, cfg, L):
+    return (s.get_logits(BOUND + 1), s.debug_read_hidden(BOUND + 1),
+            *[s.debug_read_kv(cfg.n_layers - 1, which, L, BOUND + 1) for which in (0, 1)])
+
+
+@pytest.mark.parametrize("n", [0, 3, BOUND])
+def test_parity_mode_stores_every_row_up_to_the_bound(seq, n):
+    """Rows past the draft are those of padding tokens 0, not what an earlier step left."""
+    s, cfg, L = seq
+    s.rollback(L)
+    s.set_parity_mode(True)
+    draft = [int(t) for t in np.random.default_rng(n).integers(1, cfg.vocab, n)]
+    s.verify(draft + [0] * (BOUND - n))
+    want = rows_of(s, cfg, L)
+    s.verify([7] * 24)                       # something else in every buffer
+    short_draft(s, draft)
+    y, a = s.verify(None)
+    for got, ref in zip(rows_of(s, cfg, L), want):
+        assert np.abs(got - ref).max() <= AGAIN * max(1.0, np.abs(ref).max())
+    s.set_parity_mode(False)                 # and without it the draft's own rows are the same
+    s.rollback(L)
+    short_draft(s, draft)
+    y2, a2 = s.verify(None)
+    assert list(y2[:n + 1]) == list(y[:n + 1]) and a2 == a
+    assert np.abs(s.debug_read_hidden(n + 1) - want[1][:n + 1]).max() <= AGAIN * max(1.0, np.abs(want[1]).max())
