@@ -313,11 +313,12 @@ int sdv_debug_set_draft(sdv_ctx *ctx, const int32_t *host_draft, int draft_len);
 int sdv_debug_accept(sdv_ctx *ctx, const int32_t *host_draft, int draft_len, const int32_t *host_y,
                      int *accept_len);
 
-/* Like sdv_commit, but with a caller-chosen accept length (<= draft_len of the last verify) and
- * next token: teacher forcing for step-by-step comparisons. */
+/* Like sdv_commit, but with a caller-chosen accept length (at most the length of the draft the last verify
+ * looked at, SDV_EINVAL beyond it) and next token: teacher forcing for step-by-step comparisons. */
 int sdv_debug_force_commit(sdv_ctx *ctx, int accept_len, int32_t next_token);
 
-/* The same after sdv_verify_tree: commits a caller-chosen accepted path (rows, ascending) and next token. */
+/* The same after sdv_verify_tree: commits a caller-chosen accepted path (rows of the tree's nodes,
+ * ascending) and next token. */
 int sdv_debug_force_commit_tree(sdv_ctx *ctx, const int32_t *host_path, int path_len, int32_t next_token);
 
 /* Runs the calibration's top-successor kernel on caller-supplied logits rows (host fp32 [rows][vocab],

@@ -414,6 +414,16 @@ int read_state(sdv_ctx* ctx, bool published = false) {
     return SDV_OK;
 }
 
+// Drafts (or tree nodes) of the outstanding verify step: what the device verified, which may be fewer than the host's bound
+// allowed for.  Their rows, and the pending token's, are the ones it computed.
+int verified_drafts(sdv_ctx* ctx, int* n) {
+    int rc = read_state(ctx);
+    if (rc) return rc;
+    const int dl = ctx->pinned[ST_DRAFT_LEN];
+    *n = dl < ctx->last_rows - 1 ? dl : ctx->last_rows - 1;
+    return SDV_OK;
+}
+
 int pack_op(sdv_ctx* ctx, const OpDesc& o, uint8_t* dst_base, const uint16_t* s0, int rows0, const uint16_t* s1,
             int rows1, const uint16_t* s2, int K, int mode, int t_begin, int t_end, int row_base) {
     const long long total = (long long)(t_end - t_begin) * 16 * (K / 8);
@@ -1455,9 +1465,13 @@ int sdv_debug_force_commit_tree(sdv_ctx* ctx, const int32_t* host_path, int path
     if (!ctx || path_len < 0 || (path_len && !host_path)) return SDV_EINVAL;
     if (ctx->poisoned) return SDV_ETIMEOUT;
     if (!ctx->verified || !ctx->tree_verified) return SDV_ESTATE;
-    if (path_len + 1 > ctx->last_rows || next_token < 0 || next_token >= ctx->cfg.vocab) return SDV_EINVAL;
+    if (next_token < 0 || next_token >= ctx->cfg.vocab) return SDV_EINVAL;
+    int nodes = 0;
+    int rc = verified_drafts(ctx, &nodes);
+    if (rc) return rc;
+    if (path_len > nodes) return SDV_EINVAL;
     for (int i = 0; i < path_len; ++i)
-        if (host_path[i] < 1 || host_path[i] >= ctx->last_rows || (i && host_path[i] <= host_path[i - 1])) return SDV_EINVAL;
+        if (host_path[i] < 1 || host_path[i] > nodes || (i && host_path[i] <= host_path[i - 1])) return SDV_EINVAL;
     DraftArg p;
     fill_draft_arg(p, host_path, path_len);
     set_path_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, p, next_token);
@@ -1477,8 +1491,11 @@ int sdv_debug_force_commit(sdv_ctx* ctx, int accept_len, int32_t next_token) {
     if (!ctx) return SDV_EINVAL;
     if (ctx->poisoned) return SDV_ETIMEOUT;
     if (!ctx->verified) return SDV_ESTATE;
-    if (accept_len < 0 || accept_len + 1 > ctx->last_rows || next_token < 0 || next_token >= ctx->cfg.vocab)
-        return SDV_EINVAL;
+    if (accept_len < 0 || next_token < 0 || next_token >= ctx->cfg.vocab) return SDV_EINVAL;
+    int drafts = 0;
+    int rc = verified_drafts(ctx, &drafts);
+    if (rc) return rc;
+    if (accept_len > drafts) return SDV_EINVAL;
     return commit_common(ctx, 0, accept_len, next_token, nullptr, nullptr, nullptr);
 }
 

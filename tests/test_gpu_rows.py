@@ -1,10 +1,10 @@
 """Which rows of a verify step exist: a draft held on the device may be shorter than the bound the host knows.  What the
-read-back calls return for the rows past it."""
+read-back calls return, and what the forced commits accept, for the rows past it."""
 import numpy as np
 import pytest
 
 from sdv_inputs import get_config, make_context, make_weights
-from paper_2510_15312_b200.binding import Sdv, config_from
+from paper_2510_15312_b200.binding import EINVAL, Sdv, SdvError, config_from
 
 pytestmark = pytest.mark.gpu
 
@@ -55,3 +55,30 @@ def test_parity_mode_stores_every_row_up_to_the_bound(seq, n):
     y2, a2 = s.verify(None)
     assert list(y2[:n + 1]) == list(y[:n + 1]) and a2 == a
     assert np.abs(s.debug_read_hidden(n + 1) - want[1][:n + 1]).max() <= AGAIN * max(1.0, np.abs(want[1]).max())
+
+
+@pytest.mark.parametrize("parity", [False, True])
+def test_forced_commits_stop_at_the_draft(seq, parity):
+    """No rows beyond the verified draft can be committed, whatever bound the host had for it."""
+    s, cfg, L = seq
+    s.rollback(L)
+    s.set_parity_mode(parity)
+    short_draft(s, [5, 6, 7])
+    s.verify(None, fetch=False)
+    for a in (4, BOUND, BOUND + 1):
+        with pytest.raises(SdvError) as e:
+            s.debug_force_commit(a, 9)
+        assert e.value.code == EINVAL
+    assert s.kv_len() == L
+    s.debug_force_commit(3, 9)
+    assert s.kv_len() == L + 4
+    s.rollback(L)
+    s.draft_tree(0, BOUND, fetch=False)      # no calibration: a tree of no nodes
+    s.verify_tree(fetch=False)
+    for path in ([1], [BOUND]):
+        with pytest.raises(SdvError) as e:
+            s.debug_force_commit_tree(path, 9)
+        assert e.value.code == EINVAL
+    s.debug_force_commit_tree([], 9)
+    assert s.kv_len() == L + 1
+    s.set_parity_mode(False)
