@@ -195,8 +195,8 @@ int sdv_run_kernel_ms(sdv_ctx *ctx, float *host_ms, int n);
  * Errors: SDV_EINVAL (count, duplicates, unrelated contexts, more than 32 rows), SDV_ESTATE (a sequence
  * before the end of prefill, or with a tree draft pending), SDV_ECAPACITY, SDV_ETIMEOUT. */
 /* Result of the outstanding verify step of one context (after sdv_verify, sdv_verify_tree or
- * sdv_verify_batch, before the commit): the greedy token of each of its rows into host_y (k_max + 1 ints
- * are always enough) and the accept length; either may be NULL.  Synchronises.  Errors: SDV_ESTATE when
+ * sdv_verify_batch, before the commit): the greedy tokens of the pending token's row and of each draft's
+ * into host_y (draft length + 1 ints; k_max + 1 are always enough) and the accept length; either may be NULL.  Synchronises.  Errors: SDV_ESTATE when
  * no verify result is outstanding, SDV_ETIMEOUT. */
 int sdv_get_verified(sdv_ctx *ctx, int32_t *host_y, int *accept_len);
 

@@ -1178,11 +1178,12 @@ int sdv_verify_batch(sdv_ctx* const* ctxs, int n, int* accept_len) {
 int sdv_get_verified(sdv_ctx* ctx, int32_t* host_y, int* accept_len) {
     if (!ctx) return SDV_EINVAL;
     if (!ctx->verified) return SDV_ESTATE;
-    int rc = read_state(ctx);
+    int drafts = 0;
+    int rc = verified_drafts(ctx, &drafts);
     if (rc) return rc;
     if (accept_len) *accept_len = ctx->pinned[ST_ACCEPT_LEN];
     if (host_y)
-        for (int i = 0; i < ctx->last_rows; ++i) host_y[i] = ctx->pinned[ST_Y + i];
+        for (int i = 0; i <= drafts; ++i) host_y[i] = ctx->pinned[ST_Y + i];
     return SDV_OK;
 }
 

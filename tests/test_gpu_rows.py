@@ -82,3 +82,14 @@ def test_forced_commits_stop_at_the_draft(seq, parity):
     s.debug_force_commit_tree([], 9)
     assert s.kv_len() == L + 1
     s.set_parity_mode(False)
+
+
+def test_verified_tokens_are_those_of_the_rows_that_exist(seq):
+    """sdv_get_verified writes draft length + 1 tokens, as sdv_verify does (the binding hands in zeros)."""
+    s, cfg, L = seq
+    s.rollback(L)
+    s.verify([7] * 24)
+    short_draft(s, [5, 6])
+    y, a = s.verify(None)
+    got, a2 = s.get_verified()
+    assert a2 == a and list(got[:3]) == list(y[:3]) and not got[3:].any()
