@@ -130,7 +130,8 @@ int sdv_set_database(sdv_ctx *ctx, const int32_t *host_tokens, int n);
  * host_draft != NULL: verify these draft_len tokens (0 <= draft_len <= k_max).
  * host_draft == NULL: verify the draft left by the last sdv_draft (draft_len is ignored).  The kernel
  *   takes the draft's length from the device and computes that many rows + 1; the host only knows the
- *   bound of k + 1 rows, which the capacity check uses.
+ *   bound of k + 1 rows, which the capacity check uses.  Without a draft since the last commit or rollback
+ *   the pending token's row runs alone; a draft that was handed in meanwhile has taken the drafter's place.
  * host_y (draft_len+1 ints; k_max+1 is always enough) and accept_len may be NULL; if either is
  * given the stream is synchronised.  Nothing is committed: L, T and the history are unchanged.
  * Errors: SDV_ESTATE before prefill has finished, SDV_ECAPACITY, SDV_EINVAL, SDV_ETIMEOUT. */

@@ -1091,16 +1091,19 @@ int sdv_verify(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int32_t* 
         rows = ctx->draft_pending ? ctx->draft_k + 1 : 1;
     }
     if (ctx->kv_len + rows > c.max_seq) return SDV_ECAPACITY;
+    // no draft at all: an empty one goes along, since the device may still hold the one of a verify before
+    const bool pass = host_draft || !ctx->draft_pending;
     DraftArg a;
-    if (host_draft) fill_draft_arg(a, host_draft, draft_len);
+    if (pass) fill_draft_arg(a, host_draft, host_draft ? draft_len : 0);
     const bool tree = !host_draft && ctx->tree_pending, fetch = host_y || accept_len;
     int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, tree, nullptr, false, nullptr,
-                            host_draft ? &a : nullptr);
+                            pass ? &a : nullptr);
     if (rc) return rc;
     accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0,
                                                     fetch ? ctx->pinned : nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
+    if (host_draft && ctx->draft_pending) ctx->draft_k = draft_len;   // it has taken the drafter's place on the device
     ctx->verified = true;
     ctx->tree_verified = tree;
     ctx->last_rows = rows;
@@ -1259,10 +1262,11 @@ int sdv_step(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int k_next,
     if (ctx->kv_len + rows > c.max_seq || ctx->hist_len + rows > c.max_seq + 64) return SDV_ECAPACITY;
     int* state = ctx->P.state;
     int* hist = (int*)(ctx->ws + ctx->r.hist);
+    const bool pass = host_draft || !ctx->draft_pending;   // as in sdv_verify
     DraftArg a;
-    if (host_draft) fill_draft_arg(a, host_draft, draft_len);
+    if (pass) fill_draft_arg(a, host_draft, host_draft ? draft_len : 0);
     int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, false, nullptr, false, nullptr,
-                            host_draft ? &a : nullptr);
+                            pass ? &a : nullptr);
     if (rc) return rc;
     step_tail_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, (const int*)(ctx->ws + ctx->r.db), ctx->P.cand_val, ctx->P.cand_idx,
                                                   ctx->G, c.ngram_n, c.ngram_min, k_next, c.search_history, 0, 0, k_next > 0 ? 1 : 0, 0, ctx->pinned);

@@ -422,7 +422,8 @@ __device__ __forceinline__ void accept_body(int* state, const float* cand_val, c
                                             int row0, const int* launch_state) {
     __shared__ int y_s[kMaxRows + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int dl = state[ST_DRAFT_LEN];
+    // a sequence that goes through a batched step without a draft of its own may hold one of a verify before: its row is there alone
+    const int dl = min(state[ST_DRAFT_LEN], (int)(blockDim.x >> 5) - 1);
     if (launch_state && threadIdx.x == 0 && launch_state[ST_ERR]) state[ST_ERR] = launch_state[ST_ERR];
     if (warp <= dl) {
         int bi;

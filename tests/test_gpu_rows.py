@@ -93,3 +93,31 @@ def test_verified_tokens_are_those_of_the_rows_that_exist(seq):
     y, a = s.verify(None)
     got, a2 = s.get_verified()
     assert a2 == a and list(got[:3]) == list(y[:3]) and not got[3:].any()
+
+
+def test_a_device_verify_behind_a_host_verify_looks_at_its_own_rows(seq):
+    """Without a draft of the device's own a step runs the pending token's row alone, whatever draft the verify before was
+    given; where there was one, the draft handed in has taken its place."""
+    s, cfg, L = seq
+    s.rollback(L)
+    y, _ = s.verify([])
+    story = [int(y[0])]
+    for _ in range(5):                       # the model's own continuation: accepted whole
+        y, a = s.verify(story)
+        assert a == len(story)
+        story.append(int(y[len(story)]))
+    s.rollback(L)
+    assert s.verify(story)[1] == len(story)
+    y, a = s.verify(None)
+    assert a == 0 and int(y[0]) == story[0]
+    assert s.commit()[0] == story[:1]
+    s.rollback(L)
+    s.debug_set_draft(story[:2])
+    s.verify(story)
+    y, a = s.verify(None)
+    assert a == len(story) and [int(t) for t in y[:a]] == story
+    assert s.commit()[0][:a] == story
+    for again in (lambda: s.step(None, 0)[0], lambda: Sdv.verify_batch([s]) == [0] and s.commit()[0]):
+        s.rollback(L)
+        s.verify(story)
+        assert again() == story[:1]
