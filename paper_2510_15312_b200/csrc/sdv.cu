@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "dense.cuh"
+#include "device_once.h"
 #include "forward.cuh"
 #include "layout.cuh"
 #include "small_gemm.cuh"
@@ -307,16 +308,13 @@ ForwardKernel forward_kernel(const FwdParams& P) {
 }
 cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_t stream) {
     const ForwardKernel k = forward_kernel(P);
-    static std::atomic<unsigned long long> sized[2][3];   // bit: the kernel may use all shared memory on that device
-    std::atomic<unsigned long long>& done = sized[P.hd == 128][P.nseq > 0 ? 2 : (P.tree ? 1 : 0)];
+    static DeviceOnce sized[2][3];   // the kernel may use all shared memory
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = sized[P.hd == 128][P.nseq > 0 ? 2 : (P.tree ? 1 : 0)].run(
+            dev, [&]() { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget); });
     if (e != cudaSuccess) return e;
-    if (dev >= 64 || !(done.load(std::memory_order_relaxed) >> dev & 1ull)) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-        if (e != cudaSuccess) return e;
-        if (dev < 64) done.fetch_or(1ull << dev, std::memory_order_relaxed);
-    }
     DraftArg none;
     none.n = -1;
     void* args[] = {(void*)&P, (void*)(draft ? draft : &none)};
@@ -475,15 +473,18 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_tiled_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
+    static std::atomic<EncodeTiledFn> fn{nullptr};   // the same for every thread and device
+    EncodeTiledFn known = fn.load(std::memory_order_acquire);
+    if (!known) {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
+            q == cudaDriverEntryPointSuccess) {
+            known = (EncodeTiledFn)p;
+            fn.store(known, std::memory_order_release);
+        }
     }
-    return fn;
+    return known;
 }
 // bf16 matrix [rows][K] row-major on this GPU; box = box_rows x 64 columns, 128-byte swizzle, zeros outside.
 bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t K, uint32_t box_rows) {
@@ -570,17 +571,22 @@ cudaError_t dense_product(sdv_ctx* ctx, MapIndex a, int layer, int matrix, int M
     return launch_dense_tiles<EPI_PARTIAL, 128>(ctx, m[a], m[map_at(layer, matrix, 128)], M, N, K, pl.splits, part, nullptr, 0, DenseTopOut());
 }
 
+// The dense path's kernels may use the shared memory their shapes need (an attribute of each device).
 cudaError_t dense_attributes() {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<128>::kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_SWIGLU, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_TOP, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseShape<256>::kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseAttShape<128>::kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DenseAttShape<64>::kSmemBytes);
-    done = e == cudaSuccess;
-    return e;
+    static DeviceOnce once;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return once.run(dev, []() {
+        constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 128>, attr, DenseShape<128>::kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_PARTIAL, 256>, attr, DenseShape<256>::kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_SWIGLU, 256>, attr, DenseShape<256>::kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_gemm_kernel<EPI_TOP, 256>, attr, DenseShape<256>::kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<128>, attr, DenseAttShape<128>::kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(dense_attention_kernel<64>, attr, DenseAttShape<64>::kSmemBytes);
+        return e;
+    });
 }
 
 // One sub-chunk of `rows` (1..kDenseMaxRows) context tokens at positions L..L+rows-1 through every layer:
@@ -1800,7 +1806,7 @@ int sdv_debug_timeout_probe(sdv_ctx* ctx) {
 // (small_gemm.cuh), no scratch.
 namespace {
 constexpr size_t kNaWeightBytes = (size_t)2 << 20;              // N * K * 2 <= 2 MiB
-constexpr int kNaMaxK = 4096, kNaMaxN = 4096, kNaMaxDevices = 64;
+constexpr int kNaMaxK = 4096, kNaMaxN = 4096;
 }  // namespace
 
 extern "C" {
@@ -1846,15 +1852,17 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
     cfg.numAttrs = 1;
     typedef void (*Kernel)(const float*, const uint16_t*, float*, int, int, int);
     static const Kernel kernels[4] = {small_gemm_kernel<1>, small_gemm_kernel<2>, small_gemm_kernel<3>, small_gemm_kernel<4>};
-    static std::atomic<bool> loaded[kNaMaxDevices];
-    if (dev >= kNaMaxDevices || !loaded[dev].load(std::memory_order_relaxed)) {
-        // the runtime loads a kernel's code when it is first named: all four now, so that no later call makes it take memory
-        for (int i = 0; i < 4; ++i) {
+    static DeviceOnce loaded;
+    // the runtime loads a kernel's code when it is first named: all four now, so that no later call makes it take memory
+    const cudaError_t named = loaded.run(dev, []() {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
             cudaFuncAttributes fa;
-            if (cudaFuncGetAttributes(&fa, (const void*)kernels[i]) != cudaSuccess) return SDV_ECUDA;
+            e = cudaFuncGetAttributes(&fa, (const void*)kernels[i]);
         }
-        if (dev < kNaMaxDevices) loaded[dev].store(true, std::memory_order_relaxed);
-    }
+        return e;
+    });
+    if (named != cudaSuccess) return SDV_ECUDA;
     if (cudaLaunchKernelEx(&cfg, kernels[(M - 1) / 8], dev_x, dev_w, dev_y, M, N, K) != cudaSuccess) return SDV_ECUDA;
     return cudaStreamSynchronize(s) == cudaSuccess ? SDV_OK : SDV_ECUDA;
 }
