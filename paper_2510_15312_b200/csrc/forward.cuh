@@ -131,12 +131,19 @@ __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target
 // Weight streamer (one thread).  The ring holds 128 KB of the 590 KB a layer of the 1.5B shape streams per block, and HBM
 // would idle through the attention half of a layer (24 us) once it is full.  So while the streamer waits for a free slot it reads
 // ahead into L2, at most kLookaheadBytes beyond the ring and no faster than one piece per kLookaheadCycles or kLookaheadSlow
-// (4 or 2 TB/s over the grid if nothing else ran): a burst would queue in front of the other warps' loads, which cost more than it gave, the trickle does not.
+// (4 or 3 TB/s over the grid if nothing else ran): a burst would queue in front of the other warps' loads, which cost more than it gave, the trickle does not.
 // 10050 -> 9680 us for eight steps of the 1.5B shape, 12130 -> 11970 us for four of the 7B shape; 128 KB: 9720, 256 KB: 9660.
-// The rate: where a layer is short the weights have to come during its waits.  Where the stream itself fills HBM (a block's share of a
-// layer above 2 MB), or the rows' operand builds are what a layer waits for (above 24 rows), the slower trickle disturbs less.
-// 600 against 1100 cycles: 1.5B shape 7570 / 7700 us for eight steps, 3B (17 rows) 7800 / 7860 for four; 7B 10880 / 10720, 27 rows of the
-// 1.5B shape 1452 / 1431 us a step.
+// The rate, by the time of the forward kernel at 800 cycles over that at 600 (both by turns in one context; a share is what a block streams
+// of a layer, MB of 2^20 bytes):
+//   up to 24 rows, shares up to 2.2 MB: 600.  1.5B shape (0.6 MB) 1.012 to 1.022 at 1 to 13 rows, 3B shape (1.3 MB) 1.012 to 1.022 at 1 to 17, shares
+//     of 1.4 to 1.9 MB 1.007 to 1.015 at 1 to 9 (2048 keys each); 17 to 24 rows and 8192 keys: 0.992 to 1.007.
+//   above 24 rows the operand builds are what a layer waits for: 24 rows 0.997, 25 rows 0.992, 32 rows 0.989 (1.5B shape, 2048 keys); longer
+//     layers (0.99 to 1.3 MB) 0.993 to 1.001 from 2048 keys on, 1.000 to 1.012 below.
+//   shares of 2.5 MB and more: the stream fills HBM, and the loads of the KV rows queue behind a faster trickle.  7B shape (3.0 MB), 1 to 9 rows:
+//     0.988 to 0.997 from 2560 keys on, 0.996 to 1.005 at 2048, 1.003 to 1.009 at 256.  2.5 MB: 0.989 to 0.997 at 8192 keys, 1.000 to 1.004 at
+//     2048.  2.2 MB: 0.998 to 1.002 at 8192, 1.004 to 1.009 at 2048, hence the line between these two.
+// 1100 cycles instead of 800 take up to another 0.6 % off the 7B shape at 8192 keys and 0.4 % off 27 rows of the 1.5B shape, but cost 1 to 3 % in
+// layers of 0.99 to 1.3 MB above 24 rows and about 1 % in long ones up to 2048 keys.
 struct Lookahead {   // cursor over the block's weight stream: operation by operation, each one contiguous range of bytes
     int ph, oi;
     const uint8_t* src;
@@ -168,7 +175,7 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
     Lookahead la;
     la.ph = P.ph_begin; la.oi = -1; la.begin = la.end = 0; la.src = nullptr; la.bytes = la.first = 0;
     bool more = lookahead_next(P, misc, la);
-    const uint32_t pause = P.M > 24 || P.layer_stride > (2ull << 20) * (unsigned)P.G ? kLookaheadSlow : kLookaheadCycles;
+    const uint32_t pause = P.M > kLookaheadRows || P.layer_stride > kLookaheadShare * (unsigned)P.G ? kLookaheadSlow : kLookaheadCycles;
     uint32_t last = (uint32_t)clock64();
 #pragma unroll 1
     for (int ph = P.ph_begin; ph < P.ph_end && ok; ++ph) {

@@ -45,7 +45,9 @@ constexpr int kMiscSmemBytes = 4096;
 constexpr int kMiscOff = kSmemBudget - kMiscSmemBytes;  // bookkeeping lies behind everything else, at the same place whatever the rows
 constexpr unsigned long long kLookaheadBytes = 393216;  // how far ahead of the ring the weight streamer reads into L2,
 constexpr unsigned kLookaheadPiece = 8192;             //   in pieces of this size
-constexpr int kLookaheadCycles = 600, kLookaheadSlow = 1100;   //   and no more often than this
+constexpr int kLookaheadCycles = 600, kLookaheadSlow = 800;   //   and no more often than this: the slow rate
+constexpr int kLookaheadRows = 24;                     //   above so many rows,
+constexpr unsigned long long kLookaheadShare = 19ull << 17;   //   or where a block's share of a layer has more bytes (2.375 MB)
 constexpr int kMaxDraftWords = 32;
 constexpr int kProfWords = 12;                         // timestamps per (phase, block)
 constexpr int kTmemCols = 512;
