@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(1024) dense_qkv_finish_kernel(const float* par
 // and running maximum in tensor memory and a warpgroup of its own (one tile row per thread): while one warpgroup
 // turns its scores into probabilities (written back over S as bf16, the A operand of P V), the tensor core works for the
 // other.  O is rescaled only when the maximum grew by more than 2^8 (the probabilities then stay below 2^8, the sums
-// are fp32).  The blocks of a cluster merge their rows by bulk copies between their shared memories: each finishes an
+// are fp32).  The two alternating streams with P in tensor memory and the rare rescaling are the method published as
+// FlashAttention-4; grouped heads as tile rows, keys over a cluster and the exchange are this kernel's.  The blocks of a cluster merge their rows by bulk copies between their shared memories: each finishes an
 // even share of the tile rows and is sent the others' outputs of them, with maximum and sum behind every row.  (Reading
 // them by remote loads took 4 to 6 us of a launch, 13 bytes per cycle and SM.)  Output bf16 [M][n_q * hd].
 // Bound by the exponentials (16 per cycle and SM: 1.1 us per 128 keys of both streams) and, over short contexts, by the

@@ -1,7 +1,7 @@
 // Thin wrappers over the PTX used by the kernels: mbarriers with bounded waits, bulk
-// asynchronous copies (the TMA engine, 1-D form), tcgen05 tensor-core instructions with
-// accumulators in tensor memory, ldmatrix / mma.sync bf16 tiles (attention), named barriers
-// and cache-bypassing global accesses.
+// asynchronous copies (the TMA engine, 1-D and tensor-map forms), tcgen05 tensor-core instructions with
+// accumulators in tensor memory, thread-block clusters and pairs of SMs, dependent launches, 16-byte asynchronous
+// copies, the mma.sync tile of the stand-alone GEMM, named barriers and cache-bypassing global accesses.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -95,8 +95,6 @@ __device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gmem_src, u
         ::"r"(smem_u32(smem_dst)), "l"(gmem_src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
         : "memory");
 }
-
-
 // global -> L2 only (address and size multiples of 16).
 __device__ __forceinline__ void bulk_prefetch_l2(const void* gmem, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gmem), "r"(bytes) : "memory");
@@ -110,16 +108,6 @@ __device__ __forceinline__ float ex2_ftz(float x) {
 }
 
 // ---------------------------------------------------------------- tcgen05: tensor memory and MMA
-// Shared-memory operand descriptor, K-major, no swizzle: the operand is made of 8-row x 16-byte
-// core matrices (128 contiguous bytes each); `lbo` is the byte distance between the two core
-// matrices of one 16-element K step, `sbo` the distance between consecutive 8-row groups.
-__device__ __forceinline__ uint64_t umma_smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)((lbo >> 4) & 0x3fffu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3fffu) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version of this architecture
-    return d;
-}
 // Shared-memory operand descriptor, K-major, 128-byte swizzle: rows of 64 bf16 (128 bytes), groups of
 // 8 rows 1024 bytes apart; a 16-element K step advances the start address by 32 bytes.
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
@@ -146,13 +134,13 @@ __host__ __device__ __forceinline__ uint32_t umma_idesc_bf16(uint32_t m, uint32_
     return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 __host__ __device__ __forceinline__ uint32_t umma_idesc_bf16_m128(uint32_t n) { return umma_idesc_bf16(128u, n); }
-// D[tmem] = A[smem] * B[smem]^T (first instruction of an accumulation) and D[tmem] += ..., issued by
-// one thread.  Successive column steps only advance the descriptors' address fields (the low 14
-// bits, in 16-byte units), so the issuing thread spends one addition per operand and instruction.
-// The same for operands without swizzle, given the low words of their descriptors (umma_smem_lo): successive column steps only
-// add to the address field, so the issuing thread spends one 32-bit addition per operand and instruction.
+// Operands without swizzle, K-major: made of 8-row x 16-byte core matrices (128 contiguous bytes each), 8-row groups one after the
+// other.  umma_smem_lo is the low word of such an operand's descriptor; `lbo` is the byte distance between the two core matrices of
+// one 16-element K step.  Successive column steps only add to the address field (the low 14 bits, in 16-byte units), so the thread
+// that issues umma_bf16_lo spends one 32-bit addition per operand and instruction.
 constexpr uint32_t kUmmaPlainHi = (128u >> 4) | (1u << 14);   // 8-row groups 128 bytes apart; descriptor version of this architecture
 __device__ __forceinline__ uint32_t umma_smem_lo(uint32_t saddr, uint32_t lbo) { return ((saddr >> 4) & 0x3fffu) | (((lbo >> 4) & 0x3fffu) << 16); }
+// D[tmem] = A[smem] * B[smem]^T, or += where acc != 0, issued by one thread; operands by the low words of their descriptors.
 __device__ __forceinline__ void umma_bf16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
@@ -162,6 +150,7 @@ __device__ __forceinline__ void umma_bf16_lo(uint32_t d_tmem, uint32_t a_lo, uin
         "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(acc), "r"(kUmmaPlainHi));
 }
+// The same by whole descriptors.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -338,18 +327,7 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// ---------------------------------------------------------------- tensor-core tiles
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
-                                              uint32_t& r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
+// ---------------------------------------------------------------- mma.sync tile
 // D(16x8, f32) += A(16x16, bf16, row) * B(16x8, bf16, col)
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                uint32_t b0, uint32_t b1) {
@@ -375,17 +353,11 @@ __device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
 }
 
 // ---------------------------------------------------------------- global memory, L1 bypass
-__device__ __forceinline__ float4 ldcg_f4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
 // Loads the compiler keeps in program order: a batch written as "all loads, then all uses" really
 // has all its requests in flight at once (one L2 round trip instead of one per load).
 __device__ __forceinline__ float4 ld_cg_f4_inorder(const void* p) {
     float4 v;
     asm volatile("ld.global.cg.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float4 ld_nc_f4_inorder(const void* p) {
-    float4 v;
-    asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
 // The same where n > limit; otherwise v keeps its value.
@@ -436,12 +408,7 @@ __device__ __forceinline__ void red_add_f32(float* p, float v) {
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
 
-// Offset (bytes) of element (row, col) in a [rows][64] bf16 tile whose 128-byte rows have their
-// eight 16-byte units XOR-swizzled by (row & 7): ldmatrix reads of 8 consecutive rows at one
-// unit index then touch 8 different bank groups.
-__host__ __device__ __forceinline__ uint32_t swz_off(uint32_t row, uint32_t col) {
-    return row * 128u + ((((col >> 3) ^ row) & 7u) << 4) + ((col & 7u) << 1);
-}
+// Offset (bytes) of 16-byte unit `unit` of row `row` in a tile of 128-byte rows whose eight units are XOR-swizzled by (row & 7).
 __host__ __device__ __forceinline__ uint32_t swz_unit(uint32_t row, uint32_t unit) {
     return row * 128u + (((unit ^ row) & 7u) << 4);
 }

@@ -527,7 +527,7 @@ cudaError_t launch_dependent(sdv_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, 
 
 // How a product of M x N outputs is cut: features per tile and K shares.  Model of its time in microseconds: rounds of
 // one tile per pair of SMs, each its K stages (64 columns: 0.26 us with 128 features, 0.40 with 256) and a fixed price, and
-// the partial sums, written here and read by the next kernel (about 4 bytes per us and ns of L2 time each way).
+// the fp32 partial sums, written here and read by the next kernel, each way at 6 TB/s (6e6 bytes per us).
 struct DensePlan {
     int bn, splits;
 };
