@@ -266,7 +266,7 @@ struct sdv_ctx {
     int kv_len, hist_len, n_ctx;
     bool prefill_done, weights_loaded, verified, draft_pending;
     int draft_k;    // k of the pending sdv_draft
-    int last_rows;  // rows of the last verify
+    int last_rows;  // rows of the last verify at most (a draft on the device may have been shorter)
     unsigned bar_base;  // grid-barrier counter value before the next launch (wraps; only differences are used)
     int parity;
     int profile;
