@@ -18,6 +18,9 @@
 //   warps 0..9   build the token operand at the start of an operation (normalised rows, merge of the
 //                split-KV partial results, ...) and meet the other blocks; warps 0..7 are the softmax of the attention
 //                step, whose products (scores and outputs, keys on the M side) warp 9 issues.
+// Code counts like data here: a layer's phases are 100 KB and more of instructions that every warp goes through once, so what is
+// written out twice is fetched twice.  What a phase is prepared with, its operand build and the barrier are therefore
+// written once per phase, and the stand-alone GEMM is a kernel of its own.
 // A layer is four operations separated by a bounded grid barrier: QKV projection; attention;
 // output projection (+ residual); gate|up with SwiGLU followed, inside the same block and without
 // a barrier, by the slice of the down projection (+ residual) that consumes this block's SwiGLU
@@ -98,8 +101,10 @@ static_assert(sizeof(Misc) <= kMiscSmemBytes, "misc shared memory");
 constexpr int kBarrierWarp = kWorkerWarps - 1;
 template <typename F>
 __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target, Misc* misc, int wtid, F prepare) {
-    if ((wtid >> 5) == kBarrierWarp) {
-        prepare();
+    const bool meets = (wtid >> 5) == kBarrierWarp;
+    if (!meets) named_bar_arrive(1, kWorkerThreads);
+    prepare();
+    if (meets) {
         named_bar_sync(1, kWorkerThreads);
         if ((wtid & 31) == 0) {
             red_release_add_u32(P.bar, 1u);  // no return value to wait for: polling starts at once
@@ -118,12 +123,8 @@ __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target
             }
             *(volatile int*)&misc->skip = *(volatile int*)&misc->abort_flag;
         }
-        named_bar_sync(4, kWorkerThreads);
-    } else {
-        named_bar_arrive(1, kWorkerThreads);
-        prepare();
-        named_bar_sync(4, kWorkerThreads);
     }
+    named_bar_sync(4, kWorkerThreads);
     return *(volatile int*)&misc->skip != 0;
 }
 
@@ -354,17 +355,14 @@ __device__ __forceinline__ void build_norm_operand(const FwdParams& P, NormPrep&
         for (int u = 0; u < kSegUnits; ++u) a[u] = b[u] = make_float4(0.f, 0.f, 0.f, 0.f);   // units past the segment stay zero
         const float4* src = n.src;
         int row = n.row0;
-        norm_load(n, a, src, row < M);
+        norm_load(n, b, src, row < M);
 #pragma unroll 1
         while (row < M) {
+#pragma unroll
+            for (int u = 0; u < kSegUnits; ++u) a[u] = b[u];
             src += n.step4;
             norm_load(n, b, src, row + n.row_step < M);
             norm_convert(n, a, dst + (uint32_t)row * 16u, sumsq + row, segs == 1, lane);
-            row += n.row_step;
-            if (row >= M) break;
-            src += n.step4;
-            norm_load(n, a, src, row + n.row_step < M);
-            norm_convert(n, b, dst + (uint32_t)row * 16u, sumsq + row, segs == 1, lane);
             row += n.row_step;
         }
         more += kBuilderWarps;
@@ -1295,7 +1293,7 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
 }
 
 // ------------------------------------------------------------------------------------------
-// HD: head dimension; MODE: chain, tree or batch (see attention_unit).
+// HD: head dimension; MODE: chain, tree or batch (see attention_unit), or 3: the stand-alone GEMM alone (a launch of its own).
 template <int HD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg, const __grid_constant__ DraftArg draft) {
     static_assert(sizeof(FwdParams) % 4 == 0, "parameter block is copied word by word");
@@ -1416,45 +1414,45 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     };
     const int n_layers = P.n_layers, lm = 1 + kPhasesPerLayer * n_layers;
     NormPrep prep;
-    if (ph == 0) {
-        enter();
-        embed_phase(P, draft, wtid);
-        leave();
-        meet([&]() { norm_prep<PH_QKV>(prep, P, misc, 0, wtid, 0); });
-#pragma unroll 1
-        for (int layer = 0; layer < n_layers; ++layer) {
-            int early = 0;
-            enter();
-            if (!skip) gemm_phase<HD, MODE, PH_QKV>(P, layer, prep, smem, misc, pos, wtid, pp);
-            leave();
-            meet([&]() { early = attention_early<HD, MODE>(P, layer, smem + P.u_off, wtid); });
-            enter();
-            if (!skip) attention_phase<HD, MODE>(P, misc, layer, early, smem, wtid, att_uses, pp);
-            leave();
-            meet([]() {});
-            enter();
-            if (!skip) gemm_phase<HD, MODE, PH_O>(P, layer, prep, smem, misc, pos, wtid, pp);
-            leave();
-            meet([&]() { norm_prep<PH_GUD>(prep, P, misc, layer, wtid, 0); });
-            enter();
-            if (!skip) gemm_phase<HD, MODE, PH_GUD>(P, layer, prep, smem, misc, pos, wtid, pp);
-            leave();
-            if (layer + 1 < n_layers) meet([&]() { norm_prep<PH_QKV>(prep, P, misc, layer + 1, wtid, 0); });
-        }
-        if (ph < P.ph_end) meet([&]() { norm_prep<PH_LM>(prep, P, misc, 0, wtid, 0); });
-    } else if (ph == lm) {
-        norm_prep<PH_LM>(prep, P, misc, 0, wtid, 0);
-    }
-    if (ph == lm && ph < P.ph_end) {
-        enter();
-        if (!skip) gemm_phase<HD, MODE, PH_LM>(P, 0, prep, smem, misc, pos, wtid, pp);
-        leave();
-    }
-    if (MODE == 0 && ph == lm + 1 && ph < P.ph_end) {   // the stand-alone GEMM (a launch of its own)
+    if (MODE == 3) {
         norm_prep<PH_RAW>(prep, P, misc, 0, wtid, 0);
         enter();
         gemm_phase<HD, MODE, PH_RAW>(P, 0, prep, smem, misc, pos, wtid, pp);
         leave();
+    } else {
+        if (ph == 0) {
+            enter();
+            embed_phase(P, draft, wtid);
+            leave();
+#pragma unroll 1
+            for (int layer = 0; layer < n_layers; ++layer) {
+                int early = 0;
+                meet([&]() { norm_prep<PH_QKV>(prep, P, misc, layer, wtid, 0); });
+                enter();
+                if (!skip) gemm_phase<HD, MODE, PH_QKV>(P, layer, prep, smem, misc, pos, wtid, pp);
+                leave();
+                meet([&]() { early = attention_early<HD, MODE>(P, layer, smem + P.u_off, wtid); });
+                enter();
+                if (!skip) attention_phase<HD, MODE>(P, misc, layer, early, smem, wtid, att_uses, pp);
+                leave();
+                meet([]() {});
+                enter();
+                if (!skip) gemm_phase<HD, MODE, PH_O>(P, layer, prep, smem, misc, pos, wtid, pp);
+                leave();
+                meet([&]() { norm_prep<PH_GUD>(prep, P, misc, layer, wtid, 0); });
+                enter();
+                if (!skip) gemm_phase<HD, MODE, PH_GUD>(P, layer, prep, smem, misc, pos, wtid, pp);
+                leave();
+            }
+            if (ph < P.ph_end) meet([&]() { norm_prep<PH_LM>(prep, P, misc, 0, wtid, 0); });
+        } else if (ph == lm) {
+            norm_prep<PH_LM>(prep, P, misc, 0, wtid, 0);
+        }
+        if (ph == lm && ph < P.ph_end) {
+            enter();
+            if (!skip) gemm_phase<HD, MODE, PH_LM>(P, 0, prep, smem, misc, pos, wtid, pp);
+            leave();
+        }
     }
     tc_fence_before();
     named_bar_sync(3, kWorkerThreads + 32);

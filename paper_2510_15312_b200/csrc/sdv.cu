@@ -299,20 +299,21 @@ int cuda_fail(sdv_ctx* ctx, cudaError_t e) {
     } while (0)
 
 typedef void (*ForwardKernel)(const FwdParams, const DraftArg);
-// The forward kernel compiled for this launch's head dimension and kind of attention.
+// The kind of launch the forward kernel is compiled for: chain, tree, batch, or the stand-alone GEMM alone (whatever the heads).
+int forward_mode(const FwdParams& P) { return P.ph_begin == 2 + kPhasesPerLayer * P.n_layers ? 3 : P.nseq > 0 ? 2 : P.tree ? 1 : 0; }
+// The forward kernel compiled for this launch's head dimension and kind.
 ForwardKernel forward_kernel(const FwdParams& P) {
-    const int mode = P.nseq > 0 ? 2 : (P.tree ? 1 : 0);
-    static const ForwardKernel table[2][3] = {{sdv_forward_kernel<64, 0>, sdv_forward_kernel<64, 1>, sdv_forward_kernel<64, 2>},
-                                              {sdv_forward_kernel<128, 0>, sdv_forward_kernel<128, 1>, sdv_forward_kernel<128, 2>}};
-    return table[P.hd == 128][mode];
+    static const ForwardKernel table[2][4] = {{sdv_forward_kernel<64, 0>, sdv_forward_kernel<64, 1>, sdv_forward_kernel<64, 2>, sdv_forward_kernel<64, 3>},
+                                              {sdv_forward_kernel<128, 0>, sdv_forward_kernel<128, 1>, sdv_forward_kernel<128, 2>, sdv_forward_kernel<64, 3>}};
+    return table[P.hd == 128][forward_mode(P)];
 }
 cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_t stream) {
     const ForwardKernel k = forward_kernel(P);
-    static DeviceOnce sized[2][3];   // the kernel may use all shared memory
+    static DeviceOnce sized[2][4];   // the kernel may use all shared memory
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
-        e = sized[P.hd == 128][P.nseq > 0 ? 2 : (P.tree ? 1 : 0)].run(
+        e = sized[P.hd == 128][forward_mode(P)].run(
             dev, [&]() { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget); });
     if (e != cudaSuccess) return e;
     DraftArg none;
