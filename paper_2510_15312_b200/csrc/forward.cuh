@@ -71,7 +71,7 @@ struct NormShape {
 };
 struct MmaShape {
     uint32_t idesc, blo, bstep;            // instruction descriptor; token operand's descriptor and its column step
-    int groups, last_groups, last_steps;   // column steps of a stage: groups of four, and the last stage's
+    int steps, last_steps;                 // column steps of a stage, and of the last one
 };
 struct Misc {
     uint64_t full[kMaxStages], empty[kMaxStages];
@@ -435,11 +435,15 @@ __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const P
 }
 
 // ------------------------------------------------------------------------------------------
-// Tensor-core issue, by one thread for the whole launch.  The pipe takes an instruction (M = 128, N <= 32) every 31 cycles, the
-// time shared memory needs for its 4 KB of weights, 250 cycles per 32 KB stage; the code around the instructions sets the pace: a
-// lone thread pays the full latency of every dependent instruction and branch.  So what an operation needs is worked out
-// once per launch (MmaShape), descriptors advance by 32-bit additions, the next stage's barrier is looked at (without waiting)
-// before the instructions of this one are issued, and stages run in straight groups of four column steps.
+// Tensor-core issue, by one thread for the whole launch.  Measured on the part: the pipe takes an instruction (M = 128, N <= 32) every
+// 39 cycles and a commit costs it 87, so a 32 KB stage (eight instructions, a commit) takes 399; about eight entries wait in its queue.  The
+// issuing thread pays the full latency of every dependent instruction and branch, so it keeps up only if nothing but the instructions stands
+// between a commit and the next one: an operation is one flat loop over its (pass, stage) pairs, what the next pair needs is worked
+// out and its barriers are looked at (without waiting) behind this pair's instructions and before its commits, barriers go by
+// their shared-memory addresses, and what is the same all through an operation is worked out once per launch (MmaShape).
+// Stand-alone, with nothing to wait for, in cycles (before: nested loops, commits first): gate|up of the 0.5B shape 5595 -> 3971, the 1.5B
+// shape 8569 -> 5945; down 7584 -> 4069, 3B shape 14257 -> 6945; output projection 2826 -> 1717; a 16-tile share over 160 column steps
+// 26054 -> 16473.
 // Pipeline positions: (slot, par) is the ring position (slot index and parity of the current trip round the ring), `q`
 // counts accumulator passes, `ops` token operands; all advance over the whole launch, identically in every role.
 struct PipePos {
@@ -453,87 +457,131 @@ __device__ __forceinline__ MmaShape mma_shape(const FwdParams& P, const Part& pt
     f.idesc = umma_idesc_bf16_m128(pt.slices > 1 ? (uint32_t)((brows + 15) & ~15) : (uint32_t)P.NB);
     f.blo = umma_smem_lo(operand, lbo_b);
     f.bstep = (2u * lbo_b) >> 4;                                // one column step, in descriptor address units
-    f.groups = pt.SK >> 2;                                      // a full stage: groups of four column steps (SK is a multiple of 4)
-    const int last = pt.per - (pt.nst - 1) * pt.SK;             // column steps of the last stage
-    f.last_groups = last >> 2;
-    f.last_steps = last & 3;
+    f.steps = pt.SK;
+    f.last_steps = pt.per - (pt.nst - 1) * pt.SK;
     return f;
 }
 
-// The stages of one pass; one or (TWO) two 128-row accumulators.  alo: weight descriptor of ring slot 0.
+// Barriers by their shared-memory addresses.
+__device__ __forceinline__ bool mbar_test_at(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ void umma_commit_at(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// One operation; one or (TWO) two 128-row accumulators per pass (where some passes of an operation need the second one, all are given it: its
+// instructions read on behind a shorter pass's rows, inside shared memory, into columns nobody reads).  The token operand is waited
+// for last, with everything else at hand.  due_slot, due_acc: commits that are due behind the last instructions issued.  False: a
+// wait was abandoned.
 template <bool TWO>
-__device__ __forceinline__ bool mma_pass(Misc* misc, PipePos& pos, bool& ready, uint32_t nstage, int nst, const MmaShape& f, uint32_t d, uint32_t alo,
-                                         uint32_t astep, uint64_t wait_limit) {
-    uint32_t b = f.blo, acc = 0u, slot = pos.slot, par = pos.par;
-    int groups = f.groups;
+__device__ __forceinline__ bool mma_stages(const FwdParams& P, const Part& pt, const MmaShape& fs, uint32_t ring0, Misc* misc, PipePos& pos, bool& ready, uint64_t* operand,
+                                           uint32_t operand_par) {
+    constexpr int GROUP = TWO ? 4 : 8;
+    const uint32_t bstep = fs.bstep, idesc = fs.idesc, blo = fs.blo, nstage = (uint32_t)P.nstage;
+    const int steps = fs.steps, last_steps = fs.last_steps, nst = pt.nst;
+    const uint64_t wait_limit = P.wait_limit_ns;
+    const uint32_t full0 = smem_u32(&misc->full[0]), empty0 = smem_u32(&misc->empty[0]), acc_full0 = smem_u32(&misc->tmem_full[0]), acc_empty0 = smem_u32(&misc->tmem_empty[0]);
+    const uint32_t tmem0 = misc->tmem_base, dstep = pt.slices > 1 ? 0u : kTmemBuf, dbase = tmem0 + (pt.slices > 1 ? kTmemStack : 0u);
+    const int prem = pt.prem;
+    uint32_t buf = pos.q % kAccBufs, apar = ((pos.q / kAccBufs) & 1u) ^ 1u, slot = pos.slot, par = pos.par;
+    int pi = pt.rot, p = pt.npass, st = nst;
+    uint32_t count = (uint32_t)((pt.pbase + (pi < prem ? 1 : 0)) * pt.slices), alo = umma_smem_lo(ring0, count * 256u), astep = count * 32u;
+    uint32_t d = dbase + buf * dstep, b = blo, acc = 0u, due_slot = 0u, due_acc = 0u;
+    if (!mbar_test_at(acc_empty0 + buf * 8u, apar)) {
+        const long long t0 = clock64();
+        if (!mbar_wait_bounded(&misc->tmem_empty[buf], apar, &misc->abort_flag, wait_limit)) return false;
+        pos.w_acc += (uint32_t)(clock64() - t0);
+    }
+    if (!ready) {
+        const long long t0 = clock64();
+        if (!mbar_wait_bounded(&misc->full[slot], par, &misc->abort_flag, wait_limit)) return false;
+        pos.w_full += (uint32_t)(clock64() - t0);
+    }
+    if (!mbar_wait_bounded(operand, operand_par, &misc->abort_flag, wait_limit)) return false;
 #pragma unroll 1
-    for (; nst > 0; --nst) {
+    for (;;) {
+        tc_fence_after();
+        if (due_slot) umma_commit_at(due_slot);
+        if (due_acc) umma_commit_at(due_acc);
+        due_acc = 0u;
+        uint32_t a = alo + slot * (uint32_t)(kStageBytes >> 4);
+        int left = st == 1 ? last_steps : steps;
+        if (left == GROUP) {
+#pragma unroll
+            for (int i = 0; i < GROUP; ++i) {
+                umma_bf16_lo(d, a + i * astep, b + i * bstep, idesc, i == 0 ? acc : 1u);
+                if (TWO) umma_bf16_lo(d + 32u, a + i * astep + 128u, b + i * bstep, idesc, i == 0 ? acc : 1u);   // rows 128.. of the pass
+            }
+            b += GROUP * bstep;
+        } else {
+#pragma unroll 1
+            for (; left > 1; left -= 2) {
+                umma_bf16_lo(d, a, b, idesc, acc);
+                if (TWO) umma_bf16_lo(d + 32u, a + 128u, b, idesc, acc);
+                umma_bf16_lo(d, a + astep, b + bstep, idesc, 1u);
+                if (TWO) umma_bf16_lo(d + 32u, a + astep + 128u, b + bstep, idesc, 1u);
+                acc = 1u;
+                a += 2u * astep;
+                b += 2u * bstep;
+            }
+            if (left > 0) {
+                umma_bf16_lo(d, a, b, idesc, acc);
+                if (TWO) umma_bf16_lo(d + 32u, a + 128u, b, idesc, acc);
+                b += bstep;
+            }
+        }
+        acc = 1u;
+        due_slot = empty0 + slot * 8u;
+        if (++slot == nstage) { slot = 0; par ^= 1u; }
+        ready = mbar_test_at(full0 + slot * 8u, par);   // the next stage, of this operation or the one after
+        if (--st == 0) {
+            due_acc = acc_full0 + buf * 8u;
+            buf = (buf + 1u) % kAccBufs;
+            if (buf == 0u) apar ^= 1u;
+            if (--p == 0) break;
+            st = nst;
+            b = blo;
+            acc = 0u;
+            d = dbase + buf * dstep;
+            if (prem) {
+                if (++pi == pt.npass) pi = 0;
+                count = (uint32_t)((pt.pbase + (pi < prem ? 1 : 0)) * pt.slices);
+                alo = umma_smem_lo(ring0, count * 256u);
+                astep = count * 32u;
+            }
+            if (!mbar_test_at(acc_empty0 + buf * 8u, apar)) {
+                umma_commit_at(due_slot);
+                umma_commit_at(due_acc);
+                due_slot = due_acc = 0u;
+                const long long t0 = clock64();
+                if (!mbar_wait_bounded(&misc->tmem_empty[buf], apar, &misc->abort_flag, wait_limit)) return false;
+                pos.w_acc += (uint32_t)(clock64() - t0);
+            }
+        }
         if (!ready) {
+            if (due_slot) umma_commit_at(due_slot);
+            if (due_acc) umma_commit_at(due_acc);
+            due_slot = due_acc = 0u;
             const long long t0 = clock64();
             if (!mbar_wait_bounded(&misc->full[slot], par, &misc->abort_flag, wait_limit)) return false;
             pos.w_full += (uint32_t)(clock64() - t0);
         }
-        tc_fence_after();
-        uint64_t* const done = &misc->empty[slot];
-        uint32_t a = alo + slot * (uint32_t)(kStageBytes >> 4);
-        if (++slot == nstage) { slot = 0; par ^= 1u; }
-        ready = mbar_test(&misc->full[slot], par);   // the next stage, of this operation or the one after
-        int steps = 0;
-        if (nst == 1) { groups = f.last_groups; steps = f.last_steps; }
-        auto step = [&]() {
-            umma_bf16_lo(d, a, b, f.idesc, acc);
-            if (TWO) umma_bf16_lo(d + 32u, a + 128u, b, f.idesc, acc);   // rows 128.. of the pass
-            acc = 1u;
-            a += astep;
-            b += f.bstep;
-        };
-#pragma unroll 1
-        for (int g = groups; g > 0; --g) {
-            step(); step(); step(); step();
-        }
-#pragma unroll 1
-        for (; steps > 0; --steps) step();
-        umma_commit(done);  // the slot is free once these instructions have read it
     }
+    umma_commit_at(due_slot);
+    umma_commit_at(due_acc);
     pos.slot = slot;
     pos.par = par;
+    pos.q += (uint32_t)pt.npass;
     return true;
 }
-// One operation; false: a wait was abandoned.  The token operand (`operand`, its parity) is waited for last, with everything else
-// at hand.
 __device__ __forceinline__ bool mma_op(const FwdParams& P, int op, uint32_t ring0, Misc* misc, PipePos& pos, bool& ready, uint64_t* operand,
                                        uint32_t operand_par) {
     const Part& pt = misc->part[op];
     const MmaShape f = misc->mma[op];
-    const uint32_t nstage = (uint32_t)P.nstage, tmem0 = misc->tmem_base;
-    const uint64_t wait_limit = P.wait_limit_ns;
-    const int nst = pt.nst, slices = pt.slices, npass = pt.npass, pbase = pt.pbase, prem = pt.prem, rot = pt.rot;
-#pragma unroll 1
-    for (int p = 0; p < npass; ++p, ++pos.q) {
-        const int pi = p + rot < npass ? p + rot : p + rot - npass;
-        const uint32_t count = (uint32_t)((pbase + (pi < prem ? 1 : 0)) * slices);   // row tiles of the pass, slices stacked
-        const uint32_t buf = pos.q % kAccBufs, par = ((pos.q / kAccBufs) & 1u) ^ 1u, d = tmem0 + (slices > 1 ? kTmemStack : buf * kTmemBuf);
-        if (!mbar_test(&misc->tmem_empty[buf], par)) {
-            const long long t0 = clock64();
-            if (!mbar_wait_bounded(&misc->tmem_empty[buf], par, &misc->abort_flag, wait_limit)) return false;
-            pos.w_acc += (uint32_t)(clock64() - t0);
-        }
-        const uint32_t alo = umma_smem_lo(ring0, count * 256u), astep = count * 32u;
-        if (p == 0) {
-            if (!ready) {
-                const long long t0 = clock64();
-                if (!mbar_wait_bounded(&misc->full[pos.slot], pos.par, &misc->abort_flag, wait_limit)) return false;
-                pos.w_full += (uint32_t)(clock64() - t0);
-                ready = true;
-            }
-            if (!mbar_wait_bounded(operand, operand_par, &misc->abort_flag, wait_limit)) return false;
-        }
-        if (!(count > 8u ? mma_pass<true>(misc, pos, ready, nstage, nst, f, d, alo, astep, wait_limit)
-                         : mma_pass<false>(misc, pos, ready, nstage, nst, f, d, alo, astep, wait_limit)))
-            return false;
-        umma_commit(&misc->tmem_full[buf]);
-    }
-    return true;
+    return (pt.pbase + (pt.prem > 0 ? 1 : 0)) * pt.slices > 8 ? mma_stages<true>(P, pt, f, ring0, misc, pos, ready, operand, operand_par)
+                                                              : mma_stages<false>(P, pt, f, ring0, misc, pos, ready, operand, operand_par);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1271,21 +1319,17 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
         }
         return ok;
     };
-    bool ok = true;
-    const int lm = 1 + kPhasesPerLayer * P.n_layers;
-    if (ph == 0) {
+    // q|k|v, o, gate|up, down of every layer (phases 0, 2, 3 and 3 of the layer), then the LM head; or one operation alone
+    const int lm = 1 + kPhasesPerLayer * P.n_layers, nops = ph == 0 ? 4 * P.n_layers + (P.ph_end > lm ? 1 : 0) : (P.ph_end > lm ? 1 : 0);
+    const int first = ph == 0 ? 0 : ph == lm ? OP_LM : OP_RAW;
 #pragma unroll 1
-        for (int layer = 0; layer < P.n_layers && ok; ++layer) {
-#pragma unroll 1
-            for (int i = 0; i < 4 && ok; ++i) {   // q|k|v, o, gate|up, down: phases 0, 2, 3 and 3 of the layer
-                ph = 1 + kPhasesPerLayer * layer + (i == 0 ? 0 : (i < 3 ? i + 1 : 3));
-                ok = run(OP_QKV + i);
-            }
+    for (int i = 0; i < nops; ++i) {
+        int op = first;
+        if (first == 0) {
+            op = i < 4 * P.n_layers ? i & 3 : (int)OP_LM;
+            ph = op == OP_LM ? lm : 1 + kPhasesPerLayer * (i >> 2) + (op == 0 ? 0 : op < 3 ? op + 1 : 3);
         }
-        ph = lm;
-    }
-    if (ok && P.ph_end > lm) {
-        ok = run(ph == lm ? OP_LM : OP_RAW);
+        if (!run(op)) break;
     }
     // all tensor-core work must have completed before tensor memory is returned
     umma_commit(&misc->done_bar);
