@@ -373,10 +373,12 @@ __device__ __forceinline__ void build_norm_operand(const FwdParams& P, NormPrep&
 
 // Operand of the output projection = attention output of this block's columns: the split-KV
 // partial results (un-normalised sums with their running maximum and sum) are merged on the way.
-// Four lanes share one (row, 8 columns) item, each taking every fourth partial result, TPL of them at most.
-template <int TPL>
+// LPI lanes share one (row, 8 columns) item, each taking every LPI-th partial result, TPL of them at most.  A round of items waits for one trip
+// to L2 (1.4 us, the loads of all its partial results in flight together), so the items should fit one round: four lanes an
+// item up to kWorkerThreads / 4 items, two lanes above where the results are at most 20 (1.5B shape, 2048 keys: 21 rows 6.6 -> 5.7 us
+// a phase, 32 rows 7.0 -> 6.4; at 9 rows, one round either way, four lanes are 0.1 to 0.3 us faster).
+template <int LPI, int TPL>
 __device__ __forceinline__ void build_merged_operand(const FwdParams& P, const Part& pt, uint8_t* U, int wtid) {
-    constexpr int LPI = 4;  // lanes per item
     const int S = P.att_S;
     const int M = P.M, Mp = operand_rows(P, P.M, 1), hd = P.hd;
     const int k8_0 = pt.k0 * 2, nk8 = pt.nk * 2;
@@ -1264,8 +1266,9 @@ __device__ __forceinline__ void gemm_phase(const FwdParams& P, int layer, NormPr
     if (have0) {
         if (!dead) {
             if (KIND == PH_O) {
-                if (P.att_S <= 20) build_merged_operand<5>(P, p0, U, wtid);
-                else build_merged_operand<kMaxSplits / 4>(P, p0, U, wtid);
+                if (P.att_S <= 20 && P.M * p0.nk * 2 > kWorkerThreads / 4) build_merged_operand<2, 10>(P, p0, U, wtid);
+                else if (P.att_S <= 20) build_merged_operand<4, 5>(P, p0, U, wtid);
+                else build_merged_operand<4, kMaxSplits / 4>(P, p0, U, wtid);
             } else {
                 build_norm_operand<KIND>(P, prep, layer, U, misc, pos.sums, wtid);
             }
