@@ -489,5 +489,6 @@ def gemm_noalloc(x, w_bits, y, stream=None) -> int:
     N = w_bits.shape[0]
     if tuple(w_bits.shape) != (N, K) or tuple(y.shape) != (M, N):
         raise ValueError("gemm_noalloc: shapes do not agree")
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return lib().sdv_gemm_noalloc(x.data_ptr(), w_bits.data_ptr(), y.data_ptr(), M, N, K, s.cuda_stream)
+    # the current stream's handle without a Stream object around it (3.2 -> 0.3 us of a call of 17.7)
+    s = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return lib().sdv_gemm_noalloc(x.data_ptr(), w_bits.data_ptr(), y.data_ptr(), M, N, K, s)

@@ -1850,7 +1850,7 @@ int sdv_gemm_noalloc(const float* dev_x, const uint16_t* dev_w, float* dev_y, in
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cs > 1 ? 1 : 0;   // a block alone is a cluster of its own
     typedef void (*Kernel)(const float*, const uint16_t*, float*, int, int, int);
     static const Kernel kernels[4] = {small_gemm_kernel<1>, small_gemm_kernel<2>, small_gemm_kernel<3>, small_gemm_kernel<4>};
     static DeviceOnce loaded;
