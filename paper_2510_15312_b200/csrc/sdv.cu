@@ -23,6 +23,7 @@ using namespace sdv;
 
 namespace {
 
+constexpr int kPinnedBytes = 4096;   // a context's page-locked memory
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Regions {
@@ -260,7 +261,7 @@ struct sdv_ctx {
     cudaStream_t stream;
     int G;
     FwdParams P;  // template; per-launch fields are filled at launch
-    int* pinned;  // host staging for the state block
+    int* pinned;  // page-locked copy of the state block, then room for the tokens of a run
     cudaEvent_t ev0, ev1;
     // host mirror of the device state
     int kv_len, hist_len, n_ctx;
@@ -722,7 +723,7 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
         delete ctx;
         return code;
     };
-    e = cudaHostAlloc((void**)&ctx->pinned, 4096, cudaHostAllocDefault);
+    e = cudaHostAlloc((void**)&ctx->pinned, kPinnedBytes, cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&ctx->ev1);
     if (e != cudaSuccess) return fail(SDV_ECUDA);
@@ -969,7 +970,7 @@ constexpr int kDenseMinRows = 16;  // fewer rows take the small-row kernel
 int finish_prefill(sdv_ctx* ctx, bool is_last, int row) {
     int* hist = (int*)(ctx->ws + ctx->r.hist);
     ctx->n_ctx = ctx->hist_len;
-    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 0, hist);
+    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 0, hist, ctx->pinned);
     ctx->launches++;
     CK(cudaGetLastError());
     if (!is_last) return SDV_OK;
@@ -1055,7 +1056,7 @@ int sdv_prefill_chunk(sdv_ctx* ctx, const int32_t* host_tokens, int n, int is_la
             if (rc) return rc;
         }
     }
-    return read_state(ctx);
+    return read_state(ctx, true);   // finish_prefill's kernel wrote the error word to the host
 }
 
 int sdv_draft(sdv_ctx* ctx, int k, int32_t* host_draft, int* draft_len) {
@@ -1276,7 +1277,7 @@ int sdv_step(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int k_next,
                             pass ? &a : nullptr);
     if (rc) return rc;
     step_tail_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, (const int*)(ctx->ws + ctx->r.db), ctx->P.cand_val, ctx->P.cand_idx,
-                                                  ctx->G, c.ngram_n, c.ngram_min, k_next, c.search_history, 0, 0, k_next > 0 ? 1 : 0, 0, ctx->pinned);
+                                                  ctx->G, c.ngram_n, c.ngram_min, k_next, c.search_history, 0, 0, k_next > 0 ? 1 : 0, 0, ctx->pinned, 0, 0);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->last_rows = rows;
@@ -1328,7 +1329,7 @@ int sdv_decode_steps(sdv_ctx* ctx, int k, int n_steps, int max_tokens, int ext_m
     ngram_draft_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, db, c.ngram_n, c.ngram_min, k, c.search_history, 1, nullptr);
     if (ext_max_total > 0) extend_draft_kernel<<<1, 32, 0, ctx->stream>>>(state, ext_max_total, 1);
     ctx->launches += ext_max_total > 0 ? 3 : 2;
-    const int all_phases = 2 + kPhasesPerLayer * c.n_layers;
+    const int all_phases = 2 + kPhasesPerLayer * c.n_layers, room = kPinnedBytes / 4 - ST_WORDS;
     for (int i = 0; i < n_steps; ++i) {
         // the kernel reads the KV length from the state block; the host's value (a lower bound) only shapes the attention split
         int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, all_phases, true, false, false, nullptr, true,
@@ -1337,7 +1338,8 @@ int sdv_decode_steps(sdv_ctx* ctx, int k, int n_steps, int max_tokens, int ext_m
         // accept, commit and the next step's draft in one launch
         step_tail_kernel<<<1, 1024, 0, ctx->stream>>>(state, hist, db, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, c.ngram_n,
                                                       c.ngram_min, k, c.search_history, ext_max_total, ext_max_life,
-                                                      i + 1 < n_steps ? 1 : 0, 1, nullptr);
+                                                      i + 1 < n_steps ? 1 : 0, 1, i + 1 < n_steps ? nullptr : ctx->pinned, hist_before,
+                                                      i + 1 < n_steps ? 0 : room);
         ctx->launches++;
     }
     CK(cudaGetLastError());
@@ -1346,14 +1348,16 @@ int sdv_decode_steps(sdv_ctx* ctx, int k, int n_steps, int max_tokens, int ext_m
     ctx->draft_pending = false;
     ctx->tree_pending = false;
     ctx->tree_verified = false;
-    int rc = read_state(ctx);
+    int rc = read_state(ctx, true);   // written by the last tail kernel, tokens too
     if (rc) return rc;
     ctx->kv_len = ctx->pinned[ST_KV_LEN];
     ctx->hist_len = ctx->pinned[ST_HIST_LEN];
     const int n = ctx->hist_len - hist_before;
     if (n_tokens) *n_tokens = n;
     if (kv_len) *kv_len = ctx->kv_len;
-    if (host_tokens && n > 0) {
+    if (host_tokens && n > 0 && n <= room) {
+        memcpy(host_tokens, ctx->pinned + ST_WORDS, (size_t)n * 4);
+    } else if (host_tokens && n > 0) {
         CK(cudaMemcpyAsync(host_tokens, hist + hist_before, (size_t)n * 4, cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
     }
@@ -1519,7 +1523,7 @@ int sdv_rollback(sdv_ctx* ctx, int new_kv_len) {
     int* hist = (int*)(ctx->ws + ctx->r.hist);
     ctx->kv_len = new_kv_len;
     ctx->hist_len = new_kv_len + 1;
-    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 1, hist);
+    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 1, hist, nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->verified = false;
@@ -1565,7 +1569,7 @@ int sdv_debug_set_history(sdv_ctx* ctx, const int32_t* host_hist, int hist_len, 
     ctx->hist_len = hist_len;
     ctx->kv_len = hist_len - 1;
     ctx->n_ctx = n_ctx;
-    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 1, hist);
+    set_state_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, ctx->kv_len, ctx->hist_len, ctx->n_ctx, 1, hist, nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
     ctx->prefill_done = true;

@@ -553,24 +553,36 @@ __global__ void commit_kernel(int* state, int* hist, int max_emit, int force_acc
 // scan of the step just verified, [the update of the retained segment,] its commit under the run's token
 // budget, and, unless the run ends here, the draft of the next step [and its extension].  The stages
 // meet at block barriers: what one writes to the state block and the history, the next reads.
+// host: the state block goes there as well (page-locked memory, ST_WORDS words), and behind it the history from `tokens_from` on, as far
+// as `room` words go (a run's tokens: a copy of either behind the kernels took 15 us more each).
 __global__ void __launch_bounds__(1024) step_tail_kernel(int* state, int* hist, const int* db, const float* cand_val,
                                                          const int* cand_idx, int G, int n, int n_min, int k, int search_history,
-                                                         int ext_max_total, int ext_max_life, int draft_next, int in_run, int* host) {
-    if (in_run && state[ST_BUDGET] == 0) return;   // enqueued behind the end of the run
+                                                         int ext_max_total, int ext_max_life, int draft_next, int in_run, int* host, int tokens_from,
+                                                         int room) {
+    const bool over = in_run && state[ST_BUDGET] == 0;   // enqueued behind the end of the run
+    if (over && !host) return;
     with_state(state, host, [&](int* st) {
-        accept_body(st, cand_val, cand_idx, G, 0, 0, nullptr);
-        __syncthreads();
-        if (ext_max_total > 0) {
-            if (threadIdx.x < 32) extension_update_body(st, ext_max_life);
+        auto tail = [&]() {
+            if (over) return;
+            accept_body(st, cand_val, cand_idx, G, 0, 0, nullptr);
             __syncthreads();
-        }
-        commit_body(st, hist, 0, -1, 0, in_run);
-        __syncthreads();
-        if (!draft_next || (in_run && st[ST_BUDGET] == 0)) return;
-        ngram_draft_body(st, hist, db, n, n_min, k, search_history);
-        if (ext_max_total > 0) {
+            if (ext_max_total > 0) {
+                if (threadIdx.x < 32) extension_update_body(st, ext_max_life);
+                __syncthreads();
+            }
+            commit_body(st, hist, 0, -1, 0, in_run);
             __syncthreads();
-            if (threadIdx.x < 32) extend_draft_body(st, ext_max_total);
+            if (!draft_next || (in_run && st[ST_BUDGET] == 0)) return;
+            ngram_draft_body(st, hist, db, n, n_min, k, search_history);
+            if (ext_max_total > 0) {
+                __syncthreads();
+                if (threadIdx.x < 32) extend_draft_body(st, ext_max_total);
+            }
+        };
+        tail();
+        if (room > 0) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < room && tokens_from + i < st[ST_HIST_LEN]; i += blockDim.x) host[ST_WORDS + i] = hist[tokens_from + i];
         }
     });
 }
@@ -602,9 +614,11 @@ __global__ void prefill_final_kernel(int* state, int* hist, const float* cand_va
     }
 }
 
+// host: the error word goes there as well (page-locked memory; nullptr: not asked for).
 __global__ void set_state_kernel(int* state, int kv_len, int hist_len, int n_ctx, int pending_from_hist,
-                                 const int* hist) {
+                                 const int* hist, int* host) {
     if (threadIdx.x != 0) return;
+    if (host) host[ST_ERR] = state[ST_ERR];
     state[ST_KV_LEN] = kv_len;
     state[ST_HIST_LEN] = hist_len;
     state[ST_N_CTX] = n_ctx;
