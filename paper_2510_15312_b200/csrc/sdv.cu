@@ -1164,16 +1164,21 @@ int sdv_verify_batch(sdv_ctx* const* ctxs, int n, int* accept_len) {
     CK(cudaGetLastError());
     int rc = launch_forward(ctx, rows, Lmax, 0, 0, 2 + kPhasesPerLayer * ctx->cfg.n_layers, true, false, false, &bp);
     if (rc) return rc;
+    BatchAcceptArg aa;
+    memset(&aa, 0, sizeof(aa));
     for (int b = 0; b < n; ++b) {
         sdv_ctx* c = ctxs[b];
-        accept_kernel<<<1, 32 * bp.seq[b].M, 0, ctx->stream>>>(c->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, bp.seq[b].r0,
-                                                              bstate, 0, accept_len ? c->pinned : nullptr);
-        ctx->launches++;
+        aa.state[b] = c->P.state;
+        aa.host[b] = accept_len ? c->pinned : nullptr;
+        aa.r0[b] = bp.seq[b].r0;
+        aa.M[b] = bp.seq[b].M;
         c->verified = true;
         c->tree_verified = false;
         c->last_rows = bp.seq[b].M;
         c->logits_src = ctx->P.logits + (size_t)bp.seq[b].r0 * ctx->cfg.vocab;
     }
+    accept_batch_kernel<<<n, 32 * bp.max_rows, 0, ctx->stream>>>(aa, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, bstate);
+    ctx->launches++;
     CK(cudaGetLastError());
     if (accept_len) {
         for (int b = 0; b < n; ++b) {

@@ -419,11 +419,11 @@ __global__ void extension_update_kernel(int* state, int max_life, int in_run) {
 // `row0`: the sequence's first row among the launch's rows (0 unless the step was batched); `launch_state`:
 // the state block the launch ran on when it is not `state` itself, whose error word is carried over.
 __device__ __forceinline__ void accept_body(int* state, const float* cand_val, const int* cand_idx, int G, int from_host_y,
-                                            int row0, const int* launch_state) {
+                                            int row0, const int* launch_state, int rows) {
     __shared__ int y_s[kMaxRows + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // a sequence that goes through a batched step without a draft of its own may hold one of a verify before: its row is there alone
-    const int dl = min(state[ST_DRAFT_LEN], (int)(blockDim.x >> 5) - 1);
+    const int dl = min(state[ST_DRAFT_LEN], rows - 1);
     if (launch_state && threadIdx.x == 0 && launch_state[ST_ERR]) state[ST_ERR] = launch_state[ST_ERR];
     if (warp <= dl) {
         int bi;
@@ -485,7 +485,17 @@ __device__ __forceinline__ void accept_body(int* state, const float* cand_val, c
 __global__ void accept_kernel(int* state, const float* cand_val, const int* cand_idx, int G, int from_host_y, int row0,
                               const int* launch_state, int in_run, int* host) {
     if (in_run && state[ST_BUDGET] == 0) return;
-    with_state(state, host, [&](int* st) { accept_body(st, cand_val, cand_idx, G, from_host_y, row0, launch_state); });
+    with_state(state, host, [&](int* st) { accept_body(st, cand_val, cand_idx, G, from_host_y, row0, launch_state, (int)(blockDim.x >> 5)); });
+}
+
+// The accept scans of a batched step, a block per sequence (as many launches took 8 us each).
+struct BatchAcceptArg {
+    int *state[kMaxBatch], *host[kMaxBatch];
+    int r0[kMaxBatch], M[kMaxBatch];
+};
+__global__ void accept_batch_kernel(const __grid_constant__ BatchAcceptArg a, const float* cand_val, const int* cand_idx, int G, const int* launch_state) {
+    const int b = blockIdx.x;
+    with_state(a.state[b], a.host[b], [&](int* st) { accept_body(st, cand_val, cand_idx, G, 0, a.r0[b], launch_state, a.M[b]); });
 }
 
 // Batched verify: the token rows of up to kMaxBatch sequences (each its pending token, then its draft, token 0
@@ -564,7 +574,7 @@ __global__ void __launch_bounds__(1024) step_tail_kernel(int* state, int* hist, 
     with_state(state, host, [&](int* st) {
         auto tail = [&]() {
             if (over) return;
-            accept_body(st, cand_val, cand_idx, G, 0, 0, nullptr);
+            accept_body(st, cand_val, cand_idx, G, 0, 0, nullptr, (int)(blockDim.x >> 5));
             __syncthreads();
             if (ext_max_total > 0) {
                 if (threadIdx.x < 32) extension_update_body(st, ext_max_life);
