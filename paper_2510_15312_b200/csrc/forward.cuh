@@ -22,9 +22,9 @@
 // written out twice is fetched twice.  What a phase is prepared with, its operand build and the barrier are therefore
 // written once per phase, and the stand-alone GEMM is a kernel of its own.
 // A layer is four operations separated by a bounded grid barrier: QKV projection; attention;
-// output projection (+ residual); gate|up with SwiGLU followed, inside the same block and without
-// a barrier, by the slice of the down projection (+ residual) that consumes this block's SwiGLU
-// columns.
+// output projection (+ residual); gate|up with SwiGLU followed, inside the same block (or the two blocks of a cluster, which exchange
+// their SwiGLU columns and take half of the rows each) and without a barrier, by the slice of the down projection (+ residual) that
+// consumes these SwiGLU columns.
 #pragma once
 #include <math_constants.h>
 
@@ -77,7 +77,7 @@ struct Misc {
     uint64_t full[kMaxStages], empty[kMaxStages];
     uint64_t tmem_full[kAccBufs], tmem_empty[kAccBufs];
     uint64_t op_ready;    // the token operand of this block's next operation is complete (one arrival per builder warp)
-    uint64_t act_ready;   // the SwiGLU operand of this block is complete (one arrival per epilogue warp)
+    uint64_t act_ready;   // the SwiGLU operand of this block is complete (one arrival per epilogue warp, and the other block's bytes)
     uint64_t att_bar;     // a product of the attention step has completed
     uint64_t done_bar;    // last tensor-core instruction of the launch has completed
     uint32_t tmem_base;
@@ -644,6 +644,8 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, 
     bool add = true;  // residual add (O, down)
     if (op == OP_RAW) { out = P.raw_out; stride = P.raw_N; add = P.op[OP_RAW].P_k > 1; }
     const int store_logits = P.store_logits;
+    const Part& down = misc->part[OP_DOWN];
+    const int act_col0 = op == OP_GU ? (pt.tile0 / 2 - down.k0) * 16 : 0;   // gate|up has two tiles to a column step of the down projection
 #pragma unroll 1
     for (int p = 0; p < npass; ++p, ++pos.q) {
         const int pi = op == OP_GU || LM ? p : pass_index(pt, p);   // those two have no partial sums
@@ -688,7 +690,7 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, 
                 } else if (op == OP_GU) {
                     // rows 0..7 of a tile are gate rows, 8..15 the matching up rows, 8 lanes apart: the gate
                     // lane evaluates the even token columns, the up lane the odd ones
-                    const int col = (pstart + (tt >> 4)) * 8 + (tt & 7);  // SwiGLU column within this block's slice
+                    const int col = (pstart + (tt >> 4)) * 8 + (tt & 7) + act_col0;  // SwiGLU column within the down projection's share
                     uint8_t* dst = act + operand_off(col >> 3, n0, Mp) + (col & 7) * 2;
                     if (nsel < 0) swiglu_pairs<-1>(v, rs, n0, t, valid, Mh, dst);
                     else if (nsel == 0) swiglu_pairs<0>(v, rs, n0, t, valid, Mh, dst);
@@ -709,10 +711,24 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, 
         }
     }
     if (!LM && op == OP_GU) {
-        // this warp's SwiGLU columns are written: hand them to the tensor-core thread
+        // this warp's SwiGLU columns are written: hand them to the tensor-core thread; the blocks of a pair send each other theirs, which lie
+        // one behind the other in the operand (one copy of some KB; both wait for it, so neither is ahead by more than this)
         fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&misc->act_ready);
+        const int steps = pt.ntiles / 2, theirs = down.nk - steps;
+        if (theirs > 0) {
+            named_bar_sync(2, kEpilogueWarps * 32);
+            if (warp == 0 && lane == 0) {
+                const uint32_t peer = cluster_rank() ^ 1u, at = smem_u32(act) + operand_off(act_col0 >> 3, 0, Mp), step_bytes = operand_off(2, 0, Mp);
+                mbar_arrive_expect_tx(&misc->act_ready, (uint32_t)theirs * step_bytes);
+                bulk_s2cluster(map_shared_rank(at, peer), at, (uint32_t)steps * step_bytes, map_shared_rank(smem_u32(&misc->act_ready), peer));
+            } else if (lane == 0) {
+                mbar_arrive(&misc->act_ready);
+            }
+            __syncwarp();
+        } else {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&misc->act_ready);
+        }
     }
 }
 
@@ -1394,6 +1410,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (MODE != 3) cluster_arrive();   // this block's barriers are there
     if (tid == 0) {
         if (Pg.l_from_state) misc->P.L = Pg.state[ST_KV_LEN];
         // the block's first attention unit: the same for every layer, so its index arithmetic is done here
@@ -1420,9 +1437,18 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         misc->mma[op] = mma_shape(P, misc->part[op], smem_u32(smem + (op == OP_DOWN ? P.act_off : P.u_off)));
     }
     __syncthreads();
+    if (MODE != 3) cluster_wait();
+    // a block leaves once the other one of its pair no longer copies from or to it
+    auto finish = [&]() {
+        if (MODE != 3) {
+            __syncwarp();
+            cluster_sync();
+        }
+    };
 
     if (warp == kProducerWarp) {
         if (lane == 0) producer_loop(P, smem, misc);
+        finish();
         return;
     }
     if (warp == kMmaWarp) {
@@ -1432,6 +1458,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         named_bar_sync(3, kWorkerThreads + 32);   // the workers have read the last accumulators
         tc_fence_after();
         tmem_dealloc(misc->tmem_base, kTmemCols);
+        finish();
         return;
     }
 
@@ -1506,6 +1533,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     if (*(volatile int*)&misc->abort_flag) {
         if (wtid == 0) atomicExch(P.state + ST_ERR, 1);
     }
+    finish();
 }
 
 }  // namespace sdv

@@ -41,6 +41,7 @@ constexpr int kSmemBudget = 232448;                    // 227 KB
 constexpr int kKeyChunk = 128;                         // keys per attention chunk: the rows of a tensor-core instruction
 constexpr int kAttnBytesPerDim = 640;                  // attention tiles: 64 query rows, a chunk of keys and of values; bytes per column of a head
 constexpr int kActSmemMax = 32768;                     // SwiGLU output of this block (operand of its down-projection slice) at most
+constexpr int kPairSums = 65536;                       // partial sums per row from which on pairs of blocks share the down projection
 constexpr int kMiscSmemBytes = 4096;
 constexpr int kMiscOff = kSmemBudget - kMiscSmemBytes;  // bookkeeping lies behind everything else, at the same place whatever the rows
 constexpr unsigned long long kLookaheadBytes = 393216;  // how far ahead of the ring the weight streamer reads into L2,
@@ -66,7 +67,8 @@ struct OpDesc {
     int RW;      // row tiles per pass at most (16, 8, 4, 2 or 1)
     int SK;      // column steps per stage at most (RW * SK <= 64)
     int unit;    // row partitions are multiples of this many tiles (2 for gate|up: 16 SwiGLU columns)
-    int follow;  // 1: one row partition; block i takes the columns that partition i of `gate|up` produces
+    int follow;  // 1: the columns follow `gate|up`: one row partition, block i takes the columns that its partition i produces; or two (P_row
+                 //   = 2), blocks 2 i and 2 i + 1 take half of the rows each and the columns that both of them produce
     int slices;  // K slices stacked as rows (0 or 1: none); divides K16 and the column shares
     unsigned long long w_off;  // byte offset of the operation inside its weight region
 };
@@ -118,10 +120,11 @@ __host__ __device__ inline Part make_part(const OpDesc& o, const OpDesc& gu, int
     p.pr = pr;
     p.pk = pk;
     if (o.follow) {
-        p.tile0 = 0;
-        p.ntiles = o.T;
-        p.k0 = even_start(gu.T / gu.unit, gu.P_row, pk);
-        p.nk = even_count(gu.T / gu.unit, gu.P_row, pk);
+        const int units = gu.T / gu.unit;
+        p.tile0 = even_start(o.T, o.P_row, pr);
+        p.ntiles = even_count(o.T, o.P_row, pr);
+        p.k0 = even_start(units, gu.P_row, pk * o.P_row);
+        p.nk = even_start(units, gu.P_row, (pk + 1) * o.P_row) - p.k0;
     } else {
         p.tile0 = o.unit * even_start(o.T / o.unit, o.P_row, pr);
         p.ntiles = o.unit * even_count(o.T / o.unit, o.P_row, pr);
@@ -147,7 +150,7 @@ __host__ __device__ inline Part get_part(const OpDesc& o, const OpDesc& gu, int 
         p.off = 0;
         return p;
     }
-    if (o.follow) return make_part(o, gu, 0, idx);
+    if (o.follow) return make_part(o, gu, idx % o.P_row, idx / o.P_row);
     return make_part(o, gu, idx / o.P_k, idx % o.P_k);
 }
 
@@ -157,8 +160,8 @@ __host__ __device__ inline unsigned long long weight_offset(const OpDesc& o, con
     const int t = row >> 4, ks = k8 >> 1, half = k8 & 1;
     int pr, pk;
     if (o.follow) {
-        pr = 0;
-        pk = even_find(gu.T / gu.unit, gu.P_row, ks);
+        pr = even_find(o.T, o.P_row, t);
+        pk = even_find(gu.T / gu.unit, gu.P_row, ks) / o.P_row;
     } else {
         pr = even_find(o.T / o.unit, o.P_row, t / o.unit);
         pk = even_find(o.K16, o.P_k, ks);
@@ -266,7 +269,7 @@ struct FwdParams {
     int p_off;         // exchange area of the q|k|v epilogue, probabilities of an attention unit
     int pad;           // 1: the rows of a column group in a token operand are followed by an empty one where that makes their number odd
     int plan_ks;       // what the plan follows from besides the rows: column steps of the widest token operand,
-    int plan_act;      //   SwiGLU column steps per block at most (0: no SwiGLU operand)
+    int plan_act;      //   column steps of the down projection's operand at most (0: none)
     int plan_attn;     //   bytes the attention tiles need (0: no attention)
     int rows_from_state;  // 1: at most M rows; the draft in the state block says how many
     uint8_t att_gh_rows[kMaxRows];  // att_gh for 1, 2, ... rows (rows_from_state)

@@ -203,7 +203,7 @@ SmemPlan plan_smem(FwdParams& P, int rows, bool raw_only) {
     }
     if (!raw_only) {
         const OpDesc& gu = P.op[OP_GU];
-        P.plan_act = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;  // SwiGLU column steps per block at most
+        P.plan_act = P.op[OP_DOWN].P_row * ((gu.T / gu.unit + gu.P_row - 1) / gu.P_row);
         P.plan_attn = kAttnBytesPerDim * P.hd;
     }
     plan_smem_rows(P, rows);
@@ -235,10 +235,23 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
             case OP_O: choose_partition(o, G, rows_max, true, true); break;
             case OP_GU: full_k_partition(o, G, 2); break;   // pairs of tiles: 16 SwiGLU columns = one column step of down
             case OP_LM: full_k_partition(o, G, 1); break;
-            default:  // down: every block multiplies the SwiGLU columns it produced
-                o.RW = 16; o.SK = kStageBytes / kStepBytes / 16; o.unit = 1; o.follow = 1; o.P_row = 1; o.P_k = P.op[OP_GU].P_row;
+            default: {  // down: every block multiplies the SwiGLU columns it produced, or a pair of blocks those of both
+                const OpDesc& gu = P.op[OP_GU];
+                o.RW = 16; o.SK = kStageBytes / kStepBytes / 16; o.unit = 1; o.follow = 1;
+                // In pairs each block has half of the rows, so half as many partial sums meet in L2, which the phase waits for: gate|up + down 12.6
+                // -> 12.0 us at 9 rows of the 1.5B shape, 19.1 -> 16.5 at 32, 29.1 -> 25.0 at 17 rows of the 3B shape, 7.4 -> 6.5 at 9 of the 0.5B
+                // shape.  A launch in clusters takes 2 us more, so the sums have to be many: 16 K (256 columns x 64 shares) lose 1.6 us of a launch
+                // of 53.5, 133 K (896 x 148) gain 21 of 593.  The blocks of a pair are those of a cluster: an even number of shares, beginning at an
+                // even block; and the operand of both shares has to stay within what the exchange areas take anyway.
+                const int steps = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;
+                const bool pairs = G % 2 == 0 && gu.P_row % 2 == 0 && gu.rot % 2 == 0 && o.T >= 2 && 16 * o.T * gu.P_row >= kPairSums &&
+                                   2 * steps * 32 * (rows_max | 1) <= kActSmemMax / 2;
+                o.P_row = pairs ? 2 : 1;
+                o.P_k = gu.P_row / o.P_row;
                 break;
+            }
         }
+        if (ops[i].idx == OP_GU && G % 2 == 0) rot += rot % 2;
         if (ops[i].idx != OP_QKV) fit_pass_width(o);
         if (ops[i].idx == OP_DOWN) {
             o.rot = P.op[OP_GU].rot;
@@ -320,10 +333,30 @@ cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_
     DraftArg none;
     none.n = -1;
     void* args[] = {(void*)&P, (void*)(draft ? draft : &none)};
-    // phases meet at grid barriers, so more than one phase needs all blocks co-resident
-    if (P.ph_end - P.ph_begin > 1)
-        return cudaLaunchCooperativeKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
-    return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
+    if (forward_mode(P) == 3) return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
+    // Phases meet at grid barriers, so more than one phase needs all blocks co-resident.
+    if (P.op[OP_DOWN].P_row != 2) {
+        if (P.ph_end - P.ph_begin > 1)
+            return cudaLaunchCooperativeKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
+        return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
+    }
+    // pairs of blocks share the down projection
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(P.G);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBudget;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    memset(at, 0, sizeof(at));
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;
+    at[1].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = P.ph_end - P.ph_begin > 1 ? 2 : 1;
+    return cudaLaunchKernelExC(&cfg, (const void*)k, args);
 }
 
 bool apply_plan(FwdParams& P, int rows, bool raw_only) {
@@ -713,7 +746,11 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
         return SDV_ECUDA;
     }
     if (sms > kMaxGrid) sms = kMaxGrid;
-    ctx->G = sms;  // one persistent block per SM
+    ctx->G = sms & ~1;  // one persistent block per SM, in pairs
+    if (ctx->G < 2) {
+        delete ctx;
+        return SDV_ECUDA;
+    }
     ctx->r = carve(cfg, leader == nullptr);
     // every failure below leaves through this: what was created so far is released
     auto fail = [&](int code) {
