@@ -216,6 +216,20 @@ SmemPlan plan_smem(FwdParams& P, int rows, bool raw_only) {
     return s;
 }
 
+// Whether every launch that fits with single blocks fits with pairs as well, whose down projection's operand is twice as large: for any
+// number of rows (a batched step has more than k_max + 1) and of heads per attention unit, of which a launch chooses one.
+bool pairs_fit(const FwdParams& P, int g) {
+    FwdParams one = P, two = P;
+    one.op[OP_DOWN].P_row = 1;
+    two.op[OP_DOWN].P_row = 2;
+    for (int rows = 1; rows <= kMaxRows; ++rows)
+        for (int gh = 1; gh <= g; ++gh) {
+            one.att_gh = two.att_gh = gh;
+            if (plan_smem(one, rows, false).ok && !plan_smem(two, rows, false).ok) return false;
+        }
+    return true;
+}
+
 // The operations of one layer, in streaming order, and the LM head: shapes, partitions, offsets.
 void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
     const int d = cfg->d_model, f = cfg->d_ffn, hd = cfg->head_dim;
@@ -242,7 +256,8 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
                 // -> 12.0 us at 9 rows of the 1.5B shape, 19.1 -> 16.5 at 32, 29.1 -> 25.0 at 17 rows of the 3B shape, 7.4 -> 6.5 at 9 of the 0.5B
                 // shape.  A launch in clusters takes 2 us more, so the sums have to be many: 16 K (256 columns x 64 shares) lose 1.6 us of a launch
                 // of 53.5, 133 K (896 x 148) gain 21 of 593.  The blocks of a pair are those of a cluster: an even number of shares, beginning at an
-                // even block; and the operand of both shares has to stay within what the exchange areas take anyway.
+                // even block; the operand of both shares has to stay within what the exchange areas take anyway, and must not cost a number
+                // of rows that single blocks can take (pairs_fit).
                 const int steps = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;
                 const bool pairs = G % 2 == 0 && gu.P_row % 2 == 0 && gu.rot % 2 == 0 && o.T >= 2 && 16 * o.T * gu.P_row >= kPairSums &&
                                    2 * steps * 32 * (rows_max | 1) <= kActSmemMax / 2;
@@ -261,6 +276,11 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
         }
         o.w_off = (ops[i].idx == OP_LM) ? 0 : woff;
         if (ops[i].idx != OP_LM) woff += (unsigned long long)ops[i].N * ops[i].K * 2;
+    }
+    OpDesc& down = P.op[OP_DOWN];
+    if (down.P_row == 2 && !pairs_fit(P, cfg->n_q_heads / cfg->n_kv_heads)) {
+        down.P_row = 1;
+        down.P_k = P.op[OP_GU].P_row;
     }
 }
 

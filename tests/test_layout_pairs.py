@@ -29,3 +29,16 @@ def test_who_takes_pairs(name, k, blocks):
     assert down[2] == (2 if pairs else 1) and down[2] * down[3] == gu[2]
     assert pairs == (name[0] in "ql" and blocks > 100)
     assert layout_check(down, gu, blocks) == OK
+
+
+@pytest.mark.parametrize("d,steps,k", [(1024, 28, 3), (1536, 20, 1), (2048, 12, 2), (1536, 8, 7), (896, 4, 8)])
+def test_pairs_refuse_no_rows(d, steps, k):
+    """A batched step has more rows than a draft of k_max: pairs are taken only where every number of rows fits that single blocks, whose
+    operand is half as large, can take.  147 blocks never work in pairs; the largest share has `steps` column steps there and in 148."""
+    cc = config_from(get_config("qwen1.5b"), k_max=k)
+    cc.d_model, cc.d_ffn = d, 16 * 147 * steps
+    for rows in range(1, 33):
+        (ops1, single), (ops2, pairs) = plan(cc, 147, rows), plan(cc, 148, rows)
+        assert ops1[3][2] == 1 and ops1[2][2] == 147 and ops2[2][2] == 148
+        assert pairs[5] >= single[5], (rows, ops2[3])
+    assert steps > 4 or ops2[3][2] == 2
