@@ -375,6 +375,11 @@ int sdv_debug_layout_check(const int *desc, const int *gu_desc, int n_blocks);
  * memory bytes, 1 if the plan fits. */
 int sdv_debug_plan(const sdv_config *cfg, int n_blocks, int rows, int *out);
 
+/* Host-only: what a block of a pair waits for before it leaves a launch in which a wait was abandoned, when it has sent its SwiGLU
+ * columns in `mine` phases and the other block in `sent`: bit 0: the columns of phase mine - 1 may be on their way; bit 1: those of
+ * phase `mine`, which it never prepared for, as well. */
+int sdv_debug_pair_debt(int mine, int sent);
+
 /* Number of kernels launched by this context since creation. */
 long long sdv_launch_count(const sdv_ctx *ctx);
 

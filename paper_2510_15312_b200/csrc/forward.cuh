@@ -90,6 +90,8 @@ struct Misc {
     NormShape shape[OP_COUNT];
     MmaShape mma[OP_COUNT];
     FwdParams P;          // block-local copy of the launch parameters
+    int pair_sent;        // gate|up phases in which this block has sent its SwiGLU columns to the other one of its pair (written at its end)
+    int pair_abort;       // the other one has abandoned a wait (it says so before it leaves)
 };
 static_assert(sizeof(Misc) <= kMiscSmemBytes, "misc shared memory");
 
@@ -239,10 +241,7 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
         for (uint32_t back = 0; back < nstage && back < issued; ++back) {
             if (slot == 0) { slot = nstage; par ^= 1u; }
             --slot;
-            const uint64_t t0 = global_timer_ns();
-            while (!mbar_try_wait(&misc->full[slot], par)) {
-                if (global_timer_ns() - t0 > P.wait_limit_ns) break;
-            }
+            mbar_drain(&misc->full[slot], par, P.wait_limit_ns);
         }
     }
 }
@@ -712,7 +711,8 @@ __device__ __forceinline__ void epilogue_op(const FwdParams& P, const Part& pt, 
     }
     if (!LM && op == OP_GU) {
         // this warp's SwiGLU columns are written: hand them to the tensor-core thread; the blocks of a pair send each other theirs, which lie
-        // one behind the other in the operand (one copy of some KB; both wait for it, so neither is ahead by more than this)
+        // one behind the other in the operand (one copy of some KB; both wait for it, so neither is ahead by more than this).  They are sent
+        // behind an abandoned wait as well, so that the phases prepared for and the copies sent stay the same number (pair_debt).
         fence_proxy_async_smem();
         const int steps = pt.ntiles / 2, theirs = down.nk - steps;
         if (theirs > 0) {
@@ -1356,6 +1356,20 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
 }
 
 // ------------------------------------------------------------------------------------------
+// Where a wait was abandoned in one of a pair's blocks, nobody may have waited for the other one's last columns: one thread does
+// (bounded), behind a cluster barrier (all that will be sent has been) and in front of another (what this block sent is there as well).
+__device__ __noinline__ void drain_pair(const FwdParams& P, Misc* misc) {   // out of the way: never reached in a healthy run
+    const int mine = misc->pair_sent, sent = (int)ld_cluster_u32(map_shared_rank(smem_u32(&misc->pair_sent), cluster_rank() ^ 1u));
+    const int debt = pair_debt(mine, sent);
+    if ((debt & PAIR_LAST) && !mbar_drain(&misc->act_ready, (uint32_t)(mine - 1) & 1u, P.wait_limit_ns)) return;
+    if (debt & PAIR_NEXT) {
+        mbar_arrive_expect_tx(&misc->act_ready, (uint32_t)(misc->part[OP_DOWN].nk - misc->part[OP_GU].ntiles / 2) * operand_off(2, 0, operand_rows(P, P.M, 1)));
+        for (int w = 1; w < kEpilogueWarps; ++w) mbar_arrive(&misc->act_ready);
+        mbar_drain(&misc->act_ready, (uint32_t)mine & 1u, P.wait_limit_ns);
+    }
+}
+
+// ------------------------------------------------------------------------------------------
 // HD: head dimension; MODE: chain, tree or batch (see attention_unit), or 3: the stand-alone GEMM alone (a launch of its own).
 template <int HD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_constant__ FwdParams Pg, const __grid_constant__ DraftArg draft) {
@@ -1403,6 +1417,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         mbar_init(&misc->done_bar, 1);
         misc->abort_flag = 0;
         misc->skip = 0;
+        misc->pair_abort = 0;
         for (int r = 0; r < kMaxRows; ++r) misc->sumsq[0][r] = 0.f;
         mbar_fence_init();
     }
@@ -1438,17 +1453,22 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     }
     __syncthreads();
     if (MODE != 3) cluster_wait();
-    // a block leaves once the other one of its pair no longer copies from or to it
-    auto finish = [&]() {
-        if (MODE != 3) {
-            __syncwarp();
-            cluster_sync();
-        }
+    // A block leaves once the other one of its pair no longer copies from or to it.  Where no wait was abandoned in either, each has waited for the
+    // other's columns before it gets here; otherwise they are waited for now.
+    const bool paired = MODE != 3 && P.op[OP_DOWN].P_row == 2;
+    auto finish = [&](bool worker) {
+        if (MODE == 3) return;
+        __syncwarp();
+        cluster_sync();
+        if (!paired || (*(volatile int*)&misc->abort_flag | *(volatile int*)&misc->pair_abort) == 0) return;
+        if (worker && tid == 0) drain_pair(P, misc);
+        __syncwarp();
+        cluster_sync();
     };
 
     if (warp == kProducerWarp) {
         if (lane == 0) producer_loop(P, smem, misc);
-        finish();
+        finish(false);
         return;
     }
     if (warp == kMmaWarp) {
@@ -1458,7 +1478,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         named_bar_sync(3, kWorkerThreads + 32);   // the workers have read the last accumulators
         tc_fence_after();
         tmem_dealloc(misc->tmem_base, kTmemCols);
-        finish();
+        finish(false);
         return;
     }
 
@@ -1530,10 +1550,19 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     }
     tc_fence_before();
     named_bar_sync(3, kWorkerThreads + 32);
-    if (*(volatile int*)&misc->abort_flag) {
-        if (wtid == 0) atomicExch(P.state + ST_ERR, 1);
+    if (wtid == 0 && paired) {
+        // gate|up is a layer's last phase and a phase is skipped only where all behind it are: whole layers, by the accumulator passes of this block
+        int per_layer = 0;
+        for (int op = OP_QKV; op <= OP_DOWN; ++op) per_layer += misc->part[op].npass;
+        misc->pair_sent = P.ph_begin == 0 && misc->part[OP_DOWN].nk > 0 ? min(n_layers, (int)pos.q / per_layer) : 0;
     }
-    finish();
+    if (*(volatile int*)&misc->abort_flag) {   // final by now: the tensor-core thread is done, so the streamer is or was told
+        if (wtid == 0) {
+            atomicExch(P.state + ST_ERR, 1);
+            if (paired) st_cluster_u32(map_shared_rank(smem_u32(&misc->pair_abort), cluster_rank() ^ 1u), 1u);
+        }
+    }
+    finish(true);
 }
 
 }  // namespace sdv

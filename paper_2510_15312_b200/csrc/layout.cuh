@@ -180,6 +180,17 @@ __host__ __device__ inline unsigned long long weight_offset(const OpDesc& o, con
     return stage_base + in_stage;
 }
 
+// What a block of a pair that may have abandoned a wait still has to see arrive before it leaves.  `mine`, `sent`: gate|up phases in which
+// this block and the other one have sent their SwiGLU columns.  A phase is prepared for (bytes expected, all warps arrive) exactly where its columns
+// are sent, and entered only once the phase before is over in the same block, so the two differ by one at most:
+//   sent = mine - 1: the other block never sent the last phase's; those before have been waited for.
+//   sent = mine:     the last phase's may be on their way (PAIR_LAST).
+//   sent = mine + 1: the same, and those of a phase this block never prepared for (PAIR_NEXT).
+enum PairDebt { PAIR_NONE = 0, PAIR_LAST = 1, PAIR_NEXT = 2 };
+__host__ __device__ inline int pair_debt(int mine, int sent) {
+    return (mine > 0 && sent >= mine ? PAIR_LAST : PAIR_NONE) | (sent > mine ? PAIR_NEXT : PAIR_NONE);
+}
+
 // Device state block (int32 words).
 enum StateWord {
     ST_KV_LEN = 0, ST_HIST_LEN, ST_N_CTX, ST_PENDING, ST_DRAFT_LEN, ST_ACCEPT_LEN, ST_N_EMITTED, ST_ERR,

@@ -1853,6 +1853,8 @@ int sdv_debug_plan(const sdv_config* cfg, int G, int rows, int* out) {
     return SDV_OK;
 }
 
+int sdv_debug_pair_debt(int mine, int sent) { return mine < 0 || sent < 0 ? SDV_EINVAL : pair_debt(mine, sent); }
+
 int sdv_debug_timeout_probe(sdv_ctx* ctx) {
     if (!ctx) return SDV_EINVAL;
     timeout_probe_kernel<<<1, 1, 0, ctx->stream>>>(ctx->P.state, (const int*)(ctx->ws + ctx->r.never), 5000000ull);
