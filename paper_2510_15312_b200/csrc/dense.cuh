@@ -739,6 +739,7 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
     }
     __syncwarp();
     const bool got = mbar_wait_bounded(&ctl->in_full, 0, &ctl->abort_flag, wait_limit_ns);
+    if (!got) mbar_drain(&ctl->in_full, 0, wait_limit_ns);   // a wait was given up, but the others send all the same: not into a block that has left
     __syncwarp();
     cluster_arrive();   // what was sent to this block has left its senders
     if (got) {
