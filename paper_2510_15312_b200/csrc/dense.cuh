@@ -145,14 +145,11 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     if (++s == S::kStages) { s = 0; par ^= 1u; }
                 }
             }
-            if (!ok && rank == 0) {
-                // abandoned: wait (bounded) for the copies still in flight before the pair may exit
-                for (uint32_t back = 0; back < S::kStages && back < issued; ++back) {
-                    if (s == 0) { s = S::kStages; par ^= 1u; }
-                    --s;
-                    const uint64_t t0 = global_timer_ns();
-                    while (!mbar_try_wait(&ctl->full[s], par) && global_timer_ns() - t0 < wait_limit_ns) {}
-                }
+            // the copies still in flight are waited for (bounded) before the pair may exit: where a wait was given up, here or later, nobody else does
+            for (uint32_t back = 0; rank == 0 && back < S::kStages && back < issued; ++back) {
+                if (s == 0) { s = S::kStages; par ^= 1u; }
+                --s;
+                if (!mbar_drain(&ctl->full[s], par, wait_limit_ns)) break;
             }
         }
         __syncwarp();
@@ -552,13 +549,12 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
                 for (int a = 0; a < S::kAtoms; ++a) tma_load_2d(ks + S::kTileBytes + a * 16384, &map_v, a * 64, y, &ctl->vfull[s]);
                 if (++s == S::kStages) { s = 0; par ^= 1u; }
             }
-            if (issued < nblk)   // abandoned: wait (bounded) for the copies still in flight
-                for (int back = 0; back < S::kStages && back < issued; ++back) {
-                    if (s == 0) { s = S::kStages; par ^= 1u; }
-                    --s;
-                    const uint64_t t0 = global_timer_ns();
-                    while (!(mbar_try_wait(&ctl->kfull[s], par) && mbar_try_wait(&ctl->vfull[s], par)) && global_timer_ns() - t0 < wait_limit_ns) {}
-                }
+            // the copies still in flight are waited for (bounded): where a wait was given up, here or later, nobody else does
+            for (int back = 0; back < S::kStages && back < issued; ++back) {
+                if (s == 0) { s = S::kStages; par ^= 1u; }
+                --s;
+                if (!(mbar_drain(&ctl->kfull[s], par, wait_limit_ns) && mbar_drain(&ctl->vfull[s], par, wait_limit_ns))) break;
+            }
         }
         __syncwarp();
     } else if (warp == 9) {

@@ -236,13 +236,11 @@ __device__ __forceinline__ void producer_loop(const FwdParams& P, uint8_t* smem,
             }
         }
     }
-    if (!ok) {
-        // Abandoned: wait (bounded) for the copies still in flight before the block may exit.
-        for (uint32_t back = 0; back < nstage && back < issued; ++back) {
-            if (slot == 0) { slot = nstage; par ^= 1u; }
-            --slot;
-            mbar_drain(&misc->full[slot], par, P.wait_limit_ns);
-        }
+    // The copies still in flight are waited for (bounded) before the block may exit: where a wait was given up, here or later, nobody else does.
+    for (uint32_t back = 0; back < nstage && back < issued; ++back) {
+        if (slot == 0) { slot = nstage; par ^= 1u; }
+        --slot;
+        if (!mbar_drain(&misc->full[slot], par, P.wait_limit_ns)) break;
     }
 }
 

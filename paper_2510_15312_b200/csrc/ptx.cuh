@@ -80,8 +80,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     return true;
 }
 
-// Waits for the phase whatever the abort flag says, but no longer than limit_ns: copies in flight after a wait was abandoned.
+// Waits for the phase whatever the abort flag says, but no longer than limit_ns: copies in flight that nobody else may wait for.
 __device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
+    if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = global_timer_ns();
     while (!mbar_try_wait(bar, parity))
         if (global_timer_ns() - t0 > limit_ns) return false;
