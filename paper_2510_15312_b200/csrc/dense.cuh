@@ -154,7 +154,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (rank == 0) {
+        if (rank == 0 && elect_one()) {   // one thread: lanes that a bounded wait lets go at different times could not issue together
             const uint32_t idesc = umma_idesc_bf16(256u, (uint32_t)BN);
             uint32_t s = 0, par = 0, q = 0;
             bool ok = true;
@@ -170,19 +170,16 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     tc_fence_after();
                     const uint32_t a = smem_u32(smem + s * S::kStageBytes);
                     const uint64_t da = umma_desc_sw128(a), db = umma_desc_sw128(a + S::kABytes);
-                    if (elect_one()) {
 #pragma unroll
-                        for (int k4 = 0; k4 < kDenseBK / 16; ++k4)
-                            umma_pair_bf16(d, da + (uint64_t)(2 * k4), db + (uint64_t)(2 * k4), idesc, (uint32_t)(kb | k4));
-                        umma_commit_pair(&ctl->empty[s]);   // the slot is free, in both SMs, once these instructions have read it
-                    }
-                    __syncwarp();
+                    for (int k4 = 0; k4 < kDenseBK / 16; ++k4)
+                        umma_pair_bf16(d, da + (uint64_t)(2 * k4), db + (uint64_t)(2 * k4), idesc, (uint32_t)(kb | k4));
+                    umma_commit_pair(&ctl->empty[s]);   // the slot is free, in both SMs, once these instructions have read it
                     if (++s == S::kStages) { s = 0; par ^= 1u; }
                 }
-                if (ok && elect_one()) umma_commit_pair(&ctl->acc_full[buf]);
-                __syncwarp();
+                if (ok) umma_commit_pair(&ctl->acc_full[buf]);
             }
         }
+        __syncwarp();
     } else {
         // epilogue: warp w reads accumulator lanes 32 * (w % 4) .. + 31 and CW of the columns; a thread owns a token row of
         // them and writes whole 32-byte sectors
