@@ -78,6 +78,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     struct Ctl {
         uint64_t full[S::kStages], empty[S::kStages];  // full: the leading SM's counts both SMs' bytes
         uint64_t acc_full[2], acc_empty[2];            // acc_empty: the leading SM's counts both SMs' epilogue warps
+        uint64_t stopped;                              // behind an abandoned wait: the products issued before it have completed
         uint32_t tmem_base;
         int abort_flag;
     };
@@ -100,6 +101,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             mbar_init(&ctl->acc_full[b], 1);
             mbar_init(&ctl->acc_empty[b], 8 * kHalves);
         }
+        mbar_init(&ctl->stopped, 1);
         ctl->abort_flag = 0;
         mbar_fence_init();
     }
@@ -161,7 +163,8 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             for (int t = t0; t < ntiles && ok; t += npairs, ++q) {
                 const int nkb = even_count(nkb_all, splits, t % splits);
                 const uint32_t buf = q & 1u;
-                if (!mbar_wait_bounded(&ctl->acc_empty[buf], ((q >> 1) & 1u) ^ 1u, &ctl->abort_flag, wait_limit_ns)) break;
+                ok = mbar_wait_bounded(&ctl->acc_empty[buf], ((q >> 1) & 1u) ^ 1u, &ctl->abort_flag, wait_limit_ns);
+                if (!ok) break;
                 tc_fence_after();
                 const uint32_t d = tmem + buf * 256u;
                 for (int kb = 0; kb < nkb; ++kb) {
@@ -177,6 +180,10 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     if (++s == S::kStages) { s = 0; par ^= 1u; }
                 }
                 if (ok) umma_commit_pair(&ctl->acc_full[buf]);
+            }
+            if (!ok) {   // tensor and shared memory are given back only when no product uses them any more
+                umma_commit_pair(&ctl->stopped);
+                mbar_drain(&ctl->stopped, 0, wait_limit_ns);
             }
         }
         __syncwarp();
@@ -593,8 +600,10 @@ dense_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
             __syncwarp();
             if (j + 2 < nblk) scores(j + 2);
         }
-        if (ok && elect_one()) umma_commit(&ctl->o_full);
+        // behind an abandoned wait as well: tensor and shared memory are given back only when no product uses them any more
+        if (elect_one()) umma_commit(&ctl->o_full);
         __syncwarp();
+        if (!ok) mbar_drain(&ctl->o_full, 0, wait_limit_ns);
     } else {
         const int w = warp >> 2, t = (warp & 3) * 32 + lane;   // stream, tile row
         const uint32_t ts = tmem + (uint32_t)w * 128u + ((uint32_t)((warp & 3) * 32) << 16), to = ts + 256u;
