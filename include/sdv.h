@@ -375,6 +375,12 @@ int sdv_debug_layout_check(const int *desc, const int *gu_desc, int n_blocks);
  * memory bytes, 1 if the plan fits. */
 int sdv_debug_plan(const sdv_config *cfg, int n_blocks, int rows, int *out);
 
+/* Host-only: the thread blocks a context of this configuration takes on a device of `sms` SMs that holds `clusters` pairs of blocks at once, and
+ * whether they come in pairs. */
+int sdv_debug_grid(const sdv_config *cfg, int sms, int clusters, int *blocks, int *in_pairs);
+/* The same of a context. */
+int sdv_debug_context_grid(const sdv_ctx *ctx, int *blocks, int *in_pairs);
+
 /* Host-only: what a block of a pair waits for before it leaves a launch in which a wait was abandoned, when it has sent its SwiGLU
  * columns in `mine` phases and the other block in `sent`: bit 0: the columns of phase mine - 1 may be on their way; bit 1: those of
  * phase `mine`, which it never prepared for, as well. */

@@ -19,7 +19,7 @@ EXPORTS = [
     "sdv_strerror", "sdv_last_cuda_error", "sdv_step_bytes", "sdv_debug_set_history", "sdv_debug_accept",
     "sdv_debug_force_commit", "sdv_debug_read_kv", "sdv_debug_read_hidden", "sdv_debug_gemm",
     "sdv_debug_timeout_probe", "sdv_debug_profile", "sdv_launch_count", "sdv_last_verify_ms",
-    "sdv_gemm_noalloc", "sdv_debug_layout_check", "sdv_debug_plan", "sdv_debug_pair_debt",
+    "sdv_gemm_noalloc", "sdv_debug_layout_check", "sdv_debug_plan", "sdv_debug_pair_debt", "sdv_debug_grid", "sdv_debug_context_grid",
     "sdv_set_calibration", "sdv_get_calibration", "sdv_draft_tree", "sdv_verify_tree", "sdv_debug_force_commit_tree",
     "sdv_debug_top_successors",
     "sdv_follower_workspace_bytes", "sdv_create_follower", "sdv_verify_batch", "sdv_get_verified",
@@ -105,6 +105,8 @@ def load_library(path: Optional[str] = None):
     L.sdv_gemm_noalloc.argtypes = [vp, vp, vp, C.c_int, C.c_int, C.c_int, vp]
     L.sdv_debug_layout_check.argtypes = [C.POINTER(C.c_int), C.POINTER(C.c_int), C.c_int]
     L.sdv_debug_plan.argtypes = [C.POINTER(SdvConfig), C.c_int, C.c_int, C.POINTER(C.c_int)]
+    L.sdv_debug_grid.argtypes = [C.POINTER(SdvConfig), C.c_int, C.c_int, ip, ip]
+    L.sdv_debug_context_grid.argtypes = [vp, ip, ip]
     L.sdv_debug_pair_debt.argtypes = [C.c_int, C.c_int]
     L.sdv_set_calibration.argtypes = [vp, C.c_int]
     L.sdv_get_calibration.argtypes = [vp, vp, vp, C.c_int]
@@ -452,6 +454,12 @@ class Sdv:
             raise SdvError(rc, "sdv_debug_profile")
         return out
 
+    def debug_grid(self) -> Tuple[int, bool]:
+        """(thread blocks of a launch, whether they come in pairs)."""
+        g, p = C.c_int(), C.c_int()
+        self._check(lib().sdv_debug_context_grid(self._h, C.byref(g), C.byref(p)), "sdv_debug_context_grid")
+        return g.value, bool(p.value)
+
     def debug_timeout_probe(self) -> int:
         return lib().sdv_debug_timeout_probe(self._h)
 
@@ -471,6 +479,15 @@ def plan(cconfig: SdvConfig, n_blocks: int, rows: int):
         raise SdvError(rc, "sdv_debug_plan")
     v = list(out)
     return [v[i * 8:(i + 1) * 8] for i in range(5)], v[40:46]
+
+
+def grid(cconfig: SdvConfig, sms: int, clusters: int) -> Tuple[int, bool]:
+    """Host-only: (thread blocks, whether in pairs) on a device of `sms` SMs that holds `clusters` pairs of blocks at once."""
+    g, p = C.c_int(), C.c_int()
+    rc = lib().sdv_debug_grid(C.byref(cconfig), sms, clusters, C.byref(g), C.byref(p))
+    if rc != OK:
+        raise SdvError(rc, "sdv_debug_grid")
+    return g.value, bool(p.value)
 
 
 def pair_debt(mine: int, sent: int) -> int:

@@ -230,8 +230,8 @@ bool pairs_fit(const FwdParams& P, int g) {
     return true;
 }
 
-// The operations of one layer, in streaming order, and the LM head: shapes, partitions, offsets.
-void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
+// The operations of one layer, in streaming order, and the LM head: shapes, partitions, offsets.  may_pair: blocks may come in pairs.
+void setup_ops(FwdParams& P, const sdv_config* cfg, int G, bool may_pair) {
     const int d = cfg->d_model, f = cfg->d_ffn, hd = cfg->head_dim;
     const int nq = cfg->n_q_heads * hd, nkv = cfg->n_kv_heads * hd, nqkv = nq + 2 * nkv;
     struct { int idx, N, K; } ops[5] = {{OP_QKV, nqkv, d}, {OP_O, d, nq}, {OP_GU, 2 * f, d}, {OP_DOWN, d, f},
@@ -259,7 +259,7 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
                 // even block; the operand of both shares has to stay within what the exchange areas take anyway, and must not cost a number
                 // of rows that single blocks can take (pairs_fit).
                 const int steps = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;
-                const bool pairs = G % 2 == 0 && gu.P_row % 2 == 0 && gu.rot % 2 == 0 && o.T >= 2 && 16 * o.T * gu.P_row >= kPairSums &&
+                const bool pairs = may_pair && G % 2 == 0 && gu.P_row % 2 == 0 && gu.rot % 2 == 0 && o.T >= 2 && 16 * o.T * gu.P_row >= kPairSums &&
                                    2 * steps * 32 * (rows_max | 1) <= kActSmemMax / 2;
                 o.P_row = pairs ? 2 : 1;
                 o.P_k = gu.P_row / o.P_row;
@@ -282,6 +282,19 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G) {
         down.P_row = 1;
         down.P_k = P.op[OP_GU].P_row;
     }
+}
+
+// The grid, one persistent block per SM, and its operations.  Pairs of blocks are clusters of one launch, which needs all of them at once: where
+// the device cannot hold them (`clusters_held`: how many it can), or the shape does not take pairs, the blocks are single ones on every SM.
+template <typename F>
+int setup_grid(FwdParams& P, const sdv_config* cfg, int sms, F clusters_held) {
+    const int even = sms & ~1;
+    if (even >= 2) {
+        setup_ops(P, cfg, even, true);
+        if (P.op[OP_DOWN].P_row == 2 ? clusters_held() >= even / 2 : even == sms) return even;
+    }
+    setup_ops(P, cfg, sms, false);
+    return sms;
 }
 
 }  // namespace
@@ -341,14 +354,48 @@ ForwardKernel forward_kernel(const FwdParams& P) {
                                               {sdv_forward_kernel<128, 0>, sdv_forward_kernel<128, 1>, sdv_forward_kernel<128, 2>, sdv_forward_kernel<64, 3>}};
     return table[P.hd == 128][forward_mode(P)];
 }
-cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_t stream) {
-    const ForwardKernel k = forward_kernel(P);
-    static DeviceOnce sized[2][4];   // the kernel may use all shared memory
+// The kernel may use all shared memory (an attribute of each device).
+cudaError_t size_kernel(const FwdParams& P) {
+    static DeviceOnce sized[2][4];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
         e = sized[P.hd == 128][forward_mode(P)].run(
-            dev, [&]() { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget); });
+            dev, [&]() { return cudaFuncSetAttribute(forward_kernel(P), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget); });
+    return e;
+}
+// A launch in pairs of blocks, together on the device where `together`.
+struct PairLaunch {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[2];
+    PairLaunch(const PairLaunch&) = delete;
+    PairLaunch(int G, cudaStream_t stream, bool together) {
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3(G);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = kSmemBudget;
+        cfg.stream = stream;
+        memset(at, 0, sizeof(at));
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeCooperative;
+        at[1].val.cooperative = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = together ? 2 : 1;
+    }
+};
+// Pairs of blocks of the forward kernel that the device holds at once (all its kinds have the same launch shape).
+int pairs_held(const FwdParams& P) {
+    const PairLaunch l(P.G, nullptr, false);
+    int n = 0;
+    if (size_kernel(P) == cudaSuccess && cudaOccupancyMaxActiveClusters(&n, (const void*)forward_kernel(P), &l.cfg) == cudaSuccess) return n;
+    cudaGetLastError();   // not to be reported by the next check: single blocks need no answer
+    return 0;
+}
+cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_t stream) {
+    const ForwardKernel k = forward_kernel(P);
+    const cudaError_t e = size_kernel(P);
     if (e != cudaSuccess) return e;
     DraftArg none;
     none.n = -1;
@@ -361,22 +408,8 @@ cudaError_t launch_kernel(const FwdParams& P, const DraftArg* draft, cudaStream_
         return cudaLaunchKernel((const void*)k, dim3(P.G), dim3(kThreads), args, kSmemBudget, stream);
     }
     // pairs of blocks share the down projection
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(P.G);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBudget;
-    cfg.stream = stream;
-    cudaLaunchAttribute at[2];
-    memset(at, 0, sizeof(at));
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeCooperative;
-    at[1].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = P.ph_end - P.ph_begin > 1 ? 2 : 1;
-    return cudaLaunchKernelExC(&cfg, (const void*)k, args);
+    const PairLaunch l(P.G, stream, P.ph_end - P.ph_begin > 1);
+    return cudaLaunchKernelExC(&l.cfg, (const void*)k, args);
 }
 
 bool apply_plan(FwdParams& P, int rows, bool raw_only) {
@@ -766,11 +799,6 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
         return SDV_ECUDA;
     }
     if (sms > kMaxGrid) sms = kMaxGrid;
-    ctx->G = sms & ~1;  // one persistent block per SM, in pairs
-    if (ctx->G < 2) {
-        delete ctx;
-        return SDV_ECUDA;
-    }
     ctx->r = carve(cfg, leader == nullptr);
     // every failure below leaves through this: what was created so far is released
     auto fail = [&](int code) {
@@ -792,8 +820,13 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
     P.V = cfg->vocab; P.max_seq = cfg->max_seq; P.g = cfg->n_q_heads / cfg->n_kv_heads; P.n_qkv = nqkv;
     P.eps = cfg->rms_eps;
     P.scale_log2e = (float)((1.0 / sqrt((double)hd)) * 1.4426950408889634);
+    if (leader) {  // its weights are laid out for its grid
+        ctx->G = leader->G;
+        memcpy(P.op, leader->P.op, sizeof(P.op));
+    } else {
+        ctx->G = setup_grid(P, cfg, sms, [&]() { P.G = sms & ~1; return pairs_held(P); });
+    }
     P.G = ctx->G;
-    setup_ops(P, cfg, ctx->G);
     const int rows_max = cfg->k_max + 1;
     P.layer_stride = ctx->r.layer_stride;
     uint8_t* ws = ctx->ws;
@@ -867,7 +900,7 @@ int create_context(const sdv_config* cfg, void* dev_workspace, size_t bytes, cud
     if (e != cudaSuccess) return fail(SDV_ECUDA);
     // dense prefill path: tensor maps over its activation buffers and its weight copies
     ctx->maps = new (std::nothrow) std::vector<CUtensorMap>(MAP_LAYERS + 8 * (size_t)cfg->n_layers);
-    ctx->dense_ok = ctx->maps != nullptr && d <= 16384;  // four turns of 1024 threads x 4 columns in the row-wise kernels
+    ctx->dense_ok = ctx->maps != nullptr && ctx->G >= 2 && d <= 16384;  // its products run on pairs of SMs; four turns of 1024 threads x 4 columns in the row-wise kernels
     if (ctx->dense_ok && leader) {  // the weight copies of the dense path are the leader's as well
         ctx->dense_ok = leader->dense_ok;
         if (ctx->dense_ok) *ctx->maps = *leader->maps;
@@ -1842,7 +1875,7 @@ int sdv_debug_plan(const sdv_config* cfg, int G, int rows, int* out) {
     memset(&P, 0, sizeof(P));
     P.d = cfg->d_model;
     P.hd = cfg->head_dim;
-    setup_ops(P, cfg, G);
+    setup_ops(P, cfg, G, true);
     for (int i = 0; i < 5; ++i) {
         const OpDesc& o = P.op[i];
         const int v[8] = {o.T, o.K16, o.P_row, o.P_k, o.RW, o.SK, o.unit, o.follow | (o.slices << 8)};
@@ -1850,6 +1883,24 @@ int sdv_debug_plan(const sdv_config* cfg, int G, int rows, int* out) {
     }
     const SmemPlan sp = plan_smem(P, rows, false);
     out[40] = sp.NG; out[41] = sp.NB; out[42] = sp.nstage; out[43] = sp.u_bytes; out[44] = kSmemBudget; out[45] = sp.ok ? 1 : 0;
+    return SDV_OK;
+}
+
+int sdv_debug_grid(const sdv_config* cfg, int sms, int clusters, int* blocks, int* in_pairs) {
+    if (!config_ok(cfg) || sms < 1 || sms > kMaxGrid || !blocks || !in_pairs) return SDV_EINVAL;
+    FwdParams P;
+    memset(&P, 0, sizeof(P));
+    P.d = cfg->d_model;
+    P.hd = cfg->head_dim;
+    *blocks = setup_grid(P, cfg, sms, [&]() { return clusters; });
+    *in_pairs = P.op[OP_DOWN].P_row == 2 ? 1 : 0;
+    return SDV_OK;
+}
+
+int sdv_debug_context_grid(const sdv_ctx* ctx, int* blocks, int* in_pairs) {
+    if (!ctx || !blocks || !in_pairs) return SDV_EINVAL;
+    *blocks = ctx->G;
+    *in_pairs = ctx->P.op[OP_DOWN].P_row == 2 ? 1 : 0;
     return SDV_OK;
 }
 

@@ -3,7 +3,7 @@ one and of two accumulators, shares that just make pairs, rows on both sides of 
 import pytest
 
 from sdv_inputs import get_config
-from paper_2510_15312_b200.binding import config_from, plan
+from paper_2510_15312_b200.binding import Sdv, config_from, plan
 from test_gpu_shapes import check
 
 pytestmark = pytest.mark.gpu
@@ -19,3 +19,13 @@ def test_verify_and_prefill_tiles_in_pairs(name, over, drafts):
     cfg = get_config(name).with_(chunk=13, **over)     # chunks of 13 rows take the verify kernel without its LM head
     assert plan(config_from(cfg), 148, 1)[0][3][2] == 2
     check(cfg, drafts)
+
+
+def test_a_context_takes_the_pairs_its_plan_has():
+    """The device is asked how many pairs it holds: all of them here, so that no context falls back to single blocks unseen."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for name, over, pairs in (("tiny", dict(d_model=1024, d_ffn=1024), True), ("mini_hd128", dict(d_model=448, d_ffn=7168), True), ("tiny", dict(), False)):
+        s = Sdv(config_from(get_config(name).with_(**over)))
+        assert s.debug_grid() == (sms, pairs)
+        s.close()

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from sdv_inputs import get_config
-from paper_2510_15312_b200.binding import OK, config_from, layout_check, plan
+from paper_2510_15312_b200.binding import OK, config_from, grid, layout_check, plan
 
 
 def test_pairs_cover_each_matrix_once():
@@ -42,3 +42,15 @@ def test_pairs_refuse_no_rows(d, steps, k):
         assert ops1[3][2] == 1 and ops1[2][2] == 147 and ops2[2][2] == 148
         assert pairs[5] >= single[5], (rows, ops2[3])
     assert steps > 4 or ops2[3][2] == 2
+
+
+@pytest.mark.parametrize("sms,clusters,blocks,pairs", [(148, 74, 148, True), (148, 80, 148, True), (148, 73, 148, False), (148, 0, 148, False),
+                                                       (147, 73, 146, True), (147, 72, 147, False)])
+def test_pairs_only_where_the_device_holds_them(sms, clusters, blocks, pairs):
+    """All pairs of a launch have to be on the device at once; single blocks otherwise, on every SM."""
+    assert grid(config_from(get_config("qwen1.5b")), sms, clusters) == (blocks, pairs)
+
+
+@pytest.mark.parametrize("sms", [148, 147, 16, 7, 2, 1])
+def test_single_blocks_take_every_sm(sms):
+    assert grid(config_from(get_config("tiny")), sms, sms // 2) == (sms, False)
