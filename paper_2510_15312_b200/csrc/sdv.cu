@@ -216,8 +216,11 @@ SmemPlan plan_smem(FwdParams& P, int rows, bool raw_only) {
     return s;
 }
 
-// Whether every launch that fits with single blocks fits with pairs as well, whose down projection's operand is twice as large: for any
-// number of rows (a batched step has more than k_max + 1) and of heads per attention unit, of which a launch chooses one.
+// What pairs must not cost, whose down projection's operand is twice as large, for any number of rows (a batched step has more than k_max + 1) and of
+// heads per attention unit, of which a launch chooses one: a launch that fits with single blocks, or the third ring slot.  Two slots hold the stream up:
+// layers of the 7B shape, pairs on two slots against single blocks on three, 16 rows 13 % slower at 256 and 2048 keys and 11 % at 8192, 17 rows 13 and
+// 10 %; at the numbers of rows where they have as many slots the two are within 0.6 %.  A fourth slot is worth less than the pairs mostly give: 3B
+// shape, 15 rows, pairs on three against four 0.7 to 1.1 % faster (14 and 16 rows, as many slots: 2.8 to 4 %); 0.5B, 32 rows, four against five 5.3 to 5.5 %.
 bool pairs_fit(const FwdParams& P, int g) {
     FwdParams one = P, two = P;
     one.op[OP_DOWN].P_row = 1;
@@ -225,7 +228,8 @@ bool pairs_fit(const FwdParams& P, int g) {
     for (int rows = 1; rows <= kMaxRows; ++rows)
         for (int gh = 1; gh <= g; ++gh) {
             one.att_gh = two.att_gh = gh;
-            if (plan_smem(one, rows, false).ok && !plan_smem(two, rows, false).ok) return false;
+            const SmemPlan a = plan_smem(one, rows, false), b = plan_smem(two, rows, false);
+            if ((a.ok && !b.ok) || (a.nstage >= 3 && b.nstage < 3)) return false;
         }
     return true;
 }
@@ -256,8 +260,8 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G, bool may_pair) {
                 // -> 12.0 us at 9 rows of the 1.5B shape, 19.1 -> 16.5 at 32, 29.1 -> 25.0 at 17 rows of the 3B shape, 7.4 -> 6.5 at 9 of the 0.5B
                 // shape.  A launch in clusters takes 2 us more, so the sums have to be many: 16 K (256 columns x 64 shares) lose 1.6 us of a launch
                 // of 53.5, 133 K (896 x 148) gain 21 of 593.  The blocks of a pair are those of a cluster: an even number of shares, beginning at an
-                // even block; the operand of both shares has to stay within what the exchange areas take anyway, and must not cost a number
-                // of rows that single blocks can take (pairs_fit).
+                // even block; the operand of both shares takes half of kActSmemMax at most, and must not cost a number of rows that single blocks
+                // can take, nor the third ring slot (pairs_fit).
                 const int steps = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;
                 const bool pairs = may_pair && G % 2 == 0 && gu.P_row % 2 == 0 && gu.rot % 2 == 0 && o.T >= 2 && 16 * o.T * gu.P_row >= kPairSums &&
                                    2 * steps * 32 * (rows_max | 1) <= kActSmemMax / 2;

@@ -25,6 +25,9 @@ def test_who_takes_pairs(name, k, blocks):
     """Pairs where the shares are even in number and their partial sums many; single blocks otherwise; either covers the matrix."""
     ops, sp = plan(config_from(get_config(name), k_max=k), blocks, 1)
     gu, down = ops[2], ops[3]
+    if name == "qwen7b":   # pairs would leave it two ring slots at 16 and 17 rows (below)
+        assert down[2] == 1 and down[3] == gu[2] and layout_check(down, gu, blocks) == OK
+        return
     pairs = blocks % 2 == 0 and gu[2] % 2 == 0 and 16 * down[0] * gu[2] >= 65536
     assert down[2] == (2 if pairs else 1) and down[2] * down[3] == gu[2]
     assert pairs == (name[0] in "ql" and blocks > 100)
@@ -42,6 +45,17 @@ def test_pairs_refuse_no_rows(d, steps, k):
         assert ops1[3][2] == 1 and ops1[2][2] == 147 and ops2[2][2] == 148
         assert pairs[5] >= single[5], (rows, ops2[3])
     assert steps > 4 or ops2[3][2] == 2
+
+
+@pytest.mark.parametrize("k", [4, 16, 20])
+def test_pairs_cost_no_third_ring_slot(k):
+    """The 7B shape, whose layers HBM bounds: 16 and 17 rows have three ring slots with single blocks and would have two with pairs.  (147
+    blocks never work in pairs; their largest shares are those of 148 to the column step.)"""
+    cc = config_from(get_config("qwen7b"), k_max=k)
+    for rows in range(1, 33):
+        (_, single), (ops, taken) = plan(cc, 147, rows), plan(cc, 148, rows)
+        assert ops[3][2] == 1 and min(taken[2], 3) >= min(single[2], 3), rows
+        assert taken[2] >= 3 or rows > 17
 
 
 @pytest.mark.parametrize("sms,clusters,blocks,pairs", [(148, 74, 148, True), (148, 80, 148, True), (148, 73, 148, False), (148, 0, 148, False),
