@@ -57,3 +57,16 @@ def test_no_cpu_fallback_without_gpu():
     good = SdvConfig(2, 256, 4, 4, 64, 1024, 4096, 600, 4, 0, 0, 3, 1, 0, 1e4, 1e-6)
     with pytest.raises(pkg.SdvError):
         Sdv(good)
+
+
+def test_current_stream_without_torchs_private_function(monkeypatch):
+    """The stand-alone GEMM's shortcut to the stream's handle may be missing from a torch: the public way then."""
+    import types
+    import torch
+    from paper_2510_15312_b200 import binding
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 1000 + device, raising=False)
+    assert binding._current_stream_handle(torch) == 1003
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert binding._current_stream_handle(torch) == 77
