@@ -40,7 +40,7 @@ constexpr int kMaxSplits = 40;                         // key ranges per head at
 constexpr int kSmemBudget = 232448;                    // 227 KB
 constexpr int kKeyChunk = 128;                         // keys per attention chunk: the rows of a tensor-core instruction
 constexpr int kAttnBytesPerDim = 640;                  // attention tiles: 64 query rows, a chunk of keys and of values; bytes per column of a head
-constexpr int kActSmemMax = 32768;                     // SwiGLU output of this block (operand of its down-projection slice) at most
+constexpr int kActSmemMax = 32768;                     // operand of a block's share of the down projection at most: its SwiGLU output, in pairs that of both blocks
 constexpr int kPairSums = 65536;                       // partial sums per row from which on pairs of blocks share the down projection
 constexpr int kMiscSmemBytes = 4096;
 constexpr int kMiscOff = kSmemBudget - kMiscSmemBytes;  // bookkeeping lies behind everything else, at the same place whatever the rows

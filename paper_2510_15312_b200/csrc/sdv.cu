@@ -542,7 +542,7 @@ int commit_common(sdv_ctx* ctx, int max_emit, int force_accept, int force_token,
         ctx->launches++;
         ctx->tree_verified = false;
     }
-    commit_kernel<<<1, 64, 0, ctx->stream>>>(ctx->P.state, hist, max_emit, force_accept, force_token, 0, ctx->pinned);
+    commit_kernel<<<1, 64, 0, ctx->stream>>>(ctx->P.state, hist, max_emit, force_accept, force_token, ctx->pinned);
     ctx->launches++;
     CK(cudaGetLastError());
     int rc = read_state(ctx, true);
@@ -1201,7 +1201,7 @@ int sdv_verify(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, int32_t* 
     int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, tree, nullptr, false, nullptr,
                             pass ? &a : nullptr);
     if (rc) return rc;
-    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0,
+    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0,
                                                     fetch ? ctx->pinned : nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
@@ -1335,7 +1335,7 @@ int sdv_extension_update(sdv_ctx* ctx, int max_life, int32_t* host_segment, int*
     if (!ctx || max_life < 1) return SDV_EINVAL;
     if (ctx->poisoned) return SDV_ETIMEOUT;
     if (!ctx->verified) return SDV_ESTATE;
-    extension_update_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, max_life, 0);
+    extension_update_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, max_life);
     ctx->launches++;
     CK(cudaGetLastError());
     if (host_segment || segment_len || lifetime) {
@@ -1556,7 +1556,7 @@ int sdv_verify_tree(sdv_ctx* ctx, const int32_t* host_tokens, const int32_t* hos
     int rc = launch_forward(ctx, rows, ctx->kv_len, 0, 0, 2 + kPhasesPerLayer * c.n_layers, true, false, true);
     if (rc) return rc;
     const bool fetch = host_y || host_path || path_len;
-    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0, 0, nullptr, 0,
+    accept_kernel<<<1, 32 * rows, 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 0,
                                                     fetch ? ctx->pinned : nullptr);
     ctx->launches++;
     CK(cudaGetLastError());
@@ -1705,7 +1705,7 @@ int sdv_debug_accept(sdv_ctx* ctx, const int32_t* host_draft, int draft_len, con
         ctx->launches++;
     }
     set_y_kernel<<<1, 32, 0, ctx->stream>>>(ctx->P.state, y);
-    accept_kernel<<<1, 32 * (draft_len + 1), 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 1, 0, nullptr, 0, nullptr);
+    accept_kernel<<<1, 32 * (draft_len + 1), 0, ctx->stream>>>(ctx->P.state, ctx->P.cand_val, ctx->P.cand_idx, ctx->G, 1, nullptr);
     ctx->launches += 2;
     CK(cudaGetLastError());
     ctx->verified = true;

@@ -407,17 +407,16 @@ __device__ __forceinline__ void extension_update_body(int* state, int max_life) 
         state[ST_SEG_USED] = 0;
     }
 }
-__global__ void extension_update_kernel(int* state, int max_life, int in_run) {
-    if (in_run && state[ST_BUDGET] == 0) return;
+__global__ void extension_update_kernel(int* state, int max_life) {
     extension_update_body(state, max_life);
 }
 
 // ------------------------------------------------------------------------------------------
 // Greedy tokens and accept scan.  Row j's token is the best of the per-block candidates
 // (largest logit, lowest id among equals); a = number of leading drafts equal to the model's
-// prediction; emitted = x_1..x_a, y_{a+1}.  One block of 32 * rows threads: warp j reduces row j.
+// prediction; emitted = x_1..x_a, y_{a+1}.  One block of 32 * rows threads at least: warp j reduces row j.
 // `row0`: the sequence's first row among the launch's rows (0 unless the step was batched); `launch_state`:
-// the state block the launch ran on when it is not `state` itself, whose error word is carried over.
+// the state block the launch ran on when it is not `state` itself, whose error word is carried over; `rows`: its rows at most.
 __device__ __forceinline__ void accept_body(int* state, const float* cand_val, const int* cand_idx, int G, int from_host_y,
                                             int row0, const int* launch_state, int rows) {
     __shared__ int y_s[kMaxRows + 1];
@@ -482,10 +481,8 @@ __device__ __forceinline__ void accept_body(int* state, const float* cand_val, c
         state[ST_VERIFIED] = 1;
     }
 }
-__global__ void accept_kernel(int* state, const float* cand_val, const int* cand_idx, int G, int from_host_y, int row0,
-                              const int* launch_state, int in_run, int* host) {
-    if (in_run && state[ST_BUDGET] == 0) return;
-    with_state(state, host, [&](int* st) { accept_body(st, cand_val, cand_idx, G, from_host_y, row0, launch_state, (int)(blockDim.x >> 5)); });
+__global__ void accept_kernel(int* state, const float* cand_val, const int* cand_idx, int G, int from_host_y, int* host) {
+    with_state(state, host, [&](int* st) { accept_body(st, cand_val, cand_idx, G, from_host_y, 0, nullptr, (int)(blockDim.x >> 5)); });
 }
 
 // The accept scans of a batched step, a block per sequence (as many launches took 8 us each).
@@ -555,8 +552,8 @@ __device__ __forceinline__ void commit_body(int* state, int* hist, int max_emit,
     state[ST_VERIFIED] = 0;
     state[ST_TREE_ON] = 0;
 }
-__global__ void commit_kernel(int* state, int* hist, int max_emit, int force_accept, int force_token, int in_run, int* host) {
-    with_state(state, host, [&](int* st) { commit_body(st, hist, max_emit, force_accept, force_token, in_run); });
+__global__ void commit_kernel(int* state, int* hist, int max_emit, int force_accept, int force_token, int* host) {
+    with_state(state, host, [&](int* st) { commit_body(st, hist, max_emit, force_accept, force_token, 0); });
 }
 
 // Everything between two forward kernels (of a run of enqueued steps, or of sdv_step), in one launch of 1024 threads: the accept
