@@ -178,3 +178,25 @@ def test_one_call_step_equals_draft_verify_commit(name):
     assert e.value.code == B.EINVAL
     b.close()
     a.close()
+
+
+def test_runs_longer_than_the_page_locked_copy():
+    """A run hands back up to 704 tokens with its state and copies longer ones from the history.  The LM head maps every token's embedding to its
+    successor, so that the stream is known."""
+    cfg = get_config("tiny").with_(n_ctx=40, k=3)
+    w = make_weights(cfg)
+    nxt = np.random.default_rng(3).permutation(cfg.vocab)
+    w.lm_head = np.empty_like(w.emb)
+    w.lm_head[nxt] = w.emb
+    ctx = make_context(cfg)
+    want = [int(ctx[-1])]
+    for _ in range(1002):
+        want.append(int(nxt[want[-1]]))
+    s = Sdv(config_from(cfg, max_seq=cfg.n_ctx + 1100 * (cfg.k + 1)))
+    s.load_weights(w)
+    gpu_prefill(s, ctx, cfg.chunk)
+    for budget in (703, 704, 705, 1000):
+        out, kv = s.decode_steps(cfg.k, budget, max_tokens=budget)
+        assert out == want[2:2 + budget] and kv == cfg.n_ctx + budget
+        s.rollback(cfg.n_ctx)
+    s.close()

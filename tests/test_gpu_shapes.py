@@ -5,7 +5,7 @@ import pytest
 
 from oracle import sdv_oracle as O
 from sdv_inputs import bf16_bits_to_f32, f32_to_bf16_bits, get_config, make_context, make_weights
-from paper_2510_15312_b200.binding import OK, Sdv, config_from, gemm_noalloc
+from paper_2510_15312_b200.binding import OK, Sdv, config_from, gemm_noalloc, plan
 from helpers import COS_TOL, LOGIT_TOL
 
 pytestmark = pytest.mark.gpu
@@ -74,6 +74,15 @@ def test_prefill_and_calibration_at_tile_edges(name, n_ctx, chunk):
 ])
 def test_verify_at_chunk_and_share_edges(name, over, drafts):
     check(get_config(name).with_(**over), drafts)
+
+
+def test_passes_of_nine_and_eight_tiles():
+    """Shares of 17 row tiles are walked in passes of nine and eight: two accumulators and one side by side.  Here the LM head's (half of the blocks;
+    the others have 16 tiles in one pass)."""
+    cfg = get_config("tiny").with_(vocab=16 * (148 * 16 + 74), n_ctx=40, k=16)
+    lm = plan(config_from(cfg), 148, 1)[0][4]
+    assert lm[0] == 148 * 16 + 74 and lm[2] == 148 and lm[4] == 16
+    check(cfg, (0, 8, 16))
 
 
 @pytest.mark.parametrize("M", [1, 8, 9, 16, 17, 24, 25, 32])
