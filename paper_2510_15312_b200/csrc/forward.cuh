@@ -135,18 +135,18 @@ __device__ __forceinline__ bool grid_barrier(const FwdParams& P, unsigned target
 // would idle through the attention half of a layer (24 us) once it is full.  So while the streamer waits for a free slot it reads
 // ahead into L2, at most kLookaheadBytes beyond the ring and no faster than one piece per kLookaheadCycles or kLookaheadSlow
 // (4 or 3 TB/s over the grid if nothing else ran): a burst would queue in front of the other warps' loads, which cost more than it gave, the trickle does not.
-// 10050 -> 9680 us for eight steps of the 1.5B shape, 12130 -> 11970 us for four of the 7B shape; 128 KB: 9720, 256 KB: 9660.
-// The rate, by the time of the forward kernel at 800 cycles over that at 600 (both by turns in one context; a share is what a block streams
-// of a layer, MB of 2^20 bytes):
-//   up to 24 rows, shares up to 2.2 MB: 600.  1.5B shape (0.6 MB) 1.012 to 1.022 at 1 to 13 rows, 3B shape (1.3 MB) 1.012 to 1.022 at 1 to 17, shares
-//     of 1.4 to 1.9 MB 1.007 to 1.015 at 1 to 9 (2048 keys each); 17 to 24 rows and 8192 keys: 0.992 to 1.007.
-//   above 24 rows the operand builds are what a layer waits for: 24 rows 0.997, 25 rows 0.992, 32 rows 0.989 (1.5B shape, 2048 keys); longer
-//     layers (0.99 to 1.3 MB) 0.993 to 1.001 from 2048 keys on, 1.000 to 1.012 below.
-//   shares of 2.5 MB and more: the stream fills HBM, and the loads of the KV rows queue behind a faster trickle.  7B shape (3.0 MB), 1 to 9 rows:
-//     0.988 to 0.997 from 2560 keys on, 0.996 to 1.005 at 2048, 1.003 to 1.009 at 256.  2.5 MB: 0.989 to 0.997 at 8192 keys, 1.000 to 1.004 at
-//     2048.  2.2 MB: 0.998 to 1.002 at 8192, 1.004 to 1.009 at 2048, hence the line between these two.
-// 1100 cycles instead of 800 take up to another 0.6 % off the 7B shape at 8192 keys and 0.4 % off 27 rows of the 1.5B shape, but cost 1 to 3 % in
-// layers of 0.99 to 1.3 MB above 24 rows and about 1 % in long ones up to 2048 keys.
+// Forward kernel without reading ahead, with 128, 256 and 384 KB: 1.5B shape, 9 rows, 2048 keys 956, 925, 905 and 904 us; 12 layers of the 7B
+// shape, 5 rows, 8192 keys 1226, 1216, 1212 and 1209.
+// The rate, by the time of the forward kernel at 800 cycles over that at 600 (by turns in one process, at 2048 | 8192 keys; a share is what a block
+// streams of a layer, MB of 2^20 bytes):
+//   1.5B shape (0.6 MB): 1, 5, 9 and 13 rows 1.013 1.018 1.016 1.018 | 1.008 1.007 0.988 0.990, 17 and 24 rows 1.000 1.002 | 0.981 1.026;
+//     25 and 32 rows, where the operand builds are what a layer waits for, 0.999 0.992 | 1.007 1.015.
+//   3B shape (1.3 MB): 1, 9, 17 and 24 rows 1.010 0.999 1.010 1.013 | 1.000 0.984 0.992 1.004; 25 rows 1.012 | 1.007.
+//   2.2 MB: 1, 5 and 9 rows 1.007 1.009 1.016 | 1.010 1.011 1.009.  2.5 MB: 1.007 0.999 1.004 | 1.004 1.007 1.002.
+//   7B shape (3.0 MB): 1, 5, 9 and 17 rows 1.009 1.008 1.006 1.015 | 1.002 0.998 1.001 1.002, at 256 keys 1.009 1.008 1.008 1.006.
+// The two lines were drawn where layers took longer and the slow rate won by 0.3 to 1.2 % on their far sides.  Now it does so at 25 and 32 rows of the
+// 1.5B shape up to 2048 keys, and costs up to 1.5 % elsewhere beyond them.  1100 cycles: 1.5B shape, 32 rows 0.978 | 0.969 and 25 rows 0.999 | 0.975
+// of the time at 600, 1.02 times at up to 13 rows and 2048 keys; 7B shape 1.000 to 1.016 times.
 struct Lookahead {   // cursor over the block's weight stream: operation by operation, each one contiguous range of bytes
     int ph, oi;
     const uint8_t* src;
@@ -471,7 +471,8 @@ __device__ __forceinline__ void umma_commit_at(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 // One operation; one or (TWO) two 128-row accumulators per pass (where some passes of an operation need the second one, all are given it: its
-// instructions read on behind a shorter pass's rows, inside shared memory, into columns nobody reads).  The token operand is waited
+// instructions read on behind a shorter pass's rows, inside shared memory, into columns nobody reads; only shares of 17 tiles, passes of nine and
+// eight, issue more for it).  The token operand is waited
 // for last, with everything else at hand.  due_slot, due_acc: commits that are due behind the last instructions issued.  False: a
 // wait was abandoned.
 template <bool TWO>

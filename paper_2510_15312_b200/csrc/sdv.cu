@@ -258,8 +258,10 @@ void setup_ops(FwdParams& P, const sdv_config* cfg, int G, bool may_pair) {
                 o.RW = 16; o.SK = kStageBytes / kStepBytes / 16; o.unit = 1; o.follow = 1;
                 // In pairs each block has half of the rows, so half as many partial sums meet in L2, which the phase waits for: gate|up + down 12.6
                 // -> 12.0 us at 9 rows of the 1.5B shape, 19.1 -> 16.5 at 32, 29.1 -> 25.0 at 17 rows of the 3B shape, 7.4 -> 6.5 at 9 of the 0.5B
-                // shape.  A launch in clusters takes 2 us more, so the sums have to be many: 16 K (256 columns x 64 shares) lose 1.6 us of a launch
-                // of 53.5, 133 K (896 x 148) gain 21 of 593.  The blocks of a pair are those of a cluster: an even number of shares, beginning at an
+                // shape.  A launch in clusters takes 2 us more, so the sums have to be many: with two layers 16 K (256 columns x 64 shares) lose 1.6 us of
+                // a launch of 53.5, with 24 layers 133 K (896 x 148) gain 21 of 593.  With 16 layers (5 to 32 rows, 512 keys) all that was tried gains:
+                // above the line, 64 K to 133 K sums, 0.7 to 9.3 %; below it, 32 K to 61 K, 1.3 to 5.9 % and 16 K 0.4 to 1.7 %, so the line is on the
+                // safe side for models of few layers.  The blocks of a pair are those of a cluster: an even number of shares, beginning at an
                 // even block; the operand of both shares takes half of kActSmemMax at most, and must not cost a number of rows that single blocks
                 // can take, nor the third ring slot (pairs_fit).
                 const int steps = (gu.T / gu.unit + gu.P_row - 1) / gu.P_row;
