@@ -90,8 +90,10 @@ struct Misc {
     NormShape shape[OP_COUNT];
     MmaShape mma[OP_COUNT];
     FwdParams P;          // block-local copy of the launch parameters
-    int pair_sent;        // gate|up phases in which this block has sent its SwiGLU columns to the other one of its pair (written at its end)
-    int pair_abort;       // the other one has abandoned a wait (it says so before it leaves)
+    // behind an abandoned wait, blocks of a pair only (leave_pair):
+    int pair_passes;      // accumulator passes this block, which gave up, has gone through
+    int pair_abort;       // the other one gave up; it writes this, and the next two: phases it has sent its columns in, plus one; it has all of ours
+    int pair_theirs, pair_done;
 };
 static_assert(sizeof(Misc) <= kMiscSmemBytes, "misc shared memory");
 
@@ -1355,17 +1357,36 @@ __device__ __forceinline__ void mma_loop(const FwdParams& P, uint8_t* smem, Misc
 }
 
 // ------------------------------------------------------------------------------------------
-// Where a wait was abandoned in one of a pair's blocks, nobody may have waited for the other one's last columns: one thread does
-// (bounded), behind a cluster barrier (all that will be sent has been) and in front of another (what this block sent is there as well).
-__device__ __noinline__ void drain_pair(const FwdParams& P, Misc* misc) {   // out of the way: never reached in a healthy run
-    const int mine = misc->pair_sent, sent = (int)ld_cluster_u32(map_shared_rank(smem_u32(&misc->pair_sent), cluster_rank() ^ 1u));
-    const int debt = pair_debt(mine, sent);
-    if ((debt & PAIR_LAST) && !mbar_drain(&misc->act_ready, (uint32_t)(mine - 1) & 1u, P.wait_limit_ns)) return;
-    if (debt & PAIR_NEXT) {
+// Where a wait was abandoned in one of a pair's blocks, nobody may have waited for the other one's last columns.  One thread of each block gets here,
+// behind a cluster barrier (all that will be sent has been), and keeps its block there: the two tell each other in how many phases they have
+// sent, wait for what they have been sent, and leave once the other one has done so.  Every wait has the usual limit.
+__device__ __noinline__ void leave_pair(const FwdParams& P, Misc* misc) {
+    const uint32_t other = cluster_rank() ^ 1u;
+    auto tell = [&](int* word, uint32_t v) { st_release_cluster_u32(map_shared_rank(smem_u32(word), other), v); };
+    auto hear = [&](int* word) {
+        const uint64_t t0 = global_timer_ns();
+        uint32_t v;
+        while ((v = ld_acquire_cluster_u32(smem_u32(word))) == 0u && global_timer_ns() - t0 < P.wait_limit_ns) {}
+        return v;
+    };
+    // gate|up is a layer's last phase and a phase is skipped only where all behind it are: whole layers
+    int mine = P.ph_begin == 0 && misc->part[OP_DOWN].nk > 0 ? P.n_layers : 0;
+    if (mine > 0 && *(volatile int*)&misc->abort_flag) {
+        int per_layer = 0;
+        for (int op = OP_QKV; op <= OP_DOWN; ++op) per_layer += misc->part[op].npass;
+        mine = min(mine, *(volatile int*)&misc->pair_passes / per_layer);
+    }
+    tell(&misc->pair_theirs, (uint32_t)mine + 1u);
+    const uint32_t theirs = hear(&misc->pair_theirs);
+    const int debt = theirs ? pair_debt(mine, (int)theirs - 1) : PAIR_NONE;
+    const bool last = !(debt & PAIR_LAST) || mbar_drain(&misc->act_ready, (uint32_t)(mine - 1) & 1u, P.wait_limit_ns);
+    if (last && (debt & PAIR_NEXT)) {
         mbar_arrive_expect_tx(&misc->act_ready, (uint32_t)(misc->part[OP_DOWN].nk - misc->part[OP_GU].ntiles / 2) * operand_off(2, 0, operand_rows(P, P.M, 1)));
         for (int w = 1; w < kEpilogueWarps; ++w) mbar_arrive(&misc->act_ready);
         mbar_drain(&misc->act_ready, (uint32_t)mine & 1u, P.wait_limit_ns);
     }
+    tell(&misc->pair_done, 1u);
+    hear(&misc->pair_done);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1416,7 +1437,7 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         mbar_init(&misc->done_bar, 1);
         misc->abort_flag = 0;
         misc->skip = 0;
-        misc->pair_abort = 0;
+        misc->pair_abort = misc->pair_theirs = misc->pair_done = 0;
         for (int r = 0; r < kMaxRows; ++r) misc->sumsq[0][r] = 0.f;
         mbar_fence_init();
     }
@@ -1452,22 +1473,18 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     }
     __syncthreads();
     if (MODE != 3) cluster_wait();
-    // A block leaves once the other one of its pair no longer copies from or to it.  Where no wait was abandoned in either, each has waited for the
-    // other's columns before it gets here; otherwise they are waited for now.
-    const bool paired = MODE != 3 && P.op[OP_DOWN].P_row == 2;
-    auto finish = [&](bool worker) {
-        if (MODE == 3) return;
-        __syncwarp();
-        cluster_sync();
-        if (!paired || (*(volatile int*)&misc->abort_flag | *(volatile int*)&misc->pair_abort) == 0) return;
-        if (worker && tid == 0) drain_pair(P, misc);
-        __syncwarp();
-        cluster_sync();
+    // A block leaves once the other one of its pair no longer copies from or to it: each has waited for the other's columns before it gets here
+    // unless a wait was abandoned, and then one thread stays until they are there.
+    auto finish = [&]() {
+        if (MODE != 3) {
+            __syncwarp();
+            cluster_sync();
+        }
     };
 
     if (warp == kProducerWarp) {
         if (lane == 0) producer_loop(P, smem, misc);
-        finish(false);
+        finish();
         return;
     }
     if (warp == kMmaWarp) {
@@ -1477,7 +1494,8 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
         named_bar_sync(3, kWorkerThreads + 32);   // the workers have read the last accumulators
         tc_fence_after();
         tmem_dealloc(misc->tmem_base, kTmemCols);
-        finish(false);
+        finish();
+        if (MODE != 3 && lane == 0 && P.op[OP_DOWN].P_row == 2 && (*(volatile int*)&misc->abort_flag | *(volatile int*)&misc->pair_abort) != 0) leave_pair(P, misc);
         return;
     }
 
@@ -1549,19 +1567,16 @@ __global__ void __launch_bounds__(kThreads, 1) sdv_forward_kernel(const __grid_c
     }
     tc_fence_before();
     named_bar_sync(3, kWorkerThreads + 32);
-    if (wtid == 0 && paired) {
-        // gate|up is a layer's last phase and a phase is skipped only where all behind it are: whole layers, by the accumulator passes of this block
-        int per_layer = 0;
-        for (int op = OP_QKV; op <= OP_DOWN; ++op) per_layer += misc->part[op].npass;
-        misc->pair_sent = P.ph_begin == 0 && misc->part[OP_DOWN].nk > 0 ? min(n_layers, (int)pos.q / per_layer) : 0;
-    }
     if (*(volatile int*)&misc->abort_flag) {   // final by now: the tensor-core thread is done, so the streamer is or was told
         if (wtid == 0) {
             atomicExch(P.state + ST_ERR, 1);
-            if (paired) st_cluster_u32(map_shared_rank(smem_u32(&misc->pair_abort), cluster_rank() ^ 1u), 1u);
+            if (MODE != 3 && P.op[OP_DOWN].P_row == 2) {
+                misc->pair_passes = (int)pos.q;
+                st_release_cluster_u32(map_shared_rank(smem_u32(&misc->pair_abort), cluster_rank() ^ 1u), 1u);
+            }
         }
     }
-    finish(true);
+    finish();
 }
 
 }  // namespace sdv

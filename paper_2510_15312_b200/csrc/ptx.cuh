@@ -265,10 +265,11 @@ __device__ __forceinline__ void bulk_s2cluster(uint32_t dst, uint32_t src, uint3
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
+// A word handed to another block of the cluster, and read where it was handed to.
+__device__ __forceinline__ void st_release_cluster_u32(uint32_t addr, uint32_t v) { asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ uint32_t ld_acquire_cluster_u32(uint32_t addr) {
     uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ float ld_cluster_f1(uint32_t addr) {

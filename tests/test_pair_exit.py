@@ -75,7 +75,7 @@ def act_out(rng, drains):
                 while not me.bar.over(me.mine):
                     yield
             me.arrived = LAYERS + 2
-            while other.arrived <= LAYERS + 1:     # second one
+            while other.arrived <= LAYERS + 1:     # until the other one is done waiting too
                 yield
         me.left = True
 
