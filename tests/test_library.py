@@ -64,9 +64,16 @@ def test_current_stream_without_torchs_private_function(monkeypatch):
     import types
     import torch
     from paper_2510_15312_b200 import binding
+
+    def tensor(dtype, size, *shape):
+        return types.SimpleNamespace(is_cuda=True, is_contiguous=lambda: True, dtype=dtype, element_size=lambda: size, shape=shape, data_ptr=lambda: 256)
+
+    x, w, y = tensor(torch.float32, 4, 3, 64), tensor(torch.bfloat16, 2, 16, 64), tensor(torch.float32, 4, 3, 16)
+    monkeypatch.setattr(binding, "lib", lambda: types.SimpleNamespace(sdv_gemm_noalloc=lambda *a: a[-1]))   # hands back the stream
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
     monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 1000 + device, raising=False)
-    assert binding._current_stream_handle(torch) == 1003
+    assert binding.gemm_noalloc(x, w, y) == 1003
     monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
-    assert binding._current_stream_handle(torch) == 77
+    assert binding.gemm_noalloc(x, w, y) == 77
+    assert binding.gemm_noalloc(x, w, y, stream=types.SimpleNamespace(cuda_stream=5)) == 5
