@@ -13,6 +13,16 @@ from paper_2510_15312_b200.binding import Sdv, config_from
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True)
+def nothing_left_to_free():
+    """What earlier tests left in reference cycles (a workspace that the frames of a caught exception hold) is freed here, not inside a measured call."""
+    import gc
+    gc.collect()
+    gc.disable()
+    yield
+    gc.enable()
+
+
 def _case(seed, M, N, K):
     rng = np.random.default_rng(seed)
     x = rng.standard_normal((M, K)).astype(np.float32)
